@@ -13,6 +13,11 @@
  * removes duplicates and tuples already known, and merges the survivors into
  * the full relation (Secs. Sorted-Array Pipeline and Asynchronous Fixpoint
  * Engine).  The loop runs on the device; the host sees only the end result.
+ * TC never changes a tuple's source, so a plain TC query (no flag, device loop,
+ * not profiled) over at most 2^18 vertices runs source by source: each row's
+ * delta and full relation are bit sets in shared memory, and duplicate removal,
+ * set difference and merge are one bit test and set.  The result, iteration
+ * count, per-iteration sizes and candidate count are the same.
  *
  * Conventions for every entry point
  *  - Return value: WG_OK (0) or a negative WG_E_* code.  Nothing aborts, traps
@@ -115,7 +120,8 @@ typedef struct wg_opts {
   uint32_t profile;      /* 1 = time every kernel with CUDA events (forces WG_LOOP_HOST) */
   uint32_t flags;        /* WG_FLAG_* */
   uint64_t reserve_full; /* initial capacity of the full relation, tuples; 0 = auto */
-  uint64_t reserve_cand; /* initial capacity of the candidate buffers, tuples; 0 = auto */
+  uint64_t reserve_cand; /* initial capacity of the candidate buffers, tuples; 0 = auto
+                            (nonzero: the query runs on the pipeline that has them) */
 } wg_opts;
 
 enum wg_state { WG_PENDING = 0, WG_RUNNING = 1, WG_DONE = 2, WG_FAILED = 3 };

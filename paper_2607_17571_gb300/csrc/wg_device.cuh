@@ -232,6 +232,42 @@ struct Dev {
   uint32_t zero_word;                 // always 0 (the largest segment "size" of seg_wide)
 };
 
+// ---------------------------------------------------------------- row fixpoints
+// One relation's row-by-row closure (wg_kern_rows.cu).
+struct RowInst {
+  const uint32_t* off;          // CSR
+  const uint32_t* adj;
+  const void* rec;              // adjacency records, 8 ids per vertex
+  uint32_t* bits;               // row x's bit set: words [x * words, (x + 1) * words)
+  uint32_t* cnt;                // tuples of row x
+  void* out;                    // sorted packed keys
+  unsigned long long out_cap;   // keys `out` holds
+  unsigned long long* log;      // |Delta^0|, |Delta^1|, ... (cleared before the launch)
+  uint32_t nv, w, words, row0;  // words: a multiple of 4; row0: a multiple of kRowChunk
+  uint32_t max_iters, log_cap;
+  uint32_t last;                // last iteration with new tuples
+  uint32_t fits;                // the result fits `out`
+  unsigned long long n_total, cand;
+};
+struct RowCtl {
+  uint32_t next_row, pad;
+};
+// One launch over the rows of one or more instances.
+struct RowJob {
+  RowCtl* ctl;
+  RowInst* inst;
+  const uint32_t* chunk_inst;   // row chunk -> instance (or NULL: instance 0)
+  uint32_t* csum;               // tuples per chunk of kRowChunk rows (cleared before)
+  unsigned long long* cbase;    // their exclusive prefix within the instance
+  void* queue;                  // per-CTA lists of reached vertices, queue_stride ids each
+  uint32_t queue_stride, nrows, vwords, pad;
+};
+constexpr uint32_t kRowChunk = 256;
+constexpr uint32_t kRowQueue = 1024;    // list entries kept in shared memory
+constexpr uint32_t kRecInline = 7;      // neighbours in an adjacency record
+constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
+constexpr uint32_t kRowSmemMax = 200 * 1024;
+
 // Shared-memory index with one pad word per 32: threads that walk their own
 // contiguous run (blocked order, stride 16 words) then hit distinct banks.
 __device__ __forceinline__ uint32_t pad32(uint32_t i) { return i + (i >> 5); }

@@ -309,11 +309,14 @@ struct Relation {
   uint32_t nv = 0, w = 1;
   int kb = 4;
   DBuf keys, off, adj, V;
+  DBuf rec;                       // adjacency records of the row fixpoints (up to kXSegMaxVertices)
   DBuf htab;                      // hash-join ablation: E in a linear-probing table (lazy)
   unsigned long long hmask = 0;
   uint64_t peak_cand = 0, peak_full = 0;  // capacities seen by earlier queries
+  int id_bytes() const { return nv <= 65536u ? 2 : 4; }  // of a rank in rec
   void release(wg_ctx* c) {
     keys.release(c); off.release(c); adj.release(c); V.release(c); htab.release(c);
+    rec.release(c);
   }
 };
 
@@ -337,6 +340,12 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
   launch_csr<K>((const K*)ke.p, ne, R->nv, R->w, (uint32_t*)R->off.p, (uint32_t*)R->adj.p,
                 grid_of(c, 4), c->stream);
   CK(cudaGetLastError());
+  if (R->nv <= kXSegMaxVertices) {
+    TRY(R->rec.get(c, (size_t)R->nv * 8 * R->id_bytes()));
+    launch_row_records((const uint32_t*)R->off.p, (const uint32_t*)R->adj.p, R->nv, R->rec.p,
+                       R->id_bytes(), grid_of(c, 4), c->stream);
+    CK(cudaGetLastError());
+  }
   return WG_OK;
 }
 
@@ -457,6 +466,7 @@ struct EngineBase {
   virtual uint32_t emit_tile() const = 0;
   virtual uint32_t sort_mode() const = 0;
   virtual uint32_t side_mode() const = 0;
+  virtual bool rows() const = 0;
   virtual size_t held() const = 0;       // device bytes of the engine's buffers
   virtual size_t grow_peak() const = 0;  // held() at the peak of the growth the last run asked for
   virtual void release() = 0;
@@ -545,6 +555,13 @@ struct Engine : EngineBase {
   uint32_t emit_tile_;               // merged items per join-emit tile
   uint32_t sort_mode_;               // enum wg_sort_mode (x-grouped engines)
   uint32_t side_;                    // side run of Full: 0 never, 1 with few candidates, 2 always
+  bool rows_ = false;                // row-by-row TC (wg_kern_rows.cu): none of the stages below
+  DBuf row_meta, row_bits, row_queue;
+  RowInst ri{};
+  RowJob job{};
+  size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
+  int id_bytes = 2, g_rows = 0;
+  bool expand_only = false;          // the rows are done; the result waits for a larger buffer
   Engine(wg_ctx* ctx, bool single_, uint32_t n, uint32_t bits, uint32_t logcap, bool fuse_,
          bool xseg_, bool copy_back_ = false, bool hash_join_ = false, uint32_t side = 0)
       : c(ctx), single(single_), fuse(fuse_), xseg(xseg_), n_slots(n), bits_(bits),
@@ -569,6 +586,7 @@ struct Engine : EngineBase {
   uint32_t fuse_tile() const override { return fuse_tile_; }
   uint32_t sort_mode() const override { return sort_mode_; }
   uint32_t side_mode() const override { return side_; }
+  bool rows() const override { return rows_; }
   uint32_t bits() const override { return bits_; }
   uint32_t slots() const override { return n_slots; }
 
@@ -581,7 +599,7 @@ struct Engine : EngineBase {
     ev_done = nullptr;
     DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                    &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b, &xsum_b,
-                   &mix_b, &G[0], &G[1], &xord_b};
+                   &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_queue};
     for (DBuf* b : all) b->release(c);
     capC = capF = capR = capG = 0;
     mix_tiles = 0;
@@ -604,6 +622,11 @@ struct Engine : EngineBase {
         CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
         own_st = true;
       }
+    }
+    if (rows_) {
+      hi.assign(1, Inst{});
+      CK(cudaEventCreateWithFlags(&ev_done, cudaEventDisableTiming));
+      return WG_OK;
     }
     AllocScope scope(c, st);
     TRY(b_dev.get(c, sizeof(Dev)));
@@ -801,6 +824,89 @@ struct Engine : EngineBase {
     return finish(WG_OK);
   }
 
+  // Row-by-row TC: buffers for relation R and a result of wantF keys.  A
+  // result that turns out larger only needs the expansion again (settle).
+  static size_t row_words(uint32_t nv) { return ((size_t)nv + 127) / 128 * 4; }
+  int rows_begin(Relation* Rl, uint32_t max_iters, unsigned long long wantF) {
+    AllocScope scope(c, st);
+    const uint32_t nv = Rl->nv, words = (uint32_t)row_words(nv);
+    const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
+    const uint32_t nlog = std::min<uint32_t>(1u << 16, nv + 2);
+    id_bytes = Rl->id_bytes();
+    g_rows = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(id_bytes, words)),
+                                     std::max<uint32_t>(nv, 1));
+    // control block | chunk sums | log (cleared) | instance | chunk offsets | row counts
+    auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
+    size_t end = 0;
+    const size_t o_ctl = at(end, sizeof(RowCtl)), o_sum = at(end, (size_t)nch * 4),
+                 o_log = at(end, (size_t)nlog * 8);
+    row_clear = end;
+    const size_t o_inst = at(end, sizeof(RowInst)), o_base = at(end, (size_t)nch * 8),
+                 o_cnt = at(end, (size_t)nv * 4);
+    TRY(row_meta.get(c, end));
+    TRY(row_bits.get(c, std::max<size_t>((size_t)nv * words, 1) * 4));
+    TRY(row_queue.get(c, (size_t)g_rows * std::max<uint32_t>(nv, 1) * id_bytes));
+    if (wantF > capF) {
+      TRY(F[0].get(c, wantF * sizeof(K)));
+      capF = wantF;
+    }
+    char* m = (char*)row_meta.p;
+    ri = RowInst{};
+    ri.off = (const uint32_t*)Rl->off.p; ri.adj = (const uint32_t*)Rl->adj.p;
+    ri.rec = Rl->rec.p;
+    ri.bits = (uint32_t*)row_bits.p; ri.cnt = (uint32_t*)(m + o_cnt);
+    ri.log = (unsigned long long*)(m + o_log);
+    ri.nv = nv; ri.w = Rl->w; ri.words = words;
+    ri.max_iters = max_iters; ri.log_cap = nlog;
+    job = RowJob{};
+    job.ctl = (RowCtl*)(m + o_ctl); job.inst = (RowInst*)(m + o_inst);
+    job.csum = (uint32_t*)(m + o_sum); job.cbase = (unsigned long long*)(m + o_base);
+    job.queue = row_queue.p; job.queue_stride = std::max<uint32_t>(nv, 1);
+    job.nrows = nv; job.vwords = words;
+    log_cap = nlog;
+    expand_only = false;
+    hi[0] = Inst{};
+    hi[0].state = INST_ACTIVE;
+    hi[0].log = ri.log;
+    return WG_OK;
+  }
+  int rows_launch() {
+    ri.out = F[0].p;
+    ri.out_cap = capF;
+    if (expand_only) ri.fits = 1;
+    CK(cudaMemcpyAsync(job.inst, &ri, sizeof(ri), cudaMemcpyHostToDevice, st));
+    if (!expand_only) {
+      CK(cudaMemsetAsync(row_meta.p, 0, row_clear, st));
+      if (ri.nv) launch_rows(job, id_bytes, g_rows, st);
+      launch_row_plan(job, 1, st);
+      launches_issued += ri.nv ? 2 : 1;
+    }
+    launch_row_expand<K>(job, grid_of(c, 6), st);
+    launches_issued += 1;
+    CK(cudaGetLastError());
+    CK(cudaEventRecord(ev_done, st));
+    in_flight = true;
+    return WG_OK;
+  }
+  int rows_settle(bool* again) {
+    CK(cudaMemcpyAsync(&ri, job.inst, sizeof(ri), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    Inst& I = hi[0];
+    I.n_full = ri.n_total;
+    I.cand_total = ri.cand;
+    if (!ri.fits) {
+      h.ctl.need_full = ri.n_total;
+      ++regrows;
+      *again = true;
+      expand_only = true;
+      return grow();
+    }
+    const bool capped = ri.last >= ri.max_iters;
+    I.iters_done = capped ? ri.max_iters : ri.last + 1;
+    I.state = capped ? INST_ITERCAP : INST_DONE;
+    return WG_OK;
+  }
+
   // The kernels of one semi-naive iteration (Secs. Per-Iteration Pipeline and
   // Fused Deduplication): join count -> plan -> join emit -> radix histogram ->
   // radix passes -> fused dedup + set difference -> plan (termination) -> merge.
@@ -985,6 +1091,7 @@ struct Engine : EngineBase {
   // iteration (WG_LOOP_HOST) or one per stage (WG_LOOP_HOST_STAGED).
   uint64_t host_syncs = 0;
   int launch(uint32_t budget, int mode) {
+    if (rows_) return rows_launch();
     TRY(put_passes());
     if (mode != WG_LOOP_DEVICE) {
       TRY(put_ctl(budget, false));
@@ -1016,6 +1123,7 @@ struct Engine : EngineBase {
   int settle(bool* again) {
     *again = false;
     in_flight = false;
+    if (rows_) return rows_settle(again);
     TRY(read_back());
     // kernels actually issued inside the graph: launch_iters iterations
     if (exec && h.use_cond)  // body executions: committed iterations, plus one if it aborted
@@ -1079,12 +1187,21 @@ struct Engine : EngineBase {
   int grow() {
     unsigned long long wc, wf, wr;
     grow_target(&wc, &wf, &wr);
+    if (rows_) {  // the size is exact; the result buffer holds nothing yet: free it first
+      wf = h.ctl.need_full + h.ctl.need_full / 16 + 4096;
+      AllocScope scope(c, st);
+      F[0].release(c);
+      capF = 0;
+      TRY(F[0].get(c, wf * sizeof(K)));
+      capF = wf;
+      return WG_OK;
+    }
     return ensure(wc, wf, wr, true);
   }
   size_t held() const override {
     const DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                          &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b,
-                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b};
+                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_queue};
     size_t b = 0;
     for (const DBuf* x : all) b += x->bytes;
     return b;
@@ -1095,6 +1212,8 @@ struct Engine : EngineBase {
   size_t grow_peak() const override {
     unsigned long long wantC, wantF, wantR;
     grow_target(&wantC, &wantF, &wantR);
+    if (rows_)
+      return held() - F[0].bytes + round_up((h.ctl.need_full + h.ctl.need_full / 16 + 4096) * sizeof(K));
     wantC = std::max<unsigned long long>(wantC, 1ull << 16);
     wantF = std::max<unsigned long long>(wantF, 1ull << 16);
     wantR = single ? 0 : std::max<unsigned long long>(wantR, 1ull << 16);
@@ -1174,16 +1293,18 @@ static void drop_idle_engines(wg_ctx* c, size_t bytes) {
 static EngineBase* new_engine(wg_ctx* c, int kb, bool single, uint32_t slots, uint32_t bits,
                               uint32_t logcap, bool fuse, bool xseg, int* rc,
                               bool copyback = false, bool hashjoin = false, uint32_t side = 0,
-                              cudaStream_t stream = nullptr) {
+                              cudaStream_t stream = nullptr, bool rows = false) {
   EngineBase* e;
   if (kb == 4) {
     auto* x = new Engine<uint32_t>(c, single, slots, bits, logcap, fuse, xseg, copyback, hashjoin,
                                    side);
+    x->rows_ = rows;
     *rc = x->init(stream);
     e = x;
   } else {
     auto* x = new Engine<unsigned long long>(c, single, slots, bits, logcap, fuse, xseg, copyback,
                                              hashjoin, side);
+    x->rows_ = rows;
     *rc = x->init(stream);
     e = x;
   }
@@ -1206,6 +1327,13 @@ static int single_start(wg_ctx* c, Query* q) {
       {q->opts.reserve_cand, Rl->peak_cand, 8ull * Rl->ne + Rl->nv, 1ull << 16});
   const unsigned long long wantF = std::max<unsigned long long>(
       {q->opts.reserve_full, Rl->peak_full, 4ull * Rl->ne, 1ull << 16});
+  if (E->rows_) {
+    TRY(E->rows_begin(Rl, q->opts.max_iters, wantF));
+    CK(cudaEventRecord(q->ev0, c->stream));
+    TRY(E->rows_launch());
+    q->state = WG_RUNNING;
+    return WG_OK;
+  }
   TRY(E->reset_single());
   TRY(E->ensure_nv(Rl->nv));
   TRY(E->ensure(wantC, wantF, 0, false));
@@ -2017,10 +2145,28 @@ static int make_query(wg_ctx* c, int kind, wg_rel edges, const wg_opts* opts, Qu
   return WG_OK;
 }
 
+// Whether query q runs row by row (wg_kern_rows.cu): a TC query that asks for
+// nothing of the sorted-array pipeline (its ablations, the host-driven loops,
+// a per-stage profile, the size of the candidate buffers), over a relation
+// whose bit sets and lists take at most half of the free budget -- the sorted
+// pipeline needs more than twice the result, so whatever fits there fits here.
+static bool row_query(wg_ctx* c, const Query* q) {
+  const Relation* R = q->rel;
+  if (q->kind != WG_TC || q->opts.flags || q->opts.loop != WG_LOOP_DEVICE || q->opts.profile ||
+      q->opts.reserve_cand || R->nv > kXSegMaxVertices)
+    return false;
+  size_t idle = 0;
+  for (auto& e : c->idle) idle += e->held();
+  const uint32_t words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
+  const size_t queue = (size_t)grid_of(c, occupancy_rows(R->id_bytes(), words)) * R->nv * R->id_bytes();
+  return (size_t)R->nv * words * 4 + queue <= (c->budget - c->used + idle) / 2;
+}
+
 // Give query q a single-query engine (an idle one of the same key width, pass
 // plan and stage layout, else a new one) and start its fixpoint.
 static int single_begin(wg_ctx* c, Query* q) {
   Relation* R = q->rel;
+  const bool rows = row_query(c, q);
   const int kind = q->kind;
   const bool fuse = !(q->opts.flags & WG_FLAG_SEPARATE_STAGES);
   const bool full_width = (q->opts.flags & WG_FLAG_FULL_WIDTH) != 0;
@@ -2063,7 +2209,7 @@ static int single_begin(wg_ctx* c, Query* q) {
         c->idle[i]->xgrouped() == xseg && c->idle[i]->copyback() == copyback &&
         c->idle[i]->hashjoin() == hashjoin && c->idle[i]->count_tile() == ct &&
         c->idle[i]->fuse_tile() == ft && c->idle[i]->sort_mode() == c->tune_sort[R->kb == 8] &&
-        c->idle[i]->emit_tile() == et &&
+        c->idle[i]->emit_tile() == et && c->idle[i]->rows() == rows &&
         c->idle[i]->side_mode() == side) {
       q->own = std::move(c->idle[i]);
       c->idle.erase(c->idle.begin() + i);
@@ -2071,7 +2217,7 @@ static int single_begin(wg_ctx* c, Query* q) {
   int rc = WG_OK;
   if (!q->own) {
     EngineBase* e = new_engine(c, R->kb, true, 1, bits, 1u << 16, fuse, xseg, &rc, copyback,
-                               hashjoin, side);
+                               hashjoin, side, nullptr, rows);
     if (!e) return rc;
     q->own.reset(e);
   }

@@ -12,6 +12,7 @@ int set_error(int code, const char* msg);
 struct Stage;
 struct Dev;
 struct Inst;
+struct RowJob;
 
 // sorted-array stages (wg_kern_sort.cu); K = uint32_t or unsigned long long
 template <typename K> void launch_sort_hist(Stage* st, int grid, cudaStream_t s);
@@ -61,6 +62,14 @@ void launch_plan_side(Dev* dv, cudaStream_t s);
 void launch_xseg_build(Dev* dv, cudaStream_t s);
 template <typename K>
 void launch_init_diag(Inst* inst, uint32_t first, uint32_t count, void* dpool, cudaStream_t s);
+
+// row-by-row closure (wg_kern_rows.cu); id_bytes: 2 for at most 2^16 vertices, else 4
+int occupancy_rows(int id_bytes, uint32_t vwords);
+void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s);
+void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
+template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
+void launch_row_records(const uint32_t* off, const uint32_t* adj, uint32_t nv, void* rec,
+                        int id_bytes, int grid, cudaStream_t s);
 
 // relation load and result extraction
 template <typename K>
