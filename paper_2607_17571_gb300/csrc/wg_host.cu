@@ -65,6 +65,7 @@ double now_us() {
 struct Relation;
 struct Query;
 struct EngineBase;
+struct RowLane;
 
 // ------------------------------------------------------------------ context
 struct wg_ctx {
@@ -89,6 +90,7 @@ struct wg_ctx {
   std::vector<uint64_t> completed;                // batch queries finished, not yet taken
   uint64_t excl = 0;  // batch query that runs with the whole budget (0: none), see batch_preempt
   uint64_t solo_run = 0;  // the served request running on a single-query engine (0: none)
+  std::vector<std::unique_ptr<RowLane>> lanes;    // batched row-by-row queries
   // tile shapes engines are built with, per key width (index 0: 4-byte keys,
   // 1: 8-byte); 0 = the compiled default.  Set by wg_autotune / wg_set_tiles.
   uint32_t tune_count[2] = {0, 0}, tune_fuse[2] = {0, 0}, tune_emit[2] = {0, 0};
@@ -105,11 +107,13 @@ struct wg_ctx {
 };
 
 static void drop_idle_engines(wg_ctx* c, size_t bytes);
+static void drop_idle_lanes(wg_ctx* c);
 static int dev_alloc(wg_ctx* c, size_t bytes, void** out, cudaStream_t st) {
   *out = nullptr;
   if (bytes == 0) return WG_OK;
   bytes = round_up(bytes);
   if (c->used + bytes > c->budget) drop_idle_engines(c, bytes);  // unused pools go first
+  if (c->used + bytes > c->budget) drop_idle_lanes(c);
   if (c->used + bytes > c->budget)
     return set_err(WG_E_BUDGET, "allocation of " + std::to_string(bytes) +
                                     " bytes exceeds the memory budget");
@@ -498,6 +502,8 @@ struct Query {
   bool batch = false;
   int bclass = -1;
   uint32_t slot = 0;
+  bool rowb = false;             // batched row by row (see RowLane); bclass is -1
+  bool row_alone = false;        // ... once its result did not fit beside others
   // served through a single-query engine (a large request, see solo_round)
   bool solo = false;
   bool solo_wait = false;        // paused after a growth over the budget
@@ -1558,10 +1564,12 @@ static bool solo_running(wg_ctx* c) {
   auto it = c->queries.find(c->solo_run);
   return it != c->queries.end() && it->second->state == WG_RUNNING;
 }
+static bool lanes_busy(const wg_ctx* c);
+static size_t lanes_held(const wg_ctx* c);
 static bool held_elsewhere(wg_ctx* c, int cls) {
   for (auto& kv : c->batch)
     if (kv.first != cls && kv.second) return true;
-  return solo_running(c);
+  return solo_running(c) || lanes_busy(c);
 }
 
 // Whether the growth engine e's last run asked for could fit the budget once
@@ -1570,7 +1578,7 @@ static bool held_elsewhere(wg_ctx* c, int cls) {
 // engine finished).  When it could not, waiting for them as the exclusive
 // query would only stall every other request before failing.
 static bool growth_could_fit(wg_ctx* c, const EngineBase* e) {
-  size_t others = 0;
+  size_t others = lanes_held(c);
   for (auto& kv : c->batch)
     if (kv.second && kv.second.get() != e) others += kv.second->held();
   for (auto& x : c->idle)
@@ -1628,7 +1636,7 @@ static int batch_admit(wg_ctx* c, int cls) {
   Query* x = excl_query(c);
   if (x) {  // the exclusive query only, once nothing else runs anywhere
     if (x->solo || x->state != WG_PENDING || x->bclass != cls || active > 0) return WG_OK;
-    if (solo_running(c)) return WG_OK;
+    if (solo_running(c) || lanes_busy(c)) return WG_OK;
     for (auto& kv : c->batch)
       if (kv.first != cls && batch_holds_work_any(c, kv.first)) return WG_OK;
     drop_idle_batch(c, cls);
@@ -1823,6 +1831,18 @@ static int batch_grow(wg_ctx* c, int cls) {
   return batch_preempt<K>(c, cls, rc);
 }
 
+// Release the scratch of the row lanes when they are idle; true when there was any.
+static bool drop_lanes(wg_ctx* c) {
+  if (lanes_busy(c) || !lanes_held(c)) return false;
+  drop_idle_lanes(c);
+  return true;
+}
+static bool runs_elsewhere(wg_ctx* c, int cls) {
+  for (auto& kv : c->batch)
+    if (kv.first != cls && batch_holds_work_any(c, kv.first)) return true;
+  return solo_running(c) || lanes_busy(c);
+}
+
 // One scheduling round: finish the launch in flight (grow or preempt after an
 // overflow, retire finished queries), admit queued queries, launch again.
 template <typename K>
@@ -1850,7 +1870,9 @@ static int batch_round(wg_ctx* c, int cls, uint32_t iters, bool wait_launch, boo
     }
     TRY(batch_retire<K>(c, cls));
   } else if (E->grow_wait) {  // paused: retry once memory has come back
-    if (drop_idle_batch(c, cls) || c->used < E->wait_used) {
+    // (with nothing else running no memory will come back: settle it now)
+    if (drop_idle_batch(c, cls) || drop_lanes(c) || c->used < E->wait_used ||
+        !runs_elsewhere(c, cls)) {
       TRY(batch_grow<K>(c, cls));
       if (!E->grow_wait) *progressed = true;
     }
@@ -1863,7 +1885,7 @@ static int batch_round(wg_ctx* c, int cls, uint32_t iters, bool wait_launch, boo
     // a lone query (nothing queued, nothing else running anywhere) runs to
     // its fixpoint in this one launch, as the plain loop would: capping its
     // iterations only adds host round trips while nobody waits to join
-    bool lone = active == 1 && c->pending.empty() && !solo_running(c);
+    bool lone = active == 1 && c->pending.empty() && !solo_running(c) && !lanes_busy(c);
     for (auto& kv : c->batch)
       if (lone && kv.first != cls && batch_holds_work_any(c, kv.first)) lone = false;
     TRY(E->launch(lone ? 0xFFFFFFFFu : iters, WG_LOOP_DEVICE));
@@ -1934,17 +1956,20 @@ static bool batch_busy(wg_ctx* c) {
 // while another could run: engines whose launch finished are retired,
 // admitted and relaunched; if none had finished, wait briefly and retry.
 static int solo_round(wg_ctx* c, bool* progressed, bool* busy);
+static int lanes_round(wg_ctx* c, bool* progressed);
 
 static int serve_round(wg_ctx* c, uint32_t iters) {
   for (long spin = 0;; ++spin) {
     bool progressed = false, solo_busy = false;
+    TRY(lanes_round(c, &progressed));
     TRY(solo_round(c, &progressed, &solo_busy));
     for (auto& kv : c->batch) TRY(batch_round_any(c, kv.first, iters, false, &progressed));
-    if (progressed || !(batch_busy(c) || solo_busy)) return WG_OK;
+    if (progressed || !(batch_busy(c) || solo_busy || lanes_busy(c))) return WG_OK;
     if (spin > 12000000) {  // ~10 min without any launch finishing
       return set_err(WG_E_DEVICE_TIMEOUT, "no launch finished");
     }
-    std::this_thread::sleep_for(std::chrono::microseconds(50));
+    // the small launches end within this many polls
+    if (spin >= 100) std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
 }
 
@@ -1976,6 +2001,360 @@ static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R) {
   return prc;
 }
 
+// ------------------------------------------------------------------ batched rows
+// Whether query q runs row by row (wg_kern_rows.cu): a TC query that asks for
+// nothing of the sorted-array pipeline (its ablations, the host-driven loops,
+// a per-stage profile, the size of the candidate buffers), over a relation
+// whose bit sets and lists take at most half of the free budget -- the sorted
+// pipeline needs more than twice the result, so whatever fits there fits here.
+static bool row_fits(wg_ctx* c, const Query* q) {
+  const Relation* R = q->rel;
+  if (q->kind != WG_TC || q->opts.flags || q->opts.reserve_cand || R->nv > kXSegMaxVertices)
+    return false;
+  size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
+  for (auto& e : c->idle) idle += e->held();
+  const uint32_t words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
+  const size_t queue = (size_t)grid_of(c, occupancy_rows(R->id_bytes(), words)) * R->nv * R->id_bytes();
+  return (size_t)R->nv * words * 4 + queue <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
+}
+static bool row_query(wg_ctx* c, const Query* q) {
+  return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && row_fits(c, q);
+}
+// (loop and profile are ignored in batches)
+static bool row_batched(wg_ctx* c, const Query* q) { return q->rel->nv > 0 && row_fits(c, q); }
+
+
+// Submitted row-by-row TC queries: a lane runs the rows of many relations of
+// one key width in one launch (k_rows claims rows across instances), learns
+// every result's exact size, allocates the results and expands them.  No pool
+// is shared and nothing grows: a result that does not fit beside others waits
+// until the query can run alone, as the exclusive query, and fails only then.
+// Two lanes on streams of their own, so the host's turn between a lane's
+// launches overlaps the other lane's rows.
+struct RowLane {
+  cudaStream_t st = nullptr;
+  cudaEvent_t done = nullptr;
+  int phase = 0;                   // 0 idle, 1 rows in flight, 2 expansion in flight
+  int kb = 4;
+  DBuf meta, bits, queue;
+  char* mirror = nullptr;          // page-locked copy of the cleared and uploaded parts of meta
+  size_t mirror_bytes = 0;
+  size_t o_inst = 0, o_log = 0, up_end = 0, clear = 0;
+  uint32_t n = 0, log_cap = 0;
+  RowJob job{};
+  std::vector<uint64_t> order;     // query ids as submitted
+  std::vector<uint32_t> slot;      // their instances
+  ~RowLane() {
+    if (st) cudaStreamSynchronize(st);
+    if (done) cudaEventDestroy(done);
+    if (mirror) cudaFreeHost(mirror);
+    if (st) cudaStreamDestroy(st);
+  }
+};
+static bool lanes_busy(const wg_ctx* c) {
+  for (auto& l : c->lanes)
+    if (l->phase) return true;
+  return false;
+}
+static size_t lanes_held(const wg_ctx* c) {
+  size_t b = 0;
+  for (auto& l : c->lanes) b += l->meta.bytes + l->bits.bytes + l->queue.bytes;
+  return b;
+}
+static void drop_idle_lanes(wg_ctx* c) {
+  for (auto& l : c->lanes)
+    if (l->phase == 0) { l->meta.release(c); l->bits.release(c); l->queue.release(c); }
+}
+static void release_lanes(wg_ctx* c) {
+  for (auto& l : c->lanes) {
+    if (l->st) cudaStreamSynchronize(l->st);
+    l->phase = 0;
+  }
+  drop_idle_lanes(c);
+}
+
+// Scratch of one launch: bit sets of all its instances (a launch takes about
+// this much, so that requests arriving meanwhile wait a few milliseconds at
+// most), and instances per launch.
+constexpr size_t kLaneBits = 256u << 20;
+constexpr uint32_t kLaneQueries = 1024;
+
+// Start the queued queries `ids` (one key width) on lane L.
+static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
+  AllocScope scope(c, L->st);
+  std::vector<Query*> qs;
+  for (uint64_t id : ids) qs.push_back(c->queries.find(id)->second.get());
+  L->n = (uint32_t)qs.size();
+  L->order = ids;
+  L->kb = qs[0]->rel->kb;
+  // larger relations first: their long rows must not start last
+  std::vector<uint32_t> by(L->n);
+  for (uint32_t i = 0; i < L->n; ++i) by[i] = i;
+  std::sort(by.begin(), by.end(), [&](uint32_t a, uint32_t b) {
+    return qs[a]->rel->nv != qs[b]->rel->nv ? qs[a]->rel->nv > qs[b]->rel->nv : a < b;
+  });
+  const uint32_t nv_max = qs[by[0]]->rel->nv, vwords = (uint32_t)Engine<uint32_t>::row_words(nv_max);
+  const int idb = qs[0]->rel->id_bytes();
+  uint32_t nch = 0;
+  size_t bits = 0;
+  for (Query* q : qs) {
+    nch += (q->rel->nv + kRowChunk - 1) / kRowChunk;
+    bits += (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
+  }
+  L->log_cap = std::min(kBatchLogCap, nv_max + 2);
+  const int grid = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(idb, vwords)),
+                                           (uint64_t)nch * kRowChunk);
+  auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
+  size_t end = 0;
+  const size_t o_ctl = at(end, sizeof(RowCtl)), o_sum = at(end, (size_t)nch * 4);
+  L->o_log = at(end, (size_t)L->n * L->log_cap * 8);
+  L->clear = end;
+  L->o_inst = at(end, (size_t)L->n * sizeof(RowInst));
+  const size_t o_map = at(end, (size_t)nch * 4);
+  L->up_end = end;
+  const size_t o_base = at(end, (size_t)nch * 8), o_cnt = at(end, (size_t)nch * kRowChunk * 4);
+  L->phase = 1;  // (its buffers are not to be dropped while it allocates)
+  int rc = L->meta.get(c, end);
+  if (rc == WG_OK) rc = L->bits.get(c, bits);
+  if (rc == WG_OK) rc = L->queue.get(c, (size_t)grid * nv_max * idb);
+  L->phase = 0;
+  TRY(rc);
+  if (L->up_end > L->mirror_bytes) {
+    if (L->mirror) cudaFreeHost(L->mirror);
+    L->mirror = nullptr;
+    L->mirror_bytes = 0;
+    CK(cudaMallocHost((void**)&L->mirror, 2 * L->up_end));
+    L->mirror_bytes = 2 * L->up_end;
+  }
+  char* m = (char*)L->meta.p;
+  RowInst* hi = (RowInst*)(L->mirror + L->o_inst);
+  uint32_t* hm = (uint32_t*)(L->mirror + o_map);
+  L->slot.assign(L->n, 0);
+  uint32_t ch = 0;
+  size_t wat = 0;
+  for (uint32_t k = 0; k < L->n; ++k) {
+    Query* q = qs[by[k]];
+    const Relation* R = q->rel;
+    L->slot[by[k]] = k;
+    RowInst I{};
+    I.off = (const uint32_t*)R->off.p; I.adj = (const uint32_t*)R->adj.p; I.rec = R->rec.p;
+    I.nv = R->nv; I.w = R->w; I.words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
+    I.bits = (uint32_t*)L->bits.p + wat;
+    wat += (size_t)R->nv * I.words;
+    I.row0 = ch * kRowChunk;
+    I.cnt = (uint32_t*)(m + o_cnt) + I.row0;
+    I.log = (unsigned long long*)(m + L->o_log) + (size_t)k * L->log_cap;
+    I.max_iters = q->opts.max_iters; I.log_cap = L->log_cap;
+    hi[k] = I;
+    for (uint32_t e = ch + (R->nv + kRowChunk - 1) / kRowChunk; ch < e; ++ch) hm[ch] = k;
+    q->state = WG_RUNNING;
+  }
+  RowJob& J = L->job;
+  J = RowJob{};
+  J.ctl = (RowCtl*)(m + o_ctl); J.inst = (RowInst*)(m + L->o_inst);
+  J.chunk_inst = (const uint32_t*)(m + o_map);
+  J.csum = (uint32_t*)(m + o_sum); J.cbase = (unsigned long long*)(m + o_base);
+  J.queue = L->queue.p; J.queue_stride = nv_max;
+  J.nrows = nch * kRowChunk; J.vwords = vwords;
+  CK(cudaMemcpyAsync(m + L->o_inst, L->mirror + L->o_inst, L->up_end - L->o_inst,
+                     cudaMemcpyHostToDevice, L->st));
+  CK(cudaMemsetAsync(m, 0, L->clear, L->st));
+  launch_rows(J, idb, grid, L->st);
+  launch_row_plan(J, L->n, L->st);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(L->mirror + L->o_log, m + L->o_log, L->o_inst - L->o_log + L->n * sizeof(RowInst),
+                     cudaMemcpyDeviceToHost, L->st));
+  CK(cudaEventRecord(L->done, L->st));
+  L->phase = 1;
+  return WG_OK;
+}
+
+// A row query whose result of `bytes` does not fit now: it fails if it has run
+// alone already or never could fit, else it is queued again to run alone.
+static void lane_result_refused(wg_ctx* c, RowLane* L, Query* q, size_t bytes, int why) {
+  size_t free_later = lanes_held(c);
+  for (auto& kv : c->batch)
+    if (kv.second) free_later += kv.second->held();
+  for (auto& e : c->idle) free_later += e->held();
+  if (c->solo_run) {
+    auto it = c->queries.find(c->solo_run);
+    if (it != c->queries.end() && it->second->eng) free_later += it->second->eng->held();
+  }
+  const size_t fixed = c->used > free_later ? c->used - free_later : 0;
+  const size_t own = (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
+  if ((L->n == 1 && q->row_alone) || fixed + own + bytes > c->budget) {
+    if (c->excl == q->id) c->excl = 0;
+    q->state = WG_FAILED;
+    q->error = why;
+    q->t_done_us = now_us();
+    c->completed.push_back(q->id);
+    return;
+  }
+  q->row_alone = true;
+  q->state = WG_PENDING;
+  q->regrows += 1;
+  c->pending.insert(c->pending.begin(), q->id);
+}
+
+// Rows done: allocate the results and expand the bit sets into them.
+static int lane_expand(wg_ctx* c, RowLane* L) {
+  AllocScope scope(c, L->st);
+  RowInst* hi = (RowInst*)(L->mirror + L->o_inst);
+  for (uint32_t i = 0; i < L->n; ++i) {
+    RowInst& I = hi[L->slot[i]];
+    I.fits = 0;
+    auto it = c->queries.find(L->order[i]);
+    if (it == c->queries.end()) continue;
+    Query* q = it->second.get();
+    const size_t bytes = std::max<size_t>(I.n_total, 1) * L->kb;
+    int rc = q->res_own.get(c, bytes);
+    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && drop_idle_batch(c, -1)) {
+      cudaGetLastError();
+      rc = q->res_own.get(c, bytes);
+    }
+    if (rc != WG_OK) {
+      cudaGetLastError();
+      lane_result_refused(c, L, q, bytes, rc);
+      continue;
+    }
+    const bool capped = I.last >= I.max_iters;
+    q->n_tuples = I.n_total;
+    q->candidates = I.cand;
+    q->iterations = capped ? I.max_iters : I.last + 1;
+    const unsigned long long* log =
+        (const unsigned long long*)(L->mirror + L->o_log) + (size_t)L->slot[i] * L->log_cap;
+    q->log.assign(log, log + std::min(q->iterations + 1, kBatchLogCap));
+    q->error = capped ? WG_E_ITER_CAP : WG_OK;
+    q->res_ptr = q->res_own.p;
+    I.out = q->res_own.p;
+    I.fits = 1;
+  }
+  CK(cudaMemcpyAsync((char*)L->meta.p + L->o_inst, hi, L->n * sizeof(RowInst),
+                     cudaMemcpyHostToDevice, L->st));
+  if (L->kb == 4) launch_row_expand<uint32_t>(L->job, grid_of(c, 6), L->st);
+  else launch_row_expand<unsigned long long>(L->job, grid_of(c, 6), L->st);
+  CK(cudaGetLastError());
+  CK(cudaEventRecord(L->done, L->st));
+  L->phase = 2;
+  return WG_OK;
+}
+
+static void lane_finish(wg_ctx* c, RowLane* L) {
+  for (uint64_t id : L->order) {
+    auto it = c->queries.find(id);
+    if (it == c->queries.end() || it->second->state != WG_RUNNING) continue;
+    Query* q = it->second.get();
+    if (c->excl == id) c->excl = 0;
+    q->state = q->error == WG_OK ? WG_DONE : WG_FAILED;
+    q->t_done_us = now_us();
+    c->completed.push_back(id);
+  }
+  L->phase = 0;
+}
+
+// The next launch of an idle lane: queued row queries of one key width, in
+// order, up to kLaneBits of bit sets; one query alone if it must run alone.
+static int lane_admit(wg_ctx* c, RowLane* L, bool* progressed) {
+  Query* x = excl_query(c);
+  if (x && !x->rowb) return WG_OK;  // another query waits for the whole budget
+  std::vector<uint64_t> ids;
+  size_t bits = 0;
+  int kb = 0;
+  for (uint64_t id : c->pending) {
+    auto it = c->queries.find(id);
+    if (it == c->queries.end() || !it->second->rowb) continue;
+    Query* q = it->second.get();
+    if (x && q != x) continue;
+    if (q->row_alone) {
+      if (!ids.empty()) break;
+      c->excl = id;  // nothing else is admitted until it has run
+      bool other = solo_running(c) || lanes_busy(c);
+      for (auto& kv : c->batch) other |= batch_holds_work_any(c, kv.first);
+      if (other) return WG_OK;
+      drop_idle_batch(c, -1);
+      ids.push_back(id);
+      break;
+    }
+    const size_t b = (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
+    if (kb && (q->rel->kb != kb || bits + b > kLaneBits || ids.size() >= kLaneQueries)) {
+      if (q->rel->kb != kb) continue;
+      break;
+    }
+    kb = q->rel->kb;
+    bits += b;
+    ids.push_back(id);
+  }
+  if (ids.empty()) return WG_OK;
+  int rc = lane_start(c, L, ids);
+  if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
+    cudaGetLastError();
+    if (ids.size() > 1) {  // fewer at once
+      ids.resize(1);
+      rc = lane_start(c, L, ids);
+    }
+    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && !held_elsewhere(c, -1)) {
+      // no scratch for its bit sets with nothing else running: the sorted pipeline
+      cudaGetLastError();
+      Query* q = c->queries.find(ids[0])->second.get();
+      q->rowb = false;
+      q->bclass = batch_class(q->rel);
+      if (c->excl == q->id) c->excl = 0;
+      c->batch[q->bclass];  // listed: its engine is built on demand
+      *progressed = true;
+      return WG_OK;
+    }
+    if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
+      cudaGetLastError();
+      return WG_OK;  // memory comes back when the others finish
+    }
+  }
+  TRY(rc);
+  std::vector<uint64_t> still;
+  for (uint64_t id : c->pending)
+    if (std::find(ids.begin(), ids.end(), id) == ids.end()) still.push_back(id);
+  c->pending.swap(still);
+  *progressed = true;
+  return WG_OK;
+}
+
+static int lanes_round(wg_ctx* c, bool* progressed) {
+  bool any = false;
+  for (uint64_t id : c->pending) {
+    auto it = c->queries.find(id);
+    any |= it != c->queries.end() && it->second->rowb;
+  }
+  if (!any && !lanes_busy(c)) return WG_OK;
+  while (c->lanes.size() < 2) {
+    auto l = std::make_unique<RowLane>();
+    CK(cudaStreamCreateWithFlags(&l->st, cudaStreamNonBlocking));
+    CK(cudaEventCreateWithFlags(&l->done, cudaEventDisableTiming));
+    c->lanes.push_back(std::move(l));
+  }
+  for (auto& l : c->lanes) {
+    if (l->phase) {
+      const cudaError_t e = cudaEventQuery(l->done);
+      if (e == cudaErrorNotReady) continue;
+      CK(e);
+      *progressed = true;
+      if (l->phase == 1) {
+        TRY(lane_expand(c, l.get()));
+        continue;
+      }
+      lane_finish(c, l.get());
+    }
+    TRY(lane_admit(c, l.get(), progressed));
+  }
+  return WG_OK;
+}
+
+// Wait for every launch in flight on the lanes (a query of theirs is freed).
+static void finish_lanes(wg_ctx* c) {
+  for (auto& l : c->lanes) {
+    if (l->phase == 1 && cudaEventSynchronize(l->done) == cudaSuccess) lane_expand(c, l.get());
+    if (l->phase == 2 && cudaEventSynchronize(l->done) == cudaSuccess) lane_finish(c, l.get());
+  }
+}
+
 template <typename K>
 static int copy_result(wg_ctx* c, Query* q, unsigned long long* dst, bool host) {
   const size_t n = q->n_tuples;
@@ -1988,9 +2367,13 @@ static int copy_result(wg_ctx* c, Query* q, unsigned long long* dst, bool host) 
     locked = cudaPointerGetAttributes(&pa, dst) == cudaSuccess && pa.type == cudaMemoryTypeHost;
     cudaGetLastError();  // pageable pointers are not an error
   }
-  const size_t chunk = host ? (size_t)1 << (locked ? 26 : 24) : n;
+  size_t chunk = host ? (size_t)1 << (locked ? 26 : 24) : n;
   DBuf tmp;
-  if (host) TRY(tmp.get(c, std::min(n, chunk) * 8));
+  if (host) {  // (a smaller staging buffer where the budget is nearly spent)
+    int rc;
+    while ((rc = tmp.get(c, std::min(n, chunk) * 8)) == WG_E_BUDGET && chunk > (1u << 16)) chunk /= 2;
+    TRY(rc);
+  }
   for (size_t at = 0; at < n; at += chunk) {
     const size_t m = std::min(chunk, n - at);
     unsigned long long* o = host ? (unsigned long long*)tmp.p : dst + at;
@@ -2037,6 +2420,7 @@ int wg_init(int device, size_t budget, wg_alloc_fn alloc, wg_free_fn free_fn, vo
 void wg_destroy(wg_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
+  release_lanes(c);
   for (auto& kv : c->queries) kv.second->res_own.release(c);
   for (auto& kv : c->queries) {
     Query* q = kv.second.get();
@@ -2049,6 +2433,7 @@ void wg_destroy(wg_ctx* c) {
   c->idle.clear();
   for (auto& kv : c->batch) if (kv.second) kv.second->release();
   c->batch.clear();
+  c->lanes.clear();  // (their streams: results allocated on them were freed above)
   for (auto& kv : c->class_st) {
     cudaStreamSynchronize(kv.second);
     cudaStreamDestroy(kv.second);
@@ -2143,23 +2528,6 @@ static int make_query(wg_ctx* c, int kind, wg_rel edges, const wg_opts* opts, Qu
   *out = q.get();
   c->queries[q->id] = std::move(q);
   return WG_OK;
-}
-
-// Whether query q runs row by row (wg_kern_rows.cu): a TC query that asks for
-// nothing of the sorted-array pipeline (its ablations, the host-driven loops,
-// a per-stage profile, the size of the candidate buffers), over a relation
-// whose bit sets and lists take at most half of the free budget -- the sorted
-// pipeline needs more than twice the result, so whatever fits there fits here.
-static bool row_query(wg_ctx* c, const Query* q) {
-  const Relation* R = q->rel;
-  if (q->kind != WG_TC || q->opts.flags || q->opts.loop != WG_LOOP_DEVICE || q->opts.profile ||
-      q->opts.reserve_cand || R->nv > kXSegMaxVertices)
-    return false;
-  size_t idle = 0;
-  for (auto& e : c->idle) idle += e->held();
-  const uint32_t words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
-  const size_t queue = (size_t)grid_of(c, occupancy_rows(R->id_bytes(), words)) * R->nv * R->id_bytes();
-  return (size_t)R->nv * words * 4 + queue <= (c->budget - c->used + idle) / 2;
 }
 
 // Give query q a single-query engine (an idle one of the same key width, pass
@@ -2312,12 +2680,12 @@ static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
         return WG_OK;
       }
       c->excl = q->id;
-      if (drop_idle_batch(c, -1) || c->used < q->wait_used) {
+      if (drop_idle_batch(c, -1) || drop_lanes(c) || c->used < q->wait_used) {
         TRY(k4 ? solo_resume<uint32_t>(c, q) : solo_resume<unsigned long long>(c, q));
         if (!q->solo_wait) *progressed = true;
       }
       if (q->solo_wait) {
-        bool held = false;  // memory that may still come back
+        bool held = lanes_busy(c);  // memory that may still come back
         for (auto& kv : c->batch) held |= kv.second != nullptr;
         if (!held) {
           solo_finish(c, q, WG_E_BUDGET);
@@ -2356,6 +2724,7 @@ static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
     Query* q = it->second.get();
     if (x && x != q) return WG_OK;  // only the exclusive query may start
     if (x == q) {  // once the batch engines hold no work, they go
+      if (lanes_busy(c)) return WG_OK;
       for (auto& kv : c->batch)
         if (batch_holds_work_any(c, kv.first)) return WG_OK;
       drop_idle_batch(c, -1);
@@ -2407,7 +2776,10 @@ int wg_submit(wg_ctx* c, const wg_request* reqs, size_t n, wg_query* ids) {
     q->batch = true;
     q->bclass = batch_class(q->rel);
     q->solo = q->rel->ne > kSoloEdges;
-    if (q->solo) {
+    q->rowb = !q->solo && row_batched(c, q);
+    if (q->rowb) {
+      q->bclass = -1;  // runs row by row with others (lanes_round)
+    } else if (q->solo) {
       // runs on a single-query engine (solo_round)
     } else if (!excl_query(c)) {
       TRY(ensure_batch_engine(c, q->bclass, q->rel));
@@ -2452,6 +2824,7 @@ static int progress(wg_ctx* c, Query* q, bool block) {
     // drive the batch engines until this query is retired
     if (!block) {
       bool progressed = false, busy = false;
+      TRY(lanes_round(c, &progressed));
       TRY(solo_round(c, &progressed, &busy));
       for (auto& kv : c->batch) TRY(batch_round_any(c, kv.first, 0xFFFFFFFFu, false, &progressed));
       return WG_OK;
@@ -2717,6 +3090,11 @@ void wg_query_free(wg_ctx* c, wg_query id) {
   if (it == c->queries.end()) return;
   Query* q = it->second.get();
   if (q->state == WG_RUNNING && !q->batch) progress(c, q, true);
+  if (q->rowb && q->state == WG_RUNNING) {
+    finish_lanes(c);  // its relation may go next
+    c->completed.erase(std::remove(c->completed.begin(), c->completed.end(), id),
+                       c->completed.end());
+  }
   if (q->batch && q->state == WG_PENDING) {
     c->pending.erase(std::remove(c->pending.begin(), c->pending.end(), id), c->pending.end());
   }

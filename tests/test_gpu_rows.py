@@ -108,3 +108,40 @@ def test_result_buffer_grows_and_the_engine_is_reused():
                 assert q.delta_sizes() == want.log.tolist()
                 q.free()
             rel.free()
+
+
+def _drain(ctx):
+    while ctx.serve_step(16):
+        pass
+
+
+def test_batched_rows_equal_the_batched_pipeline():
+    """Submitted queries row by row (rows of many relations of both rank widths
+    in one launch, chunks of 256 rows that end mid-way, iteration caps, more
+    iterations than the batch keeps sizes of) against the same queries on the
+    batch engines' sorted-array pipeline, and a query freed while it runs."""
+    from paper_2607_17571_gb300 import wg
+    gs = [I.path(1100), I.path(2), I.er_graph(255, 500, 1), I.er_graph(700, 1500, 2),
+          I.er_graph(70_000, 60_000, 3), I.cycle(257), I.rmat_dag(11, 5000, 4),
+          I.er_graph(80_000, 50_000, 5), I.path(300)]
+    caps = [0, 0, 0, 3, 0, 100, 0, 2, 64]
+    with wg.Context(0) as c:
+        rels = [c.load(g.src, g.dst) for g in gs]
+        got = []
+        for kw in ({}, dict(side_run="never")):
+            hs = c.submit([(wg.WG_TC, r, dict(max_iters=m, **kw)) for r, m in zip(rels, caps)])
+            extra = c.submit([(wg.WG_TC, rels[3], kw)])[0]
+            c.serve_step(1)
+            extra.free()
+            _drain(c)
+            assert sorted(c.take_completed()) == sorted(h.id for h in hs)
+            out = []
+            for h in hs:
+                st = h.poll()
+                out.append((st.state, st.error, st.n_tuples, st.iterations, st.candidates,
+                            h.delta_sizes(), h.digest() if st.state == wg.WG_DONE else None))
+                h.free()
+            got.append(out)
+        assert got[0] == got[1]
+        for r in rels:
+            r.free()
