@@ -237,7 +237,9 @@ struct Dev {
 struct RowInst {
   const uint32_t* off;          // CSR
   const uint32_t* adj;
-  const void* rec;              // adjacency records, 8 ids per vertex
+  const void* rec;              // vertex records, 32 bytes each
+  const uint32_t* ns;           // bit set of the vertices with out-edges
+  const void* units;            // adjacency past the records, in 16-byte units
   uint32_t* bits;               // row x's bit set: words [x * words, (x + 1) * words)
   uint32_t* cnt;                // tuples of row x
   void* out;                    // sorted packed keys
@@ -259,12 +261,10 @@ struct RowJob {
   const uint32_t* chunk_inst;   // row chunk -> instance (or NULL: instance 0)
   uint32_t* csum;               // tuples per chunk of kRowChunk rows (cleared before)
   unsigned long long* cbase;    // their exclusive prefix within the instance
-  void* queue;                  // per-CTA lists of reached vertices, queue_stride ids each
-  uint32_t queue_stride, nrows, vwords, pad;
+  uint32_t nrows, vwords;       // vwords: words of the widest instance's rows
 };
 constexpr uint32_t kRowChunk = 256;
-constexpr uint32_t kRowQueue = 1024;    // list entries kept in shared memory
-constexpr uint32_t kRecInline = 7;      // neighbours in an adjacency record
+constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are expanded
 constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
 constexpr uint32_t kRowSmemMax = 200 * 1024;
 

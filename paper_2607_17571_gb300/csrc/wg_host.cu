@@ -313,14 +313,25 @@ struct Relation {
   uint32_t nv = 0, w = 1;
   int kb = 4;
   DBuf keys, off, adj, V;
-  DBuf rec;                       // adjacency records of the row fixpoints (up to kXSegMaxVertices)
+  DBuf rowv;                      // row fixpoints (up to kXSegMaxVertices): vertex records,
+  size_t o_ns = 0, o_units = 0;   // out-edge bit set and adjacency units at these offsets
   DBuf htab;                      // hash-join ablation: E in a linear-probing table (lazy)
   unsigned long long hmask = 0;
   uint64_t peak_cand = 0, peak_full = 0;  // capacities seen by earlier queries
-  int id_bytes() const { return nv <= 65536u ? 2 : 4; }  // of a rank in rec
+  int id_bytes() const { return nv <= 65536u ? 2 : 4; }  // of a rank in the units
+  uint32_t row_words() const { return (nv + 127) / 128 * 4; }  // of a row's bit set
+  size_t row_bits() const { return (size_t)nv * row_words() * 4; }  // bytes of all rows' sets
+  void row_inst(RowInst* I) const {
+    *I = RowInst{};
+    I->off = (const uint32_t*)off.p; I->adj = (const uint32_t*)adj.p;
+    I->rec = rowv.p;
+    I->ns = (const uint32_t*)((const char*)rowv.p + o_ns);
+    I->units = (const char*)rowv.p + o_units;
+    I->nv = nv; I->w = w; I->words = row_words();
+  }
   void release(wg_ctx* c) {
     keys.release(c); off.release(c); adj.release(c); V.release(c); htab.release(c);
-    rec.release(c);
+    rowv.release(c);
   }
 };
 
@@ -344,10 +355,14 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
   launch_csr<K>((const K*)ke.p, ne, R->nv, R->w, (uint32_t*)R->off.p, (uint32_t*)R->adj.p,
                 grid_of(c, 4), c->stream);
   CK(cudaGetLastError());
-  if (R->nv <= kXSegMaxVertices) {
-    TRY(R->rec.get(c, (size_t)R->nv * 8 * R->id_bytes()));
-    launch_row_records((const uint32_t*)R->off.p, (const uint32_t*)R->adj.p, R->nv, R->rec.p,
-                       R->id_bytes(), grid_of(c, 4), c->stream);
+  if (R->nv <= kXSegMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
+    R->o_ns = round_up((size_t)R->nv * 32);
+    R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
+    TRY(R->rowv.get(c, R->o_units + row_units(ne, R->nv, R->id_bytes()) * 16));
+    char* v = (char*)R->rowv.p;
+    launch_row_layout<K>((const K*)ke.p, (uint32_t)ne, R->w, (const uint32_t*)R->off.p,
+                         (const uint32_t*)R->adj.p, R->nv, v, (uint32_t*)(v + R->o_ns),
+                         R->row_words(), v + R->o_units, R->id_bytes(), grid_of(c, 8), c->stream);
     CK(cudaGetLastError());
   }
   return WG_OK;
@@ -562,7 +577,7 @@ struct Engine : EngineBase {
   uint32_t sort_mode_;               // enum wg_sort_mode (x-grouped engines)
   uint32_t side_;                    // side run of Full: 0 never, 1 with few candidates, 2 always
   bool rows_ = false;                // row-by-row TC (wg_kern_rows.cu): none of the stages below
-  DBuf row_meta, row_bits, row_queue;
+  DBuf row_meta, row_bits;
   RowInst ri{};
   RowJob job{};
   size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
@@ -605,7 +620,7 @@ struct Engine : EngineBase {
     ev_done = nullptr;
     DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                    &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b, &xsum_b,
-                   &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_queue};
+                   &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits};
     for (DBuf* b : all) b->release(c);
     capC = capF = capR = capG = 0;
     mix_tiles = 0;
@@ -832,10 +847,9 @@ struct Engine : EngineBase {
 
   // Row-by-row TC: buffers for relation R and a result of wantF keys.  A
   // result that turns out larger only needs the expansion again (settle).
-  static size_t row_words(uint32_t nv) { return ((size_t)nv + 127) / 128 * 4; }
   int rows_begin(Relation* Rl, uint32_t max_iters, unsigned long long wantF) {
     AllocScope scope(c, st);
-    const uint32_t nv = Rl->nv, words = (uint32_t)row_words(nv);
+    const uint32_t nv = Rl->nv, words = Rl->row_words();
     const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
     const uint32_t nlog = std::min<uint32_t>(1u << 16, nv + 2);
     id_bytes = Rl->id_bytes();
@@ -850,24 +864,19 @@ struct Engine : EngineBase {
     const size_t o_inst = at(end, sizeof(RowInst)), o_base = at(end, (size_t)nch * 8),
                  o_cnt = at(end, (size_t)nv * 4);
     TRY(row_meta.get(c, end));
-    TRY(row_bits.get(c, std::max<size_t>((size_t)nv * words, 1) * 4));
-    TRY(row_queue.get(c, (size_t)g_rows * std::max<uint32_t>(nv, 1) * id_bytes));
+    TRY(row_bits.get(c, std::max<size_t>(Rl->row_bits(), 16)));
     if (wantF > capF) {
       TRY(F[0].get(c, wantF * sizeof(K)));
       capF = wantF;
     }
     char* m = (char*)row_meta.p;
-    ri = RowInst{};
-    ri.off = (const uint32_t*)Rl->off.p; ri.adj = (const uint32_t*)Rl->adj.p;
-    ri.rec = Rl->rec.p;
+    Rl->row_inst(&ri);
     ri.bits = (uint32_t*)row_bits.p; ri.cnt = (uint32_t*)(m + o_cnt);
     ri.log = (unsigned long long*)(m + o_log);
-    ri.nv = nv; ri.w = Rl->w; ri.words = words;
     ri.max_iters = max_iters; ri.log_cap = nlog;
     job = RowJob{};
     job.ctl = (RowCtl*)(m + o_ctl); job.inst = (RowInst*)(m + o_inst);
     job.csum = (uint32_t*)(m + o_sum); job.cbase = (unsigned long long*)(m + o_base);
-    job.queue = row_queue.p; job.queue_stride = std::max<uint32_t>(nv, 1);
     job.nrows = nv; job.vwords = words;
     log_cap = nlog;
     expand_only = false;
@@ -1207,7 +1216,7 @@ struct Engine : EngineBase {
   size_t held() const override {
     const DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                          &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b,
-                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_queue};
+                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits};
     size_t b = 0;
     for (const DBuf* x : all) b += x->bytes;
     return b;
@@ -2005,23 +2014,21 @@ static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R) {
 // Whether query q runs row by row (wg_kern_rows.cu): a TC query that asks for
 // nothing of the sorted-array pipeline (its ablations, the host-driven loops,
 // a per-stage profile, the size of the candidate buffers), over a relation
-// whose bit sets and lists take at most half of the free budget -- the sorted
+// whose bit sets take at most half of the free budget -- the sorted
 // pipeline needs more than twice the result, so whatever fits there fits here.
 static bool row_fits(wg_ctx* c, const Query* q) {
   const Relation* R = q->rel;
-  if (q->kind != WG_TC || q->opts.flags || q->opts.reserve_cand || R->nv > kXSegMaxVertices)
+  if (q->kind != WG_TC || q->opts.flags || q->opts.reserve_cand || !R->rowv.p)
     return false;
   size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
   for (auto& e : c->idle) idle += e->held();
-  const uint32_t words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
-  const size_t queue = (size_t)grid_of(c, occupancy_rows(R->id_bytes(), words)) * R->nv * R->id_bytes();
-  return (size_t)R->nv * words * 4 + queue <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
+  return R->row_bits() <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
 }
 static bool row_query(wg_ctx* c, const Query* q) {
   return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && row_fits(c, q);
 }
 // (loop and profile are ignored in batches)
-static bool row_batched(wg_ctx* c, const Query* q) { return q->rel->nv > 0 && row_fits(c, q); }
+static bool row_batched(wg_ctx* c, const Query* q) { return row_fits(c, q); }
 
 
 // Submitted row-by-row TC queries: a lane runs the rows of many relations of
@@ -2036,7 +2043,7 @@ struct RowLane {
   cudaEvent_t done = nullptr;
   int phase = 0;                   // 0 idle, 1 rows in flight, 2 expansion in flight
   int kb = 4;
-  DBuf meta, bits, queue;
+  DBuf meta, bits;
   char* mirror = nullptr;          // page-locked copy of the cleared and uploaded parts of meta
   size_t mirror_bytes = 0;
   size_t o_inst = 0, o_log = 0, up_end = 0, clear = 0;
@@ -2058,12 +2065,12 @@ static bool lanes_busy(const wg_ctx* c) {
 }
 static size_t lanes_held(const wg_ctx* c) {
   size_t b = 0;
-  for (auto& l : c->lanes) b += l->meta.bytes + l->bits.bytes + l->queue.bytes;
+  for (auto& l : c->lanes) b += l->meta.bytes + l->bits.bytes;
   return b;
 }
 static void drop_idle_lanes(wg_ctx* c) {
   for (auto& l : c->lanes)
-    if (l->phase == 0) { l->meta.release(c); l->bits.release(c); l->queue.release(c); }
+    if (l->phase == 0) { l->meta.release(c); l->bits.release(c); }
 }
 static void release_lanes(wg_ctx* c) {
   for (auto& l : c->lanes) {
@@ -2093,13 +2100,13 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   std::sort(by.begin(), by.end(), [&](uint32_t a, uint32_t b) {
     return qs[a]->rel->nv != qs[b]->rel->nv ? qs[a]->rel->nv > qs[b]->rel->nv : a < b;
   });
-  const uint32_t nv_max = qs[by[0]]->rel->nv, vwords = (uint32_t)Engine<uint32_t>::row_words(nv_max);
+  const uint32_t nv_max = qs[by[0]]->rel->nv, vwords = qs[by[0]]->rel->row_words();
   const int idb = qs[0]->rel->id_bytes();
   uint32_t nch = 0;
   size_t bits = 0;
   for (Query* q : qs) {
     nch += (q->rel->nv + kRowChunk - 1) / kRowChunk;
-    bits += (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
+    bits += q->rel->row_bits();
   }
   L->log_cap = std::min(kBatchLogCap, nv_max + 2);
   const int grid = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(idb, vwords)),
@@ -2116,7 +2123,6 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   L->phase = 1;  // (its buffers are not to be dropped while it allocates)
   int rc = L->meta.get(c, end);
   if (rc == WG_OK) rc = L->bits.get(c, bits);
-  if (rc == WG_OK) rc = L->queue.get(c, (size_t)grid * nv_max * idb);
   L->phase = 0;
   TRY(rc);
   if (L->up_end > L->mirror_bytes) {
@@ -2136,9 +2142,8 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
     Query* q = qs[by[k]];
     const Relation* R = q->rel;
     L->slot[by[k]] = k;
-    RowInst I{};
-    I.off = (const uint32_t*)R->off.p; I.adj = (const uint32_t*)R->adj.p; I.rec = R->rec.p;
-    I.nv = R->nv; I.w = R->w; I.words = (uint32_t)Engine<uint32_t>::row_words(R->nv);
+    RowInst I;
+    R->row_inst(&I);
     I.bits = (uint32_t*)L->bits.p + wat;
     wat += (size_t)R->nv * I.words;
     I.row0 = ch * kRowChunk;
@@ -2154,7 +2159,6 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   J.ctl = (RowCtl*)(m + o_ctl); J.inst = (RowInst*)(m + L->o_inst);
   J.chunk_inst = (const uint32_t*)(m + o_map);
   J.csum = (uint32_t*)(m + o_sum); J.cbase = (unsigned long long*)(m + o_base);
-  J.queue = L->queue.p; J.queue_stride = nv_max;
   J.nrows = nch * kRowChunk; J.vwords = vwords;
   CK(cudaMemcpyAsync(m + L->o_inst, L->mirror + L->o_inst, L->up_end - L->o_inst,
                      cudaMemcpyHostToDevice, L->st));
@@ -2181,8 +2185,7 @@ static void lane_result_refused(wg_ctx* c, RowLane* L, Query* q, size_t bytes, i
     if (it != c->queries.end() && it->second->eng) free_later += it->second->eng->held();
   }
   const size_t fixed = c->used > free_later ? c->used - free_later : 0;
-  const size_t own = (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
-  if ((L->n == 1 && q->row_alone) || fixed + own + bytes > c->budget) {
+  if ((L->n == 1 && q->row_alone) || fixed + q->rel->row_bits() + bytes > c->budget) {
     if (c->excl == q->id) c->excl = 0;
     q->state = WG_FAILED;
     q->error = why;
@@ -2275,7 +2278,7 @@ static int lane_admit(wg_ctx* c, RowLane* L, bool* progressed) {
       ids.push_back(id);
       break;
     }
-    const size_t b = (size_t)q->rel->nv * Engine<uint32_t>::row_words(q->rel->nv) * 4;
+    const size_t b = q->rel->row_bits();
     if (kb && (q->rel->kb != kb || bits + b > kLaneBits || ids.size() >= kLaneQueries)) {
       if (q->rel->kb != kb) continue;
       break;

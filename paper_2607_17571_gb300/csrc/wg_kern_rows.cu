@@ -26,34 +26,57 @@
 
 namespace wg {
 
-// Adjacency record of a vertex: out-degree and the first kRecInline neighbours,
-// 16 bytes with 16-bit ranks, 32 bytes (one sector) with 32-bit ranks.  One
-// load gives most vertices' whole adjacency; longer ones continue in the CSR.
-__device__ __forceinline__ uint32_t rec_id(const uint4& a, const uint4&, int s, uint16_t) {
-  const uint32_t v = s == 0 ? a.x : s <= 2 ? a.y : s <= 4 ? a.z : a.w;
-  return (s & 1) ? (v & 0xFFFFu) : (v >> 16);
-}
-__device__ __forceinline__ uint32_t rec_id(const uint4& a, const uint4& b, int s, uint32_t) {
-  return s == 0 ? a.y : s == 1 ? a.z : s == 2 ? a.w : s == 3 ? b.x : s == 4 ? b.y : s == 5 ? b.z : b.w;
-}
-__device__ __forceinline__ void rec_load(const uint4* rec, uint32_t y, uint4& a, uint4& b, uint16_t) {
-  a = __ldg(rec + y);
-  b = a;
-}
-__device__ __forceinline__ void rec_load(const uint4* rec, uint32_t y, uint4& a, uint4& b, uint32_t) {
-  a = __ldg(rec + 2 * (size_t)y);
-  b = __ldg(rec + 2 * (size_t)y + 1);
-}
-__device__ __forceinline__ uint32_t rec_deg(const uint4& a, uint16_t) { return a.x & 0xFFFFu; }
-__device__ __forceinline__ uint32_t rec_deg(const uint4& a, uint32_t) { return a.x; }
-
+// Adjacency in units of 16 bytes (8 16-bit or 4 32-bit ranks).  Each vertex has
+// a 32-byte record (one sector): {first further unit, degree, -, -} and its
+// first unit, so one access gives most vertices' whole adjacency.  Its further
+// units start at (off[v] + (U-1) v + U-1) / U: room for every vertex before it
+// without a scan.  A unit's unused places repeat the vertex's last neighbour
+// (setting a bit twice is harmless), so no place needs a test.
+template <typename IdT> struct Unit { static constexpr uint32_t n = 16 / sizeof(IdT); };
 template <typename IdT>
-__global__ void k_row_records(const uint32_t* off, const uint32_t* adj, uint32_t nv, IdT* rec) {
-  constexpr uint32_t kTop = sizeof(IdT) == 2 ? 0xFFFFu : 0xFFFFFFFFu;
-  const uint32_t n = nv * 8u;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t v = i >> 3, s = i & 7u, o = off[v], d = off[v + 1] - o;
-    rec[i] = (IdT)(s == 0 ? min(d, kTop) : s <= d ? adj[o + s - 1] : 0u);
+__device__ __forceinline__ uint32_t unit_start(uint32_t off, uint32_t v) {
+  constexpr uint32_t U = Unit<IdT>::n;
+  return (off + (U - 1) * (v + 1)) / U;
+}
+// The bits of places [2p, 2p + 2) of a unit (16-bit ranks) or place p (32-bit).
+__device__ __forceinline__ void set_bit(uint32_t* n, uint32_t byte_off, uint32_t z) {
+  atomicOr((uint32_t*)((char*)n + byte_off), __funnelshift_l(0u, 1u, z));  // 1 << (z & 31)
+}
+__device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint16_t) {
+  set_bit(n, (v >> 3) & 0x1FFCu, v);
+  set_bit(n, (v >> 19) & 0x1FFCu, v >> 16);
+}
+__device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint32_t) {
+  set_bit(n, (v >> 3) & ~3u, v);
+}
+
+// The vertex records, the bit set of vertices with out-edges, and the further
+// units of a relation (edges in source order, the source of edge i is E[i] >> w).
+template <typename K, typename IdT>
+__global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne, uint32_t w,
+                                                         const uint32_t* off, const uint32_t* adj,
+                                                         uint32_t nv, uint4* rec, uint32_t* ns,
+                                                         uint32_t words, IdT* units) {
+  const uint32_t stride = gridDim.x * kThreads, t = blockIdx.x * kThreads + threadIdx.x;
+  for (uint32_t v = t; v < words * 32; v += stride) {
+    uint32_t o = 0, d = 0;
+    if (v < nv) {
+      o = off[v];
+      d = off[v + 1] - o;
+      rec[2 * (size_t)v] = uint4{unit_start<IdT>(o, v), d, 0, 0};
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, d > 0);
+    if ((v & 31) == 0) ns[v >> 5] = m;
+  }
+  for (uint32_t i = t; i < ne; i += stride) {
+    constexpr uint32_t U = Unit<IdT>::n;
+    const uint32_t x = (uint32_t)(E[i] >> w), o = off[x], j = i - o;
+    IdT* to = j < U ? (IdT*)(rec + 2 * (size_t)x + 1) + j
+                    : units + (size_t)unit_start<IdT>(o, x) * U + (j - U);
+    const IdT z = (IdT)adj[i];
+    *to = z;
+    if (i + 1 == off[x + 1])
+      for (uint32_t r = j % U + 1; r < U; ++r) *++to = z;
   }
 }
 
@@ -66,41 +89,95 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
   return v;
 }
 
-// One CTA takes a row through its whole fixpoint.  Shared memory: the row's
-// bit set and the head of its list of reached vertices in order of discovery
-// (the rest of the list, past kRowQueue entries, lies in the CTA's part of
-// `gq`, which stays in L2); a level is the range of the list pushed by the one
-// before it.  Per level each warp takes 32 frontier vertices at a time: their
-// records in one load per lane, then the neighbours past the inline ones of
-// all 32 as one strip of edges (each lane finds its edge's vertex by a search
-// over the lanes' prefix sums), so hubs are spread over the warp.
-template <typename IdT>
-__global__ void __launch_bounds__(kThreads, 6) k_rows(RowJob J) {
-  extern __shared__ uint32_t sm[];
+// One CTA takes a row through its whole fixpoint.  Shared memory: the row's bit
+// set S and the candidates' bit set N of the next iteration.
+// An iteration: the threads take 128 bits of N at a time, drop what S has, merge
+// the rest (the delta) into S and list the delta's vertices that have out-edges
+// (on the R-MAT workloads 4 to 5 in 10 have none); the warps then expand the
+// list 32 vertices at a time: each lane its vertex's record, then the vertices'
+// further units as one strip, 32 units per step, a lane finding its unit's
+// vertex from the bit mask of the strip's first units.  Setting a bit in the
+// next N needs no answer, so a candidate costs one shared atomic and no list of
+// winners is kept; scanning N costs words / 128 lane steps per iteration.  Two
+// barriers per iteration; a delta of more than kRowList such vertices takes
+// several rounds, the bits not yet listed waiting in the row's place in `bits`.
+//
+// Bound by issue slots and by the barriers (ncu: 58% of the issue slots, DRAM
+// idle).  What it measured on R-MAT 2^17 / 400k, whole call: winners of each
+// bit listed by an answering atomic, records of 7 neighbours and single edges
+// past them 16.1 ms; candidate bits without an answer, edges in 16-byte units,
+// a list per warp (one barrier, but it waited for the warp with the most to
+// expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0.
+template <typename IdT, int T, int kMin>
+__global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
+  constexpr uint32_t U = Unit<IdT>::n, kW = T / 32;
+  extern __shared__ uint4 sm4[];
   __shared__ RowInst I;
   __shared__ unsigned long long s_log[kRowLog];
-  __shared__ uint32_t s_row[2], s_push[3];
-  uint32_t* V = sm;
-  IdT* sq = (IdT*)(sm + J.vwords);
-  IdT* gq = (IdT*)J.queue + (size_t)blockIdx.x * J.queue_stride;
+  __shared__ uint32_t s_row[2], s_cnt[2], s_len[2];
+  uint32_t* S = (uint32_t*)sm4;
+  uint32_t* N = S + J.vwords;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* strip = N + J.vwords + warp * 32;
+  IdT* list = (IdT*)(N + J.vwords + kW * 32);
+  const uint32_t upto = 0xFFFFFFFFu >> (31 - lane);
   unsigned long long cand = 0;
   uint32_t cur = 0xFFFFFFFFu;
-  for (uint32_t i = tid; i < J.vwords; i += kThreads) V[i] = 0;
-  if (tid < kRowLog) s_log[tid] = 0;
+  for (uint32_t i = tid; i < 2 * J.vwords; i += T) S[i] = 0;
+  for (uint32_t i = tid; i < kRowLog; i += T) s_log[i] = 0;
   if (tid == 0) s_row[0] = atomicAdd(&J.ctl->next_row, 1u);
   __syncthreads();
-  auto put = [&](uint32_t p, uint32_t z) {
-    if (p < kRowQueue) sq[p] = (IdT)z; else gq[p] = (IdT)z;
-  };
   auto flush = [&]() {  // the counters of the current instance
     for (int o = 16; o > 0; o >>= 1) cand += __shfl_xor_sync(0xffffffffu, cand, o);
     if (lane == 0 && cand) atomicAdd(&J.inst[cur].cand, cand);
     cand = 0;
-    if (tid < kRowLog && s_log[tid]) {
-      if (tid < I.log_cap) atomicAdd(I.log + tid, s_log[tid]);
-      s_log[tid] = 0;
+    for (uint32_t i = tid; i < kRowLog; i += T) {
+      if (s_log[i] && i < I.log_cap) atomicAdd(I.log + i, s_log[i]);
+      s_log[i] = 0;
     }
+  };
+  constexpr uint32_t P = U / 4;  // places in a word of a unit
+  // the bits of the neighbours of vertices l[0..n), n <= 32, into N
+  auto expand = [&](const IdT* l, uint32_t n) {
+    uint32_t us = 0, deg = 0;
+    uint4 u = {0, 0, 0, 0};
+    if (lane < n) {
+      const uint4* r = (const uint4*)I.rec + 2 * (size_t)l[lane];
+      const uint2 t = __ldg((const uint2*)r);
+      u = __ldg(r + 1);
+      us = t.x;
+      deg = t.y;
+    }
+    cand += deg;
+    const uint32_t most = __reduce_max_sync(0xffffffffu, deg);
+    if (lane < n) {
+      set_part(N, u.x, IdT());
+      if (most > P) set_part(N, u.y, IdT());
+      if (most > 2 * P) set_part(N, u.z, IdT());
+      if (most > 3 * P) set_part(N, u.w, IdT());
+    }
+    if (most <= U) return;
+    const uint32_t more = deg > U ? (deg - 1) / U : 0u;  // further units
+    const uint32_t has = __ballot_sync(0xffffffffu, more > 0);
+    const uint32_t in = warp_incl_scan(more, lane);
+    const uint32_t tot = __shfl_sync(0xffffffffu, in, 31), st = in - more;
+    if (more) strip[__popc(has & upto) - 1] = us - st;
+    __syncwarp();
+    uint32_t prev = 0;  // vertices whose units begin before this step
+    for (uint32_t e0 = 0; e0 < tot; e0 += 32) {
+      const uint32_t sh = st - e0, e = e0 + lane;
+      const uint32_t m = __reduce_or_sync(0xffffffffu, more && sh < 32u ? 1u << sh : 0u);
+      const uint32_t t = strip[prev + __popc(m & upto) - 1];
+      prev += __popc(m);
+      if (e < tot) {
+        u = __ldg((const uint4*)I.units + (t + e));
+        set_part(N, u.x, IdT());
+        set_part(N, u.y, IdT());
+        set_part(N, u.z, IdT());
+        set_part(N, u.w, IdT());
+      }
+    }
+    __syncwarp();
   };
   for (uint32_t p = 0;; p ^= 1) {
     const uint32_t row = s_row[p];
@@ -116,117 +193,97 @@ __global__ void __launch_bounds__(kThreads, 6) k_rows(RowJob J) {
     }
     if (tid == 0) s_row[p ^ 1] = atomicAdd(&J.ctl->next_row, 1u);
     const uint32_t x = row - I.row0;
-    uint32_t o = 0, end = 0;
+    uint32_t o = 0, deg = 0;
     if (x < I.nv) {  // (rows of an instance are padded to whole chunks)
       o = I.off[x];
-      end = I.off[x + 1] - o;
+      deg = I.off[x + 1] - o;
     }
-    if (end == 0) {
+    if (deg == 0) {
       if (tid == 0 && x < I.nv) I.cnt[x] = 0;
     } else {
-      if (tid == 0) s_push[0] = 0;
-      for (uint32_t i = tid; i < end; i += kThreads) {
+      const uint32_t words = I.words, quads = words / 4;
+      if (tid == 0) { s_cnt[0] = 0; s_len[0] = 0; cand += deg; }
+      for (uint32_t i = tid; i < deg; i += T) {
         const uint32_t z = I.adj[o + i];
-        atomicOr(V + (z >> 5), 1u << (z & 31));
-        put(i, z);
+        atomicOr(N + (z >> 5), 1u << (z & 31));
       }
-      if (tid == 0) { cand += end; s_log[0] += end; }
       __syncthreads();
-      uint32_t start = 0, lvl = 0;
-      while (lvl < I.max_iters) {
-        uint32_t* push = s_push + lvl % 3;
-        if (tid == 0) s_push[(lvl + 1) % 3] = 0;
-        for (uint32_t b = start + warp * 32; b < end; b += kThreads) {
-          const uint32_t i = b + lane;
-          uint4 ra = {0, 0, 0, 0}, rb = ra;
-          uint32_t y = 0;
-          if (i < end) {
-            y = i < kRowQueue ? sq[i] : gq[i];
-            rec_load((const uint4*)I.rec, y, ra, rb, IdT());
-          }
-          const uint32_t deg = rec_deg(ra, IdT());
-          const uint32_t inl = min(deg, kRecInline);
-          uint32_t fo = 0, r = 0;
-          if (deg > kRecInline) {  // (a 16-bit degree field saturates)
-            fo = I.off[y];
-            r = I.off[y + 1] - fo - kRecInline;
-            fo += kRecInline;
-          }
-          cand += inl + r;
-          uint32_t m = 0;
-          const uint32_t most = __reduce_max_sync(0xffffffffu, inl);
-#pragma unroll
-          for (int s = 0; s < (int)kRecInline; ++s) {
-            if (s >= most) break;
-            if (s < inl) {
-              const uint32_t z = rec_id(ra, rb, s, IdT()), bit = 1u << (z & 31);
-              if (!(V[z >> 5] & bit) && !(atomicOr(V + (z >> 5), bit) & bit)) m |= 1u << s;
+      uint32_t lvl = 0, total = 0, turn = 0;
+      uint4* const n4 = (uint4*)N;
+      uint4* const out = (uint4*)(I.bits + (size_t)x * words);
+      for (;; ++lvl) {
+        uint32_t listed = 0, wait = 0;  // wait: this thread's steps with bits not yet listed
+        for (uint32_t round = 0;; ++round, turn ^= 1) {
+          if (tid == 0) s_len[turn ^ 1] = 0;
+          uint32_t got = 0;
+          uint4 nd = {0, 0, 0, 0};
+          if (round == 0 && tid < quads) nd = n4[tid];
+          for (uint32_t g = warp * 32, step = 1; g < quads; g += T, step <<= 1) {
+            const uint32_t w = g + lane;
+            uint4 d = nd;
+            if (round == 0) {
+              nd = w + T < quads ? n4[w + T] : uint4{0, 0, 0, 0};
+              if (d.x | d.y | d.z | d.w) {
+                n4[w] = uint4{0, 0, 0, 0};
+                const uint4 s = sm4[w], ns = __ldg((const uint4*)I.ns + w);
+                d.x &= ~s.x; d.y &= ~s.y; d.z &= ~s.z; d.w &= ~s.w;
+                sm4[w] = uint4{s.x | d.x, s.y | d.y, s.z | d.z, s.w | d.w};
+                got += __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+                d.x &= ns.x; d.y &= ns.y; d.z &= ns.z; d.w &= ns.w;
+                if (lvl >= I.max_iters) d = uint4{0, 0, 0, 0};
+              }
+            } else if (wait & step) {
+              d = out[w];
+            }
+            if (!__any_sync(0xffffffffu, d.x | d.y | d.z | d.w)) continue;
+            const uint32_t c = __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+            const uint32_t in = warp_incl_scan(c, lane);
+            uint32_t at = 0;
+            if (lane == 31) at = atomicAdd(s_len + turn, in);
+            at = __shfl_sync(0xffffffffu, at, 31) + in - c;
+            auto put = [&](uint32_t& m, uint32_t base) {
+              while (m && at < kRowList) {
+                list[at++] = (IdT)(base + __ffs(m) - 1);
+                m &= m - 1;
+              }
+            };
+            put(d.x, w * 128); put(d.y, w * 128 + 32); put(d.z, w * 128 + 64); put(d.w, w * 128 + 96);
+            wait &= ~step;
+            if (d.x | d.y | d.z | d.w) {
+              out[w] = d;
+              wait |= step;
             }
           }
-          {
-            const uint32_t c = __popc(m), in = warp_incl_scan(c, lane);
-            const uint32_t tot = __shfl_sync(0xffffffffu, in, 31);
-            if (tot) {
-              uint32_t at = 0;
-              if (lane == 0) at = atomicAdd(push, tot);
-              at = end + __shfl_sync(0xffffffffu, at, 0) + in - c;
-#pragma unroll
-              for (int s = 0; s < (int)kRecInline; ++s)
-                if (m >> s & 1u) put(at++, rec_id(ra, rb, s, IdT()));
-            }
-          }
-          if (__any_sync(0xffffffffu, r)) {
-            const uint32_t in = warp_incl_scan(r, lane);
-            const uint32_t R = __shfl_sync(0xffffffffu, in, 31);
-            const uint32_t fe = fo - (in - r);  // edge e of the strip is adj[fe_owner + e]
-            for (uint32_t e0 = 0; e0 < R; e0 += 32) {
-              const uint32_t e = e0 + lane;
-              uint32_t ow = 0;  // lanes whose inclusive prefix is <= e
-#pragma unroll
-              for (int st = 16; st > 0; st >>= 1) {
-                const uint32_t v = __shfl_sync(0xffffffffu, in, ow + st - 1);
-                if (v <= e) ow += st;
-              }
-              const uint32_t a = __shfl_sync(0xffffffffu, fe, ow & 31);
-              uint32_t z = 0;
-              bool win = false;
-              if (e < R) {
-                z = I.adj[a + e];
-                const uint32_t bit = 1u << (z & 31);
-                win = !(V[z >> 5] & bit) && !(atomicOr(V + (z >> 5), bit) & bit);
-              }
-              const uint32_t bal = __ballot_sync(0xffffffffu, win);
-              if (bal) {
-                uint32_t at = 0;
-                if (lane == 0) at = atomicAdd(push, (uint32_t)__popc(bal));
-                at = end + __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1));
-                if (win) put(at, z);
-              }
-            }
-          }
+          got = __reduce_add_sync(0xffffffffu, got);
+          if (lane == 0 && got) atomicAdd(s_cnt + (lvl & 1), got);
+          __syncthreads();
+          const uint32_t len = s_len[turn], n = min(len, kRowList);
+          if (round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
+          listed |= len;
+          if (len == 0) break;
+          for (uint32_t b = warp * 32; b < n; b += T) expand(list + b, min(32u, n - b));
+          __syncthreads();
+          if (len <= kRowList) break;
         }
-        __syncthreads();
-        const uint32_t n = *push;
+        const uint32_t n = s_cnt[lvl & 1];
         if (n == 0) break;
-        ++lvl;
+        total += n;
         if (tid == 0) {
           if (lvl < kRowLog) s_log[lvl] += n;
           else if (lvl < I.log_cap) atomicAdd(I.log + lvl, (unsigned long long)n);
         }
-        start = end;
-        end += n;
+        if (listed == 0) { ++lvl; break; }  // nothing of this delta joins any edge
+        turn ^= 1;
       }
-      if (tid == 0) {
-        atomicMax(&J.inst[q].last, lvl);
-        I.cnt[x] = end;
-        atomicAdd(J.csum + row / kRowChunk, end);
+      if (tid == 0) {  // (the delta of iteration lvl - 1 was the last that is not empty)
+        atomicMax(&J.inst[q].last, lvl - 1);
+        I.cnt[x] = total;
+        atomicAdd(J.csum + row / kRowChunk, total);
       }
       // the row's bit set out, and cleared for the next row
-      uint4* out = (uint4*)(I.bits + (size_t)x * I.words);
-      uint4* v4 = (uint4*)V;
-      for (uint32_t i = tid; i < I.words / 4; i += kThreads) {
-        out[i] = v4[i];
-        v4[i] = uint4{0, 0, 0, 0};
+      for (uint32_t i = tid; i < quads; i += T) {
+        out[i] = sm4[i];
+        sm4[i] = uint4{0, 0, 0, 0};
       }
     }
     __syncthreads();
@@ -328,27 +385,42 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
 }
 
 // ------------------------------------------------------------------ launchers
-uint32_t row_smem(uint32_t vwords, int id_bytes) { return vwords * 4 + kRowQueue * id_bytes; }
+static uint32_t row_smem(uint32_t vwords, int id_bytes, int threads) {
+  return 2 * vwords * 4 + (threads / 32) * 32 * 4 + kRowList * id_bytes;
+}
+// Threads per CTA: a CTA waits twice per iteration for its slowest warp, so the
+// smaller the better while its bit sets leave room for enough CTAs per SM
+// (64 / 128 / 256 / 512 threads, whole call: R-MAT 2^17 / 400k 7.3 / 7.0 / 7.2 /
+// 8.4 ms; R-MAT 2^19 / 400k, 31 KB of bit sets, 22.7 / 16.8 / 15.2 / 16.9 ms;
+// the 64-query batch 15.8 / 16.0 / 18.7 / 24.4 ms).
+static int row_threads(uint32_t vwords) { return vwords <= 2048 ? 128 : vwords <= 4096 ? 256 : 512; }
 
-template <typename IdT>
-static int rows_occ(uint32_t smem) {
-  static int max_set = 0;  // (the attribute is per process and device, raised once)
-  if (!max_set) {
-    cudaFuncSetAttribute(k_rows<IdT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemMax);
-    max_set = 1;
-  }
-  int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rows<IdT>, kThreads, smem);
-  return occ;
+template <typename F>
+static auto rows_kernel(uint32_t vwords, int id_bytes, F f) {
+  const int t = row_threads(vwords);
+  if (id_bytes == 2) return f(k_rows<uint16_t, 128, 10>);  // (at most 2,048 words)
+  return t == 128   ? f(k_rows<uint32_t, 128, 10>)
+         : t == 256 ? f(k_rows<uint32_t, 256, 5>)
+                    : f(k_rows<uint32_t, 512, 2>);
 }
 int occupancy_rows(int id_bytes, uint32_t vwords) {
-  const uint32_t smem = row_smem(vwords, id_bytes);
-  return id_bytes == 2 ? rows_occ<uint16_t>(smem) : rows_occ<uint32_t>(smem);
+  const int t = row_threads(vwords);
+  const uint32_t smem = row_smem(vwords, id_bytes, t);
+  return rows_kernel(vwords, id_bytes, [&](auto k) {
+    if (smem > 48 * 1024)
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, t, smem);
+    return occ;
+  });
 }
 void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s) {
-  const uint32_t smem = row_smem(J.vwords, id_bytes);
-  if (id_bytes == 2) k_rows<uint16_t><<<grid, kThreads, smem, s>>>(J);
-  else k_rows<uint32_t><<<grid, kThreads, smem, s>>>(J);
+  const int t = row_threads(J.vwords);
+  const uint32_t smem = row_smem(J.vwords, id_bytes, t);
+  rows_kernel(J.vwords, id_bytes, [&](auto k) {
+    k<<<grid, t, smem, s>>>(J);
+    return 0;
+  });
 }
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s) {
   k_row_plan<<<n_inst, 1024, 0, s>>>(J);
@@ -357,12 +429,29 @@ template <typename K>
 void launch_row_expand(const RowJob& J, int grid, cudaStream_t s) {
   k_row_expand<K><<<grid, kThreads, 0, s>>>(J);
 }
-void launch_row_records(const uint32_t* off, const uint32_t* adj, uint32_t nv, void* rec,
-                        int id_bytes, int grid, cudaStream_t s) {
-  if (id_bytes == 2) k_row_records<uint16_t><<<grid, kThreads, 0, s>>>(off, adj, nv, (uint16_t*)rec);
-  else k_row_records<uint32_t><<<grid, kThreads, 0, s>>>(off, adj, nv, (uint32_t*)rec);
+size_t row_units(uint64_t ne, uint32_t nv, int id_bytes) {
+  const uint64_t U = 16 / id_bytes;
+  return (size_t)((ne + (U - 1) * ((uint64_t)nv + 1)) / U + 1);
+}
+template <typename K>
+void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
+                       const uint32_t* adj, uint32_t nv, void* rec, uint32_t* ns, uint32_t words,
+                       void* units, int id_bytes, int grid, cudaStream_t s) {
+  if (id_bytes == 2)
+    k_row_layout<K, uint16_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
+                                                        words, (uint16_t*)units);
+  else
+    k_row_layout<K, uint32_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
+                                                        words, (uint32_t*)units);
 }
 template void launch_row_expand<uint32_t>(const RowJob&, int, cudaStream_t);
 template void launch_row_expand<unsigned long long>(const RowJob&, int, cudaStream_t);
+template void launch_row_layout<uint32_t>(const uint32_t*, uint32_t, uint32_t, const uint32_t*,
+                                          const uint32_t*, uint32_t, void*, uint32_t*, uint32_t,
+                                          void*, int, int, cudaStream_t);
+template void launch_row_layout<unsigned long long>(const unsigned long long*, uint32_t, uint32_t,
+                                                    const uint32_t*, const uint32_t*, uint32_t,
+                                                    void*, uint32_t*, uint32_t, void*, int, int,
+                                                    cudaStream_t);
 
 }  // namespace wg

@@ -68,8 +68,13 @@ int occupancy_rows(int id_bytes, uint32_t vwords);
 void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
-void launch_row_records(const uint32_t* off, const uint32_t* adj, uint32_t nv, void* rec,
-                        int id_bytes, int grid, cudaStream_t s);
+// adjacency units of a relation: their number, and the layout of vertex records
+// (32 bytes each), out-edge bit set (words) and further units (16 bytes each)
+size_t row_units(uint64_t ne, uint32_t nv, int id_bytes);
+template <typename K>
+void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
+                       const uint32_t* adj, uint32_t nv, void* rec, uint32_t* ns, uint32_t words,
+                       void* units, int id_bytes, int grid, cudaStream_t s);
 
 // relation load and result extraction
 template <typename K>
