@@ -268,6 +268,26 @@ constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are
 constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
 constexpr uint32_t kRowSmemMax = 200 * 1024;
 
+// ---------------------------------------------------------------- triangle counting
+struct TriCtl {
+  unsigned long long paths, hits;  // two-paths (a,b,c); those with E(c,a)
+  uint32_t room, next, tasks, pad;
+};
+struct TriJob {  // wg_kern_tri.cu
+  TriCtl* ctl;                     // cleared, with ideg, before the launch
+  uint32_t *ideg, *ioff, *ifill, *iadj;  // the transposed edges
+  const uint32_t *off, *adj;
+  uint2* task;                     // tri_tasks() of them at most
+  uint32_t nv, words;
+  uint32_t chunk;                  // neighbours per task, at least kTriChunk
+};
+constexpr uint32_t kTriChunk = 64;
+__host__ __device__ inline unsigned long long tri_tasks(unsigned long long ne, uint32_t nv) {
+  return 2ull * nv + 2 * ne / kTriChunk;
+}
+constexpr uint32_t kTriSmem = 200 * 1024;
+constexpr uint32_t kTriMaxVertices = 1500000;  // their bit set fits a CTA's shared memory
+
 // Shared-memory index with one pad word per 32: threads that walk their own
 // contiguous run (blocked order, stride 16 words) then hit distinct banks.
 __device__ __forceinline__ uint32_t pad32(uint32_t i) { return i + (i >> 5); }

@@ -13,6 +13,7 @@ struct Stage;
 struct Dev;
 struct Inst;
 struct RowJob;
+struct TriJob;
 
 // sorted-array stages (wg_kern_sort.cu); K = uint32_t or unsigned long long
 template <typename K> void launch_sort_hist(Stage* st, int grid, cudaStream_t s);
@@ -75,6 +76,10 @@ template <typename K>
 void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
                        const uint32_t* adj, uint32_t nv, void* rec, uint32_t* ns, uint32_t words,
                        void* units, int id_bytes, int grid, cudaStream_t s);
+
+// triangle counting by set intersection (wg_kern_tri.cu): transpose and count
+template <typename K>
+void launch_tri(const K* E, uint32_t ne, uint32_t w, const TriJob& J, int sms, cudaStream_t s);
 
 // relation load and result extraction
 template <typename K>
