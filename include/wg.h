@@ -14,7 +14,7 @@
  * the full relation (Secs. Sorted-Array Pipeline and Asynchronous Fixpoint
  * Engine).  The loop runs on the device; the host sees only the end result.
  * TC never changes a tuple's source, so a plain TC query (no flag, device loop,
- * not profiled) over at most 2^18 vertices runs source by source: each row's
+ * not profiled) over at most 786,432 vertices runs source by source: each row's
  * delta and full relation are bit sets in shared memory, and duplicate removal,
  * set difference and merge are one bit test and set.  The result, iteration
  * count, per-iteration sizes and candidate count are the same.

@@ -249,6 +249,7 @@ struct RowInst {
   uint32_t max_iters, log_cap;
   uint32_t last;                // last iteration with new tuples
   uint32_t fits;                // the result fits `out`
+  uint32_t n_big, pad;          // rows k_rows_small left to k_rows
   unsigned long long n_total, cand;
 };
 struct RowCtl {
@@ -262,11 +263,20 @@ struct RowJob {
   uint32_t* csum;               // tuples per chunk of kRowChunk rows (cleared before)
   unsigned long long* cbase;    // their exclusive prefix within the instance
   uint32_t nrows, vwords;       // vwords: words of the widest instance's rows
+  // small rows first (one instance): the rows left to k_rows, of which `bits`
+  // has room for `slots`, and kSmallRow ids per row (or NULL, 0, NULL)
+  uint32_t* rows;
+  uint32_t* small;
+  uint32_t slots, pad;
 };
 constexpr uint32_t kRowChunk = 256;
 constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are expanded
 constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
-constexpr uint32_t kRowSmemMax = 200 * 1024;
+constexpr uint32_t kRowSmemMax = 216 * 1024;
+// Tuples of a row k_rows_small takes (128 / 256 / 512, whole call: ER 400,000 /
+// 360,000 1.74 / 1.08 / 1.08 ms, R-MAT 2^19 / 400k 12.6 / 12.7 / 13.1 ms).
+constexpr uint32_t kSmallRow = 256;
+constexpr uint32_t kRowMaxVertices = 786432;  // two bit sets of them fit a CTA's shared memory
 
 // ---------------------------------------------------------------- triangle counting
 struct TriCtl {

@@ -313,7 +313,7 @@ struct Relation {
   uint32_t nv = 0, w = 1;
   int kb = 4;
   DBuf keys, off, adj, V;
-  DBuf rowv;                      // row fixpoints (up to kXSegMaxVertices): vertex records,
+  DBuf rowv;                      // row fixpoints (up to kRowMaxVertices): vertex records,
   size_t o_ns = 0, o_units = 0;   // out-edge bit set and adjacency units at these offsets
   DBuf htab;                      // hash-join ablation: E in a linear-probing table (lazy)
   unsigned long long hmask = 0;
@@ -321,6 +321,11 @@ struct Relation {
   int id_bytes() const { return nv <= 65536u ? 2 : 4; }  // of a rank in the units
   uint32_t row_words() const { return (nv + 127) / 128 * 4; }  // of a row's bit set
   size_t row_bits() const { return (size_t)nv * row_words() * 4; }  // bytes of all rows' sets
+  // Single queries over wide relations take the small rows apart (k_rows_small):
+  // with 32-bit ranks, where a row's bit set takes 8 KB and more (sparse ER
+  // 400,000 / 360,000: 15.5 -> 1.1 ms; dense R-MAT 2^19 / 400k: no change).
+  bool small_rows() const { return nv > 65536u; }
+  bool no_rows = false;           // the rows' bit sets did not fit the budget
   void row_inst(RowInst* I) const {
     *I = RowInst{};
     I->off = (const uint32_t*)off.p; I->adj = (const uint32_t*)adj.p;
@@ -355,7 +360,7 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
   launch_csr<K>((const K*)ke.p, ne, R->nv, R->w, (uint32_t*)R->off.p, (uint32_t*)R->adj.p,
                 grid_of(c, 4), c->stream);
   CK(cudaGetLastError());
-  if (R->nv <= kXSegMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
+  if (R->nv <= kRowMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
     R->o_ns = round_up((size_t)R->nv * 32);
     R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
     TRY(R->rowv.get(c, R->o_units + row_units(ne, R->nv, R->id_bytes()) * 16));
@@ -618,12 +623,13 @@ struct Engine : EngineBase {
   uint32_t sort_mode_;               // enum wg_sort_mode (x-grouped engines)
   uint32_t side_;                    // side run of Full: 0 never, 1 with few candidates, 2 always
   bool rows_ = false;                // row-by-row TC (wg_kern_rows.cu): none of the stages below
-  DBuf row_meta, row_bits;
+  DBuf row_meta, row_bits, row_small;
   RowInst ri{};
   RowJob job{};
   size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
   int id_bytes = 2, g_rows = 0;
   bool expand_only = false;          // the rows are done; the result waits for a larger buffer
+  bool row_short = false;            // the long rows' bit sets did not fit the budget
   Engine(wg_ctx* ctx, bool single_, uint32_t n, uint32_t bits, uint32_t logcap, bool fuse_,
          bool xseg_, bool copy_back_ = false, bool hash_join_ = false, uint32_t side = 0)
       : c(ctx), single(single_), fuse(fuse_), xseg(xseg_), n_slots(n), bits_(bits),
@@ -661,7 +667,7 @@ struct Engine : EngineBase {
     ev_done = nullptr;
     DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                    &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b, &xsum_b,
-                   &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits};
+                   &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_small};
     for (DBuf* b : all) b->release(c);
     capC = capF = capR = capG = 0;
     mix_tiles = 0;
@@ -893,6 +899,7 @@ struct Engine : EngineBase {
     const uint32_t nv = Rl->nv, words = Rl->row_words();
     const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
     const uint32_t nlog = std::min<uint32_t>(1u << 16, nv + 2);
+    const bool small = Rl->small_rows();
     id_bytes = Rl->id_bytes();
     g_rows = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(id_bytes, words)),
                                      std::max<uint32_t>(nv, 1));
@@ -903,9 +910,17 @@ struct Engine : EngineBase {
                  o_log = at(end, (size_t)nlog * 8);
     row_clear = end;
     const size_t o_inst = at(end, sizeof(RowInst)), o_base = at(end, (size_t)nch * 8),
-                 o_cnt = at(end, (size_t)nv * 4);
+                 o_cnt = at(end, (size_t)nv * 4), o_rows = at(end, small ? (size_t)nv * 4 : 0);
     TRY(row_meta.get(c, end));
-    TRY(row_bits.get(c, std::max<size_t>(Rl->row_bits(), 16)));
+    // bit sets of every row, or (small rows apart) of as many as a quarter of
+    // the free budget holds: more are made room for when they turn up (settle)
+    size_t sets = std::max<size_t>(Rl->row_bits(), 16);
+    if (small) {
+      TRY(row_small.get(c, (size_t)nv * kSmallRow * 4));
+      const size_t room = (c->budget - std::min(c->budget, c->used) + row_bits.bytes) / 4;
+      sets = std::max(std::min(sets, room), (size_t)words * 4);
+    }
+    TRY(row_bits.get(c, sets));
     if (wantF > capF) {
       TRY(F[0].get(c, wantF * sizeof(K)));
       capF = wantF;
@@ -919,11 +934,29 @@ struct Engine : EngineBase {
     job.ctl = (RowCtl*)(m + o_ctl); job.inst = (RowInst*)(m + o_inst);
     job.csum = (uint32_t*)(m + o_sum); job.cbase = (unsigned long long*)(m + o_base);
     job.nrows = nv; job.vwords = words;
+    if (small) {
+      job.rows = (uint32_t*)(m + o_rows);
+      job.small = (uint32_t*)row_small.p;
+      job.slots = (uint32_t)std::min<size_t>(nv, row_bits.bytes / ((size_t)words * 4));
+    }
     log_cap = nlog;
     expand_only = false;
     hi[0] = Inst{};
     hi[0].state = INST_ACTIVE;
     hi[0].log = ri.log;
+    return WG_OK;
+  }
+  // Room for the bit sets of the long rows the last run found.
+  int rows_room() {
+    AllocScope scope(c, st);
+    const size_t set = (size_t)ri.words * 4;
+    row_bits.release(c);
+    row_short = true;
+    TRY(row_bits.get(c, std::min((size_t)ri.n_big + ri.n_big / 16 + 64, (size_t)ri.nv) * set));
+    row_short = false;
+    ri.bits = (uint32_t*)row_bits.p;
+    job.slots = (uint32_t)std::min<size_t>(ri.nv, row_bits.bytes / set);
+    ri.n_big = 0; ri.last = 0; ri.cand = 0;
     return WG_OK;
   }
   int rows_launch() {
@@ -933,6 +966,10 @@ struct Engine : EngineBase {
     CK(cudaMemcpyAsync(job.inst, &ri, sizeof(ri), cudaMemcpyHostToDevice, st));
     if (!expand_only) {
       CK(cudaMemsetAsync(row_meta.p, 0, row_clear, st));
+      if (job.rows) {
+        launch_rows_small(job, grid_of(c, 6), st);
+        launches_issued += 2;  // (and k_row_expand_small)
+      }
       if (ri.nv) launch_rows(job, id_bytes, g_rows, st);
       launch_row_plan(job, 1, st);
       launches_issued += ri.nv ? 2 : 1;
@@ -950,6 +987,11 @@ struct Engine : EngineBase {
     Inst& I = hi[0];
     I.n_full = ri.n_total;
     I.cand_total = ri.cand;
+    if (job.rows && ri.n_big > job.slots) {  // more long rows than bit sets: start over
+      ++regrows;
+      *again = true;
+      return rows_room();
+    }
     if (!ri.fits) {
       h.ctl.need_full = ri.n_total;
       ++regrows;
@@ -1243,6 +1285,7 @@ struct Engine : EngineBase {
   int grow() {
     unsigned long long wc, wf, wr;
     grow_target(&wc, &wf, &wr);
+    if (rows_ && row_short) return rows_room();
     if (rows_) {  // the size is exact; the result buffer holds nothing yet: free it first
       wf = h.ctl.need_full + h.ctl.need_full / 16 + 4096;
       AllocScope scope(c, st);
@@ -1257,7 +1300,7 @@ struct Engine : EngineBase {
   size_t held() const override {
     const DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                          &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b,
-                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits};
+                         &xsum_b, &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_small};
     size_t b = 0;
     for (const DBuf* x : all) b += x->bytes;
     return b;
@@ -1268,6 +1311,7 @@ struct Engine : EngineBase {
   size_t grow_peak() const override {
     unsigned long long wantC, wantF, wantR;
     grow_target(&wantC, &wantF, &wantR);
+    if (rows_ && row_short) return held() + ((size_t)ri.n_big + 64) * ri.words * 4;
     if (rows_)
       return held() - F[0].bytes + round_up((h.ctl.need_full + h.ctl.need_full / 16 + 4096) * sizeof(K));
     wantC = std::max<unsigned long long>(wantC, 1ull << 16);
@@ -1477,6 +1521,9 @@ static int single_start(wg_ctx* c, Query* q) {
   return WG_OK;
 }
 
+extern "C" {
+static int single_begin(wg_ctx* c, Query* q);
+}
 template <typename K>
 static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget = false) {
   auto* E = static_cast<Engine<K>*>(q->eng);
@@ -1492,6 +1539,18 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     }
     bool again = false;
     int rc = E->settle(&again);
+    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->row_short) {
+      // the long rows' bit sets do not fit: the sorted-array pipeline takes it
+      cudaGetLastError();
+      q->rel->no_rows = true;
+      q->own.reset();
+      q->eng = nullptr;
+      rc = single_begin(c, q);
+      if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
+      q->state = WG_FAILED;
+      q->error = rc;
+      return rc;
+    }
     if (rc != WG_OK && pause_on_budget && (rc == WG_E_BUDGET || rc == WG_E_NOMEM)) {
       cudaGetLastError();  // the pools stay whole at their old capacities
       q->solo_wait = true;
@@ -2057,19 +2116,22 @@ static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R) {
 // a per-stage profile, the size of the candidate buffers), over a relation
 // whose bit sets take at most half of the free budget -- the sorted
 // pipeline needs more than twice the result, so whatever fits there fits here.
-static bool row_fits(wg_ctx* c, const Query* q) {
+static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
   const Relation* R = q->rel;
   if (q->kind != WG_TC || q->opts.flags || q->opts.reserve_cand || !R->rowv.p)
     return false;
   size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
   for (auto& e : c->idle) idle += e->held();
-  return R->row_bits() <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
+  // (small rows apart: their lists, and bit sets for whatever is left)
+  const size_t need = R->small_rows() && !batched ? (size_t)R->nv * kSmallRow * 8 : R->row_bits();
+  return need <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
 }
 static bool row_query(wg_ctx* c, const Query* q) {
-  return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && row_fits(c, q);
+  return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->rel->no_rows &&
+         row_fits(c, q, false);
 }
 // (loop and profile are ignored in batches)
-static bool row_batched(wg_ctx* c, const Query* q) { return row_fits(c, q); }
+static bool row_batched(wg_ctx* c, const Query* q) { return row_fits(c, q, true); }
 
 
 // Submitted row-by-row TC queries: a lane runs the rows of many relations of

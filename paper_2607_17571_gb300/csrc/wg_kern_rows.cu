@@ -179,9 +179,13 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
     }
     __syncwarp();
   };
+  // listed rows (k_rows_small's leftovers): their bit sets lie in list order
+  const uint32_t nrows = J.rows ? J.inst->n_big : J.nrows;
+  if (J.rows && nrows > J.slots) return;  // no room: the host grows it and starts over
   for (uint32_t p = 0;; p ^= 1) {
-    const uint32_t row = s_row[p];
-    if (row >= J.nrows) break;
+    const uint32_t at_row = s_row[p];
+    if (at_row >= nrows) break;
+    const uint32_t row = J.rows ? J.rows[at_row] : at_row;
     const uint32_t q = J.chunk_inst ? J.chunk_inst[row / kRowChunk] : 0u;
     if (q != cur) {
       __syncthreads();
@@ -210,7 +214,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
       __syncthreads();
       uint32_t lvl = 0, total = 0, turn = 0;
       uint4* const n4 = (uint4*)N;
-      uint4* const out = (uint4*)(I.bits + (size_t)x * words);
+      uint4* const out = (uint4*)(I.bits + (size_t)(J.rows ? at_row : x) * words);
       for (;; ++lvl) {
         uint32_t listed = 0, wait = 0;  // wait: this thread's steps with bits not yet listed
         for (uint32_t round = 0;; ++round, turn ^= 1) {
@@ -291,6 +295,152 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   if (cur != 0xFFFFFFFFu) flush();
 }
 
+// Rows of at most kSmallRow tuples, for relations whose bit sets are wide (one
+// instance, 32-bit ranks): one warp per row, the reached vertices in a hash set
+// and a list in shared memory, the sorted list out to small + row * kSmallRow.  A row
+// that turns out longer is listed for k_rows.  Without it a sparse relation pays
+// a bit set per row to hold a few vertices: ER 400,000 vertices / 360,000 edges,
+// 335,000 rows of 9 tuples on average against bit sets of 42 KB, 15.5 ms on the
+// sorted-array pipeline, 1.08 ms here (0.39 this kernel, 0.38 k_rows).  Bound by
+// the latency of the gathered CSR entries.
+__global__ void __launch_bounds__(kThreads) k_rows_small(RowJob J) {
+  constexpr uint32_t kSlots = 2 * kSmallRow, kNone = 0xFFFFFFFFu;
+  static_assert(kSlots >= kSmallRow + 64 && (kSlots & (kSlots - 1)) == 0, "the probes must end");
+  __shared__ uint32_t s_hash[kWarps][kSlots], s_list[kWarps][kSmallRow], s_end[kWarps][kSmallRow + 1];
+  __shared__ unsigned long long s_log[kRowLog];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* hash = s_hash[warp];
+  uint32_t* list = s_list[warp];
+  uint32_t* ends = s_end[warp];  // list length after each level
+  const RowInst& I = *J.inst;
+  const uint32_t* off = I.off;
+  const uint32_t* adj = I.adj;
+  const uint32_t nv = I.nv, max_iters = I.max_iters;
+  for (uint32_t i = tid; i < kRowLog; i += kThreads) s_log[i] = 0;
+  for (uint32_t i = lane; i < kSlots; i += 32) hash[i] = kNone;
+  __syncthreads();
+  unsigned long long cand = 0;
+  uint32_t last = 0;
+  for (uint32_t x = blockIdx.x * kWarps + warp; x < nv; x += gridDim.x * kWarps) {
+    const uint32_t o = off[x], deg = off[x + 1] - o;
+    if (deg == 0) {
+      if (lane == 0) I.cnt[x] = 0;
+      continue;
+    }
+    uint32_t n = 0, lvl = 0, mine = lane == 0 ? deg : 0;
+    // adds the lanes' vertices z that are new to the list; false when it is full
+    auto add = [&](uint32_t z, bool valid) {
+      bool fresh = false;
+      if (valid) {
+        uint32_t h = (z * 2654435761u) >> 16 & (kSlots - 1);
+        for (;;) {  // (at most kSmallRow + 32 of the slots are taken)
+          const uint32_t old = atomicCAS(hash + h, kNone, z);
+          if (old == kNone) { fresh = true; break; }
+          if (old == z) break;
+          h = (h + 1) & (kSlots - 1);
+        }
+      }
+      const uint32_t m = __ballot_sync(0xffffffffu, fresh);
+      const uint32_t at = n + __popc(m & ((1u << lane) - 1));
+      n += __popc(m);
+      if (n > kSmallRow) return false;
+      if (fresh) list[at] = z;
+      return true;
+    };
+    bool fits = deg <= kSmallRow;
+    for (uint32_t i = 0; i < deg && fits; i += 32) fits = add(i + lane < deg ? adj[o + i + lane] : 0u, i + lane < deg);
+    uint32_t start = 0;
+    while (fits) {
+      __syncwarp();
+      if (lane == 0) ends[lvl] = n;
+      const uint32_t end = n;
+      if (lvl >= max_iters) { ++lvl; break; }
+      for (uint32_t b = start; b < end && fits; b += 32) {
+        uint32_t fo = 0, d = 0;
+        if (b + lane < end) {
+          const uint32_t y = list[b + lane];
+          fo = off[y];
+          d = off[y + 1] - fo;
+        }
+        const uint32_t in = warp_incl_scan(d, lane), tot = __shfl_sync(0xffffffffu, in, 31);
+        mine += d;
+        const uint32_t fe = fo - (in - d);  // edge e of the strip is adj[fe of its vertex + e]
+        for (uint32_t e0 = 0; e0 < tot && fits; e0 += 32) {
+          const uint32_t e = e0 + lane;
+          uint32_t ow = 0;  // lanes whose edges all come before e
+#pragma unroll
+          for (int st = 16; st > 0; st >>= 1) {
+            const uint32_t v = __shfl_sync(0xffffffffu, in, ow + st - 1);
+            if (v <= e) ow += st;
+          }
+          const uint32_t a = __shfl_sync(0xffffffffu, fe, ow & 31);
+          fits = add(e < tot ? adj[a + e] : 0u, e < tot);
+        }
+      }
+      ++lvl;
+      if (n == end) break;  // an empty delta
+      start = end;
+    }
+    if (fits) {
+      // the list in order: each lane ranks its vertices against all
+      __syncwarp();
+      uint32_t* to = J.small + (size_t)x * kSmallRow;
+      for (uint32_t i = lane; i < n; i += 32) {
+        const uint32_t v = list[i];
+        uint32_t r = 0;
+        for (uint32_t j = 0; j < n; ++j) r += list[j] < v;
+        to[r] = v;
+      }
+      cand += mine;
+      last = max(last, lvl - 1);
+      for (uint32_t l = lane; l < lvl; l += 32) {
+        const unsigned long long c = ends[l] - (l ? ends[l - 1] : 0u);
+        if (l < kRowLog) atomicAdd(s_log + l, c);
+        else if (l < I.log_cap) atomicAdd(I.log + l, c);
+      }
+      if (lane == 0) {
+        I.cnt[x] = n;
+        atomicAdd(J.csum + x / kRowChunk, n);
+      }
+    } else if (lane == 0) {
+      J.rows[atomicAdd(&J.inst->n_big, 1u)] = x;
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < kSlots; i += 32) hash[i] = kNone;
+    __syncwarp();
+  }
+  for (int o = 16; o > 0; o >>= 1) cand += __shfl_xor_sync(0xffffffffu, cand, o);
+  if (lane == 0) {
+    if (cand) atomicAdd(&J.inst->cand, cand);
+    atomicMax(&J.inst->last, last);
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < kRowLog; i += kThreads)
+    if (s_log[i] && i < I.log_cap) atomicAdd(I.log + i, s_log[i]);
+}
+
+// Small rows -> sorted packed keys: a warp takes 32 rows.
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_row_expand_small(RowJob J) {
+  const uint32_t lane = threadIdx.x & 31;
+  const RowInst& I = *J.inst;
+  if (!I.fits) return;
+  for (uint32_t r = (blockIdx.x * kThreads + threadIdx.x) & ~31u; r < I.nv; r += gridDim.x * kThreads) {
+    const uint32_t r0 = r / kRowChunk * kRowChunk;
+    uint32_t before = 0;
+    for (uint32_t i = r0 + lane; i < r; i += 32) before += I.cnt[i];
+    before = __reduce_add_sync(0xffffffffu, before);
+    const uint32_t c = r + lane < I.nv ? I.cnt[r + lane] : 0u, in = warp_incl_scan(c, lane);
+    K* out = (K*)I.out + J.cbase[r / kRowChunk] + before;
+    for (uint32_t k = 0; k < 32; ++k) {
+      const uint32_t n = __shfl_sync(0xffffffffu, c, k), at = __shfl_sync(0xffffffffu, in, k) - n;
+      if (n > kSmallRow) continue;
+      for (uint32_t i = lane; i < n; i += 32)
+        out[at + i] = ((K)(r + k) << I.w) | J.small[(size_t)(r + k) * kSmallRow + i];
+    }
+  }
+}
+
 // Row offsets at chunk granularity, totals and the capacity check: one CTA per
 // instance scans its chunk sums in place (counts in, exclusive offsets out).
 __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
@@ -327,7 +477,7 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
   if (threadIdx.x == 0) {
     I->n_total = carry;
     // an output buffer that is too small: the expansion waits for a larger one
-    I->fits = carry <= I->out_cap ? 1u : 0u;
+    I->fits = carry <= I->out_cap && !(J.rows && I->n_big > J.slots) ? 1u : 0u;
   }
 }
 
@@ -338,8 +488,9 @@ template <typename K>
 __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
   __shared__ uint16_t buf[kWarps][2048];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t stride = gridDim.x * kWarps;
-  for (uint32_t row = blockIdx.x * kWarps + warp; row < J.nrows; row += stride) {
+  const uint32_t stride = gridDim.x * kWarps, nrows = J.rows ? J.inst->n_big : J.nrows;
+  for (uint32_t i = blockIdx.x * kWarps + warp; i < nrows; i += stride) {
+    const uint32_t row = J.rows ? J.rows[i] : i;
     const uint32_t ch = row / kRowChunk;
     const RowInst* I = J.inst + (J.chunk_inst ? J.chunk_inst[ch] : 0u);
     const uint32_t x = row - I->row0;
@@ -349,10 +500,10 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
     // this row's offset: the chunk's, and the rows before it in the chunk
     const uint32_t r0 = x / kRowChunk * kRowChunk;
     uint32_t before = 0;
-    for (uint32_t i = r0 + lane; i < x; i += 32) before += I->cnt[i];
+    for (uint32_t r = r0 + lane; r < x; r += 32) before += I->cnt[r];
     before = __reduce_add_sync(0xffffffffu, before);
     K* out = (K*)I->out + J.cbase[ch] + before;
-    const uint2* w2 = (const uint2*)(I->bits + (size_t)x * I->words);
+    const uint2* w2 = (const uint2*)(I->bits + (size_t)(J.rows ? i : x) * I->words);
     const uint32_t np = I->words / 2;
     const K hi = (K)x << I->w;
     uint2 v = lane < np ? w2[lane] : uint2{0, 0};
@@ -392,8 +543,12 @@ static uint32_t row_smem(uint32_t vwords, int id_bytes, int threads) {
 // smaller the better while its bit sets leave room for enough CTAs per SM
 // (64 / 128 / 256 / 512 threads, whole call: R-MAT 2^17 / 400k 7.3 / 7.0 / 7.2 /
 // 8.4 ms; R-MAT 2^19 / 400k, 31 KB of bit sets, 22.7 / 16.8 / 15.2 / 16.9 ms;
-// the 64-query batch 15.8 / 16.0 / 18.7 / 24.4 ms).
-static int row_threads(uint32_t vwords) { return vwords <= 2048 ? 128 : vwords <= 4096 ? 256 : 512; }
+// the 64-query batch 15.8 / 16.0 / 18.7 / 24.4 ms).  From 131,072 vertices two CTAs
+// of 512 share an SM while their bit sets allow (k_rows on ER 400,000 / 360,000:
+// 0.95 against 1.48 ms with one of 1,024).
+static int row_threads(uint32_t vwords) {
+  return vwords <= 2048 ? 128 : vwords <= 4096 ? 256 : vwords <= 12800 ? 512 : 1024;
+}
 
 template <typename F>
 static auto rows_kernel(uint32_t vwords, int id_bytes, F f) {
@@ -401,7 +556,8 @@ static auto rows_kernel(uint32_t vwords, int id_bytes, F f) {
   if (id_bytes == 2) return f(k_rows<uint16_t, 128, 10>);  // (at most 2,048 words)
   return t == 128   ? f(k_rows<uint32_t, 128, 10>)
          : t == 256 ? f(k_rows<uint32_t, 256, 5>)
-                    : f(k_rows<uint32_t, 512, 2>);
+         : t == 512 ? f(k_rows<uint32_t, 512, 2>)
+                    : f(k_rows<uint32_t, 1024, 1>);
 }
 int occupancy_rows(int id_bytes, uint32_t vwords) {
   const int t = row_threads(vwords);
@@ -425,8 +581,12 @@ void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s) {
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s) {
   k_row_plan<<<n_inst, 1024, 0, s>>>(J);
 }
+void launch_rows_small(const RowJob& J, int grid, cudaStream_t s) {
+  k_rows_small<<<grid, kThreads, 0, s>>>(J);
+}
 template <typename K>
 void launch_row_expand(const RowJob& J, int grid, cudaStream_t s) {
+  if (J.rows) k_row_expand_small<K><<<grid, kThreads, 0, s>>>(J);
   k_row_expand<K><<<grid, kThreads, 0, s>>>(J);
 }
 size_t row_units(uint64_t ne, uint32_t nv, int id_bytes) {

@@ -67,6 +67,7 @@ void launch_init_diag(Inst* inst, uint32_t first, uint32_t count, void* dpool, c
 // row-by-row closure (wg_kern_rows.cu); id_bytes: 2 for at most 2^16 vertices, else 4
 int occupancy_rows(int id_bytes, uint32_t vwords);
 void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s);
+void launch_rows_small(const RowJob& J, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
 // adjacency units of a relation: their number, and the layout of vertex records

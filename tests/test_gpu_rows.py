@@ -145,3 +145,57 @@ def test_batched_rows_equal_the_batched_pipeline():
         assert got[0] == got[1]
         for r in rels:
             r.free()
+
+
+def _small_rows_graph(nv, seed):
+    """nv vertices, most reaching few others; chains, stars and hubs whose rows
+    have 254 to 258 tuples (the small rows end at 256), a few rows of thousands
+    and one cycle."""
+    rng = np.random.default_rng(seed)
+    s, d = [np.arange(0, nv - 1, 2)], [np.arange(1, nv, 2)]
+    at = nv // 2
+    for n in (254, 255, 256, 257, 258):
+        chain = np.arange(at, at + n + 1)           # rows of n, n - 1, ... tuples
+        s.append(chain[:-1]); d.append(chain[1:])
+        at += n + 1
+        s.append(np.full(n, at)); d.append(np.arange(at + 1, at + 1 + n))  # a star of n leaves
+        at += n + 1
+    s.append(np.full(3000, at)); d.append(rng.integers(0, nv, 3000))
+    s.append(np.arange(20, 140)); d.append(np.arange(21, 141) % 140 + (np.arange(21, 141) >= 140) * 20)
+    s.append(rng.integers(0, nv, nv // 3)); d.append(rng.integers(0, nv, nv // 3))
+    return np.concatenate(s), np.concatenate(d)
+
+
+# bit sets of 8 to 96 KB (each CTA shape), the widest relation that has them and
+# the narrowest that has none
+@pytest.mark.parametrize("nv", [65_538, 140_000, 262_146, 300_000, 786_432, 786_434])
+def test_small_rows_apart(ctx, nv):
+    _check(ctx, *_small_rows_graph(nv, nv))
+
+
+@pytest.mark.parametrize("cap", [1, 3, 64, 255, 256, 257])
+def test_small_rows_iteration_caps(ctx, cap):
+    _check(ctx, *_small_rows_graph(70_000, 5), max_iters=cap)
+
+
+@pytest.mark.parametrize("rows,budget_mb", [(9000, 6000), (9000, 1900), (26_000, 1900)])
+def test_long_rows_and_the_budget(rows, budget_mb):
+    # rows of 261 tuples over 400,000 vertices need bit sets of 50 KB each.  A
+    # quarter of the budget holds them; or it does not and they are made room
+    # for when they turn up; or they do not fit at all (1.3 GB beside the small
+    # rows' 0.4) and the sorted-array pipeline takes the query
+    from oracle import oracle_tc_reach
+    from paper_2607_17571_gb300 import wg
+    i, hubs = np.arange(rows), np.arange(30_000, 30_010)
+    src = np.concatenate([np.arange(0, 400_000, 2), i, np.repeat(hubs, 260)]).astype(np.uint32)
+    dst = np.concatenate([np.arange(1, 400_001, 2), 30_000 + i % 10,
+                          np.tile(np.arange(50_000, 50_260), 10)]).astype(np.uint32)
+    n, iters, log, dg = oracle_tc_reach(src, dst, n_threads=8)
+    with wg.Context(0, mem_budget=budget_mb << 20) as c:
+        rel = c.load(src, dst)
+        for _ in range(2):
+            q = c.tc(rel)
+            st = q.wait()
+            assert (st.n_tuples, st.iterations, q.digest()) == (n, iters, dg)
+            assert q.delta_sizes() == list(log)
+            q.free()
