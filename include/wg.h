@@ -16,8 +16,10 @@
  * TC never changes a tuple's source, so a plain TC query (no flag, device loop,
  * not profiled) over at most 786,432 vertices runs source by source: each row's
  * delta and full relation are bit sets in shared memory, and duplicate removal,
- * set difference and merge are one bit test and set.  The result, iteration
- * count, per-iteration sizes and candidate count are the same.
+ * set difference and merge are one bit test and set.  A plain SG query over at
+ * most 131,072 vertices keeps such rows in device memory and gives all children
+ * of a row the same candidate set at once.  The result, iteration count,
+ * per-iteration sizes and candidate count are the same.
  *
  * Conventions for every entry point
  *  - Return value: WG_OK (0) or a negative WG_E_* code.  Nothing aborts, traps

@@ -240,6 +240,7 @@ struct RowInst {
   const void* rec;              // vertex records, 32 bytes each
   const uint32_t* ns;           // bit set of the vertices with out-edges
   const void* units;            // adjacency past the records, in 16-byte units
+  const uint32_t* mp;           // bit set of the vertices with several parents
   uint32_t* bits;               // row x's bit set: words [x * words, (x + 1) * words)
   uint32_t* cnt;                // tuples of row x
   void* out;                    // sorted packed keys
@@ -268,6 +269,7 @@ struct RowJob {
   uint32_t* rows;
   uint32_t* small;
   uint32_t slots, pad;
+  const struct SgInst* sg;      // same-generation: which pieces of the rows are valid (or NULL)
 };
 constexpr uint32_t kRowChunk = 256;
 constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are expanded
@@ -277,6 +279,30 @@ constexpr uint32_t kRowSmemMax = 216 * 1024;
 // 360,000 1.74 / 1.08 / 1.08 ms, R-MAT 2^19 / 400k 12.6 / 12.7 / 13.1 ms).
 constexpr uint32_t kSmallRow = 256;
 constexpr uint32_t kRowMaxVertices = 786432;  // two bit sets of them fit a CTA's shared memory
+
+// Same-generation over the same rows (wg_kern_sg.cu).  A row's bit set is taken
+// in pieces of 128 bits; a mask of `mw` words says which hold valid data.
+struct SgInst {
+  uint4* d[2];                  // delta rows, read and written in turn
+  uint32_t* fm;                 // valid pieces of the relation's rows (RowInst::bits)
+  uint32_t* dm[2];              // ... and of the delta rows
+  uint32_t* act;                // iteration a row was last listed for
+  uint32_t mw, pad;
+};
+struct SgCtl {                  // cleared before the launch, with fm, dm and act
+  uint32_t arrived, error;
+  uint32_t next[3], count[3];   // items claimed / listed, by iteration mod 3
+};
+struct SgJob {
+  RowJob rows;
+  SgCtl* ctl;
+  SgInst* sg;
+  uint32_t* list[2];            // rows with a non-empty delta, by iteration mod 2
+};
+constexpr int kSgThreads = 64;
+constexpr uint32_t kSgList = 1024;            // vertices of 8 pieces
+constexpr uint32_t kSgMaxVertices = 131072;   // 32 mask words
+constexpr uint32_t kSgSpinLimit = 1u << 24;   // polls before the barrier gives up
 
 // ---------------------------------------------------------------- triangle counting
 struct TriCtl {

@@ -314,7 +314,8 @@ struct Relation {
   int kb = 4;
   DBuf keys, off, adj, V;
   DBuf rowv;                      // row fixpoints (up to kRowMaxVertices): vertex records,
-  size_t o_ns = 0, o_units = 0;   // out-edge bit set and adjacency units at these offsets
+  size_t o_ns = 0, o_units = 0, o_mp = 0;  // out-edge bit set, adjacency units, bit set of the
+                                  // vertices with several parents at these offsets
   DBuf htab;                      // hash-join ablation: E in a linear-probing table (lazy)
   unsigned long long hmask = 0;
   uint64_t peak_cand = 0, peak_full = 0;  // capacities seen by earlier queries
@@ -326,12 +327,17 @@ struct Relation {
   // 400,000 / 360,000: 15.5 -> 1.1 ms; dense R-MAT 2^19 / 400k: no change).
   bool small_rows() const { return nv > 65536u; }
   bool no_rows = false;           // the rows' bit sets did not fit the budget
+  // Same-generation rows (wg_kern_sg.cu): mask words of a row, and bytes beside
+  // the bit sets: two deltas as large, three masks, iteration marks, row lists.
+  uint32_t sg_mask_words() const { return (row_words() / 4 + 31) / 32; }
+  size_t sg_masks() const { return (size_t)nv * sg_mask_words() * 4; }
   void row_inst(RowInst* I) const {
     *I = RowInst{};
     I->off = (const uint32_t*)off.p; I->adj = (const uint32_t*)adj.p;
     I->rec = rowv.p;
     I->ns = (const uint32_t*)((const char*)rowv.p + o_ns);
     I->units = (const char*)rowv.p + o_units;
+    I->mp = (const uint32_t*)((const char*)rowv.p + o_mp);
     I->nv = nv; I->w = w; I->words = row_words();
   }
   void release(wg_ctx* c) {
@@ -363,11 +369,13 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
   if (R->nv <= kRowMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
     R->o_ns = round_up((size_t)R->nv * 32);
     R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
-    TRY(R->rowv.get(c, R->o_units + row_units(ne, R->nv, R->id_bytes()) * 16));
+    R->o_mp = R->o_units + round_up(row_units(ne, R->nv, R->id_bytes()) * 16);
+    TRY(R->rowv.get(c, R->o_mp + (size_t)R->row_words() * 8));
     char* v = (char*)R->rowv.p;
     launch_row_layout<K>((const K*)ke.p, (uint32_t)ne, R->w, (const uint32_t*)R->off.p,
                          (const uint32_t*)R->adj.p, R->nv, v, (uint32_t*)(v + R->o_ns),
-                         R->row_words(), v + R->o_units, R->id_bytes(), grid_of(c, 8), c->stream);
+                         R->row_words(), v + R->o_units, (uint32_t*)(v + R->o_mp), R->id_bytes(),
+                         grid_of(c, 8), c->stream);
     CK(cudaGetLastError());
   }
   return WG_OK;
@@ -626,6 +634,9 @@ struct Engine : EngineBase {
   DBuf row_meta, row_bits, row_small;
   RowInst ri{};
   RowJob job{};
+  bool row_sg = false;               // the query is same-generation
+  SgJob sg{};
+  SgInst sgi{};
   size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
   int id_bytes = 2, g_rows = 0;
   bool expand_only = false;          // the rows are done; the result waits for a larger buffer
@@ -894,23 +905,30 @@ struct Engine : EngineBase {
 
   // Row-by-row TC: buffers for relation R and a result of wantF keys.  A
   // result that turns out larger only needs the expansion again (settle).
-  int rows_begin(Relation* Rl, uint32_t max_iters, unsigned long long wantF) {
+  int rows_begin(Relation* Rl, int kind, uint32_t max_iters, unsigned long long wantF) {
     AllocScope scope(c, st);
     const uint32_t nv = Rl->nv, words = Rl->row_words();
     const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
     const uint32_t nlog = std::min<uint32_t>(1u << 16, nv + 2);
-    const bool small = Rl->small_rows();
+    row_sg = kind == WG_SG;
+    const bool small = !row_sg && Rl->small_rows();
     id_bytes = Rl->id_bytes();
-    g_rows = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(id_bytes, words)),
-                                     std::max<uint32_t>(nv, 1));
-    // control block | chunk sums | log (cleared) | instance | chunk offsets | row counts
+    g_rows = (int)std::min<uint64_t>(
+        grid_of(c, row_sg ? occupancy_sg(id_bytes, words) : occupancy_rows(id_bytes, words)),
+        std::max<uint32_t>(nv, 1));
+    // control block | chunk sums | log | same-generation: masks, marks (cleared) |
+    // instance | chunk offsets | row counts | row lists
     auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
     size_t end = 0;
-    const size_t o_ctl = at(end, sizeof(RowCtl)), o_sum = at(end, (size_t)nch * 4),
-                 o_log = at(end, (size_t)nlog * 8);
+    const size_t o_ctl = at(end, sizeof(RowCtl) + sizeof(SgCtl)), o_sum = at(end, (size_t)nch * 4),
+                 o_log = at(end, (size_t)nlog * 8), masks = row_sg ? Rl->sg_masks() : 0,
+                 o_fm = at(end, masks), o_dm0 = at(end, masks), o_dm1 = at(end, masks),
+                 o_act = at(end, row_sg ? (size_t)nv * 4 : 0);
     row_clear = end;
-    const size_t o_inst = at(end, sizeof(RowInst)), o_base = at(end, (size_t)nch * 8),
-                 o_cnt = at(end, (size_t)nv * 4), o_rows = at(end, small ? (size_t)nv * 4 : 0);
+    const size_t o_inst = at(end, sizeof(RowInst)), o_sgi = at(end, sizeof(SgInst)),
+                 o_base = at(end, (size_t)nch * 8), o_cnt = at(end, (size_t)nv * 4),
+                 o_rows = at(end, small || row_sg ? (size_t)nv * 4 : 0),
+                 o_rows1 = at(end, row_sg ? (size_t)nv * 4 : 0);
     TRY(row_meta.get(c, end));
     // bit sets of every row, or (small rows apart) of as many as a quarter of
     // the free budget holds: more are made room for when they turn up (settle)
@@ -920,6 +938,7 @@ struct Engine : EngineBase {
       const size_t room = (c->budget - std::min(c->budget, c->used) + row_bits.bytes) / 4;
       sets = std::max(std::min(sets, room), (size_t)words * 4);
     }
+    if (row_sg) sets = 3 * std::max<size_t>(Rl->row_bits(), 16);
     TRY(row_bits.get(c, sets));
     if (wantF > capF) {
       TRY(F[0].get(c, wantF * sizeof(K)));
@@ -938,6 +957,21 @@ struct Engine : EngineBase {
       job.rows = (uint32_t*)(m + o_rows);
       job.small = (uint32_t*)row_small.p;
       job.slots = (uint32_t)std::min<size_t>(nv, row_bits.bytes / ((size_t)words * 4));
+    }
+    if (row_sg) {
+      sgi = SgInst{};
+      sgi.d[0] = (uint4*)((char*)row_bits.p + Rl->row_bits());
+      sgi.d[1] = (uint4*)((char*)row_bits.p + 2 * Rl->row_bits());
+      sgi.fm = (uint32_t*)(m + o_fm);
+      sgi.dm[0] = (uint32_t*)(m + o_dm0); sgi.dm[1] = (uint32_t*)(m + o_dm1);
+      sgi.act = (uint32_t*)(m + o_act);
+      sgi.mw = Rl->sg_mask_words();
+      job.sg = (SgInst*)(m + o_sgi);
+      sg = SgJob{};
+      sg.rows = job;
+      sg.ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
+      sg.sg = (SgInst*)(m + o_sgi);
+      sg.list[0] = (uint32_t*)(m + o_rows); sg.list[1] = (uint32_t*)(m + o_rows1);
     }
     log_cap = nlog;
     expand_only = false;
@@ -970,9 +1004,16 @@ struct Engine : EngineBase {
         launch_rows_small(job, grid_of(c, 6), st);
         launches_issued += 2;  // (and k_row_expand_small)
       }
-      if (ri.nv) launch_rows(job, id_bytes, g_rows, st);
+      if (row_sg) {
+        CK(cudaMemcpyAsync(sg.sg, &sgi, sizeof(sgi), cudaMemcpyHostToDevice, st));
+        CK(launch_sg(sg, id_bytes, g_rows, c->num_sms, st));
+        launches_issued += 3;
+      } else if (ri.nv) {
+        launch_rows(job, id_bytes, g_rows, st);
+        launches_issued += 1;
+      }
       launch_row_plan(job, 1, st);
-      launches_issued += ri.nv ? 2 : 1;
+      launches_issued += 1;
     }
     launch_row_expand<K>(job, grid_of(c, 6), st);
     launches_issued += 1;
@@ -983,7 +1024,11 @@ struct Engine : EngineBase {
   }
   int rows_settle(bool* again) {
     CK(cudaMemcpyAsync(&ri, job.inst, sizeof(ri), cudaMemcpyDeviceToHost, st));
+    SgCtl sc{};
+    if (row_sg && !expand_only)
+      CK(cudaMemcpyAsync(&sc, sg.ctl, sizeof(sc), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (sc.error) return set_err(WG_E_DEVICE_TIMEOUT, "a bounded device wait gave up");
     Inst& I = hi[0];
     I.n_full = ri.n_total;
     I.cand_total = ri.cand;
@@ -1428,7 +1473,7 @@ static int single_start(wg_ctx* c, Query* q) {
   const unsigned long long wantF = std::max<unsigned long long>(
       {q->opts.reserve_full, Rl->peak_full, 4ull * Rl->ne, 1ull << 16});
   if (E->rows_) {
-    TRY(E->rows_begin(Rl, q->opts.max_iters, wantF));
+    TRY(E->rows_begin(Rl, q->kind, q->opts.max_iters, wantF));
     CK(cudaEventRecord(q->ev0, c->stream));
     TRY(E->rows_launch());
     q->state = WG_RUNNING;
@@ -2111,19 +2156,21 @@ static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R) {
 }
 
 // ------------------------------------------------------------------ batched rows
-// Whether query q runs row by row (wg_kern_rows.cu): a TC query that asks for
+// Whether query q runs row by row (wg_kern_rows.cu, wg_kern_sg.cu): one that asks for
 // nothing of the sorted-array pipeline (its ablations, the host-driven loops,
 // a per-stage profile, the size of the candidate buffers), over a relation
 // whose bit sets take at most half of the free budget -- the sorted
 // pipeline needs more than twice the result, so whatever fits there fits here.
 static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
   const Relation* R = q->rel;
-  if (q->kind != WG_TC || q->opts.flags || q->opts.reserve_cand || !R->rowv.p)
-    return false;
+  if (q->opts.flags || q->opts.reserve_cand || !R->rowv.p) return false;
+  if (q->kind == WG_SG && R->nv > kSgMaxVertices) return false;
   size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
   for (auto& e : c->idle) idle += e->held();
   // (small rows apart: their lists, and bit sets for whatever is left)
-  const size_t need = R->small_rows() && !batched ? (size_t)R->nv * kSmallRow * 8 : R->row_bits();
+  const size_t need = q->kind == WG_SG ? 3 * (R->row_bits() + R->sg_masks()) + (size_t)R->nv * 16
+                      : R->small_rows() && !batched ? (size_t)R->nv * kSmallRow * 8
+                                                    : R->row_bits();
   return need <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
 }
 static bool row_query(wg_ctx* c, const Query* q) {
@@ -2134,8 +2181,8 @@ static bool row_query(wg_ctx* c, const Query* q) {
 static bool row_batched(wg_ctx* c, const Query* q) { return row_fits(c, q, true); }
 
 
-// Submitted row-by-row TC queries: a lane runs the rows of many relations of
-// one key width in one launch (k_rows claims rows across instances), learns
+// Submitted row-by-row queries: a lane runs the rows of many relations of one
+// kind and key width in one launch (rows are claimed across instances), learns
 // every result's exact size, allocates the results and expands them.  No pool
 // is shared and nothing grows: a result that does not fit beside others waits
 // until the query can run alone, as the exclusive query, and fails only then.
@@ -2146,10 +2193,12 @@ struct RowLane {
   cudaEvent_t done = nullptr;
   int phase = 0;                   // 0 idle, 1 rows in flight, 2 expansion in flight
   int kb = 4;
+  bool sg = false;                 // same-generation queries (else TC)
   DBuf meta, bits;
   char* mirror = nullptr;          // page-locked copy of the cleared and uploaded parts of meta
   size_t mirror_bytes = 0;
-  size_t o_inst = 0, o_log = 0, up_end = 0, clear = 0;
+  size_t o_ctl = 0, o_inst = 0, o_log = 0, up_end = 0, clear = 0;
+  char* host(size_t at) { return mirror + (at - o_ctl); }
   uint32_t n = 0, log_cap = 0;
   RowJob job{};
   std::vector<uint64_t> order;     // query ids as submitted
@@ -2197,6 +2246,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   L->n = (uint32_t)qs.size();
   L->order = ids;
   L->kb = qs[0]->rel->kb;
+  L->sg = qs[0]->kind == WG_SG;
   // larger relations first: their long rows must not start last
   std::vector<uint32_t> by(L->n);
   for (uint32_t i = 0; i < L->n; ++i) by[i] = i;
@@ -2206,41 +2256,52 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   const uint32_t nv_max = qs[by[0]]->rel->nv, vwords = qs[by[0]]->rel->row_words();
   const int idb = qs[0]->rel->id_bytes();
   uint32_t nch = 0;
-  size_t bits = 0;
+  size_t bits = 0, masks = 0;
   for (Query* q : qs) {
     nch += (q->rel->nv + kRowChunk - 1) / kRowChunk;
     bits += q->rel->row_bits();
+    masks += q->rel->sg_masks();
   }
   L->log_cap = std::min(kBatchLogCap, nv_max + 2);
-  const int grid = (int)std::min<uint64_t>(grid_of(c, occupancy_rows(idb, vwords)),
-                                           (uint64_t)nch * kRowChunk);
+  const int grid = (int)std::min<uint64_t>(
+      grid_of(c, L->sg ? occupancy_sg(idb, vwords) : occupancy_rows(idb, vwords)),
+      (uint64_t)nch * kRowChunk);
   auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
   size_t end = 0;
-  const size_t o_ctl = at(end, sizeof(RowCtl)), o_sum = at(end, (size_t)nch * 4);
+  const size_t rows4 = (size_t)nch * kRowChunk * 4;
+  if (!L->sg) masks = 0;
+  const size_t o_sum = at(end, (size_t)nch * 4), o_fm = at(end, masks), o_dm0 = at(end, masks),
+               o_dm1 = at(end, masks), o_act = at(end, L->sg ? rows4 : 0),
+               o_ctl = at(end, sizeof(RowCtl) + sizeof(SgCtl));
+  L->o_ctl = o_ctl;
   L->o_log = at(end, (size_t)L->n * L->log_cap * 8);
   L->clear = end;
   L->o_inst = at(end, (size_t)L->n * sizeof(RowInst));
-  const size_t o_map = at(end, (size_t)nch * 4);
+  const size_t o_map = at(end, (size_t)nch * 4),
+               o_sgi = at(end, L->sg ? (size_t)L->n * sizeof(SgInst) : 0);
   L->up_end = end;
-  const size_t o_base = at(end, (size_t)nch * 8), o_cnt = at(end, (size_t)nch * kRowChunk * 4);
+  const size_t o_base = at(end, (size_t)nch * 8), o_cnt = at(end, rows4),
+               o_l0 = at(end, L->sg ? rows4 : 0), o_l1 = at(end, L->sg ? rows4 : 0);
   L->phase = 1;  // (its buffers are not to be dropped while it allocates)
   int rc = L->meta.get(c, end);
-  if (rc == WG_OK) rc = L->bits.get(c, bits);
+  if (rc == WG_OK) rc = L->bits.get(c, L->sg ? 3 * bits : bits);
   L->phase = 0;
   TRY(rc);
-  if (L->up_end > L->mirror_bytes) {
+  // the mirror holds meta from the control block on (the masks before it stay here)
+  if (L->up_end - o_ctl > L->mirror_bytes) {
     if (L->mirror) cudaFreeHost(L->mirror);
     L->mirror = nullptr;
     L->mirror_bytes = 0;
-    CK(cudaMallocHost((void**)&L->mirror, 2 * L->up_end));
-    L->mirror_bytes = 2 * L->up_end;
+    CK(cudaMallocHost((void**)&L->mirror, 2 * (L->up_end - o_ctl)));
+    L->mirror_bytes = 2 * (L->up_end - o_ctl);
   }
   char* m = (char*)L->meta.p;
-  RowInst* hi = (RowInst*)(L->mirror + L->o_inst);
-  uint32_t* hm = (uint32_t*)(L->mirror + o_map);
+  RowInst* hi = (RowInst*)L->host(L->o_inst);
+  uint32_t* hm = (uint32_t*)L->host(o_map);
+  SgInst* hs = (SgInst*)L->host(o_sgi);
   L->slot.assign(L->n, 0);
   uint32_t ch = 0;
-  size_t wat = 0;
+  size_t wat = 0, mat = 0;
   for (uint32_t k = 0; k < L->n; ++k) {
     Query* q = qs[by[k]];
     const Relation* R = q->rel;
@@ -2254,6 +2315,17 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
     I.log = (unsigned long long*)(m + L->o_log) + (size_t)k * L->log_cap;
     I.max_iters = q->opts.max_iters; I.log_cap = L->log_cap;
     hi[k] = I;
+    if (L->sg) {
+      SgInst g{};
+      g.d[0] = (uint4*)((char*)I.bits + bits);
+      g.d[1] = (uint4*)((char*)I.bits + 2 * bits);
+      g.fm = (uint32_t*)(m + o_fm + mat);
+      g.dm[0] = (uint32_t*)(m + o_dm0 + mat); g.dm[1] = (uint32_t*)(m + o_dm1 + mat);
+      g.act = (uint32_t*)(m + o_act) + I.row0;
+      g.mw = R->sg_mask_words();
+      mat += R->sg_masks();
+      hs[k] = g;
+    }
     for (uint32_t e = ch + (R->nv + kRowChunk - 1) / kRowChunk; ch < e; ++ch) hm[ch] = k;
     q->state = WG_RUNNING;
   }
@@ -2263,13 +2335,23 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   J.chunk_inst = (const uint32_t*)(m + o_map);
   J.csum = (uint32_t*)(m + o_sum); J.cbase = (unsigned long long*)(m + o_base);
   J.nrows = nch * kRowChunk; J.vwords = vwords;
-  CK(cudaMemcpyAsync(m + L->o_inst, L->mirror + L->o_inst, L->up_end - L->o_inst,
+  CK(cudaMemcpyAsync(m + L->o_inst, L->host(L->o_inst), L->up_end - L->o_inst,
                      cudaMemcpyHostToDevice, L->st));
   CK(cudaMemsetAsync(m, 0, L->clear, L->st));
-  launch_rows(J, idb, grid, L->st);
+  if (L->sg) {
+    J.sg = (SgInst*)(m + o_sgi);
+    SgJob S{};
+    S.rows = J;
+    S.ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
+    S.sg = (SgInst*)(m + o_sgi);
+    S.list[0] = (uint32_t*)(m + o_l0); S.list[1] = (uint32_t*)(m + o_l1);
+    CK(launch_sg(S, idb, grid, c->num_sms, L->st));
+  } else {
+    launch_rows(J, idb, grid, L->st);
+  }
   launch_row_plan(J, L->n, L->st);
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(L->mirror + L->o_log, m + L->o_log, L->o_inst - L->o_log + L->n * sizeof(RowInst),
+  CK(cudaMemcpyAsync(L->mirror, m + o_ctl, L->o_inst - o_ctl + L->n * sizeof(RowInst),
                      cudaMemcpyDeviceToHost, L->st));
   CK(cudaEventRecord(L->done, L->st));
   L->phase = 1;
@@ -2288,7 +2370,8 @@ static void lane_result_refused(wg_ctx* c, RowLane* L, Query* q, size_t bytes, i
     if (it != c->queries.end() && it->second->eng) free_later += it->second->eng->held();
   }
   const size_t fixed = c->used > free_later ? c->used - free_later : 0;
-  if ((L->n == 1 && q->row_alone) || fixed + q->rel->row_bits() + bytes > c->budget) {
+  const size_t sets = (q->kind == WG_SG ? 3 : 1) * q->rel->row_bits();
+  if ((L->n == 1 && q->row_alone) || fixed + sets + bytes > c->budget) {
     if (c->excl == q->id) c->excl = 0;
     q->state = WG_FAILED;
     q->error = why;
@@ -2305,7 +2388,18 @@ static void lane_result_refused(wg_ctx* c, RowLane* L, Query* q, size_t bytes, i
 // Rows done: allocate the results and expand the bit sets into them.
 static int lane_expand(wg_ctx* c, RowLane* L) {
   AllocScope scope(c, L->st);
-  RowInst* hi = (RowInst*)(L->mirror + L->o_inst);
+  RowInst* hi = (RowInst*)L->host(L->o_inst);
+  if (L->sg && ((const SgCtl*)(L->mirror + sizeof(RowCtl)))->error) {
+    for (uint64_t id : L->order) {
+      auto it = c->queries.find(id);
+      if (it == c->queries.end()) continue;
+      it->second->state = WG_FAILED;
+      it->second->error = WG_E_DEVICE_TIMEOUT;
+      c->completed.push_back(id);
+    }
+    L->phase = 0;
+    return set_err(WG_E_DEVICE_TIMEOUT, "a bounded device wait gave up");
+  }
   for (uint32_t i = 0; i < L->n; ++i) {
     RowInst& I = hi[L->slot[i]];
     I.fits = 0;
@@ -2328,7 +2422,7 @@ static int lane_expand(wg_ctx* c, RowLane* L) {
     q->candidates = I.cand;
     q->iterations = capped ? I.max_iters : I.last + 1;
     const unsigned long long* log =
-        (const unsigned long long*)(L->mirror + L->o_log) + (size_t)L->slot[i] * L->log_cap;
+        (const unsigned long long*)L->host(L->o_log) + (size_t)L->slot[i] * L->log_cap;
     q->log.assign(log, log + std::min(q->iterations + 1, kBatchLogCap));
     q->error = capped ? WG_E_ITER_CAP : WG_OK;
     q->res_ptr = q->res_own.p;
@@ -2358,14 +2452,14 @@ static void lane_finish(wg_ctx* c, RowLane* L) {
   L->phase = 0;
 }
 
-// The next launch of an idle lane: queued row queries of one key width, in
+// The next launch of an idle lane: queued row queries of one kind and key width, in
 // order, up to kLaneBits of bit sets; one query alone if it must run alone.
 static int lane_admit(wg_ctx* c, RowLane* L, bool* progressed) {
   Query* x = excl_query(c);
   if (x && !x->rowb) return WG_OK;  // another query waits for the whole budget
   std::vector<uint64_t> ids;
   size_t bits = 0;
-  int kb = 0;
+  int kb = 0, kind = 0;
   for (uint64_t id : c->pending) {
     auto it = c->queries.find(id);
     if (it == c->queries.end() || !it->second->rowb) continue;
@@ -2381,12 +2475,11 @@ static int lane_admit(wg_ctx* c, RowLane* L, bool* progressed) {
       ids.push_back(id);
       break;
     }
-    const size_t b = q->rel->row_bits();
-    if (kb && (q->rel->kb != kb || bits + b > kLaneBits || ids.size() >= kLaneQueries)) {
-      if (q->rel->kb != kb) continue;
-      break;
-    }
+    const size_t b = (q->kind == WG_SG ? 3 : 1) * q->rel->row_bits();
+    if (kb && (q->rel->kb != kb || q->kind != kind)) continue;
+    if (kb && (bits + b > kLaneBits || ids.size() >= kLaneQueries)) break;
     kb = q->rel->kb;
+    kind = q->kind;
     bits += b;
     ids.push_back(id);
   }

@@ -23,40 +23,18 @@
 //   k_row_expand  bit sets -> sorted packed keys
 #include "wg_device.cuh"
 #include "wg_launch.h"
+#include "wg_rows.cuh"
 
 namespace wg {
 
-// Adjacency in units of 16 bytes (8 16-bit or 4 32-bit ranks).  Each vertex has
-// a 32-byte record (one sector): {first further unit, degree, -, -} and its
-// first unit, so one access gives most vertices' whole adjacency.  Its further
-// units start at (off[v] + (U-1) v + U-1) / U: room for every vertex before it
-// without a scan.  A unit's unused places repeat the vertex's last neighbour
-// (setting a bit twice is harmless), so no place needs a test.
-template <typename IdT> struct Unit { static constexpr uint32_t n = 16 / sizeof(IdT); };
-template <typename IdT>
-__device__ __forceinline__ uint32_t unit_start(uint32_t off, uint32_t v) {
-  constexpr uint32_t U = Unit<IdT>::n;
-  return (off + (U - 1) * (v + 1)) / U;
-}
-// The bits of places [2p, 2p + 2) of a unit (16-bit ranks) or place p (32-bit).
-__device__ __forceinline__ void set_bit(uint32_t* n, uint32_t byte_off, uint32_t z) {
-  atomicOr((uint32_t*)((char*)n + byte_off), __funnelshift_l(0u, 1u, z));  // 1 << (z & 31)
-}
-__device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint16_t) {
-  set_bit(n, (v >> 3) & 0x1FFCu, v);
-  set_bit(n, (v >> 19) & 0x1FFCu, v >> 16);
-}
-__device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint32_t) {
-  set_bit(n, (v >> 3) & ~3u, v);
-}
-
 // The vertex records, the bit set of vertices with out-edges, and the further
-// units of a relation (edges in source order, the source of edge i is E[i] >> w).
+// units of a relation (edges in source order, the source of edge i is E[i] >> w);
+// the bit set mp of the vertices with several parents.
 template <typename K, typename IdT>
 __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne, uint32_t w,
                                                          const uint32_t* off, const uint32_t* adj,
                                                          uint32_t nv, uint4* rec, uint32_t* ns,
-                                                         uint32_t words, IdT* units) {
+                                                         uint32_t words, IdT* units, uint32_t* mp) {
   const uint32_t stride = gridDim.x * kThreads, t = blockIdx.x * kThreads + threadIdx.x;
   for (uint32_t v = t; v < words * 32; v += stride) {
     uint32_t o = 0, d = 0;
@@ -74,19 +52,12 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
     IdT* to = j < U ? (IdT*)(rec + 2 * (size_t)x + 1) + j
                     : units + (size_t)unit_start<IdT>(o, x) * U + (j - U);
     const IdT z = (IdT)adj[i];
+    const uint32_t bit = 1u << (z & 31);  // (mp: several parents; after it: at least one)
+    if (atomicOr(mp + words + (z >> 5), bit) & bit) atomicOr(mp + (z >> 5), bit);
     *to = z;
     if (i + 1 == off[x + 1])
       for (uint32_t r = j % U + 1; r < U; ++r) *++to = z;
   }
-}
-
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= (uint32_t)o) v += y;
-  }
-  return v;
 }
 
 // One CTA takes a row through its whole fixpoint.  Shared memory: the row's bit
@@ -110,7 +81,7 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
 // expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0.
 template <typename IdT, int T, int kMin>
 __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
-  constexpr uint32_t U = Unit<IdT>::n, kW = T / 32;
+  constexpr uint32_t kW = T / 32;
   extern __shared__ uint4 sm4[];
   __shared__ RowInst I;
   __shared__ unsigned long long s_log[kRowLog];
@@ -120,7 +91,6 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* strip = N + J.vwords + warp * 32;
   IdT* list = (IdT*)(N + J.vwords + kW * 32);
-  const uint32_t upto = 0xFFFFFFFFu >> (31 - lane);
   unsigned long long cand = 0;
   uint32_t cur = 0xFFFFFFFFu;
   for (uint32_t i = tid; i < 2 * J.vwords; i += T) S[i] = 0;
@@ -135,49 +105,6 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
       if (s_log[i] && i < I.log_cap) atomicAdd(I.log + i, s_log[i]);
       s_log[i] = 0;
     }
-  };
-  constexpr uint32_t P = U / 4;  // places in a word of a unit
-  // the bits of the neighbours of vertices l[0..n), n <= 32, into N
-  auto expand = [&](const IdT* l, uint32_t n) {
-    uint32_t us = 0, deg = 0;
-    uint4 u = {0, 0, 0, 0};
-    if (lane < n) {
-      const uint4* r = (const uint4*)I.rec + 2 * (size_t)l[lane];
-      const uint2 t = __ldg((const uint2*)r);
-      u = __ldg(r + 1);
-      us = t.x;
-      deg = t.y;
-    }
-    cand += deg;
-    const uint32_t most = __reduce_max_sync(0xffffffffu, deg);
-    if (lane < n) {
-      set_part(N, u.x, IdT());
-      if (most > P) set_part(N, u.y, IdT());
-      if (most > 2 * P) set_part(N, u.z, IdT());
-      if (most > 3 * P) set_part(N, u.w, IdT());
-    }
-    if (most <= U) return;
-    const uint32_t more = deg > U ? (deg - 1) / U : 0u;  // further units
-    const uint32_t has = __ballot_sync(0xffffffffu, more > 0);
-    const uint32_t in = warp_incl_scan(more, lane);
-    const uint32_t tot = __shfl_sync(0xffffffffu, in, 31), st = in - more;
-    if (more) strip[__popc(has & upto) - 1] = us - st;
-    __syncwarp();
-    uint32_t prev = 0;  // vertices whose units begin before this step
-    for (uint32_t e0 = 0; e0 < tot; e0 += 32) {
-      const uint32_t sh = st - e0, e = e0 + lane;
-      const uint32_t m = __reduce_or_sync(0xffffffffu, more && sh < 32u ? 1u << sh : 0u);
-      const uint32_t t = strip[prev + __popc(m & upto) - 1];
-      prev += __popc(m);
-      if (e < tot) {
-        u = __ldg((const uint4*)I.units + (t + e));
-        set_part(N, u.x, IdT());
-        set_part(N, u.y, IdT());
-        set_part(N, u.z, IdT());
-        set_part(N, u.w, IdT());
-      }
-    }
-    __syncwarp();
   };
   // listed rows (k_rows_small's leftovers): their bit sets lie in list order
   const uint32_t nrows = J.rows ? J.inst->n_big : J.nrows;
@@ -195,7 +122,9 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
       cur = q;
       __syncthreads();
     }
-    if (tid == 0) s_row[p ^ 1] = atomicAdd(&J.ctl->next_row, 1u);
+    // the next row, claimed here and stored at the end: nothing waits for it
+    uint32_t next = 0;
+    if (tid == 0) next = atomicAdd(&J.ctl->next_row, 1u);
     const uint32_t x = row - I.row0;
     uint32_t o = 0, deg = 0;
     if (x < I.nv) {  // (rows of an instance are padded to whole chunks)
@@ -265,7 +194,8 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
           if (round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
           listed |= len;
           if (len == 0) break;
-          for (uint32_t b = warp * 32; b < n; b += T) expand(list + b, min(32u, n - b));
+          for (uint32_t b = warp * 32; b < n; b += T)
+            cand += expand_vertices(I, list + b, min(32u, n - b), N, strip);
           __syncthreads();
           if (len <= kRowList) break;
         }
@@ -290,6 +220,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
         sm4[i] = uint4{0, 0, 0, 0};
       }
     }
+    if (tid == 0) s_row[p ^ 1] = next;
     __syncthreads();
   }
   if (cur != 0xFFFFFFFFu) flush();
@@ -483,16 +414,30 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
 
 // Bit sets -> sorted packed keys (x << w) | z, one warp per row: 64 words at a
 // time, each lane lists the set bits of its two words at its prefix in the
-// warp's shared buffer, then the warp writes the list coalesced.
-template <typename K>
+// warp's shared buffer, then the warp writes the list coalesced.  kMasked
+// (same-generation): of each row the 128-bit pieces marked valid only, 16 at a
+// time.  A step that is half full is written a word at a time by the whole warp.
+// 7.5e7 same-generation tuples, rows of nearly full pieces: 0.31 -> 0.18 ms with
+// the padding and the word steps (ncu had the buffer's bank conflicts at 87% of
+// the L1 pipe).
+template <typename K, bool kMasked>
 __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
-  __shared__ uint16_t buf[kWarps][2048];
+  __shared__ uint16_t s_buf[kWarps][2048 + 64], s_list[kMasked ? kWarps : 1][kMasked ? kSgMaxVertices / 128 : 1];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1;
+  constexpr uint32_t kDense = 1024;  // of 2,048 bits
+  // (valid pieces are often nearly full, so lanes list some 64 places apart: two
+  // places of padding spread the banks; unmasked rows are sparser, and it costs
+  // them more than it saves: 0.62 against 0.56 ms for 4.8e8 tuples)
+  auto pad = [](uint32_t at) { return kMasked ? at + (at >> 6) * 2 : at; };
+  uint16_t* buf = s_buf[warp];
+  uint16_t* list = s_list[kMasked ? warp : 0];
   const uint32_t stride = gridDim.x * kWarps, nrows = J.rows ? J.inst->n_big : J.nrows;
   for (uint32_t i = blockIdx.x * kWarps + warp; i < nrows; i += stride) {
     const uint32_t row = J.rows ? J.rows[i] : i;
     const uint32_t ch = row / kRowChunk;
-    const RowInst* I = J.inst + (J.chunk_inst ? J.chunk_inst[ch] : 0u);
+    const uint32_t q = J.chunk_inst ? J.chunk_inst[ch] : 0u;
+    const RowInst* I = J.inst + q;
     const uint32_t x = row - I->row0;
     if (x >= I->nv || !I->fits) continue;
     const uint32_t n = I->cnt[x];
@@ -504,34 +449,48 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
     before = __reduce_add_sync(0xffffffffu, before);
     K* out = (K*)I->out + J.cbase[ch] + before;
     const uint2* w2 = (const uint2*)(I->bits + (size_t)(J.rows ? i : x) * I->words);
-    const uint32_t np = I->words / 2;
+    uint32_t np = I->words / 2;  // pairs of words to list
+    if (kMasked) {
+      const SgInst* G = J.sg + q;
+      np = 2 * list_pieces(lane < G->mw ? G->fm[(size_t)x * G->mw + lane] : 0u, list);
+      __syncwarp();
+    }
+    // the place in the row of the p-th pair listed
+    auto place = [&](uint32_t p) { return kMasked ? 2u * list[p >> 1] + (p & 1u) : p; };
     const K hi = (K)x << I->w;
-    uint2 v = lane < np ? w2[lane] : uint2{0, 0};
+    uint2 v = lane < np ? w2[place(lane)] : uint2{0, 0};
     for (uint32_t b = 0; b < np; b += 32) {
       const uint32_t nx = b + 32 + lane;
-      const uint2 nextv = nx < np ? w2[nx] : uint2{0, 0};
+      const uint2 nextv = nx < np ? w2[place(nx)] : uint2{0, 0};
       const uint32_t c = __popc(v.x) + __popc(v.y), in = warp_incl_scan(c, lane);
       const uint32_t tot = __shfl_sync(0xffffffffu, in, 31);
-      if (tot) {
-        uint32_t at = in - c;
-        uint32_t m = v.x;
-        while (m) {
-          buf[warp][at++] = (uint16_t)(lane * 64 + __ffs(m) - 1);
-          m &= m - 1;
+      if (tot >= kDense) {
+        // dense: the warp takes a word at a time, a lane per bit
+        uint32_t off = 0;
+        for (uint32_t j = 0; j < 64; ++j) {
+          const uint32_t m = __shfl_sync(0xffffffffu, j & 1 ? v.y : v.x, j >> 1);
+          if (m >> lane & 1u)
+            out[off + __popc(m & below)] = hi + (K)place(b + (j >> 1)) * 64 + ((j & 1u) * 32 + lane);
+          off += __popc(m);
         }
-        m = v.y;
-        while (m) {
-          buf[warp][at++] = (uint16_t)(lane * 64 + 31 + __ffs(m));
-          m &= m - 1;
-        }
+        out += tot;
+      } else if (tot) {
+        auto put = [&](uint32_t at, uint32_t m, uint32_t base) {
+          for (; m; m &= m - 1, ++at) buf[pad(at)] = (uint16_t)(base + __ffs(m) - 1);
+        };
+        put(in - c, v.x, lane * 64);
+        put(in - __popc(v.y), v.y, lane * 64 + 32);
         __syncwarp();
-        const K base = hi + (K)b * 64;
-        for (uint32_t j = lane; j < tot; j += 32) out[j] = base + buf[warp][j];
+        for (uint32_t j = lane; j < tot; j += 32) {
+          const uint32_t t = buf[pad(j)];
+          out[j] = hi + (K)place(b + (t >> 6)) * 64 + (t & 63u);
+        }
         out += tot;
         __syncwarp();
       }
       v = nextv;
     }
+    if (kMasked) __syncwarp();
   }
 }
 
@@ -587,7 +546,8 @@ void launch_rows_small(const RowJob& J, int grid, cudaStream_t s) {
 template <typename K>
 void launch_row_expand(const RowJob& J, int grid, cudaStream_t s) {
   if (J.rows) k_row_expand_small<K><<<grid, kThreads, 0, s>>>(J);
-  k_row_expand<K><<<grid, kThreads, 0, s>>>(J);
+  if (J.sg) k_row_expand<K, true><<<grid, kThreads, 0, s>>>(J);
+  else k_row_expand<K, false><<<grid, kThreads, 0, s>>>(J);
 }
 size_t row_units(uint64_t ne, uint32_t nv, int id_bytes) {
   const uint64_t U = 16 / id_bytes;
@@ -596,22 +556,23 @@ size_t row_units(uint64_t ne, uint32_t nv, int id_bytes) {
 template <typename K>
 void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
                        const uint32_t* adj, uint32_t nv, void* rec, uint32_t* ns, uint32_t words,
-                       void* units, int id_bytes, int grid, cudaStream_t s) {
+                       void* units, uint32_t* mp, int id_bytes, int grid, cudaStream_t s) {
+  cudaMemsetAsync(mp, 0, (size_t)words * 8, s);
   if (id_bytes == 2)
     k_row_layout<K, uint16_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
-                                                        words, (uint16_t*)units);
+                                                        words, (uint16_t*)units, mp);
   else
     k_row_layout<K, uint32_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
-                                                        words, (uint32_t*)units);
+                                                        words, (uint32_t*)units, mp);
 }
 template void launch_row_expand<uint32_t>(const RowJob&, int, cudaStream_t);
 template void launch_row_expand<unsigned long long>(const RowJob&, int, cudaStream_t);
 template void launch_row_layout<uint32_t>(const uint32_t*, uint32_t, uint32_t, const uint32_t*,
                                           const uint32_t*, uint32_t, void*, uint32_t*, uint32_t,
-                                          void*, int, int, cudaStream_t);
+                                          void*, uint32_t*, int, int, cudaStream_t);
 template void launch_row_layout<unsigned long long>(const unsigned long long*, uint32_t, uint32_t,
                                                     const uint32_t*, const uint32_t*, uint32_t,
-                                                    void*, uint32_t*, uint32_t, void*, int, int,
-                                                    cudaStream_t);
+                                                    void*, uint32_t*, uint32_t, void*, uint32_t*,
+                                                    int, int, cudaStream_t);
 
 }  // namespace wg

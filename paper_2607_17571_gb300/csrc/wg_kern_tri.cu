@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(1024, 1) k_tri_count(TriJob J) {
   for (uint32_t p = 0;; p ^= 1) {
     const uint32_t t = s_t[p];
     if (t >= J.ctl->tasks) break;
-    if (tid == 0) s_t[p ^ 1] = atomicAdd(&J.ctl->next, 1u);
+    uint32_t next = 0;
+    if (tid == 0) next = atomicAdd(&J.ctl->next, 1u);
     const uint2 task = J.task[t];
     const uint32_t v = task.x, odd = task.y & 1u;
     const uint32_t oo = J.off[v], od = J.off[v + 1] - oo, io = J.ioff[v], id = J.ideg[v];
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(1024, 1) k_tri_count(TriJob J) {
     hits += mine;
     __syncthreads();
     for (uint32_t i = tid; i < sd; i += T) bits[sadj[so + i] >> 5] = 0;
+    if (tid == 0) s_t[p ^ 1] = next;
     __syncthreads();
   }
   for (int o = 16; o > 0; o >>= 1) hits += __shfl_xor_sync(0xffffffffu, hits, o);

@@ -14,6 +14,7 @@ struct Dev;
 struct Inst;
 struct RowJob;
 struct TriJob;
+struct SgJob;
 
 // sorted-array stages (wg_kern_sort.cu); K = uint32_t or unsigned long long
 template <typename K> void launch_sort_hist(Stage* st, int grid, cudaStream_t s);
@@ -71,12 +72,17 @@ void launch_rows_small(const RowJob& J, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
 // adjacency units of a relation: their number, and the layout of vertex records
-// (32 bytes each), out-edge bit set (words) and further units (16 bytes each)
+// (32 bytes each), out-edge bit set (words), further units (16 bytes each), bit set
+// of the vertices with several parents (words; followed by as many of scratch)
 size_t row_units(uint64_t ne, uint32_t nv, int id_bytes);
 template <typename K>
 void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
                        const uint32_t* adj, uint32_t nv, void* rec, uint32_t* ns, uint32_t words,
-                       void* units, int id_bytes, int grid, cudaStream_t s);
+                       void* units, uint32_t* mp, int id_bytes, int grid, cudaStream_t s);
+
+// same-generation over rows (wg_kern_sg.cu): every iteration, and the row counts
+int occupancy_sg(int id_bytes, uint32_t vwords);
+cudaError_t launch_sg(const SgJob& J, int id_bytes, int grid, int sms, cudaStream_t s);
 
 // triangle counting by set intersection (wg_kern_tri.cu): transpose and count
 template <typename K>
