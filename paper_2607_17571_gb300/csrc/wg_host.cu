@@ -268,15 +268,41 @@ static int prim_unique(wg_ctx* c, const K* in, size_t n, const K* full, size_t n
                        size_t* n_out) {
   *n_out = 0;
   if (n == 0) return WG_OK;
-  const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
-  TRY(prim_scratch(c, 0, ntiles));
+  // One merge-path pass over both arrays (the fused stage's kernel without a
+  // Full'), unless `full` is empty or so much longer than `in` that a search per
+  // key (k_unique_diff) reads less.  64-bit keys, n = 2^20, n_full = 1 / 8 / 64 n:
+  // search 196 / 281 / 747 us, merge 54 / 101 / 412 us (it grows with n_full, and
+  // would lose from some 128 n); 2^24 against 2^24 keys 918 -> 254 us; 1,000
+  // against 64,000 87 -> 42 us.  The splits go to the sort's buffer.
+  constexpr uint32_t T = FuseTile<K>::T;
+  const uint64_t tiles = ((uint64_t)n + nf + T - 1) / T;
+  bool merged = nf > 0 && nf <= 64 * (uint64_t)n && tiles < (1u << 31);
+  if (merged) {  // (a status word per tile: fewer than prim_scratch's per digit)
+    const int rc = prim_scratch(c, (tiles + 1) * 8, tiles / kRadix + 1);
+    if (rc != WG_OK && rc != WG_E_BUDGET && rc != WG_E_NOMEM) return rc;
+    if (rc != WG_OK) cudaGetLastError();
+    merged = rc == WG_OK;
+  }
   Seg sg{};
-  sg.n = n; sg.aux_n = nf; sg.ntiles = ntiles;
-  TRY(prim_seg(c, sg));
-  Stage u = prim_stage(c, ntiles);
-  u.in = in; u.aux = full; u.out = out; u.epoch = prim_epoch(c);
-  TRY(prim_put(c, S_UNIQ, u));
-  launch_unique_diff<K>(c->s_stage + S_UNIQ, grid_of(c, occupancy_sort<K>(2)), c->stream);
+  if (merged) {
+    sg.n = nf; sg.aux_n = n; sg.ntiles = (uint32_t)tiles;
+    TRY(prim_seg(c, sg));
+    Stage f = prim_stage(c, (uint32_t)tiles);
+    f.in = full; f.aux = in; f.out = out; f.epoch = prim_epoch(c);
+    f.splits = (unsigned long long*)c->s_tmp;
+    TRY(prim_put(c, S_FUSE, f));
+    launch_partition<K>(c->s_stage + S_FUSE, 0, T, c->num_sms * 4, c->stream);
+    launch_diff_merge<K>(c->s_stage + S_FUSE, grid_of(c, occupancy_sort<K>(4)), c->stream, T);
+  } else {
+    const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
+    TRY(prim_scratch(c, 0, ntiles));
+    sg.n = n; sg.aux_n = nf; sg.ntiles = ntiles;
+    TRY(prim_seg(c, sg));
+    Stage u = prim_stage(c, ntiles);
+    u.in = in; u.aux = full; u.out = out; u.epoch = prim_epoch(c);
+    TRY(prim_put(c, S_UNIQ, u));
+    launch_unique_diff<K>(c->s_stage + S_UNIQ, grid_of(c, occupancy_sort<K>(2)), c->stream);
+  }
   CK(cudaGetLastError());
   Seg back{};
   Ctl ctl{};
@@ -295,13 +321,23 @@ template <typename K>
 static int prim_merge(wg_ctx* c, const K* a, size_t na, const K* b, size_t nb, K* out) {
   if (na + nb == 0) return WG_OK;
   const uint32_t ntiles = (uint32_t)((na + nb + kTileM - 1) / kTileM);
-  TRY(prim_scratch(c, 0, 0));
+  // the tiles' splits, found in parallel (in the sort's buffer); without room
+  // for them each tile searches its own
+  const int rc = prim_scratch(c, ((size_t)ntiles + 1) * 8, 0);
+  if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
+    cudaGetLastError();
+    TRY(prim_scratch(c, 0, 0));
+  } else {
+    TRY(rc);
+  }
   Seg sg{};
   sg.n = na; sg.aux_n = nb; sg.ntiles = ntiles;
   TRY(prim_seg(c, sg));
   Stage m = prim_stage(c, ntiles);
   m.in = a; m.aux = b; m.out = out;
+  m.splits = rc == WG_OK ? (unsigned long long*)c->s_tmp : nullptr;
   TRY(prim_put(c, S_MERGE, m));
+  if (m.splits) launch_partition<K>(c->s_stage + S_MERGE, 0, kTileM, c->num_sms * 4, c->stream);
   launch_merge<K>(c->s_stage + S_MERGE, grid_of(c, occupancy_sort<K>(3)), c->stream);
   CK(cudaGetLastError());
   return WG_OK;

@@ -856,9 +856,13 @@ __device__ __forceinline__ unsigned long long merge_path(const K* A, unsigned lo
   return lo;
 }
 
+// A tile's inputs are staged in shared memory; each thread takes 16 consecutive
+// outputs, one merge-path search for their start and then one comparison each,
+// and the tile goes out through shared memory, coalesced.  (A search per output:
+// 0.28 ms for 2.8e7 64-bit keys, now 0.15.)
 template <typename K>
 __global__ void __launch_bounds__(kThreads) k_merge(Stage* stp) {
-  __shared__ K sm[kTileM];
+  __shared__ K sm[Padded<kTileM>::n];
   __shared__ unsigned long long s_a0, s_a1;
   __shared__ uint32_t s_t;
   Ctl* ctl = stp->ctl;
@@ -913,21 +917,46 @@ __global__ void __launch_bounds__(kThreads) k_merge(Stage* stp) {
 #pragma unroll
         for (int e = 0; e < kTileM / kThreads; ++e) {
           const uint32_t i = threadIdx.x + e * kThreads;
-          if (i < la + lb) sm[i] = v[e];
+          if (i < la + lb) sm[pad32(i)] = v[e];
         }
       }
       __syncthreads();
-      const K* SA = sm;
-      const K* SB = sm + la;
-      for (uint32_t q = threadIdx.x; q < la + lb; q += kThreads) {
-        uint32_t lo = q > lb ? q - lb : 0, hi = q < la ? q : la;
-        while (lo < hi) {
-          const uint32_t m = (lo + hi) >> 1;
-          if (SA[m] < SB[q - 1 - m]) lo = m + 1; else hi = m;
+      constexpr int E = kTileM / kThreads;
+      const uint32_t L = la + lb, q0 = threadIdx.x * E;
+      K val[E];
+      if (q0 < L) {
+        auto SA = [&](uint32_t i) { return sm[pad32(i)]; };
+        auto SB = [&](uint32_t j) { return sm[pad32(la + j)]; };
+        uint32_t i = q0 > lb ? q0 - lb : 0, hi = q0 < la ? q0 : la;
+        while (i < hi) {
+          const uint32_t m = (i + hi) >> 1;
+          if (SA(m) < SB(q0 - 1 - m)) i = m + 1; else hi = m;
         }
-        const uint32_t ib = q - lo;
-        const bool takeA = lo < la && (ib >= lb || SA[lo] < SB[ib]);
-        out[d0 + q] = takeA ? SA[lo] : SB[ib];
+        uint32_t j = q0 - i;
+        K a = SA(i), b = SB(j);  // (index la + lb <= kTileM lies in sm; unused then)
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          val[e] = 0;
+          if (q0 + e < L) {
+            const bool takeA = i < la && (j >= lb || a < b);
+            val[e] = takeA ? a : b;
+            const K w = sm[pad32(takeA ? i + 1 : la + j + 1)];
+            i += takeA ? 1u : 0u;
+            j += takeA ? 0u : 1u;
+            a = takeA ? w : a;
+            b = takeA ? b : w;
+          }
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (q0 + e < L) sm[pad32(q0 + e)] = val[e];
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const uint32_t i = threadIdx.x + e * kThreads;
+        if (i < L) out[d0 + i] = sm[pad32(i)];
       }
     }
     __syncthreads();
@@ -1079,6 +1108,7 @@ __device__ __forceinline__ void fuse_classify(Stage* stp, uint32_t j, K* sbuf, u
       }
     }
   }
+  if (!stp->out2) kept = isN;  // no Full' is written: only the new tuples are kept
   // one scan for both counts: N in the high half, kept in the low half
   unsigned long long tot;
   const unsigned long long both = ((unsigned long long)__popc(isN) << 32) | __popc(kept);
@@ -1111,6 +1141,16 @@ __device__ __forceinline__ void fuse_write(Stage* stp, const K* sbuf, const uint
   // new tuples are few: each thread stores its own run of them directly,
   // visiting only the set bits (a new tuple's place among the kept elements
   // is the number of kept bits below it)
+  if (!Fall) {  // the pass only finds what Full lacks: the kept elements, coalesced
+    K* no = Nall + sg.out_off + exN;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const uint32_t i = threadIdx.x + e * kThreads;
+      if (i < m.totN) no[i] = sbuf[pad32(i)];
+    }
+    if (threadIdx.x == 0 && m.last) stp->segs[m.k].res = exN + m.totN;
+    return;
+  }
   const uint32_t mk = smask[threadIdx.x], pr = spre[threadIdx.x];
   const uint32_t kept = mk & 0xFFFFu, wk0 = pr & 0xFFFFu;
   K* no = Nall + sg.out_off + exN + (pr >> 16);
@@ -1118,13 +1158,11 @@ __device__ __forceinline__ void fuse_write(Stage* stp, const K* sbuf, const uint
     const uint32_t e = __ffs(nb) - 1;
     *no++ = sbuf[pad32(wk0 + __popc(kept & ((1u << e) - 1u)))];
   }
-  if (Fall) {  // no Full' when the pass only finds what the main run lacks (side iteration)
-    K* fo = Fall + sg.out2_off + m.a0 + exN;
+  K* fo = Fall + sg.out2_off + m.a0 + exN;
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const uint32_t i = threadIdx.x + e * kThreads;
-      if (i < m.totK) fo[i] = sbuf[pad32(i)];
-    }
+  for (int e = 0; e < E; ++e) {
+    const uint32_t i = threadIdx.x + e * kThreads;
+    if (i < m.totK) fo[i] = sbuf[pad32(i)];
   }
   if (threadIdx.x == 0 && m.last) stp->segs[m.k].res = exN + m.totN;
 }
