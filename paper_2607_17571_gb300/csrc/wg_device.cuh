@@ -237,9 +237,9 @@ struct Dev {
 struct RowInst {
   const uint32_t* off;          // CSR
   const uint32_t* adj;
-  const void* rec;              // vertex records, 32 bytes each
+  const void* rec;              // vertex records, 16 bytes each
   const uint32_t* ns;           // bit set of the vertices with out-edges
-  const void* units;            // adjacency past the records, in 16-byte units
+  const void* units;            // neighbours past the records, in 16-byte units
   const uint32_t* mp;           // bit set of the vertices with several parents
   uint32_t* bits;               // row x's bit set: words [x * words, (x + 1) * words)
   uint32_t* cnt;                // tuples of row x

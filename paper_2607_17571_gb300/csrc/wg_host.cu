@@ -403,7 +403,7 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
                 grid_of(c, 4), c->stream);
   CK(cudaGetLastError());
   if (R->nv <= kRowMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
-    R->o_ns = round_up((size_t)R->nv * 32);
+    R->o_ns = round_up((size_t)R->nv * 16);
     R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
     R->o_mp = R->o_units + round_up(row_units(ne, R->nv, R->id_bytes()) * 16);
     TRY(R->rowv.get(c, R->o_mp + (size_t)R->row_words() * 8));

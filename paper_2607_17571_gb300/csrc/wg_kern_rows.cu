@@ -33,30 +33,30 @@ namespace wg {
 template <typename K, typename IdT>
 __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne, uint32_t w,
                                                          const uint32_t* off, const uint32_t* adj,
-                                                         uint32_t nv, uint4* rec, uint32_t* ns,
+                                                         uint32_t nv, IdT* rec, uint32_t* ns,
                                                          uint32_t words, IdT* units, uint32_t* mp) {
+  constexpr uint32_t U = Unit<IdT>::n, kRecIds = U - 1, kTop = sizeof(IdT) == 2 ? 0xFFFFu : 0xFFFFFFFFu;
   const uint32_t stride = gridDim.x * kThreads, t = blockIdx.x * kThreads + threadIdx.x;
   for (uint32_t v = t; v < words * 32; v += stride) {
-    uint32_t o = 0, d = 0;
+    uint32_t d = 0;
     if (v < nv) {
-      o = off[v];
-      d = off[v + 1] - o;
-      rec[2 * (size_t)v] = uint4{unit_start<IdT>(o, v), d, 0, 0};
+      d = off[v + 1] - off[v];
+      rec[U * (size_t)v] = (IdT)min(d, kTop);
     }
     const uint32_t m = __ballot_sync(0xffffffffu, d > 0);
     if ((v & 31) == 0) ns[v >> 5] = m;
   }
   for (uint32_t i = t; i < ne; i += stride) {
-    constexpr uint32_t U = Unit<IdT>::n;
-    const uint32_t x = (uint32_t)(E[i] >> w), o = off[x], j = i - o;
-    IdT* to = j < U ? (IdT*)(rec + 2 * (size_t)x + 1) + j
-                    : units + (size_t)unit_start<IdT>(o, x) * U + (j - U);
-    const IdT z = (IdT)adj[i];
+    const uint32_t x = (uint32_t)(E[i] >> w), o = off[x], j = i - o, z = adj[i];
     const uint32_t bit = 1u << (z & 31);  // (mp: several parents; after it: at least one)
     if (atomicOr(mp + words + (z >> 5), bit) & bit) atomicOr(mp + (z >> 5), bit);
-    *to = z;
-    if (i + 1 == off[x + 1])
-      for (uint32_t r = j % U + 1; r < U; ++r) *++to = z;
+    IdT* to = j < kRecIds ? rec + U * (size_t)x + 1 + j
+                          : units + (size_t)unit_start<IdT>(o, x) * U + (j - kRecIds);
+    *to = (IdT)z;
+    if (i + 1 == off[x + 1]) {
+      const uint32_t room = j < kRecIds ? kRecIds - 1 - j : U - 1 - (j - kRecIds) % U;
+      for (uint32_t r = 0; r < room; ++r) *++to = (IdT)z;
+    }
   }
 }
 
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
 // the rest (the delta) into S and list the delta's vertices that have out-edges
 // (on the R-MAT workloads 4 to 5 in 10 have none); the warps then expand the
 // list 32 vertices at a time: each lane its vertex's record, then the vertices'
-// further units as one strip, 32 units per step, a lane finding its unit's
+// units as one strip, 32 units per step, a lane finding its unit's
 // vertex from the bit mask of the strip's first units.  Setting a bit in the
 // next N needs no answer, so a candidate costs one shared atomic and no list of
 // winners is kept; scanning N costs words / 128 lane steps per iteration.  Two
@@ -559,10 +559,10 @@ void launch_row_layout(const K* E, uint32_t ne, uint32_t w, const uint32_t* off,
                        void* units, uint32_t* mp, int id_bytes, int grid, cudaStream_t s) {
   cudaMemsetAsync(mp, 0, (size_t)words * 8, s);
   if (id_bytes == 2)
-    k_row_layout<K, uint16_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
+    k_row_layout<K, uint16_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint16_t*)rec, ns,
                                                         words, (uint16_t*)units, mp);
   else
-    k_row_layout<K, uint32_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint4*)rec, ns,
+    k_row_layout<K, uint32_t><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, nv, (uint32_t*)rec, ns,
                                                         words, (uint32_t*)units, mp);
 }
 template void launch_row_expand<uint32_t>(const RowJob&, int, cudaStream_t);

@@ -72,7 +72,7 @@ void launch_rows_small(const RowJob& J, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
 // adjacency units of a relation: their number, and the layout of vertex records
-// (32 bytes each), out-edge bit set (words), further units (16 bytes each), bit set
+// (16 bytes each), out-edge bit set (words), further units (16 bytes each), bit set
 // of the vertices with several parents (words; followed by as many of scratch)
 size_t row_units(uint64_t ne, uint32_t nv, int id_bytes);
 template <typename K>

@@ -5,22 +5,22 @@
 
 namespace wg {
 
-// Adjacency in units of 16 bytes (8 16-bit or 4 32-bit ranks).  Each vertex has
-// a 32-byte record (one sector): {first further unit, degree, -, -} and its
-// first unit, so one access gives most vertices' whole adjacency.  Its further
-// units start at (off[v] + (U-1) v + U-1) / U: room for every vertex before it
-// without a scan.  A unit's unused places repeat the vertex's last neighbour
-// (setting a bit twice is harmless), so no place needs a test.
+// Adjacency in units of 16 bytes (U = 8 16-bit or 4 32-bit ranks).  Each vertex
+// has a record {degree (16 bits saturate), its first U-1 neighbours}: one load
+// gives most vertices' whole adjacency.  Its further neighbours lie in units from
+// (off[v] + (U-1) v + U-1) / U: room for every vertex before it without a scan.
+// Unused places repeat the vertex's last neighbour (setting a bit twice is
+// harmless).
 template <typename IdT> struct Unit { static constexpr uint32_t n = 16 / sizeof(IdT); };
 template <typename IdT>
 __device__ __forceinline__ uint32_t unit_start(uint32_t off, uint32_t v) {
   constexpr uint32_t U = Unit<IdT>::n;
   return (off + (U - 1) * (v + 1)) / U;
 }
-// The bits of places [2p, 2p + 2) of a unit (16-bit ranks) or place p (32-bit).
 __device__ __forceinline__ void set_bit(uint32_t* n, uint32_t byte_off, uint32_t z) {
   atomicOr((uint32_t*)((char*)n + byte_off), __funnelshift_l(0u, 1u, z));  // 1 << (z & 31)
 }
+// The bits of the two 16-bit ranks, or the 32-bit rank, in a word.
 __device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint16_t) {
   set_bit(n, (v >> 3) & 0x1FFCu, v);
   set_bit(n, (v >> 19) & 0x1FFCu, v >> 16);
@@ -28,6 +28,29 @@ __device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint16_t) {
 __device__ __forceinline__ void set_part(uint32_t* n, uint32_t v, uint32_t) {
   set_bit(n, (v >> 3) & ~3u, v);
 }
+// A vertex's record: its degree, and the bits of its neighbours there (pairs by
+// the lane's own degree: the shared atomics, not the tests, are the scarce part).
+template <typename IdT> struct Rec;
+template <> struct Rec<uint16_t> {
+  uint4 a;
+  __device__ __forceinline__ void load(const void* rec, uint32_t v) { a = __ldg((const uint4*)rec + v); }
+  __device__ __forceinline__ uint32_t deg() const { return a.x & 0xFFFFu; }
+  __device__ __forceinline__ void set(uint32_t* n, uint32_t deg) const {
+    set_bit(n, (a.x >> 19) & 0x1FFCu, a.x >> 16);
+    if (deg > 1) set_part(n, a.y, uint16_t());
+    if (deg > 3) set_part(n, a.z, uint16_t());
+    if (deg > 5) set_part(n, a.w, uint16_t());
+  }
+};
+template <> struct Rec<uint32_t> {
+  uint4 a;
+  __device__ __forceinline__ void load(const void* rec, uint32_t v) { a = __ldg((const uint4*)rec + v); }
+  __device__ __forceinline__ uint32_t deg() const { return a.x; }
+  __device__ __forceinline__ void set(uint32_t* n, uint32_t deg) const {
+    set_part(n, a.y, uint32_t());
+    if (deg > 1) { set_part(n, a.z, uint32_t()); set_part(n, a.w, uint32_t()); }
+  }
+};
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
 #pragma unroll
@@ -40,33 +63,34 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
 
 // The bits of the neighbours of vertices l[0..n), 1 <= n <= 32, each with at
 // least one, into the bit set N (shared memory): one warp, each lane its vertex's
-// record, then the vertices' further units as one strip, 32 units per step, a
+// record, then the vertices' units as one strip, 32 units per step, a
 // lane finding its unit's vertex from the bit mask of the strip's first units.
 // strip: 32 words of the warp.  Returns the degree of the lane's vertex.
 template <typename IdT>
 __device__ __forceinline__ uint32_t expand_vertices(const RowInst& I, const IdT* l, uint32_t n,
                                                     uint32_t* N, uint32_t* strip) {
-  constexpr uint32_t U = Unit<IdT>::n, P = U / 4;  // places in a unit, and in a word of one
+  constexpr uint32_t U = Unit<IdT>::n, kRecIds = U - 1;
   const uint32_t lane = threadIdx.x & 31, upto = 0xFFFFFFFFu >> (31 - lane);
   uint32_t us = 0, deg = 0;
-  uint4 u = {0, 0, 0, 0};
   if (lane < n) {
-    const uint4* r = (const uint4*)I.rec + 2 * (size_t)l[lane];
-    const uint2 t = __ldg((const uint2*)r);
-    u = __ldg(r + 1);
-    us = t.x;
-    deg = t.y;
+    const uint32_t v = l[lane];
+    Rec<IdT> r;
+    r.load(I.rec, v);
+    deg = r.deg();
+    uint32_t o = 0, o1 = 0;
+    if (deg > kRecIds) {
+      o = __ldg(I.off + v);
+      o1 = __ldg(I.off + v + 1);
+    }
+    r.set(N, deg);
+    if (deg > kRecIds) {
+      deg = o1 - o;
+      us = unit_start<IdT>(o, v);
+    }
   }
-  const uint32_t most = __reduce_max_sync(0xffffffffu, deg);
-  if (lane < n) {
-    set_part(N, u.x, IdT());
-    if (most > P) set_part(N, u.y, IdT());
-    if (most > 2 * P) set_part(N, u.z, IdT());
-    if (most > 3 * P) set_part(N, u.w, IdT());
-  }
-  if (most <= U) return deg;
-  const uint32_t more = deg > U ? (deg - 1) / U : 0u;  // further units
+  const uint32_t more = deg > kRecIds ? (deg - kRecIds + U - 1) / U : 0u;  // units
   const uint32_t has = __ballot_sync(0xffffffffu, more > 0);
+  if (!has) return deg;
   const uint32_t in = warp_incl_scan(more, lane);
   const uint32_t tot = __shfl_sync(0xffffffffu, in, 31), st = in - more;
   if (more) strip[__popc(has & upto) - 1] = us - st;
@@ -78,7 +102,7 @@ __device__ __forceinline__ uint32_t expand_vertices(const RowInst& I, const IdT*
     const uint32_t t = strip[prev + __popc(m & upto) - 1];
     prev += __popc(m);
     if (e < tot) {
-      u = __ldg((const uint4*)I.units + (t + e));
+      const uint4 u = __ldg((const uint4*)I.units + (t + e));
       set_part(N, u.x, IdT());
       set_part(N, u.y, IdT());
       set_part(N, u.z, IdT());

@@ -65,7 +65,7 @@ def test_vertex_counts(ctx, nv):
     _check(ctx, *_pairs(nv, [(top, 0), (0, 1 % nv), (top, top)]))
 
 
-@pytest.mark.parametrize("deg", [1, 6, 7, 8, 9, 31, 38, 39, 40, 71, 1023, 1024, 1025, 3000])
+@pytest.mark.parametrize("deg", [1, 6, 7, 8, 9, 11, 12, 15, 16, 31, 39, 40, 71, 1023, 1024, 1025, 3000])
 def test_degrees(ctx, deg):
     _check(ctx, *_star(deg, min(deg, 40)))
     # the hub reached from others, itself among its own successors
