@@ -256,6 +256,13 @@ struct RowInst {
 struct RowCtl {
   uint32_t next_row, pad;
 };
+constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
+// What a single query's run found, in page-locked host memory.
+struct RowReport {
+  unsigned long long n_total, cand;
+  uint32_t last, fits, n_big, error;
+  unsigned long long log[kRowLog];
+};
 // One launch over the rows of one or more instances.
 struct RowJob {
   RowCtl* ctl;
@@ -270,10 +277,11 @@ struct RowJob {
   uint32_t* small;
   uint32_t slots, pad;
   const struct SgInst* sg;      // same-generation: which pieces of the rows are valid (or NULL)
+  const struct SgCtl* sg_ctl;   // ... and its control block (or NULL)
+  RowReport* report;            // written by k_row_plan (or NULL)
 };
 constexpr uint32_t kRowChunk = 256;
 constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are expanded
-constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
 constexpr uint32_t kRowSmemMax = 216 * 1024;
 // Tuples of a row k_rows_small takes (128 / 256 / 512, whole call: ER 400,000 /
 // 360,000 1.74 / 1.08 / 1.08 ms, R-MAT 2^19 / 400k 12.6 / 12.7 / 13.1 ms).

@@ -91,6 +91,10 @@ struct wg_ctx {
   uint64_t excl = 0;  // batch query that runs with the whole budget (0: none), see batch_preempt
   uint64_t solo_run = 0;  // the served request running on a single-query engine (0: none)
   std::vector<std::unique_ptr<RowLane>> lanes;    // batched row-by-row queries
+  std::map<uint64_t, int> occ;            // resident CTAs per SM by kernel (see occ_of)
+  std::vector<cudaEvent_t> events;        // timing events of freed queries
+  std::vector<RowReport*> reports;        // unused reports, from page-locked slabs
+  std::vector<void*> report_slabs;
   // tile shapes engines are built with, per key width (index 0: 4-byte keys,
   // 1: 8-byte); 0 = the compiled default.  Set by wg_autotune / wg_set_tiles.
   uint32_t tune_count[2] = {0, 0}, tune_fuse[2] = {0, 0}, tune_emit[2] = {0, 0};
@@ -170,6 +174,49 @@ struct DBuf {
 };
 
 static int grid_of(wg_ctx* c, int occ) { return c->num_sms * std::max(1, occ); }
+
+// Occupancies are asked for once per context: the query costs microseconds, a
+// small fixpoint tens of them.
+template <typename F>
+static int occ_of(wg_ctx* c, uint64_t family, uint64_t key, F ask) {
+  auto it = c->occ.emplace(family << 48 | key, 0);
+  if (it.second) it.first->second = ask();
+  return it.first->second;
+}
+template <typename K> static int occ_sort(wg_ctx* c, int which) {
+  return occ_of(c, 1, sizeof(K) << 8 | which, [&] { return occupancy_sort<K>(which); });
+}
+template <typename K> static int occ_join(wg_ctx* c, int which) {
+  return occ_of(c, 2, sizeof(K) << 8 | which, [&] { return occupancy_join<K>(which); });
+}
+static int occ_rows(wg_ctx* c, bool sg, int id_bytes, uint32_t words) {
+  return occ_of(c, sg ? 3 : 4, (uint64_t)words << 8 | id_bytes, [&] {
+    return sg ? occupancy_sg(id_bytes, words) : occupancy_rows(id_bytes, words);
+  });
+}
+
+// Timing events and page-locked reports are kept for the next query or engine.
+static int take_event(wg_ctx* c, cudaEvent_t* e) {
+  if (c->events.empty()) {
+    CK(cudaEventCreate(e));
+  } else {
+    *e = c->events.back();
+    c->events.pop_back();
+  }
+  return WG_OK;
+}
+static int take_report(wg_ctx* c, RowReport** r) {
+  if (c->reports.empty()) {
+    constexpr int n = 64;
+    RowReport* slab = nullptr;
+    CK(cudaMallocHost((void**)&slab, n * sizeof(RowReport)));
+    c->report_slabs.push_back(slab);
+    for (int i = 0; i < n; ++i) c->reports.push_back(slab + i);
+  }
+  *r = c->reports.back();
+  c->reports.pop_back();
+  return WG_OK;
+}
 
 // ------------------------------------------------------------------ primitives
 // Standalone segmented stages on one segment (relation load, wg_sort_keys,
@@ -255,9 +302,9 @@ static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
     s.shift = p * dbits; s.pass = p; s.epoch = prim_epoch(c);
     TRY(prim_put(c, S_PASS0 + p, s));
   }
-  launch_sort_hist<K>(c->s_stage + S_HIST, grid_of(c, occupancy_sort<K>(0)), c->stream);
+  launch_sort_hist<K>(c->s_stage + S_HIST, grid_of(c, occ_sort<K>(c, 0)), c->stream);
   for (uint32_t p = 0; p < passes; ++p)
-    launch_sort_pass<K>(c->s_stage + S_PASS0 + p, grid_of(c, occupancy_sort<K>(1)), c->stream, dbits);
+    launch_sort_pass<K>(c->s_stage + S_PASS0 + p, grid_of(c, occ_sort<K>(c, 1)), c->stream, dbits);
   CK(cudaGetLastError());
   if (passes & 1) CK(cudaMemcpyAsync(keys, c->s_tmp, n * sizeof(K), cudaMemcpyDeviceToDevice, c->stream));
   return WG_OK;
@@ -292,7 +339,7 @@ static int prim_unique(wg_ctx* c, const K* in, size_t n, const K* full, size_t n
     f.splits = (unsigned long long*)c->s_tmp;
     TRY(prim_put(c, S_FUSE, f));
     launch_partition<K>(c->s_stage + S_FUSE, 0, T, c->num_sms * 4, c->stream);
-    launch_diff_merge<K>(c->s_stage + S_FUSE, grid_of(c, occupancy_sort<K>(4)), c->stream, T);
+    launch_diff_merge<K>(c->s_stage + S_FUSE, grid_of(c, occ_sort<K>(c, 4)), c->stream, T);
   } else {
     const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
     TRY(prim_scratch(c, 0, ntiles));
@@ -301,7 +348,7 @@ static int prim_unique(wg_ctx* c, const K* in, size_t n, const K* full, size_t n
     Stage u = prim_stage(c, ntiles);
     u.in = in; u.aux = full; u.out = out; u.epoch = prim_epoch(c);
     TRY(prim_put(c, S_UNIQ, u));
-    launch_unique_diff<K>(c->s_stage + S_UNIQ, grid_of(c, occupancy_sort<K>(2)), c->stream);
+    launch_unique_diff<K>(c->s_stage + S_UNIQ, grid_of(c, occ_sort<K>(c, 2)), c->stream);
   }
   CK(cudaGetLastError());
   Seg back{};
@@ -338,7 +385,7 @@ static int prim_merge(wg_ctx* c, const K* a, size_t na, const K* b, size_t nb, K
   m.splits = rc == WG_OK ? (unsigned long long*)c->s_tmp : nullptr;
   TRY(prim_put(c, S_MERGE, m));
   if (m.splits) launch_partition<K>(c->s_stage + S_MERGE, 0, kTileM, c->num_sms * 4, c->stream);
-  launch_merge<K>(c->s_stage + S_MERGE, grid_of(c, occupancy_sort<K>(3)), c->stream);
+  launch_merge<K>(c->s_stage + S_MERGE, grid_of(c, occ_sort<K>(c, 3)), c->stream);
   CK(cudaGetLastError());
   return WG_OK;
 }
@@ -517,7 +564,7 @@ static int tri_count(wg_ctx* c, Relation* R, unsigned long long* count) {
   k.in = R->keys.p; k.inst = (Inst*)inst.p; k.pos = (unsigned long long*)pos.p;
   k.epoch = prim_epoch(c);
   TRY(prim_put(c, S_COUNT, k));
-  launch_join_count<K>(c->s_stage + S_COUNT, grid_of(c, occupancy_join<K>(0)), c->stream, kTileD);
+  launch_join_count<K>(c->s_stage + S_COUNT, grid_of(c, occ_join<K>(c, 0)), c->stream, kTileD);
   CK(cudaGetLastError());
   Seg back{};
   Ctl ctl{};
@@ -539,7 +586,7 @@ static int tri_count(wg_ctx* c, Relation* R, unsigned long long* count) {
     e.splits = (unsigned long long*)spl.p; e.probe = (unsigned long long*)hits.p;
     TRY(prim_put(c, S_EMIT, e));
     launch_partition<K>(c->s_stage + S_EMIT, 1, kTileC, c->num_sms * 4, c->stream);
-    launch_tri_probe<K>(c->s_stage + S_EMIT, grid_of(c, occupancy_join<K>(2)), c->stream);
+    launch_tri_probe<K>(c->s_stage + S_EMIT, grid_of(c, occ_join<K>(c, 2)), c->stream);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(count, hits.p, 8, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(&ctl, c->s_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
@@ -673,6 +720,7 @@ struct Engine : EngineBase {
   bool row_sg = false;               // the query is same-generation
   SgJob sg{};
   SgInst sgi{};
+  RowReport* report = nullptr;       // page-locked: what a run found, written by k_row_plan
   size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
   int id_bytes = 2, g_rows = 0;
   bool expand_only = false;          // the rows are done; the result waits for a larger buffer
@@ -712,6 +760,8 @@ struct Engine : EngineBase {
     exec = nullptr; graph = nullptr;
     if (ev_done) cudaEventDestroy(ev_done);
     ev_done = nullptr;
+    if (report) c->reports.push_back(report);
+    report = nullptr;
     DBuf* all[] = {&b_dev, &b_inst, &b_seg, &b_log, &D[0], &D[1], &C[0], &C[1], &F[0], &F[1],
                    &R, &pos, &st_s, &st_k, &hist, &spl, &xlen_b, &segx_b, &tseg_b, &xsum_b,
                    &mix_b, &G[0], &G[1], &xord_b, &row_meta, &row_bits, &row_small};
@@ -741,6 +791,7 @@ struct Engine : EngineBase {
     if (rows_) {
       hi.assign(1, Inst{});
       CK(cudaEventCreateWithFlags(&ev_done, cudaEventDisableTiming));
+      TRY(take_report(c, &report));
       return WG_OK;
     }
     AllocScope scope(c, st);
@@ -775,15 +826,15 @@ struct Engine : EngineBase {
     for (int i = 0; i < S_NUM; ++i) h.st[i].ctl = (Ctl*)((char*)dv + offsetof(Dev, ctl));
     CK(cudaMemcpyAsync(dv, &h, sizeof(Dev), cudaMemcpyHostToDevice, st));
     CK(cudaEventCreateWithFlags(&ev_done, cudaEventDisableTiming));
-    g_count = grid_of(c, occupancy_join<K>(count_tile_ == (uint32_t)kTileD ? 0 : 3));
-    g_emit = grid_of(c, occupancy_join<K>(emit_tile_ == (uint32_t)kTileC ? 1 : 4));
-    g_hist = grid_of(c, occupancy_sort<K>(0));
-    g_pass = grid_of(c, occupancy_sort<K>(1));
-    g_seg = grid_of(c, occupancy_sort<K>(sort_mode_ == WG_SORT_SEGMENT8 ? 7
+    g_count = grid_of(c, occ_join<K>(c, count_tile_ == (uint32_t)kTileD ? 0 : 3));
+    g_emit = grid_of(c, occ_join<K>(c, emit_tile_ == (uint32_t)kTileC ? 1 : 4));
+    g_hist = grid_of(c, occ_sort<K>(c, 0));
+    g_pass = grid_of(c, occ_sort<K>(c, 1));
+    g_seg = grid_of(c, occ_sort<K>(c, sort_mode_ == WG_SORT_SEGMENT8 ? 7
                                          : sort_mode_ == WG_SORT_SEGMENT_WIDE ? 8 : 6));
-    g_uniq = grid_of(c, occupancy_sort<K>(2));
-    g_merge = grid_of(c, occupancy_sort<K>(3));
-    g_fuse = grid_of(c, occupancy_sort<K>(fuse_tile_ == (uint32_t)FuseTile<K>::T ? 4 : 5));
+    g_uniq = grid_of(c, occ_sort<K>(c, 2));
+    g_merge = grid_of(c, occ_sort<K>(c, 3));
+    g_fuse = grid_of(c, occ_sort<K>(c, fuse_tile_ == (uint32_t)FuseTile<K>::T ? 4 : 5));
     return WG_OK;
   }
 
@@ -950,7 +1001,7 @@ struct Engine : EngineBase {
     const bool small = !row_sg && Rl->small_rows();
     id_bytes = Rl->id_bytes();
     g_rows = (int)std::min<uint64_t>(
-        grid_of(c, row_sg ? occupancy_sg(id_bytes, words) : occupancy_rows(id_bytes, words)),
+        grid_of(c, occ_rows(c, row_sg, id_bytes, words)),
         std::max<uint32_t>(nv, 1));
     // control block | chunk sums | log | same-generation: masks, marks (cleared) |
     // instance | chunk offsets | row counts | row lists
@@ -989,6 +1040,7 @@ struct Engine : EngineBase {
     job.ctl = (RowCtl*)(m + o_ctl); job.inst = (RowInst*)(m + o_inst);
     job.csum = (uint32_t*)(m + o_sum); job.cbase = (unsigned long long*)(m + o_base);
     job.nrows = nv; job.vwords = words;
+    job.report = report;
     if (small) {
       job.rows = (uint32_t*)(m + o_rows);
       job.small = (uint32_t*)row_small.p;
@@ -1003,6 +1055,7 @@ struct Engine : EngineBase {
       sgi.act = (uint32_t*)(m + o_act);
       sgi.mw = Rl->sg_mask_words();
       job.sg = (SgInst*)(m + o_sgi);
+      job.sg_ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
       sg = SgJob{};
       sg.rows = job;
       sg.ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
@@ -1033,15 +1086,14 @@ struct Engine : EngineBase {
     ri.out = F[0].p;
     ri.out_cap = capF;
     if (expand_only) ri.fits = 1;
-    CK(cudaMemcpyAsync(job.inst, &ri, sizeof(ri), cudaMemcpyHostToDevice, st));
+    launch_row_begin(job, ri, sgi, row_meta.p, expand_only ? 0 : row_clear, c->num_sms, st);
+    launches_issued += 1;
     if (!expand_only) {
-      CK(cudaMemsetAsync(row_meta.p, 0, row_clear, st));
       if (job.rows) {
         launch_rows_small(job, grid_of(c, 6), st);
         launches_issued += 2;  // (and k_row_expand_small)
       }
       if (row_sg) {
-        CK(cudaMemcpyAsync(sg.sg, &sgi, sizeof(sgi), cudaMemcpyHostToDevice, st));
         CK(launch_sg(sg, id_bytes, g_rows, c->num_sms, st));
         launches_issued += 3;
       } else if (ri.nv) {
@@ -1059,12 +1111,15 @@ struct Engine : EngineBase {
     return WG_OK;
   }
   int rows_settle(bool* again) {
-    CK(cudaMemcpyAsync(&ri, job.inst, sizeof(ri), cudaMemcpyDeviceToHost, st));
-    SgCtl sc{};
-    if (row_sg && !expand_only)
-      CK(cudaMemcpyAsync(&sc, sg.ctl, sizeof(sc), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (sc.error) return set_err(WG_E_DEVICE_TIMEOUT, "a bounded device wait gave up");
+    // (the launch is over: the caller waited for ev_done)
+    if (!expand_only) {
+      ri.n_total = report->n_total;
+      ri.cand = report->cand;
+      ri.last = report->last;
+      ri.fits = report->fits;
+      ri.n_big = report->n_big;
+    }
+    if (!expand_only && report->error) return set_err(WG_E_DEVICE_TIMEOUT, "a bounded device wait gave up");
     Inst& I = hi[0];
     I.n_full = ri.n_total;
     I.cand_total = ri.cand;
@@ -1083,6 +1138,14 @@ struct Engine : EngineBase {
     const bool capped = ri.last >= ri.max_iters;
     I.iters_done = capped ? ri.max_iters : ri.last + 1;
     I.state = capped ? INST_ITERCAP : INST_DONE;
+    return WG_OK;
+  }
+
+  // The first n delta sizes of the run.
+  int rows_log(uint32_t n, unsigned long long* to) {
+    std::memcpy(to, report->log, std::min(n, kRowLog) * 8);
+    if (n > kRowLog)
+      CK(cudaMemcpy(to + kRowLog, ri.log + kRowLog, (n - kRowLog) * 8, cudaMemcpyDeviceToHost));
     return WG_OK;
   }
 
@@ -1512,6 +1575,7 @@ static int single_start(wg_ctx* c, Query* q) {
     TRY(E->rows_begin(Rl, q->kind, q->opts.max_iters, wantF));
     CK(cudaEventRecord(q->ev0, c->stream));
     TRY(E->rows_launch());
+    CK(cudaEventRecord(q->ev1, c->stream));
     q->state = WG_RUNNING;
     return WG_OK;
   }
@@ -1645,10 +1709,11 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     }
     if (again) {
       TRY(E->launch(0xFFFFFFFFu, loop_mode(q)));
+      if (E->rows_) CK(cudaEventRecord(q->ev1, c->stream));
       continue;
     }
     const Inst& I = E->hi[0];
-    if (!q->opts.profile) CK(cudaEventRecord(q->ev1, c->stream));
+    if (!q->opts.profile && !E->rows_) CK(cudaEventRecord(q->ev1, c->stream));
     CK(cudaEventSynchronize(q->ev1));
     float ms = 0;
     cudaEventElapsedTime(&ms, q->ev0, q->ev1);
@@ -1661,7 +1726,8 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     q->res_ptr = (const K*)E->pool_ptr(I.res_pool) + I.res_off;
     const uint32_t nlog = std::min<uint32_t>(I.iters_done + 1, E->log_cap);
     q->log.assign(nlog, 0);
-    CK(cudaMemcpy(q->log.data(), I.log, nlog * 8, cudaMemcpyDeviceToHost));
+    if (E->rows_) TRY(E->rows_log(nlog, q->log.data()));
+    else CK(cudaMemcpy(q->log.data(), I.log, nlog * 8, cudaMemcpyDeviceToHost));
     q->rel->peak_cand = std::max<uint64_t>(q->rel->peak_cand, E->capC);
     q->rel->peak_full = std::max<uint64_t>(q->rel->peak_full, E->capF);
     if (I.state == INST_ITERCAP) {
@@ -2300,7 +2366,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   }
   L->log_cap = std::min(kBatchLogCap, nv_max + 2);
   const int grid = (int)std::min<uint64_t>(
-      grid_of(c, L->sg ? occupancy_sg(idb, vwords) : occupancy_rows(idb, vwords)),
+      grid_of(c, occ_rows(c, L->sg, idb, vwords)),
       (uint64_t)nch * kRowChunk);
   auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
   size_t end = 0;
@@ -2677,6 +2743,8 @@ void wg_destroy(wg_ctx* c) {
   g_binfo.erase(c);
   for (auto& kv : c->rels) kv.second->release(c);
   c->rels.clear();
+  for (cudaEvent_t e : c->events) cudaEventDestroy(e);
+  for (void* p : c->report_slabs) cudaFreeHost(p);
   dev_free(c, c->s_tmp, c->s_tmp_bytes);
   dev_free(c, c->s_status, c->s_status_n * 8);
   dev_free(c, c->s_hist, sizeof(unsigned long long) * kMaxPasses * kRadix);
@@ -2757,8 +2825,8 @@ static int make_query(wg_ctx* c, int kind, wg_rel edges, const wg_opts* opts, Qu
   q->rel_id = edges;
   if (opts) q->opts = *opts;
   if (q->opts.max_iters == 0) q->opts.max_iters = 1u << 20;
-  CK(cudaEventCreate(&q->ev0));
-  CK(cudaEventCreate(&q->ev1));
+  TRY(take_event(c, &q->ev0));
+  TRY(take_event(c, &q->ev1));
   q->t_submit_us = now_us();
   *out = q.get();
   c->queries[q->id] = std::move(q);
@@ -2877,7 +2945,9 @@ static int solo_resume(wg_ctx* c, Query* q) {
   }
   TRY(rc);
   q->solo_wait = false;
-  return E->launch(0xFFFFFFFFu, loop_mode(q));
+  TRY(E->launch(0xFFFFFFFFu, loop_mode(q)));
+  if (E->rows_) CK(cudaEventRecord(q->ev1, c->stream));
+  return WG_OK;
 }
 
 static void solo_requeue(wg_ctx* c, Query* q) {
@@ -3335,8 +3405,8 @@ void wg_query_free(wg_ctx* c, wg_query id) {
   }
   cudaStreamSynchronize(c->stream);
   q->res_own.release(c);
-  if (q->ev0) cudaEventDestroy(q->ev0);
-  if (q->ev1) cudaEventDestroy(q->ev1);
+  if (q->ev0) c->events.push_back(q->ev0);
+  if (q->ev1) c->events.push_back(q->ev1);
   if (q->own) c->idle.push_back(std::move(q->own));  // keep pools and graph for the next query
   c->queries.erase(it);
 }

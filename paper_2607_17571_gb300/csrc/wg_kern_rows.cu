@@ -372,6 +372,18 @@ __global__ void __launch_bounds__(kThreads) k_row_expand_small(RowJob J) {
   }
 }
 
+// The start of a single query: its instance, from the launch's arguments, and the
+// cleared scratch (one launch in place of two small copies and a memset).
+__global__ void __launch_bounds__(kThreads) k_row_begin(RowJob J, RowInst I, SgInst G, uint4* clear,
+                                                        size_t n) {
+  const size_t t = (size_t)blockIdx.x * kThreads + threadIdx.x;
+  if (t == 0) {
+    *J.inst = I;
+    if (J.sg) *(SgInst*)J.sg = G;
+  }
+  for (size_t i = t; i < n; i += (size_t)gridDim.x * kThreads) clear[i] = uint4{0, 0, 0, 0};
+}
+
 // Row offsets at chunk granularity, totals and the capacity check: one CTA per
 // instance scans its chunk sums in place (counts in, exclusive offsets out).
 __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
@@ -409,7 +421,17 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
     I->n_total = carry;
     // an output buffer that is too small: the expansion waits for a larger one
     I->fits = carry <= I->out_cap && !(J.rows && I->n_big > J.slots) ? 1u : 0u;
+    if (RowReport* r = J.report) {
+      r->n_total = carry;
+      r->cand = I->cand;
+      r->last = I->last;
+      r->fits = I->fits;
+      r->n_big = I->n_big;
+      r->error = J.sg_ctl ? J.sg_ctl->error : 0u;
+    }
   }
+  if (J.report && threadIdx.x < kRowLog)
+    J.report->log[threadIdx.x] = threadIdx.x < I->log_cap ? I->log[threadIdx.x] : 0ull;
 }
 
 // Bit sets -> sorted packed keys (x << w) | z, one warp per row: 64 words at a
@@ -539,6 +561,12 @@ void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s) {
 }
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s) {
   k_row_plan<<<n_inst, 1024, 0, s>>>(J);
+}
+void launch_row_begin(const RowJob& J, const RowInst& I, const SgInst& G, void* clear,
+                      size_t bytes, int sms, cudaStream_t s) {
+  const size_t n = bytes / 16, ctas = (n + kThreads - 1) / kThreads;
+  k_row_begin<<<(int)min(max(ctas, (size_t)1), (size_t)sms * 8), kThreads, 0, s>>>(J, I, G,
+                                                                                 (uint4*)clear, n);
 }
 void launch_rows_small(const RowJob& J, int grid, cudaStream_t s) {
   k_rows_small<<<grid, kThreads, 0, s>>>(J);

@@ -15,6 +15,8 @@ struct Inst;
 struct RowJob;
 struct TriJob;
 struct SgJob;
+struct RowInst;
+struct SgInst;
 
 // sorted-array stages (wg_kern_sort.cu); K = uint32_t or unsigned long long
 template <typename K> void launch_sort_hist(Stage* st, int grid, cudaStream_t s);
@@ -68,6 +70,9 @@ void launch_init_diag(Inst* inst, uint32_t first, uint32_t count, void* dpool, c
 // row-by-row closure (wg_kern_rows.cu); id_bytes: 2 for at most 2^16 vertices, else 4
 int occupancy_rows(int id_bytes, uint32_t vwords);
 void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s);
+// writes a single query's instance and clears `bytes` (a multiple of 16) of scratch
+void launch_row_begin(const RowJob& J, const RowInst& I, const SgInst& G, void* clear,
+                      size_t bytes, int sms, cudaStream_t s);
 void launch_rows_small(const RowJob& J, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
