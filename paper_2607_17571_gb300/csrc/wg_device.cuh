@@ -281,7 +281,10 @@ struct RowJob {
   RowReport* report;            // written by k_row_plan (or NULL)
 };
 constexpr uint32_t kRowChunk = 256;
-constexpr uint32_t kRowList = 2048;     // delta vertices listed before they are expanded
+// delta vertices a CTA of k_rows lists before they are expanded
+__host__ __device__ constexpr uint32_t row_list(int threads) {
+  return threads < 128 ? 16u * threads : 2048u;
+}
 constexpr uint32_t kRowSmemMax = 216 * 1024;
 // Tuples of a row k_rows_small takes (128 / 256 / 512, whole call: ER 400,000 /
 // 360,000 1.74 / 1.08 / 1.08 ms, R-MAT 2^19 / 400k 12.6 / 12.7 / 13.1 ms).

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
 // vertex from the bit mask of the strip's first units.  Setting a bit in the
 // next N needs no answer, so a candidate costs one shared atomic and no list of
 // winners is kept; scanning N costs words / 128 lane steps per iteration.  Two
-// barriers per iteration; a delta of more than kRowList such vertices takes
+// barriers per iteration; a delta of more than row_list(T) such vertices takes
 // several rounds, the bits not yet listed waiting in the row's place in `bits`.
 //
 // Bound by issue slots and by the barriers (ncu: 58% of the issue slots, DRAM
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
 // expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0.
 template <typename IdT, int T, int kMin>
 __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
-  constexpr uint32_t kW = T / 32;
+  constexpr uint32_t kW = T / 32, kList = row_list(T);
   extern __shared__ uint4 sm4[];
   __shared__ RowInst I;
   __shared__ unsigned long long s_log[kRowLog];
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
             if (lane == 31) at = atomicAdd(s_len + turn, in);
             at = __shfl_sync(0xffffffffu, at, 31) + in - c;
             auto put = [&](uint32_t& m, uint32_t base) {
-              while (m && at < kRowList) {
+              while (m && at < kList) {
                 list[at++] = (IdT)(base + __ffs(m) - 1);
                 m &= m - 1;
               }
@@ -190,14 +190,14 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
           got = __reduce_add_sync(0xffffffffu, got);
           if (lane == 0 && got) atomicAdd(s_cnt + (lvl & 1), got);
           __syncthreads();
-          const uint32_t len = s_len[turn], n = min(len, kRowList);
+          const uint32_t len = s_len[turn], n = min(len, kList);
           if (round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
           listed |= len;
           if (len == 0) break;
           for (uint32_t b = warp * 32; b < n; b += T)
             cand += expand_vertices(I, list + b, min(32u, n - b), N, strip);
           __syncthreads();
-          if (len <= kRowList) break;
+          if (len <= kList) break;
         }
         const uint32_t n = s_cnt[lvl & 1];
         if (n == 0) break;
@@ -518,25 +518,34 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
 
 // ------------------------------------------------------------------ launchers
 static uint32_t row_smem(uint32_t vwords, int id_bytes, int threads) {
-  return 2 * vwords * 4 + (threads / 32) * 32 * 4 + kRowList * id_bytes;
+  return 2 * vwords * 4 + (threads / 32) * 32 * 4 + row_list(threads) * id_bytes;
 }
 // Threads per CTA: a CTA waits twice per iteration for its slowest warp, so the
-// smaller the better while its bit sets leave room for enough CTAs per SM
-// (64 / 128 / 256 / 512 threads, whole call: R-MAT 2^17 / 400k 7.3 / 7.0 / 7.2 /
-// 8.4 ms; R-MAT 2^19 / 400k, 31 KB of bit sets, 22.7 / 16.8 / 15.2 / 16.9 ms;
-// the 64-query batch 15.8 / 16.0 / 18.7 / 24.4 ms).  From 131,072 vertices two CTAs
-// of 512 share an SM while their bit sets allow (k_rows on ER 400,000 / 360,000:
-// 0.95 against 1.48 ms with one of 1,024).
+// smaller the better while its bit sets leave room for enough CTAs per SM.
+// Whole calls, 32 / 64 / 128 / 256 / 512 threads: chain of 1,000 (32 words) 1.07 /
+// 1.18 / 1.17 / 2.1 / 2.4 ms; the 64-query batch (up to 512) 12.3 / 12.3 / 13.1 ms;
+// R-MAT 2^15 / 100k (750) - / 537 / 510 us; R-MAT 2^17 / 400k (1,900) - / 7.3 / 7.0 /
+// 7.2 / 8.4 ms and 2^19 / 400k (3,900 words) - / 22.7 / 16.8 / 15.2 / 16.9 ms (both
+// before the 16-byte records).  From 131,072 vertices two CTAs of 512 share an SM
+// while their bit sets allow (k_rows on ER 400,000 / 360,000: 0.95 against 1.48 ms
+// with one of 1,024).
 static int row_threads(uint32_t vwords) {
-  return vwords <= 2048 ? 128 : vwords <= 4096 ? 256 : vwords <= 12800 ? 512 : 1024;
+  return vwords <= 128    ? 32
+         : vwords <= 512  ? 64
+         : vwords <= 2048 ? 128
+         : vwords <= 4096 ? 256
+         : vwords <= 12800 ? 512
+                           : 1024;
 }
 
 template <typename F>
 static auto rows_kernel(uint32_t vwords, int id_bytes, F f) {
   const int t = row_threads(vwords);
-  if (id_bytes == 2) return f(k_rows<uint16_t, 128, 10>);  // (at most 2,048 words)
-  return t == 128   ? f(k_rows<uint32_t, 128, 10>)
-         : t == 256 ? f(k_rows<uint32_t, 256, 5>)
+  if (id_bytes == 2)  // (at most 2,048 words)
+    return t == 32   ? f(k_rows<uint16_t, 32, 32>)
+           : t == 64 ? f(k_rows<uint16_t, 64, 20>)
+                     : f(k_rows<uint16_t, 128, 10>);
+  return t == 256   ? f(k_rows<uint32_t, 256, 5>)  // (more than 2,048)
          : t == 512 ? f(k_rows<uint32_t, 512, 2>)
                     : f(k_rows<uint32_t, 1024, 1>);
 }
