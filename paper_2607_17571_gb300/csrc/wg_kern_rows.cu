@@ -438,7 +438,8 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
 // time, each lane lists the set bits of its two words at its prefix in the
 // warp's shared buffer, then the warp writes the list coalesced.  kMasked
 // (same-generation): of each row the 128-bit pieces marked valid only, 16 at a
-// time.  A step that is half full is written a word at a time by the whole warp.
+// time; a step that is a quarter full is written a word at a time by the whole
+// warp (unmasked rows of low-degree graphs, 2/3 full, lose 5% by that).
 // 7.5e7 same-generation tuples, rows of nearly full pieces: 0.31 -> 0.18 ms with
 // the padding and the word steps (ncu had the buffer's bank conflicts at 87% of
 // the L1 pipe).
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
   __shared__ uint16_t s_buf[kWarps][2048 + 64], s_list[kMasked ? kWarps : 1][kMasked ? kSgMaxVertices / 128 : 1];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1;
-  constexpr uint32_t kDense = 1024;  // of 2,048 bits
+  constexpr uint32_t kDense = 512;  // of 2,048 bits
   // (valid pieces are often nearly full, so lanes list some 64 places apart: two
   // places of padding spread the banks; unmasked rows are sparser, and it costs
   // them more than it saves: 0.62 against 0.56 ms for 4.8e8 tuples)
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
       const uint2 nextv = nx < np ? w2[place(nx)] : uint2{0, 0};
       const uint32_t c = __popc(v.x) + __popc(v.y), in = warp_incl_scan(c, lane);
       const uint32_t tot = __shfl_sync(0xffffffffu, in, 31);
-      if (tot >= kDense) {
+      if (kMasked && tot >= kDense) {
         // dense: the warp takes a word at a time, a lane per bit
         uint32_t off = 0;
         for (uint32_t j = 0; j < 64; ++j) {
@@ -505,7 +506,7 @@ __global__ void __launch_bounds__(kThreads) k_row_expand(RowJob J) {
         __syncwarp();
         for (uint32_t j = lane; j < tot; j += 32) {
           const uint32_t t = buf[pad(j)];
-          out[j] = hi + (K)place(b + (t >> 6)) * 64 + (t & 63u);
+          out[j] = kMasked ? hi + (K)place(b + (t >> 6)) * 64 + (t & 63u) : hi + (K)b * 64 + t;
         }
         out += tot;
         __syncwarp();
