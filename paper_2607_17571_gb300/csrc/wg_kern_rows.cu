@@ -194,8 +194,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
           if (round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
           listed |= len;
           if (len == 0) break;
-          for (uint32_t b = warp * 32; b < n; b += T)
-            cand += expand_vertices(I, list + b, min(32u, n - b), N, strip);
+          cand += expand_vertices<IdT, false>(I, list, warp * 32, n, T, N, strip);
           __syncthreads();
           if (len <= kList) break;
         }

@@ -86,13 +86,15 @@ __device__ __forceinline__ bool sg_barrier(SgCtl* c, uint32_t target) {
   return s_ok != 0;
 }
 
+constexpr uint32_t kSgKids = 1024;  // children whose listing goes through shared memory
+
 template <typename IdT>
 __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
   constexpr uint32_t kW = kSgThreads / 32;
   extern __shared__ uint4 S4[];
   __shared__ RowInst I;
   __shared__ SgInst G;
-  __shared__ uint32_t s_row[2], s_nq, s_nz;
+  __shared__ uint32_t s_row[2], s_nq, s_nz, s_kids[kSgKids / 32];  // children with new tuples
   constexpr uint32_t kNone = 0xFFFFFFFFu;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* S = (uint32_t*)S4;
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
   IdT* list = (IdT*)(vql + J.rows.vwords / 4) + warp * kSgList;
   for (uint32_t i = tid; i < J.rows.vwords / 4; i += kSgThreads) S4[i] = uint4{0, 0, 0, 0};
   if (tid == 0) s_nz = 0;
+  if (tid < kSgKids / 32) s_kids[tid] = 0;
   unsigned long long cand = 0, got = 0;
   uint32_t cur = 0xFFFFFFFFu;
   SgCtl* ctl = J.ctl;
@@ -127,8 +130,10 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
       ctl->count[(k + 2) % 3] = 0;
       ctl->next[(k + 2) % 3] = 0;
     }
+    const uint32_t* const listed = in ? J.list[1] : J.list[0];
+    uint32_t* const to_list = in ? J.list[0] : J.list[1];
     auto row_of = [&](uint32_t i) {
-      return i >= n ? kNone : k == 0 ? i : __ldcg(J.list[in] + i);
+      return i >= n ? kNone : k == 0 ? i : __ldcg(listed + i);
     };
     if (tid == 0) s_row[0] = row_of(atomicAdd(&ctl->next[k % 3], 1u));
     __syncthreads();
@@ -195,8 +200,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
           };
           put(v.x, w * 128); put(v.y, w * 128 + 32); put(v.z, w * 128 + 64); put(v.w, w * 128 + 96);
           __syncwarp();
-          for (uint32_t b = 0; b < len; b += 32)
-            dsum += expand_vertices(I, list + b, min(32u, len - b), S, strip);
+          dsum += expand_vertices<IdT, true>(I, list, 0, len, 32, S, strip);
           __syncwarp();
         }
         cand += (unsigned long long)dsum * deg;
@@ -231,9 +235,9 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
         uint4* F = (uint4*)I.bits + at;
         uint4 d = s;
         if (!bit_of(I.mp, x)) {
+          uint4 old = __ldcg(F);  // (beside the mask, not after it: unused if not valid)
           const bool old_valid = (__ldcg(G.fm + mat) & bit) != 0;
-          uint4 old = {0, 0, 0, 0};
-          if (old_valid) old = __ldcg(F);
+          if (!old_valid) old = uint4{0, 0, 0, 0};
           d.x &= ~old.x; d.y &= ~old.y; d.z &= ~old.z; d.w &= ~old.w;
           if (!any4(d)) continue;
           *F = uint4{old.x | d.x, old.y | d.y, old.z | d.z, old.w | d.w};
@@ -257,14 +261,24 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
         got += popc4(d);
         if (on) {
           atomicOr(G.dm[out] + mat, bit);
-          if (__ldcg(G.act + x) != k + 1 && atomicExch(G.act + x, k + 1) != k + 1)
-            J.list[out][atomicAdd(next_n, 1u)] = I.row0 + x;
+          if (c < kSgKids) atomicOr(s_kids + (c >> 5), 1u << (c & 31));
+          else if (__ldcg(G.act + x) != k + 1 && atomicExch(G.act + x, k + 1) != k + 1)
+            to_list[atomicAdd(next_n, 1u)] = I.row0 + x;
         }
       }
       __syncthreads();
+      // list the children with new tuples: a child of one parent only here, so
+      // without asking; one of several once per iteration
+      for (uint32_t c = tid; c < min(deg, kSgKids); c += kSgThreads) {
+        if (!(s_kids[c >> 5] >> (c & 31) & 1u)) continue;
+        const uint32_t x = __ldg(adj + c);
+        if (!bit_of(I.mp, x) || atomicExch(G.act + x, k + 1) != k + 1)
+          to_list[atomicAdd(next_n, 1u)] = I.row0 + x;
+      }
       for (uint32_t i = tid; i < nz; i += kSgThreads) S4[nzl[i]] = uint4{0, 0, 0, 0};
       if (tid == 0) { s_nz = 0; s_row[p ^ 1] = next; }
-      __syncthreads();
+      __syncthreads();  // (every read of s_kids is done)
+      if (tid < kSgKids / 32) s_kids[tid] = 0;
     }
     if (cur != 0xFFFFFFFFu) flush();
     if (!sg_barrier(ctl, (k + 1) * gridDim.x)) return;

@@ -61,22 +61,18 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
   return v;
 }
 
-// The bits of the neighbours of vertices l[0..n), 1 <= n <= 32, each with at
-// least one, into the bit set N (shared memory): one warp, each lane its vertex's
-// record, then the vertices' units as one strip, 32 units per step, a
-// lane finding its unit's vertex from the bit mask of the strip's first units.
-// strip: 32 words of the warp.  Returns the degree of the lane's vertex.
+// The bits of the neighbours of a warp's vertices (lane: vertex v with record r of
+// degree deg, 0: none) into the bit set N (shared memory): the records' own, then
+// the vertices' units as one strip, 32 units per step, a lane finding its unit's
+// vertex from the bit mask of the strip's first units.  strip: 32 words of the
+// warp.  Returns the degree of the lane's vertex.
 template <typename IdT>
-__device__ __forceinline__ uint32_t expand_vertices(const RowInst& I, const IdT* l, uint32_t n,
-                                                    uint32_t* N, uint32_t* strip) {
+__device__ __forceinline__ uint32_t expand_strip(const RowInst& I, uint32_t v, uint32_t deg,
+                                                 const Rec<IdT>& r, uint32_t* N, uint32_t* strip) {
   constexpr uint32_t U = Unit<IdT>::n, kRecIds = U - 1;
   const uint32_t lane = threadIdx.x & 31, upto = 0xFFFFFFFFu >> (31 - lane);
-  uint32_t us = 0, deg = 0;
-  if (lane < n) {
-    const uint32_t v = l[lane];
-    Rec<IdT> r;
-    r.load(I.rec, v);
-    deg = r.deg();
+  uint32_t us = 0;
+  if (deg) {
     uint32_t o = 0, o1 = 0;
     if (deg > kRecIds) {
       o = __ldg(I.off + v);
@@ -111,6 +107,36 @@ __device__ __forceinline__ uint32_t expand_vertices(const RowInst& I, const IdT*
   }
   __syncwarp();
   return deg;
+}
+
+// The bits of the neighbours of the vertices l[b..n), l[b + step..n), ..., 32 at
+// most each, every one with neighbours.  One warp; returns the sum of the degrees
+// of the lane's vertices.  kAhead: the next 32 records are loaded before the bits
+// of these are set (same-generation rows, few warps per SM: 1.35 -> 1.32 ms; TC rows
+// gain nothing and R-MAT 2^17 / 400k loses 1%).
+template <typename IdT, bool kAhead>
+__device__ __forceinline__ uint32_t expand_vertices(const RowInst& I, const IdT* l, uint32_t b,
+                                                    uint32_t n, uint32_t step, uint32_t* N,
+                                                    uint32_t* strip) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t sum = 0, v = 0;
+  Rec<IdT> r;
+  auto load = [&](uint32_t at) {
+    r.a = uint4{0, 0, 0, 0};
+    if (at + lane < n) {
+      v = l[at + lane];
+      r.load(I.rec, v);
+    }
+  };
+  if (kAhead) load(b);
+  for (; b < n; b += step) {
+    if (!kAhead) load(b);
+    const uint32_t v0 = v;
+    const Rec<IdT> r0 = r;
+    if (kAhead) load(b + step);
+    sum += expand_strip<IdT>(I, v0, r0.deg(), r0, N, strip);
+  }
+  return sum;
 }
 
 // The set bits of a row's mask (at most 32 words) as an ordered list; returns
