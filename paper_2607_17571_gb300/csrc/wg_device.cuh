@@ -315,6 +315,20 @@ constexpr uint32_t kSgList = 1024;            // vertices of 8 pieces
 constexpr uint32_t kSgMaxVertices = 131072;   // 32 mask words
 constexpr uint32_t kSgSpinLimit = 1u << 24;   // polls before the barrier gives up
 
+// ---------------------------------------------------------------- sort by top digit first
+struct MsdState { uint32_t ok, next; };  // the keys suit it; bins claimed
+struct MsdJob {                          // wg_kern_msd.cu
+  const void* in;                        // the keys
+  void* tmp;                             // partitioned keys
+  void* out;                             // sorted keys (may be `in`)
+  uint32_t *cnt, *off, *cur;             // 2^top each
+  MsdState* state;
+  uint32_t n, bits, top, pad;
+};
+constexpr uint32_t kMsdTile = 16384, kMsdCap = 8192, kMsdTopMax = 14;
+constexpr int kMsdThreads = 512;
+constexpr uint32_t kMsdMin = 1u << 23;   // keys (see prim_sort)
+
 // ---------------------------------------------------------------- triangle counting
 struct TriCtl {
   unsigned long long paths, hits;  // two-paths (a,b,c); those with E(c,a)

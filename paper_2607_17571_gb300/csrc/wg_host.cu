@@ -278,20 +278,58 @@ static void pass_plan(uint32_t bits, uint32_t* passes, uint32_t* dbits) {
   *dbits = (bits + *passes - 1) / *passes;
 }
 
+// Large arrays of 64-bit keys by their top digit first (wg_kern_msd.cu), when a
+// sample and then the exact count find that their bins fit; *sorted says whether.
+// Even 34-bit keys, 2^22 / 2^23 / 2^24: 325 -> 217, 554 -> 371, 1035 -> 660 us (48
+// bits 403 -> 282, 686 -> 478, 1230 -> 858); 32-bit keys gain nothing (26 bits, 2^24:
+// 531 -> 502, 32 bits 582 -> 604 us).  A skewed array pays the sample and its
+// read-back, 18 us: 6% / 4% / 2% at those sizes, so the line lies at 2^23 keys.
+template <typename K>
+static int prim_sort_msd(wg_ctx* c, K* keys, size_t n, uint32_t bits, uint32_t top, size_t key_bytes,
+                         size_t bin_bytes, bool* sorted) {
+  if constexpr (sizeof(K) == 8) {
+    char* x = (char*)c->s_tmp + key_bytes;
+    MsdJob M{};
+    M.in = keys; M.tmp = c->s_tmp; M.out = keys;
+    M.cnt = (uint32_t*)x; M.off = (uint32_t*)(x + bin_bytes); M.cur = (uint32_t*)(x + 2 * bin_bytes);
+    M.state = (MsdState*)(x + 3 * bin_bytes);
+    M.n = (uint32_t)n; M.bits = bits; M.top = top;
+    MsdState h{1, 0};
+    for (int step = 0; step < 2 && h.ok; ++step) {
+      launch_msd_sort<K>(M, step, c->num_sms, c->stream);
+      CK(cudaMemcpyAsync(&h, M.state, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+    }
+    if (h.ok) launch_msd_sort<K>(M, 2, c->num_sms, c->stream);
+    CK(cudaGetLastError());
+    *sorted = h.ok != 0;
+  }
+  return WG_OK;
+}
+
 template <typename K>
 static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
   if (n <= 1) return WG_OK;
   const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
-  TRY(prim_scratch(c, n * sizeof(K), ntiles));
+  uint32_t top = 1;  // the top digit: bins of at most 5,000 keys on average (of kMsdCap)
+  while (top < 31 && (n >> top) > 5000) ++top;
+  const bool msd = sizeof(K) == 8 && n >= kMsdMin && top <= kMsdTopMax && top < bits;
+  const size_t key_bytes = round_up(n * sizeof(K)), bin_bytes = msd ? (size_t)4 << top : 0;
+  TRY(prim_scratch(c, msd ? key_bytes + 3 * bin_bytes + 256 : n * sizeof(K), ntiles));
+  // a wait that gave up in an earlier primitive must not make these passes
+  // skip their work: the control block starts clear (the caller reads it after)
+  CK(cudaMemsetAsync(c->s_ctl, 0, sizeof(Ctl), c->stream));
+  if (msd) {
+    bool sorted = false;
+    TRY(prim_sort_msd<K>(c, keys, n, bits, top, key_bytes, bin_bytes, &sorted));
+    if (sorted) return WG_OK;
+  }
   uint32_t passes, dbits;
   pass_plan(bits, &passes, &dbits);
   Seg sg{};
   sg.n = n; sg.tile0 = 0; sg.ntiles = ntiles;
   TRY(prim_seg(c, sg));
   CK(cudaMemsetAsync(c->s_hist, 0, sizeof(unsigned long long) * passes * kRadix, c->stream));
-  // a wait that gave up in an earlier primitive must not make these passes
-  // skip their work: the control block starts clear (the caller reads it after)
-  CK(cudaMemsetAsync(c->s_ctl, 0, sizeof(Ctl), c->stream));
   Stage h = prim_stage(c, ntiles);
   h.in = keys; h.passes = passes; h.dbits = dbits;
   TRY(prim_put(c, S_HIST, h));

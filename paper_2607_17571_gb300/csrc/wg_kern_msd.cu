@@ -1,0 +1,277 @@
+// wg_kern_msd.cu -- radix sort of a large array by its top digit first (sm_103a).
+//
+// The lookback passes (k_sort_pass) read and write every key once per 7 or 8 bits
+// and must keep their order from the second pass on.  Here one pass partitions
+// the keys by their top B bits -- in any order within a bin, so it needs neither
+// stable ranks nor a lookback: each tile counts its bins in shared memory and
+// reserves its places with one global atomic per bin -- and then a CTA sorts each
+// bin, which fits its shared memory, on the remaining bits: three sweeps over HBM
+// in all (count, partition, bins) whatever the key width.  Keys whose top bits are
+// skewed (a bin over kMsdCap keys) go to the lookback passes: a sample finds most
+// of them in a few microseconds, the exact count the rest.
+//
+// 2^24 uniform 64-bit keys on 34 bits: count 24, partition 179, bins 372 us, against
+// 950 us for the lookback passes' five.  The bins are bound by shared memory and the
+// barriers of their passes, the partition by its scattered 16-byte writes.
+#include "wg_device.cuh"
+#include "wg_launch.h"
+
+namespace wg {
+
+template <typename K>
+__device__ __forceinline__ uint32_t msd_bin(const MsdJob& J, K k) {
+  return (uint32_t)(k >> (J.bits - J.top)) & ((1u << J.top) - 1);
+}
+
+// A sample of the keys: are 2^8 (or fewer) bins of the top bits about even?
+template <typename K>
+__global__ void __launch_bounds__(1024) k_msd_probe(MsdJob J) {
+  constexpr uint32_t kSample = 4096;
+  __shared__ uint32_t cnt[256], s_max;
+  const K* in = (const K*)J.in;
+  const uint32_t t = threadIdx.x, coarse = min(J.top, 8u);
+  if (t < 256) cnt[t] = 0;
+  if (t == 0) s_max = 0;
+  __syncthreads();
+  const uint32_t step = J.n / kSample;  // (at least 1: n >= kMsdMin)
+#pragma unroll
+  for (uint32_t i = t; i < kSample; i += 1024)
+    atomicAdd(cnt + (msd_bin(J, in[(size_t)i * step]) >> (J.top - coarse)), 1u);
+  __syncthreads();
+  if (t < 256) atomicMax(&s_max, cnt[t]);
+  __syncthreads();
+  if (t == 0) {
+    // twice the even share and some: a fuller bin would rarely fit
+    J.state->ok = s_max <= 2 * (kSample >> coarse) + 16 ? 1u : 0u;
+    J.state->next = 0;
+  }
+}
+
+// Keys per bin (cnt is cleared before).
+template <typename K>
+__global__ void __launch_bounds__(1024) k_msd_count(MsdJob J) {
+  extern __shared__ uint32_t cnt[];
+  const uint32_t nb = 1u << J.top;
+  for (uint32_t i = threadIdx.x; i < nb; i += 1024) cnt[i] = 0;
+  __syncthreads();
+  const K* in = (const K*)J.in;
+  for (uint32_t t = blockIdx.x * kMsdTile; t < J.n; t += gridDim.x * kMsdTile) {
+    K k[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const uint32_t i = t + threadIdx.x + e * 1024;
+      k[e] = i < J.n ? __ldcs(in + i) : (K)0;
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+      if (t + threadIdx.x + e * 1024 < J.n) atomicAdd(cnt + msd_bin(J, k[e]), 1u);
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < nb; i += 1024)
+    if (cnt[i]) atomicAdd(J.cnt + i, cnt[i]);
+}
+
+// Bin offsets, and whether every bin fits.
+__global__ void __launch_bounds__(1024) k_msd_plan(MsdJob J) {
+  __shared__ uint32_t sh[32], s_max;
+  const uint32_t nb = 1u << J.top, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t per = (nb + 1023) / 1024, b0 = t * per;
+  if (t == 0) s_max = 0;
+  __syncthreads();
+  uint32_t sum = 0, top = 0;
+  for (uint32_t i = b0; i < min(b0 + per, nb); ++i) {
+    const uint32_t c = J.cnt[i];
+    sum += c;
+    top = max(top, c);
+  }
+  atomicMax(&s_max, top);
+  uint32_t in = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, in, o);
+    if (lane >= (uint32_t)o) in += y;
+  }
+  if (lane == 31) sh[warp] = in;
+  __syncthreads();
+  uint32_t before = in - sum;
+  for (uint32_t w = 0; w < warp; ++w) before += sh[w];
+  for (uint32_t i = b0; i < min(b0 + per, nb); ++i) {
+    J.off[i] = before;
+    J.cur[i] = before;
+    before += J.cnt[i];
+  }
+  if (t == 0) {
+    J.state->ok = s_max <= kMsdCap ? 1u : 0u;
+  }
+}
+
+// Keys to their bins, in any order.
+template <typename K>
+__global__ void __launch_bounds__(1024) k_msd_partition(MsdJob J) {
+  extern __shared__ uint32_t cnt[];  // keys of the tile per bin, then their first place
+  const uint32_t nb = 1u << J.top;
+  const K* in = (const K*)J.in;
+  K* out = (K*)J.tmp;
+  for (uint32_t t = blockIdx.x * kMsdTile; t < J.n; t += gridDim.x * kMsdTile) {
+    for (uint32_t i = threadIdx.x; i < nb; i += 1024) cnt[i] = 0;
+    __syncthreads();
+    K k[16];
+    uint32_t rank[8];  // two 16-bit ranks each
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const uint32_t i = t + threadIdx.x + e * 1024;
+      k[e] = i < J.n ? __ldcs(in + i) : (K)0;
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      uint32_t r = 0;
+      if (t + threadIdx.x + e * 1024 < J.n) r = atomicAdd(cnt + msd_bin(J, k[e]), 1u);
+      rank[e >> 1] = e & 1 ? rank[e >> 1] | r << 16 : r;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nb; i += 1024) {
+      const uint32_t c = cnt[i];
+      if (c) cnt[i] = atomicAdd(J.cur + i, c);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+      if (t + threadIdx.x + e * 1024 < J.n)
+        out[cnt[msd_bin(J, k[e])] + (rank[e >> 1] >> (e & 1 ? 16 : 0) & 0xFFFFu)] = k[e];
+    __syncthreads();
+  }
+}
+
+// Each bin sorted on the bits below its own, in shared memory: LSD radix passes
+// of at most 8 bits, stable (a warp ranks its consecutive keys with match_any).
+template <typename K>
+__global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
+  extern __shared__ unsigned long long smem_bins[];  // [kMsdCap] keys | [warps][256] counters
+  constexpr uint32_t kW = kMsdThreads / 32, kItems = kMsdCap / kMsdThreads;
+  __shared__ uint32_t s_sum[8], s_bin;
+  K* buf = (K*)smem_bins;
+  uint32_t* cnt = (uint32_t*)(buf + kMsdCap);
+  const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5, below = (1u << lane) - 1;
+  uint32_t* mine = cnt + warp * 256;
+  const uint32_t low = J.bits - J.top, passes = (low + 7) / 8, dbits = passes ? (low + passes - 1) / passes : 0;
+  const uint32_t mask = (1u << dbits) - 1;
+  const K* in = (const K*)J.tmp;
+  K* out = (K*)J.out;
+  for (;;) {
+    if (t == 0) s_bin = atomicAdd(&J.state->next, 1u);
+    __syncthreads();
+    const uint32_t b = s_bin;
+    __syncthreads();
+    if (b >= 1u << J.top) return;
+    const uint32_t o = J.off[b], m = J.cnt[b];
+    if (m == 0) continue;
+    // warp w holds keys [w * run, (w + 1) * run) of the bin, 32 at a time
+    const uint32_t items = (m + kMsdThreads - 1) / kMsdThreads, run = items * 32, w0 = warp * run;
+    K k[kItems];
+#pragma unroll
+    for (uint32_t e = 0; e < kItems; ++e) {
+      if (e >= items) break;
+      const uint32_t i = w0 + e * 32 + lane;
+      k[e] = i < m ? __ldcs(in + o + i) : (K)0;
+    }
+    for (uint32_t p = 0; p < passes; ++p) {
+      const uint32_t shift = p * dbits;
+      for (uint32_t i = lane; i < 256; i += 32) mine[i] = 0;
+      __syncwarp();
+      uint32_t rank[kItems / 2];  // two 16-bit ranks within the warp's digit each
+#pragma unroll
+      for (uint32_t e = 0; e < kItems; ++e) {
+        if (e >= items) break;
+        const bool on = w0 + e * 32 + lane < m;
+        const uint32_t d = on ? (uint32_t)(k[e] >> shift) & mask : 256u;
+        const uint32_t same = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = on ? mine[d] : 0u;
+        __syncwarp();
+        if (on && !(same & below)) mine[d] = before + __popc(same);
+        __syncwarp();
+        const uint32_t r = before + __popc(same & below);
+        rank[e >> 1] = e & 1 ? rank[e >> 1] | r << 16 : r;
+      }
+      __syncthreads();
+      // each digit's places: before it all smaller digits, then the warps in order
+      if (t < 256) {
+        uint32_t sum = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < kW; ++w) {
+          const uint32_t c = cnt[w * 256 + t];
+          cnt[w * 256 + t] = sum;
+          sum += c;
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int q = 1; q < 32; q <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, q);
+          if (lane >= (uint32_t)q) inc += y;
+        }
+        if (lane == 31) s_sum[warp] = inc;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        uint32_t base = inc - sum;
+        for (uint32_t w = 0; w < warp; ++w) base += s_sum[w];
+#pragma unroll
+        for (uint32_t w = 0; w < kW; ++w) cnt[w * 256 + t] += base;
+      }
+      __syncthreads();
+#pragma unroll
+      for (uint32_t e = 0; e < kItems; ++e) {
+        if (e >= items) break;
+        if (w0 + e * 32 + lane < m) {
+          const uint32_t d = (uint32_t)(k[e] >> shift) & mask;
+          buf[mine[d] + (rank[e >> 1] >> (e & 1 ? 16 : 0) & 0xFFFFu)] = k[e];
+        }
+      }
+      __syncthreads();
+      if (p + 1 < passes) {
+#pragma unroll
+        for (uint32_t e = 0; e < kItems; ++e) {
+          if (e >= items) break;
+          const uint32_t i = w0 + e * 32 + lane;
+          if (i < m) k[e] = buf[i];
+        }
+        __syncthreads();
+      }
+    }
+    if (passes) {
+      for (uint32_t i = t; i < m; i += kMsdThreads) out[o + i] = buf[i];
+    } else {
+#pragma unroll
+      for (uint32_t e = 0; e < kItems; ++e) {
+        if (e >= items) break;
+        const uint32_t i = w0 + e * 32 + lane;
+        if (i < m) out[o + i] = k[e];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Step 0: the sample (state->ok); 1: count and plan (state->ok); 2: the sort.  The
+// caller reads state->ok after steps 0 and 1: with a skewed array it pays the
+// sample and one read-back.
+template <typename K>
+void launch_msd_sort(const MsdJob& J, int step, int sms, cudaStream_t s) {
+  const uint32_t nb = 1u << J.top;
+  if (step == 0) {
+    k_msd_probe<K><<<1, 1024, 0, s>>>(J);
+  } else if (step == 1) {
+    cudaFuncSetAttribute(k_msd_count<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << kMsdTopMax);
+    cudaMemsetAsync(J.cnt, 0, nb * 4, s);
+    k_msd_count<K><<<sms, 1024, nb * 4, s>>>(J);
+    k_msd_plan<<<1, 1024, 0, s>>>(J);
+  } else {
+    const uint32_t bins = kMsdCap * sizeof(K) + kMsdThreads / 32 * 256 * 4;
+    cudaFuncSetAttribute(k_msd_partition<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << kMsdTopMax);
+    cudaFuncSetAttribute(k_msd_bins<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bins);
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_msd_bins<K>, kMsdThreads, bins);
+    k_msd_partition<K><<<sms, 1024, nb * 4, s>>>(J);
+    k_msd_bins<K><<<sms * max(1, occ), kMsdThreads, bins, s>>>(J);
+  }
+}
+template void launch_msd_sort<unsigned long long>(const MsdJob&, int, int, cudaStream_t);
+
+}  // namespace wg

@@ -15,6 +15,7 @@ struct Inst;
 struct RowJob;
 struct TriJob;
 struct SgJob;
+struct MsdJob;
 struct RowInst;
 struct SgInst;
 
@@ -37,6 +38,9 @@ void launch_partition(Stage* consumer, int mode, uint32_t tile, int grid, cudaSt
 template <typename K> int occupancy_sort(int which);  // 0 hist, 1 pass, 2 uniq, 3 merge, 4 fused,
                                                       // 5 fused with half tiles, 6 / 7 segment sort
                                                       // of 16 / 8 keys per thread
+
+// sort of a large array by its top digit first (wg_kern_msd.cu), in three steps
+template <typename K> void launch_msd_sort(const MsdJob& J, int step, int sms, cudaStream_t s);
 
 // join and engine control (wg_kern_join.cu)
 // tile: delta tuples per count tile, kTileD or kTileD / 2
