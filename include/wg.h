@@ -119,7 +119,8 @@ enum wg_loop {
 typedef struct wg_opts {
   uint32_t max_iters;    /* iteration cap; 0 = 1<<20 */
   uint32_t loop;         /* enum wg_loop */
-  uint32_t profile;      /* 1 = time every kernel with CUDA events (forces WG_LOOP_HOST) */
+  uint32_t profile;      /* 1 = time every kernel with CUDA events (forces WG_LOOP_HOST,
+                            so the sorted-array pipeline) */
   uint32_t flags;        /* WG_FLAG_* */
   uint64_t reserve_full; /* initial capacity of the full relation, tuples; 0 = auto */
   uint64_t reserve_cand; /* initial capacity of the candidate buffers, tuples; 0 = auto
@@ -278,7 +279,8 @@ void wg_query_free(wg_ctx* ctx, wg_query q);
  * count, the join emit, the radix sort and the fused stage timed with CUDA
  * events) and keep
  * the fastest choice of each stage in the context for the relation's key
- * width: every engine created afterwards (single, batched, served) uses it.  `out` may be
+ * width: every engine of the sorted-array pipeline created afterwards (single,
+ * batched, served) uses it; queries run as rows have no tiles.  `out` may be
  * NULL.  Synchronous; runs on the context stream.  Errors: WG_E_INVAL (bad
  * handle or kind), WG_E_NOMEM / WG_E_BUDGET (a run's pools do not fit),
  * WG_E_CUDA.  On an error the context keeps its previous shapes.
@@ -345,7 +347,9 @@ int wg_selftest_wait_timeout(wg_ctx* ctx);
  * higher bits must be zero), in place (Sec. Buffer Routing and Adaptive Radix
  * Sort: histogram, prefix sum, scatter per digit).  Every pass after the
  * first is stable; keys equal on the sorted bits are identical, so the
- * result is the unique sorted sequence. */
+ * result is the unique sorted sequence.  From 2^23 64-bit keys the top digit
+ * goes first (one unordered partition), then every bin is sorted in shared
+ * memory; keys too unevenly spread for that take the passes. */
 int wg_sort_keys(wg_ctx* ctx, void* d_keys, size_t n, int key_bytes, uint32_t bits);
 /* wg_unique_diff: out = { c in sorted `cand` : c differs from its predecessor
  * and c is not in sorted `full` } in input order (Sec. Fused Deduplication and

@@ -14,9 +14,9 @@
 // relation.
 //
 // Measured on GB300, fixpoint and result in device memory, sorted-array
-// pipeline -> rows: R-MAT 2^17 / 400k edges (4.8e8 tuples) 67.6 -> 16.3 ms,
-// R-MAT 2^19 / 400k (1.0e9 tuples, 64-bit keys) 165 -> 27.6 ms, ER 1,000 /
-// 3,000 2.53 -> 0.15 ms, a chain of 1,000 vertices 145 -> 1.8 ms.
+// pipeline -> rows: R-MAT 2^17 / 400k edges (4.8e8 tuples) 68.0 -> 5.35 ms (k_rows
+// 3.50), R-MAT 2^19 / 400k (1.0e9 tuples, 64-bit keys) 164 -> 12.6 ms (7.69), ER
+// 1,000 / 3,000 2.55 -> 0.10 ms, a chain of 1,000 vertices 147 -> 1.1 ms.
 //
 //   k_rows        the fixpoints of all rows (one CTA per row, rows claimed)
 //   k_row_plan    row offsets (scan of the row counts), totals, capacity check
@@ -73,12 +73,14 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
 // barriers per iteration; a delta of more than row_list(T) such vertices takes
 // several rounds, the bits not yet listed waiting in the row's place in `bits`.
 //
-// Bound by issue slots and by the barriers (ncu: 58% of the issue slots, DRAM
-// idle).  What it measured on R-MAT 2^17 / 400k, whole call: winners of each
+// Bound by the L1 / shared pipe, issue slots and barriers (ncu on R-MAT 2^15 / 100k,
+// 324 us: pipe 76%, issue 62%, DRAM 0.05%; on ER 16,384 / 34,000 82% and 68%).
+// What it measured on R-MAT 2^17 / 400k, whole call: winners of each
 // bit listed by an answering atomic, records of 7 neighbours and single edges
 // past them 16.1 ms; candidate bits without an answer, edges in 16-byte units,
 // a list per warp (one barrier, but it waited for the warp with the most to
-// expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0.
+// expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0; vertex
+// records of 16 bytes 5.35.
 template <typename IdT, int T, int kMin>
 __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   constexpr uint32_t kW = T / 32, kList = row_list(T);
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
 // that turns out longer is listed for k_rows.  Without it a sparse relation pays
 // a bit set per row to hold a few vertices: ER 400,000 vertices / 360,000 edges,
 // 335,000 rows of 9 tuples on average against bit sets of 42 KB, 15.5 ms on the
-// sorted-array pipeline, 1.08 ms here (0.39 this kernel, 0.38 k_rows).  Bound by
+// sorted-array pipeline, 1.03 ms here (0.39 this kernel, 0.38 k_rows).  Bound by
 // the latency of the gathered CSR entries.
 __global__ void __launch_bounds__(kThreads) k_rows_small(RowJob J) {
   constexpr uint32_t kSlots = 2 * kSmallRow, kNone = 0xFFFFFFFFu;

@@ -21,8 +21,8 @@
 // Bound by the latency of an item's steps (delta pieces, records, row pieces) and
 // the barriers between them (ncu: 24% of the issue slots, DRAM 1%), so CTAs are
 // small: 256 / 128 / 64 / 32 threads 1.71 / 1.05 / 0.86 / 0.88 ms on the forest of
-// 60,000 vertices (7.5e7 tuples, 12 iterations); whole call 5.85 ms on the
-// sorted-array pipeline, 1.38 here.
+// 60,000 vertices (7.5e7 tuples, 12 iterations; 0.83 since records are loaded
+// ahead); whole call 6.5 ms on the sorted-array pipeline, 1.3-1.4 here.
 #include "wg_device.cuh"
 #include "wg_launch.h"
 #include "wg_rows.cuh"
