@@ -325,7 +325,7 @@ struct MsdJob {                          // wg_kern_msd.cu
   MsdState* state;
   uint32_t n, bits, top, pad;
 };
-constexpr uint32_t kMsdTile = 16384, kMsdCap = 8192, kMsdTopMax = 14;
+constexpr uint32_t kMsdTile = 16384, kMsdCap = 8192, kMsdTopMax = 14, kMsdFine = 12;
 constexpr int kMsdThreads = 512;
 constexpr uint32_t kMsdMin = 1u << 23;   // keys (see prim_sort)
 

@@ -10,9 +10,10 @@
 // skewed (a bin over kMsdCap keys) go to the lookback passes: a sample finds most
 // of them in a few microseconds, the exact count the rest.
 //
-// 2^24 uniform 64-bit keys on 34 bits: count 24, partition 179, bins 372 us, against
-// 950 us for the lookback passes' five.  The bins are bound by shared memory and the
-// barriers of their passes, the partition by its scattered 16-byte writes.
+// 2^24 uniform 64-bit keys on 34 bits: whole call 399 us (652 with the bins sorted by
+// three LSD passes, 990 with the lookback passes' five; 48 bits 396, 864 and 1,190);
+// count 24, partition 179 us.  The bins are bound by shared memory, the partition by
+// its scattered 16-byte writes.
 #include "wg_device.cuh"
 #include "wg_launch.h"
 
@@ -142,29 +143,44 @@ __global__ void __launch_bounds__(1024) k_msd_partition(MsdJob J) {
   }
 }
 
-// Each bin sorted on the bits below its own, in shared memory: LSD radix passes
-// of at most 8 bits, stable (a warp ranks its consecutive keys with match_any).
+// Each bin sorted on the bits below its own, in shared memory.  Equal keys are
+// alike, so no order has to be kept: the next kMsdFine bits split the bin into
+// about as many buckets as it has keys (one shared atomic per key), and a key's
+// place in its bucket is the number of smaller ones, found by comparing.  A bin
+// whose buckets would take more than about eight comparisons per key, or that has
+// one of more than 64, goes through LSD passes of at most 8 bits instead (a warp
+// ranks its consecutive keys with match_any).
 template <typename K>
 __global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
-  extern __shared__ unsigned long long smem_bins[];  // [kMsdCap] keys | [warps][256] counters
+  extern __shared__ __align__(16) unsigned long long smem_bins[];  // [kMsdCap] keys | [warps][256] counters
   constexpr uint32_t kW = kMsdThreads / 32, kItems = kMsdCap / kMsdThreads;
-  __shared__ uint32_t s_sum[8], s_bin;
+  __shared__ uint32_t s_sum[kW], s_bin, s_cost;
   K* buf = (K*)smem_bins;
   uint32_t* cnt = (uint32_t*)(buf + kMsdCap);
   const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5, below = (1u << lane) - 1;
   uint32_t* mine = cnt + warp * 256;
   const uint32_t low = J.bits - J.top, passes = (low + 7) / 8, dbits = passes ? (low + passes - 1) / passes : 0;
   const uint32_t mask = (1u << dbits) - 1;
+  constexpr uint32_t kFine = 1u << kMsdFine, kPer = kFine / kMsdThreads;
+  static_assert(kFine <= kW * 256 && kPer % 4 == 0, "the buckets' counters take the passes' room");
+  const uint32_t fshift = low > kMsdFine ? low - kMsdFine : 0;  // (low >= 1)
+  const uint32_t fmask = (1u << min(low, kMsdFine)) - 1;
   const K* in = (const K*)J.tmp;
   K* out = (K*)J.out;
   for (;;) {
-    if (t == 0) s_bin = atomicAdd(&J.state->next, 1u);
+    if (t == 0) {
+      s_bin = atomicAdd(&J.state->next, 1u);
+      s_cost = 0;
+    }
+    for (uint32_t i = t; i < kFine / 4; i += kMsdThreads) ((uint4*)cnt)[i] = uint4{0, 0, 0, 0};
     __syncthreads();
     const uint32_t b = s_bin;
-    __syncthreads();
     if (b >= 1u << J.top) return;
     const uint32_t o = J.off[b], m = J.cnt[b];
-    if (m == 0) continue;
+    if (m == 0) {
+      __syncthreads();
+      continue;
+    }
     // warp w holds keys [w * run, (w + 1) * run) of the bin, 32 at a time
     const uint32_t items = (m + kMsdThreads - 1) / kMsdThreads, run = items * 32, w0 = warp * run;
     K k[kItems];
@@ -174,11 +190,74 @@ __global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
       const uint32_t i = w0 + e * 32 + lane;
       k[e] = i < m ? __ldcs(in + o + i) : (K)0;
     }
+    uint32_t rank[kItems / 2];  // two 16-bit ranks within the digit each
+    uint32_t cost = 0;
+#pragma unroll
+    for (uint32_t e = 0; e < kItems; ++e) {
+      if (e >= items) break;
+      uint32_t r = 0;
+      if (w0 + e * 32 + lane < m) r = atomicAdd(cnt + ((uint32_t)(k[e] >> fshift) & fmask), 1u);
+      cost += r < 64 ? r : 4 * kMsdCap;
+      rank[e >> 1] = e & 1 ? rank[e >> 1] | r << 16 : r;
+    }
+    cost = __reduce_add_sync(0xffffffffu, cost);
+    if (lane == 0 && cost) atomicAdd(&s_cost, cost);
+    __syncthreads();
+    const bool fine = !fshift || s_cost <= 4 * m;  // (twice s_cost comparisons)
+    if (fine) {
+      uint32_t c[kPer], sum = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; i += 4) *(uint4*)(c + i) = *(const uint4*)(cnt + t * kPer + i);
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) {
+        const uint32_t v = c[i];
+        c[i] = sum;
+        sum += v;
+      }
+      uint32_t inc = sum;
+#pragma unroll
+      for (int q = 1; q < 32; q <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, q);
+        if (lane >= (uint32_t)q) inc += y;
+      }
+      if (lane == 31) s_sum[warp] = inc;
+      __syncthreads();
+      uint32_t ws = lane < kW ? s_sum[lane] : 0u;
+      ws = lane < warp ? ws : 0u;
+      const uint32_t base = __reduce_add_sync(0xffffffffu, ws) + inc - sum;
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) c[i] += base;
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; i += 4) *(uint4*)(cnt + t * kPer + i) = *(const uint4*)(c + i);
+      __syncthreads();
+#pragma unroll
+      for (uint32_t e = 0; e < kItems; ++e) {
+        if (e >= items) break;
+        if (w0 + e * 32 + lane < m)
+          buf[cnt[(uint32_t)(k[e] >> fshift) & fmask] + (rank[e >> 1] >> (e & 1 ? 16 : 0) & 0xFFFFu)] = k[e];
+      }
+      __syncthreads();
+      for (uint32_t i = t; i < m; i += kMsdThreads) {
+        const K key = buf[i];
+        uint32_t at = i;
+        if (fshift) {
+          const uint32_t d = (uint32_t)(key >> fshift) & fmask;
+          const uint32_t j0 = cnt[d], j1 = d < kFine - 1 ? cnt[d + 1] : m;
+          at = j0;
+          for (uint32_t j = j0; j < j1; ++j) {
+            const K other = buf[j];
+            at += other < key || (other == key && j < i);
+          }
+        }
+        out[o + at] = key;
+      }
+      __syncthreads();
+      continue;
+    }
     for (uint32_t p = 0; p < passes; ++p) {
       const uint32_t shift = p * dbits;
       for (uint32_t i = lane; i < 256; i += 32) mine[i] = 0;
       __syncwarp();
-      uint32_t rank[kItems / 2];  // two 16-bit ranks within the warp's digit each
 #pragma unroll
       for (uint32_t e = 0; e < kItems; ++e) {
         if (e >= items) break;
@@ -235,16 +314,7 @@ __global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
         __syncthreads();
       }
     }
-    if (passes) {
-      for (uint32_t i = t; i < m; i += kMsdThreads) out[o + i] = buf[i];
-    } else {
-#pragma unroll
-      for (uint32_t e = 0; e < kItems; ++e) {
-        if (e >= items) break;
-        const uint32_t i = w0 + e * 32 + lane;
-        if (i < m) out[o + i] = k[e];
-      }
-    }
+    for (uint32_t i = t; i < m; i += kMsdThreads) out[o + i] = buf[i];
     __syncthreads();
   }
 }

@@ -73,3 +73,21 @@ def test_skewed_keys_fall_back(ctx, bits):
         idx = other[torch.randperm(other.numel(), device="cuda")[:held]]
         b[idx] = (5 << sh) | (b[idx] & rest)
         _sort(ctx, b, bits)
+
+
+@pytest.mark.parametrize("copies", [1, 7, 8, 9, 17, 63, 64, 65, 300])
+@pytest.mark.parametrize("bits", [24, 36])
+def test_buckets_within_a_bin(ctx, bits, copies):
+    """Few distinct values below the top digit, each several times (around the
+    fullest bucket that is ordered by comparing, and around the mean that is),
+    in all bins and in one of them alone."""
+    n = MIN + 4_099
+    a = _uniform(n, 8, bits, copies)
+    low = bits - 11                                 # 11 top bits, 4,096 keys a bin
+    rest = (1 << low) - 1
+    few = (a & rest) % max(1, 4096 // copies) * (rest // 4096 + 1)
+    _sort(ctx, ((a >> low) << low) | (few & rest), bits)
+    b = a.clone()
+    one = ((a >> low) == 9).nonzero().flatten()[:copies]
+    b[one] = (9 << low) | (b[one] & 1)              # one full bucket, keys out of order
+    _sort(ctx, b, bits)
