@@ -10,10 +10,10 @@
 // skewed (a bin over kMsdCap keys) go to the lookback passes: a sample finds most
 // of them in a few microseconds, the exact count the rest.
 //
-// 2^24 uniform 64-bit keys on 34 bits: whole call 399 us (652 with the bins sorted by
-// three LSD passes, 990 with the lookback passes' five; 48 bits 396, 864 and 1,190);
-// count 24, partition 179 us.  The bins are bound by shared memory, the partition by
-// its scattered 16-byte writes.
+// 2^24 uniform 64-bit keys on 34 bits: whole call 297 us (990 with the lookback
+// passes' five; 399 with the partition's keys written from where they were read, 652
+// with the bins also sorted by three LSD passes); 48 bits 299, 1,190, 396 and 864.
+// Bound by shared memory: one counting atomic and two staged moves a key and kernel.
 #include "wg_device.cuh"
 #include "wg_launch.h"
 
@@ -106,39 +106,80 @@ __global__ void __launch_bounds__(1024) k_msd_plan(MsdJob J) {
   }
 }
 
-// Keys to their bins, in any order.
+// Keys to their bins, in any order.  A tile is put in bin order in shared memory
+// first, so that a bin's keys (4 on average at 2^12 bins) leave as one run; the
+// next tile's loads are in flight meanwhile.
 template <typename K>
 __global__ void __launch_bounds__(1024) k_msd_partition(MsdJob J) {
-  extern __shared__ uint32_t cnt[];  // keys of the tile per bin, then their first place
-  const uint32_t nb = 1u << J.top;
+  extern __shared__ __align__(16) unsigned long long smem_part[];  // [kMsdTile] keys | [bins]
+  __shared__ uint32_t s_sum[32];
+  K* buf = (K*)smem_part;
+  uint32_t* cnt = (uint32_t*)(buf + kMsdTile);  // keys of the bin; first place in buf | keys << 16; to out
+  static_assert(kMsdTile < 1u << 16, "a place and a count share a word");
+  const uint32_t nb = 1u << J.top, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t per = (nb + 1023) / 1024;
   const K* in = (const K*)J.in;
   K* out = (K*)J.tmp;
-  for (uint32_t t = blockIdx.x * kMsdTile; t < J.n; t += gridDim.x * kMsdTile) {
-    for (uint32_t i = threadIdx.x; i < nb; i += 1024) cnt[i] = 0;
+  K k[16];
+  auto load = [&](size_t tile) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const size_t i = tile + t + e * 1024;
+      k[e] = i < J.n ? __ldcs(in + i) : (K)0;
+    }
+  };
+  size_t tile = (size_t)blockIdx.x * kMsdTile;
+  load(tile);
+  for (; tile < J.n; tile += (size_t)gridDim.x * kMsdTile) {
+    const uint32_t m = (uint32_t)min((size_t)kMsdTile, J.n - tile);
+    for (uint32_t i = t; i < nb; i += 1024) cnt[i] = 0;
     __syncthreads();
-    K k[16];
     uint32_t rank[8];  // two 16-bit ranks each
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
-      const uint32_t i = t + threadIdx.x + e * 1024;
-      k[e] = i < J.n ? __ldcs(in + i) : (K)0;
-    }
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
       uint32_t r = 0;
-      if (t + threadIdx.x + e * 1024 < J.n) r = atomicAdd(cnt + msd_bin(J, k[e]), 1u);
+      if (t + e * 1024 < m) r = atomicAdd(cnt + msd_bin(J, k[e]), 1u);
       rank[e >> 1] = e & 1 ? rank[e >> 1] | r << 16 : r;
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < nb; i += 1024) {
+    const uint32_t b0 = min(t * per, nb), b1 = min(b0 + per, nb);
+    uint32_t sum = 0;
+    for (uint32_t i = b0; i < b1; ++i) sum += cnt[i];
+    uint32_t inc = sum;
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, q);
+      if (lane >= (uint32_t)q) inc += y;
+    }
+    if (lane == 31) s_sum[warp] = inc;
+    __syncthreads();
+    const uint32_t ws = s_sum[lane];
+    uint32_t at = __reduce_add_sync(0xffffffffu, lane < warp ? ws : 0u) + inc - sum;
+    for (uint32_t i = b0; i < b1; ++i) {
       const uint32_t c = cnt[i];
-      if (c) cnt[i] = atomicAdd(J.cur + i, c);
+      cnt[i] = at | c << 16;
+      at += c;
     }
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; ++e)
-      if (t + threadIdx.x + e * 1024 < J.n)
-        out[cnt[msd_bin(J, k[e])] + (rank[e >> 1] >> (e & 1 ? 16 : 0) & 0xFFFFu)] = k[e];
+      if (t + e * 1024 < m)
+        buf[(cnt[msd_bin(J, k[e])] & 0xFFFFu) + (rank[e >> 1] >> (e & 1 ? 16 : 0) & 0xFFFFu)] = k[e];
+    load(tile + (size_t)gridDim.x * kMsdTile);
+    __syncthreads();
+    for (uint32_t i = t; i < nb; i += 1024) {
+      const uint32_t v = cnt[i], c = v >> 16;
+      if (c) cnt[i] = atomicAdd(J.cur + i, c) - (v & 0xFFFFu);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const uint32_t i = t + e * 1024;
+      if (i < m) {
+        const K key = buf[i];
+        out[cnt[msd_bin(J, key)] + i] = key;
+      }
+    }
     __syncthreads();
   }
 }
@@ -334,11 +375,13 @@ void launch_msd_sort(const MsdJob& J, int step, int sms, cudaStream_t s) {
     k_msd_plan<<<1, 1024, 0, s>>>(J);
   } else {
     const uint32_t bins = kMsdCap * sizeof(K) + kMsdThreads / 32 * 256 * 4;
-    cudaFuncSetAttribute(k_msd_partition<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << kMsdTopMax);
+    const uint32_t part = kMsdTile * sizeof(K);  // (and the bins' words: at most 192 KB)
+    cudaFuncSetAttribute(k_msd_partition<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(part + (4 << kMsdTopMax)));
     cudaFuncSetAttribute(k_msd_bins<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bins);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_msd_bins<K>, kMsdThreads, bins);
-    k_msd_partition<K><<<sms, 1024, nb * 4, s>>>(J);
+    k_msd_partition<K><<<sms, 1024, part + nb * 4, s>>>(J);
     k_msd_bins<K><<<sms * max(1, occ), kMsdThreads, bins, s>>>(J);
   }
 }
