@@ -323,11 +323,12 @@ struct MsdJob {                          // wg_kern_msd.cu
   void* out;                             // sorted keys (may be `in`)
   uint32_t *cnt, *off, *cur;             // 2^top each
   MsdState* state;
+  uint32_t* report;                      // page-locked: 0 / 1 once the fit is known
   uint32_t n, bits, top, pad;
 };
 constexpr uint32_t kMsdTile = 16384, kMsdCap = 8192, kMsdTopMax = 14, kMsdFine = 12;
 constexpr int kMsdThreads = 512;
-constexpr uint32_t kMsdMin = 1u << 23;   // keys (see prim_sort)
+constexpr uint32_t kMsdMin = 1u << 22;   // keys (see prim_sort)
 
 // ---------------------------------------------------------------- triangle counting
 struct TriCtl {

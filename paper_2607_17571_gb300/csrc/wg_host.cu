@@ -93,6 +93,7 @@ struct wg_ctx {
   std::vector<std::unique_ptr<RowLane>> lanes;    // batched row-by-row queries
   std::map<uint64_t, int> occ;            // resident CTAs per SM by kernel (see occ_of)
   std::vector<cudaEvent_t> events;        // timing events of freed queries
+  RowReport* s_report = nullptr;          // a large sort's, once it has one
   std::vector<RowReport*> reports;        // unused reports, from page-locked slabs
   std::vector<void*> report_slabs;
   // tile shapes engines are built with, per key width (index 0: 4-byte keys,
@@ -278,32 +279,38 @@ static void pass_plan(uint32_t bits, uint32_t* passes, uint32_t* dbits) {
   *dbits = (bits + *passes - 1) / *passes;
 }
 
-// Large arrays of 64-bit keys by their top digit first (wg_kern_msd.cu), when a
-// sample and then the exact count find that their bins fit; *sorted says whether.
-// Even 34-bit keys, 2^22 / 2^23 / 2^24: 325 -> 217, 554 -> 371, 1035 -> 660 us (48
-// bits 403 -> 282, 686 -> 478, 1230 -> 858); 32-bit keys gain nothing (26 bits, 2^24:
-// 531 -> 502, 32 bits 582 -> 604 us).  A skewed array pays the sample and its
-// read-back, 18 us: 6% / 4% / 2% at those sizes, so the line lies at 2^23 keys.
+// Large arrays by their top digit first (wg_kern_msd.cu), when a sample and then
+// the exact count find that their bins fit; *sorted says whether.  Even keys,
+// lookback passes -> top digit first, 2^21 / 2^22 / 2^23 / 2^24: 34 bits of 64
+// 208 -> 76, 311 -> 95, 551 -> 162, 1,054 -> 276 us; 48 bits 251 -> 78, 390 -> 94,
+// 687 -> 160, 1,227 -> 276; 32-bit keys 152 -> 66, 214 -> 91, 339 -> 130, 573 ->
+// 218.  A skewed array pays the sample until its report, 10 us: at 32-bit keys 8% /
+// 5% / 3% / 2%, half of which the single copy of the passes' records gives back, so
+// the line lies at 2^22 keys.
 template <typename K>
 static int prim_sort_msd(wg_ctx* c, K* keys, size_t n, uint32_t bits, uint32_t top, size_t key_bytes,
                          size_t bin_bytes, bool* sorted) {
-  if constexpr (sizeof(K) == 8) {
-    char* x = (char*)c->s_tmp + key_bytes;
-    MsdJob M{};
-    M.in = keys; M.tmp = c->s_tmp; M.out = keys;
-    M.cnt = (uint32_t*)x; M.off = (uint32_t*)(x + bin_bytes); M.cur = (uint32_t*)(x + 2 * bin_bytes);
-    M.state = (MsdState*)(x + 3 * bin_bytes);
-    M.n = (uint32_t)n; M.bits = bits; M.top = top;
-    MsdState h{1, 0};
-    for (int step = 0; step < 2 && h.ok; ++step) {
-      launch_msd_sort<K>(M, step, c->num_sms, c->stream);
-      CK(cudaMemcpyAsync(&h, M.state, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-      CK(cudaStreamSynchronize(c->stream));
-    }
-    if (h.ok) launch_msd_sort<K>(M, 2, c->num_sms, c->stream);
-    CK(cudaGetLastError());
-    *sorted = h.ok != 0;
+  char* x = (char*)c->s_tmp + key_bytes;
+  MsdJob M{};
+  M.in = keys; M.tmp = c->s_tmp; M.out = keys;
+  M.cnt = (uint32_t*)x; M.off = (uint32_t*)(x + bin_bytes); M.cur = (uint32_t*)(x + 2 * bin_bytes);
+  M.state = (MsdState*)(x + 3 * bin_bytes);
+  M.n = (uint32_t)n; M.bits = bits; M.top = top;
+  if (!c->s_report) TRY(take_report(c, &c->s_report));
+  M.report = &c->s_report->fits;
+  volatile uint32_t* fits = M.report;
+  *fits = 2;
+  launch_msd_sort<K>(M, 0, c->num_sms, c->stream);
+  CK(cudaGetLastError());
+  while (*fits == 2) {  // (at the latest when these kernels are done)
+    const cudaError_t q = cudaStreamQuery(c->stream);
+    if (q == cudaErrorNotReady) continue;
+    CK(q);
+    break;
   }
+  *sorted = *fits == 1;
+  if (*sorted) launch_msd_sort<K>(M, 1, c->num_sms, c->stream);
+  CK(cudaGetLastError());
   return WG_OK;
 }
 
@@ -313,7 +320,7 @@ static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
   const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
   uint32_t top = 1;  // the top digit: bins of at most 5,000 keys on average (of kMsdCap)
   while (top < 31 && (n >> top) > 5000) ++top;
-  const bool msd = sizeof(K) == 8 && n >= kMsdMin && top <= kMsdTopMax && top < bits;
+  const bool msd = n >= kMsdMin && top <= kMsdTopMax && top < bits;
   const size_t key_bytes = round_up(n * sizeof(K)), bin_bytes = msd ? (size_t)4 << top : 0;
   TRY(prim_scratch(c, msd ? key_bytes + 3 * bin_bytes + 256 : n * sizeof(K), ntiles));
   // a wait that gave up in an earlier primitive must not make these passes
@@ -330,16 +337,19 @@ static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
   sg.n = n; sg.tile0 = 0; sg.ntiles = ntiles;
   TRY(prim_seg(c, sg));
   CK(cudaMemsetAsync(c->s_hist, 0, sizeof(unsigned long long) * passes * kRadix, c->stream));
-  Stage h = prim_stage(c, ntiles);
+  Stage st[S_SORT_END - S_HIST] = {};  // the histogram's record and the passes': one copy
+  Stage& h = st[0];
+  h = prim_stage(c, ntiles);
   h.in = keys; h.passes = passes; h.dbits = dbits;
-  TRY(prim_put(c, S_HIST, h));
   K* buf[2] = {keys, (K*)c->s_tmp};
   for (uint32_t p = 0; p < passes; ++p) {
     Stage s = h;
     s.in = buf[p & 1]; s.out = buf[(p + 1) & 1];
     s.shift = p * dbits; s.pass = p; s.epoch = prim_epoch(c);
-    TRY(prim_put(c, S_PASS0 + p, s));
+    st[S_PASS0 - S_HIST + p] = s;
   }
+  CK(cudaMemcpyAsync(c->s_stage + S_HIST, st, (S_PASS0 - S_HIST + passes) * sizeof(Stage),
+                     cudaMemcpyHostToDevice, c->stream));
   launch_sort_hist<K>(c->s_stage + S_HIST, grid_of(c, occ_sort<K>(c, 0)), c->stream);
   for (uint32_t p = 0; p < passes; ++p)
     launch_sort_pass<K>(c->s_stage + S_PASS0 + p, grid_of(c, occ_sort<K>(c, 1)), c->stream, dbits);

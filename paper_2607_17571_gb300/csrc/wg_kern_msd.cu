@@ -10,10 +10,11 @@
 // skewed (a bin over kMsdCap keys) go to the lookback passes: a sample finds most
 // of them in a few microseconds, the exact count the rest.
 //
-// 2^24 uniform 64-bit keys on 34 bits: whole call 297 us (990 with the lookback
+// 2^24 uniform 64-bit keys on 34 bits: whole call 276 us (1,054 with the lookback
 // passes' five; 399 with the partition's keys written from where they were read, 652
-// with the bins also sorted by three LSD passes); 48 bits 299, 1,190, 396 and 864.
-// Bound by shared memory: one counting atomic and two staged moves a key and kernel.
+// with the bins also sorted by three LSD passes, both with two read-backs); 48 bits
+// 276, 1,227, 396 and 864.  Bound by shared memory: one counting atomic and two
+// staged moves a key and kernel.
 #include "wg_device.cuh"
 #include "wg_launch.h"
 
@@ -24,7 +25,8 @@ __device__ __forceinline__ uint32_t msd_bin(const MsdJob& J, K k) {
   return (uint32_t)(k >> (J.bits - J.top)) & ((1u << J.top) - 1);
 }
 
-// A sample of the keys: are 2^8 (or fewer) bins of the top bits about even?
+// A sample of the keys: are 2^8 (or fewer) bins of the top bits about even?  Clears
+// the bins' counts too.
 template <typename K>
 __global__ void __launch_bounds__(1024) k_msd_probe(MsdJob J) {
   constexpr uint32_t kSample = 4096;
@@ -33,6 +35,7 @@ __global__ void __launch_bounds__(1024) k_msd_probe(MsdJob J) {
   const uint32_t t = threadIdx.x, coarse = min(J.top, 8u);
   if (t < 256) cnt[t] = 0;
   if (t == 0) s_max = 0;
+  for (uint32_t i = t; i < 1u << J.top; i += 1024) J.cnt[i] = 0;
   __syncthreads();
   const uint32_t step = J.n / kSample;  // (at least 1: n >= kMsdMin)
 #pragma unroll
@@ -43,16 +46,19 @@ __global__ void __launch_bounds__(1024) k_msd_probe(MsdJob J) {
   __syncthreads();
   if (t == 0) {
     // twice the even share and some: a fuller bin would rarely fit
-    J.state->ok = s_max <= 2 * (kSample >> coarse) + 16 ? 1u : 0u;
+    const uint32_t ok = s_max <= 2 * (kSample >> coarse) + 16 ? 1u : 0u;
+    J.state->ok = ok;
     J.state->next = 0;
+    if (!ok) *J.report = 0;
   }
 }
 
-// Keys per bin (cnt is cleared before).
+// Keys per bin.
 template <typename K>
 __global__ void __launch_bounds__(1024) k_msd_count(MsdJob J) {
   extern __shared__ uint32_t cnt[];
   const uint32_t nb = 1u << J.top;
+  if (!J.state->ok) return;
   for (uint32_t i = threadIdx.x; i < nb; i += 1024) cnt[i] = 0;
   __syncthreads();
   const K* in = (const K*)J.in;
@@ -77,6 +83,7 @@ __global__ void __launch_bounds__(1024) k_msd_plan(MsdJob J) {
   __shared__ uint32_t sh[32], s_max;
   const uint32_t nb = 1u << J.top, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const uint32_t per = (nb + 1023) / 1024, b0 = t * per;
+  if (!J.state->ok) return;
   if (t == 0) s_max = 0;
   __syncthreads();
   uint32_t sum = 0, top = 0;
@@ -102,7 +109,7 @@ __global__ void __launch_bounds__(1024) k_msd_plan(MsdJob J) {
     before += J.cnt[i];
   }
   if (t == 0) {
-    J.state->ok = s_max <= kMsdCap ? 1u : 0u;
+    J.state->ok = *J.report = s_max <= kMsdCap ? 1u : 0u;
   }
 }
 
@@ -192,7 +199,7 @@ __global__ void __launch_bounds__(1024) k_msd_partition(MsdJob J) {
 // one of more than 64, goes through LSD passes of at most 8 bits instead (a warp
 // ranks its consecutive keys with match_any).
 template <typename K>
-__global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
+__global__ void __launch_bounds__(kMsdThreads, sizeof(K) == 4 ? 3 : 2) k_msd_bins(MsdJob J) {
   extern __shared__ __align__(16) unsigned long long smem_bins[];  // [kMsdCap] keys | [warps][256] counters
   constexpr uint32_t kW = kMsdThreads / 32, kItems = kMsdCap / kMsdThreads;
   __shared__ uint32_t s_sum[kW], s_bin, s_cost;
@@ -360,17 +367,14 @@ __global__ void __launch_bounds__(kMsdThreads) k_msd_bins(MsdJob J) {
   }
 }
 
-// Step 0: the sample (state->ok); 1: count and plan (state->ok); 2: the sort.  The
-// caller reads state->ok after steps 0 and 1: with a skewed array it pays the
-// sample and one read-back.
+// Step 0: the sample, then count and plan (state->ok: the bins fit); 1: the sort.
+// The caller waits for the report between them; a skewed array skips the count.
 template <typename K>
 void launch_msd_sort(const MsdJob& J, int step, int sms, cudaStream_t s) {
   const uint32_t nb = 1u << J.top;
   if (step == 0) {
     k_msd_probe<K><<<1, 1024, 0, s>>>(J);
-  } else if (step == 1) {
     cudaFuncSetAttribute(k_msd_count<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << kMsdTopMax);
-    cudaMemsetAsync(J.cnt, 0, nb * 4, s);
     k_msd_count<K><<<sms, 1024, nb * 4, s>>>(J);
     k_msd_plan<<<1, 1024, 0, s>>>(J);
   } else {
@@ -385,6 +389,7 @@ void launch_msd_sort(const MsdJob& J, int step, int sms, cudaStream_t s) {
     k_msd_bins<K><<<sms * max(1, occ), kMsdThreads, bins, s>>>(J);
   }
 }
+template void launch_msd_sort<uint32_t>(const MsdJob&, int, int, cudaStream_t);
 template void launch_msd_sort<unsigned long long>(const MsdJob&, int, int, cudaStream_t);
 
 }  // namespace wg

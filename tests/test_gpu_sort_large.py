@@ -91,3 +91,14 @@ def test_buckets_within_a_bin(ctx, bits, copies):
     one = ((a >> low) == 9).nonzero().flatten()[:copies]
     b[one] = (9 << low) | (b[one] & 1)              # one full bucket, keys out of order
     _sort(ctx, b, bits)
+
+
+@pytest.mark.parametrize("kb,bits", [(4, 12), (4, 26), (4, 32), (8, 13), (8, 34)])
+@pytest.mark.parametrize("n", [(1 << 22) - 1, 1 << 22, (1 << 22) + 16_383])
+def test_first_sizes(ctx, kb, bits, n):
+    """Around the first size of the top-digit-first form, even keys, one key, and
+    few values with the top bits unused."""
+    a = _uniform(n, kb, bits, n + bits)
+    _sort(ctx, a, bits)
+    _sort(ctx, a[:1].repeat(n), bits)
+    _sort(ctx, a & ((1 << (bits - 6)) - 1), bits)
