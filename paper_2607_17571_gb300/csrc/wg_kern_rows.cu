@@ -16,7 +16,7 @@
 // Measured on GB300, fixpoint and result in device memory, sorted-array
 // pipeline -> rows: R-MAT 2^17 / 400k edges (4.8e8 tuples) 68.0 -> 5.35 ms (k_rows
 // 3.50), R-MAT 2^19 / 400k (1.0e9 tuples, 64-bit keys) 164 -> 12.6 ms (7.69), ER
-// 1,000 / 3,000 2.55 -> 0.10 ms, a chain of 1,000 vertices 147 -> 1.1 ms.
+// 1,000 / 3,000 2.55 -> 0.10 ms, a chain of 1,000 vertices 147 -> 0.72 ms.
 //
 //   k_rows        the fixpoints of all rows (one CTA per row, rows claimed)
 //   k_row_plan    row offsets (scan of the row counts), totals, capacity check
@@ -60,6 +60,12 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
   }
 }
 
+template <int T>
+__device__ __forceinline__ void cta_sync() {
+  if (T == 32) __syncwarp();
+  else __syncthreads();
+}
+
 // One CTA takes a row through its whole fixpoint.  Shared memory: the row's bit
 // set S and the candidates' bit set N of the next iteration.
 // An iteration: the threads take 128 bits of N at a time, drop what S has, merge
@@ -80,10 +86,15 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
 // past them 16.1 ms; candidate bits without an answer, edges in 16-byte units,
 // a list per warp (one barrier, but it waited for the warp with the most to
 // expand) 8.3; one list per CTA 7.5; one N instead of two, no test per place 7.0; vertex
-// records of 16 bytes 5.35.
+// records of 16 bytes 5.35.  With one warp (T = 32) an iteration is a chain of
+// dependent instructions: a chain of 1,000 vertices took 1.09 ms with the counts in
+// shared memory and one global atomic per iteration past its log, 1.02 with 32
+// iterations' counts to an atomic, 0.84 with the list's length and the delta's size
+// in registers, 0.72 without scan and barriers where no lane has two new vertices.
 template <typename IdT, int T, int kMin>
 __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   constexpr uint32_t kW = T / 32, kList = row_list(T);
+  constexpr bool kOne = kW == 1;  // one warp: counts stay in registers
   extern __shared__ uint4 sm4[];
   __shared__ RowInst I;
   __shared__ unsigned long long s_log[kRowLog];
@@ -144,13 +155,19 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
       }
       __syncthreads();
       uint32_t lvl = 0, total = 0, turn = 0;
+      // iterations past the log in shared memory: warp 0's lanes hold 32 of them
+      uint32_t held = 0;
+      auto log_held = [&](uint32_t first) {
+        if (held && first + lane < I.log_cap) atomicAdd(I.log + first + lane, (unsigned long long)held);
+        held = 0;
+      };
       uint4* const n4 = (uint4*)N;
       uint4* const out = (uint4*)(I.bits + (size_t)(J.rows ? at_row : x) * words);
       for (;; ++lvl) {
-        uint32_t listed = 0, wait = 0;  // wait: this thread's steps with bits not yet listed
+        uint32_t listed = 0, cnt = 0, wait = 0;  // wait: this thread's steps with bits not yet listed
         for (uint32_t round = 0;; ++round, turn ^= 1) {
-          if (tid == 0) s_len[turn ^ 1] = 0;
-          uint32_t got = 0;
+          if (!kOne && tid == 0) s_len[turn ^ 1] = 0;
+          uint32_t got = 0, len = 0;
           uint4 nd = {0, 0, 0, 0};
           if (round == 0 && tid < quads) nd = n4[tid];
           for (uint32_t g = warp * 32, step = 1; g < quads; g += T, step <<= 1) {
@@ -170,12 +187,24 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
             } else if (wait & step) {
               d = out[w];
             }
-            if (!__any_sync(0xffffffffu, d.x | d.y | d.z | d.w)) continue;
+            const uint32_t any = d.x | d.y | d.z | d.w;
+            const uint32_t has = __ballot_sync(0xffffffffu, any != 0);
+            if (!has) continue;
             const uint32_t c = __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+            if (kOne && round == 0 && len + 32 <= kList && !__any_sync(0xffffffffu, c > 1)) {
+              // at most one vertex a lane (a deep relation's deltas): no scan
+              if (any)
+                list[len + __popc(has & ((1u << lane) - 1))] =
+                    (IdT)(w * 128 + (d.x ? 0 : d.y ? 32 : d.z ? 64 : 96) + __ffs(any) - 1);
+              len += __popc(has);
+              continue;
+            }
             const uint32_t in = warp_incl_scan(c, lane);
             uint32_t at = 0;
-            if (lane == 31) at = atomicAdd(s_len + turn, in);
-            at = __shfl_sync(0xffffffffu, at, 31) + in - c;
+            if (kOne) at = len, len += __shfl_sync(0xffffffffu, in, 31);
+            else if (lane == 31) at = atomicAdd(s_len + turn, in);
+            if (!kOne) at = __shfl_sync(0xffffffffu, at, 31);
+            at += in - c;
             auto put = [&](uint32_t& m, uint32_t base) {
               while (m && at < kList) {
                 list[at++] = (IdT)(base + __ffs(m) - 1);
@@ -190,26 +219,31 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
             }
           }
           got = __reduce_add_sync(0xffffffffu, got);
-          if (lane == 0 && got) atomicAdd(s_cnt + (lvl & 1), got);
-          __syncthreads();
-          const uint32_t len = s_len[turn], n = min(len, kList);
-          if (round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
+          if (!kOne && lane == 0 && got) atomicAdd(s_cnt + (lvl & 1), got);
+          cnt += got;  // (kOne)
+          cta_sync<T>();
+          if (!kOne) len = s_len[turn];
+          const uint32_t n = min(len, kList);
+          if (!kOne && round == 0 && tid == 0) s_cnt[~lvl & 1] = 0;
           listed |= len;
           if (len == 0) break;
           cand += expand_vertices<IdT, false>(I, list, warp * 32, n, T, N, strip);
-          __syncthreads();
+          cta_sync<T>();
           if (len <= kList) break;
         }
-        const uint32_t n = s_cnt[lvl & 1];
+        const uint32_t n = kOne ? cnt : s_cnt[lvl & 1];
         if (n == 0) break;
         total += n;
-        if (tid == 0) {
-          if (lvl < kRowLog) s_log[lvl] += n;
-          else if (lvl < I.log_cap) atomicAdd(I.log + lvl, (unsigned long long)n);
+        if (lvl < kRowLog) {
+          if (tid == 0) s_log[lvl] += n;
+        } else if (warp == 0) {
+          if (lane == (lvl & 31)) held = n;
+          if ((lvl & 31) == 31) log_held(lvl & ~31u);
         }
         if (listed == 0) { ++lvl; break; }  // nothing of this delta joins any edge
         turn ^= 1;
       }
+      if (warp == 0 && lvl > kRowLog) log_held((lvl - 1) & ~31u);
       if (tid == 0) {  // (the delta of iteration lvl - 1 was the last that is not empty)
         atomicMax(&J.inst[q].last, lvl - 1);
         I.cnt[x] = total;
@@ -524,7 +558,7 @@ static uint32_t row_smem(uint32_t vwords, int id_bytes, int threads) {
 }
 // Threads per CTA: a CTA waits twice per iteration for its slowest warp, so the
 // smaller the better while its bit sets leave room for enough CTAs per SM.
-// Whole calls, 32 / 64 / 128 / 256 / 512 threads: chain of 1,000 (32 words) 1.07 /
+// Whole calls, 32 / 64 / 128 / 256 / 512 threads: chain of 1,000 (32 words) 0.72 /
 // 1.18 / 1.17 / 2.1 / 2.4 ms; the 64-query batch (up to 512) 12.3 / 12.3 / 13.1 ms;
 // R-MAT 2^15 / 100k (750) - / 537 / 510 us; R-MAT 2^17 / 400k (1,900) - / 7.3 / 7.0 /
 // 7.2 / 8.4 ms and 2^19 / 400k (3,900 words) - / 22.7 / 16.8 / 15.2 / 16.9 ms (both
