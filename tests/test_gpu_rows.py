@@ -199,3 +199,14 @@ def test_long_rows_and_the_budget(rows, budget_mb):
             assert (st.n_tuples, st.iterations, q.digest()) == (n, iters, dg)
             assert q.delta_sizes() == list(log)
             q.free()
+
+
+@pytest.mark.parametrize("n", [63, 64, 65, 66, 95, 96, 97, 129, 161])
+@pytest.mark.parametrize("wide", [0, 5_000, 70_000])
+def test_iterations_past_the_shared_log(ctx, n, wide):
+    """A path of n edges, alone (one warp a row) and beside wide single edges (more
+    warps, 32-bit ranks): its iterations past 64 are logged 32 at a time."""
+    g = I.path(n + 1)
+    at = int(max(g.src.max(), g.dst.max())) + 1
+    b = np.arange(at, at + wide, dtype=np.uint32)
+    _check(ctx, np.concatenate([g.src, b[0::2]]), np.concatenate([g.dst, b[1::2]]))
