@@ -251,6 +251,17 @@ static int prim_scratch(wg_ctx* c, size_t tmp_bytes, size_t ntiles) {
   }
   return WG_OK;
 }
+// Scratch of a form that can be done without: *ok says whether there was room, and
+// without it the keys' buffer is given back.
+static int prim_scratch_if(wg_ctx* c, size_t tmp_bytes, size_t ntiles, bool* ok) {
+  const int rc = prim_scratch(c, tmp_bytes, ntiles);
+  *ok = rc == WG_OK;
+  if (rc != WG_E_BUDGET && rc != WG_E_NOMEM) return rc;
+  cudaGetLastError();
+  dev_free(c, c->s_tmp, c->s_tmp_bytes);
+  c->s_tmp = nullptr; c->s_tmp_bytes = 0;
+  return WG_OK;
+}
 static uint32_t prim_epoch(wg_ctx* c) {
   if (++c->s_epoch >= (1u << 23)) {  // epochs wrap at 24 bits: clear the words first
     cudaMemsetAsync(c->s_status, 0, c->s_status_n * 8, c->stream);
@@ -320,9 +331,10 @@ static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
   const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
   uint32_t top = 1;  // the top digit: bins of at most 5,000 keys on average (of kMsdCap)
   while (top < 31 && (n >> top) > 5000) ++top;
-  const bool msd = n >= kMsdMin && top <= kMsdTopMax && top < bits;
+  bool msd = n >= kMsdMin && top <= kMsdTopMax && top < bits;
   const size_t key_bytes = round_up(n * sizeof(K)), bin_bytes = msd ? (size_t)4 << top : 0;
-  TRY(prim_scratch(c, msd ? key_bytes + 3 * bin_bytes + 256 : n * sizeof(K), ntiles));
+  if (msd) TRY(prim_scratch_if(c, key_bytes + 3 * bin_bytes + 256, ntiles, &msd));
+  if (!msd) TRY(prim_scratch(c, n * sizeof(K), ntiles));
   // a wait that gave up in an earlier primitive must not make these passes
   // skip their work: the control block starts clear (the caller reads it after)
   CK(cudaMemsetAsync(c->s_ctl, 0, sizeof(Ctl), c->stream));
@@ -372,12 +384,8 @@ static int prim_unique(wg_ctx* c, const K* in, size_t n, const K* full, size_t n
   constexpr uint32_t T = FuseTile<K>::T;
   const uint64_t tiles = ((uint64_t)n + nf + T - 1) / T;
   bool merged = nf > 0 && nf <= 64 * (uint64_t)n && tiles < (1u << 31);
-  if (merged) {  // (a status word per tile: fewer than prim_scratch's per digit)
-    const int rc = prim_scratch(c, (tiles + 1) * 8, tiles / kRadix + 1);
-    if (rc != WG_OK && rc != WG_E_BUDGET && rc != WG_E_NOMEM) return rc;
-    if (rc != WG_OK) cudaGetLastError();
-    merged = rc == WG_OK;
-  }
+  // (a status word per tile: fewer than prim_scratch's per digit)
+  if (merged) TRY(prim_scratch_if(c, (tiles + 1) * 8, tiles / kRadix + 1, &merged));
   Seg sg{};
   if (merged) {
     sg.n = nf; sg.aux_n = n; sg.ntiles = (uint32_t)tiles;
@@ -418,19 +426,15 @@ static int prim_merge(wg_ctx* c, const K* a, size_t na, const K* b, size_t nb, K
   const uint32_t ntiles = (uint32_t)((na + nb + kTileM - 1) / kTileM);
   // the tiles' splits, found in parallel (in the sort's buffer); without room
   // for them each tile searches its own
-  const int rc = prim_scratch(c, ((size_t)ntiles + 1) * 8, 0);
-  if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
-    cudaGetLastError();
-    TRY(prim_scratch(c, 0, 0));
-  } else {
-    TRY(rc);
-  }
+  bool split = true;
+  TRY(prim_scratch_if(c, ((size_t)ntiles + 1) * 8, 0, &split));
+  if (!split) TRY(prim_scratch(c, 0, 0));
   Seg sg{};
   sg.n = na; sg.aux_n = nb; sg.ntiles = ntiles;
   TRY(prim_seg(c, sg));
   Stage m = prim_stage(c, ntiles);
   m.in = a; m.aux = b; m.out = out;
-  m.splits = rc == WG_OK ? (unsigned long long*)c->s_tmp : nullptr;
+  m.splits = split ? (unsigned long long*)c->s_tmp : nullptr;
   TRY(prim_put(c, S_MERGE, m));
   if (m.splits) launch_partition<K>(c->s_stage + S_MERGE, 0, kTileM, c->num_sms * 4, c->stream);
   launch_merge<K>(c->s_stage + S_MERGE, grid_of(c, occ_sort<K>(c, 3)), c->stream);

@@ -102,3 +102,28 @@ def test_first_sizes(ctx, kb, bits, n):
     _sort(ctx, a, bits)
     _sort(ctx, a[:1].repeat(n), bits)
     _sort(ctx, a & ((1 << (bits - 6)) - 1), bits)
+
+
+@pytest.mark.parametrize("kb", [4, 8])
+def test_needs_no_larger_budget_than_the_passes(kb):
+    from paper_2607_17571_gb300 import wg
+
+    def least(n):
+        """The smallest budget, in units of 256 bytes, that sorts n keys."""
+        a = _uniform(n, kb, 8 * kb - 2, n)
+        lo, hi = 16, n * kb * 2 // 256
+        while lo < hi:
+            mid = (lo + hi) // 2
+            with wg.Context(0, mem_budget=mid * 256) as c:
+                t = a.clone()
+                torch.cuda.synchronize()
+                try:
+                    c.sort_keys(t.data_ptr(), n, kb, 8 * kb - 2)
+                    assert torch.equal(t, a.sort().values)
+                    hi = mid
+                except wg.WgError as e:
+                    assert "BUDGET" in str(e)
+                    lo = mid + 1
+        return lo
+
+    assert least(1 << 22) == least((1 << 22) - 1)  # the first takes the counts if it can
