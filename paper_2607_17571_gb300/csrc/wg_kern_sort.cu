@@ -859,20 +859,20 @@ __device__ __forceinline__ unsigned long long merge_path(const K* A, unsigned lo
 // A tile's inputs are staged in shared memory; each thread takes 16 consecutive
 // outputs, one merge-path search for their start and then one comparison each,
 // and the tile goes out through shared memory, coalesced.  (A search per output:
-// 0.28 ms for 2.8e7 64-bit keys, now 0.15.)
+// 0.28 ms for 2.8e7 64-bit keys, now 0.13.)  Tiles are dealt out by CTA and the
+// splits read by every thread, so nothing waits before the loads; at 5 CTAs an SM
+// the registers just fit (whole call, 2^24 + 2^24 64-bit keys: claimed tiles and 4
+// CTAs 229 us, dealt out 223, and 5 CTAs 201; 32-bit keys 140, 136, 134).
 template <typename K>
-__global__ void __launch_bounds__(kThreads) k_merge(Stage* stp) {
+__global__ void __launch_bounds__(kThreads, 5) k_merge(Stage* stp) {
   __shared__ K sm[Padded<kTileM>::n];
   __shared__ unsigned long long s_a0, s_a1;
-  __shared__ uint32_t s_t;
   Ctl* ctl = stp->ctl;
   if (*(volatile uint32_t*)&ctl->abort) return;
   const K* A_all = (const K*)stp->in;
   const K* B_all = (const K*)stp->aux;
   const uint32_t nseg = stp->nseg, ntiles = stp->ntiles;
-  for (;;) {
-    const uint32_t t = claim_tile(stp, &s_t);
-    if (t >= ntiles) return;
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t k = find_seg(stp->segs, nseg, t, stp->tile_seg);
     const Seg sg = stp->segs[k];
     const K* A = A_all + sg.in_off;
@@ -882,15 +882,18 @@ __global__ void __launch_bounds__(kThreads) k_merge(Stage* stp) {
     const unsigned long long d0 = (unsigned long long)(t - sg.tile0) * kTileM;
     const unsigned long long d1 = min(d0 + kTileM, na + nb);
     const bool last = t == sg.tile0 + sg.ntiles - 1;
-    if (stp->splits) {
-      if (threadIdx.x == 0) s_a0 = stp->splits[t];
-      if (threadIdx.x == 32) s_a1 = last ? na : stp->splits[t + 1];
+    unsigned long long a0, a1;
+    if (stp->splits) {  // every thread reads them: no barrier before the loads
+      a0 = stp->splits[t];
+      a1 = last ? na : stp->splits[t + 1];
     } else {
       if (threadIdx.x == 0) s_a0 = merge_path(A, na, B, nb, d0);
       if (threadIdx.x == 32) s_a1 = merge_path(A, na, B, nb, d1);
+      __syncthreads();
+      a0 = s_a0;
+      a1 = s_a1;
     }
-    __syncthreads();
-    const unsigned long long a0 = s_a0, a1 = s_a1, b0 = d0 - a0, b1 = d1 - a1;
+    const unsigned long long b0 = d0 - a0, b1 = d1 - a1;
     const uint32_t la = (uint32_t)(a1 - a0), lb = (uint32_t)(b1 - b0);
     if (lb == 0 || la == 0) {  // one side only: a straight copy
       const K* src = lb == 0 ? A + a0 : B + b0;
