@@ -347,7 +347,7 @@ int wg_selftest_wait_timeout(wg_ctx* ctx);
  * higher bits must be zero), in place (Sec. Buffer Routing and Adaptive Radix
  * Sort: histogram, prefix sum, scatter per digit).  Every pass after the
  * first is stable; keys equal on the sorted bits are identical, so the
- * result is the unique sorted sequence.  From 2^22 keys the top digit
+ * result is the unique sorted sequence.  From 2^17 64-bit or 2^22 32-bit keys the top digit
  * goes first (one unordered partition), then every bin is sorted in shared
  * memory; keys too unevenly spread for that take the passes. */
 int wg_sort_keys(wg_ctx* ctx, void* d_keys, size_t n, int key_bytes, uint32_t bits);

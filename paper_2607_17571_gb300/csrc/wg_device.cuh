@@ -328,7 +328,7 @@ struct MsdJob {                          // wg_kern_msd.cu
 };
 constexpr uint32_t kMsdTile = 16384, kMsdCap = 8192, kMsdTopMax = 14, kMsdFine = 12;
 constexpr int kMsdThreads = 512;
-constexpr uint32_t kMsdMin = 1u << 22;   // keys (see prim_sort)
+constexpr uint32_t kMsdMin[2] = {1u << 22, 1u << 17};  // 32- and 64-bit keys (see prim_sort_msd)
 
 // ---------------------------------------------------------------- triangle counting
 struct TriCtl {

@@ -292,12 +292,13 @@ static void pass_plan(uint32_t bits, uint32_t* passes, uint32_t* dbits) {
 
 // Large arrays by their top digit first (wg_kern_msd.cu), when a sample and then
 // the exact count find that their bins fit; *sorted says whether.  Even keys,
-// lookback passes -> top digit first, 2^21 / 2^22 / 2^23 / 2^24: 34 bits of 64
-// 208 -> 76, 311 -> 95, 551 -> 162, 1,054 -> 276 us; 48 bits 251 -> 78, 390 -> 94,
-// 687 -> 160, 1,227 -> 276; 32-bit keys 152 -> 66, 214 -> 91, 339 -> 130, 573 ->
-// 218.  A skewed array pays the sample until its report, 10 us: at 32-bit keys 8% /
-// 5% / 3% / 2%, half of which the single copy of the passes' records gives back, so
-// the line lies at 2^22 keys.
+// lookback passes -> top digit first, 2^17 / 2^20 / 2^22 / 2^24: 34 bits of 64
+// 164 -> 62, 184 -> 67, 324 -> 99, 1,054 -> 276 us; 48 bits 193 -> 59, 230 -> 71,
+// 393 -> 96, 1,227 -> 276; 32-bit keys 124 -> 59, 140 -> 70, 222 -> 85, 573 -> 218.
+// A skewed array pays the sample until its report, 10 us, half of which the single
+// copy of the passes' records gives back: 156 -> 159, 177 -> 183, 304 -> 315 us of
+// 64-bit keys, and with 32-bit keys' fewer passes 113 -> 120, 130 -> 140, 209 -> 216.
+// So the line lies at 2^17 64-bit and 2^22 32-bit keys.
 template <typename K>
 static int prim_sort_msd(wg_ctx* c, K* keys, size_t n, uint32_t bits, uint32_t top, size_t key_bytes,
                          size_t bin_bytes, bool* sorted) {
@@ -331,7 +332,7 @@ static int prim_sort(wg_ctx* c, K* keys, size_t n, uint32_t bits) {
   const uint32_t ntiles = (uint32_t)((n + kTileC - 1) / kTileC);
   uint32_t top = 1;  // the top digit: bins of at most 5,000 keys on average (of kMsdCap)
   while (top < 31 && (n >> top) > 5000) ++top;
-  bool msd = n >= kMsdMin && top <= kMsdTopMax && top < bits;
+  bool msd = n >= kMsdMin[sizeof(K) / 8] && top <= kMsdTopMax && top < bits;
   const size_t key_bytes = round_up(n * sizeof(K)), bin_bytes = msd ? (size_t)4 << top : 0;
   if (msd) TRY(prim_scratch_if(c, key_bytes + 3 * bin_bytes + 256, ntiles, &msd));
   if (!msd) TRY(prim_scratch(c, n * sizeof(K), ntiles));

@@ -127,3 +127,13 @@ def test_needs_no_larger_budget_than_the_passes(kb):
         return lo
 
     assert least(1 << 22) == least((1 << 22) - 1)  # the first takes the counts if it can
+
+
+@pytest.mark.parametrize("bits", [6, 13, 18, 34, 62, 64])
+@pytest.mark.parametrize("n", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1, 200_003, (1 << 19) + 5])
+def test_first_sizes_of_64_bit_keys(ctx, bits, n):
+    """Few bins: fewer than the sample's, than a CTA's threads, than CTAs."""
+    a = _uniform(n, 8, bits, n + bits)
+    _sort(ctx, a, bits)
+    _sort(ctx, a[:1].repeat(n), bits)
+    _sort(ctx, a & ((1 << (bits - 4)) - 1) if bits < 64 else a >> 1, bits)
