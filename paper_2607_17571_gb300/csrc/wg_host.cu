@@ -2393,6 +2393,13 @@ static void release_lanes(wg_ctx* c) {
 constexpr size_t kLaneBits = 256u << 20;
 constexpr uint32_t kLaneQueries = 1024;
 
+// Per-iteration sizes to keep for a query over nv vertices, at most `cap`: a TC
+// row's levels are distinct vertices, an SG pair's distinct pairs (two cycles of
+// lengths 31 and 32 under one parent: 64 vertices, 992 iterations).
+static uint32_t row_log_len(int kind, uint64_t nv, uint32_t cap) {
+  return (uint32_t)std::min<uint64_t>(cap, (kind == WG_SG ? nv * nv : nv) + 2);
+}
+
 // Start the queued queries `ids` (one key width) on lane L.
 static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   AllocScope scope(c, L->st);
@@ -2417,7 +2424,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
     bits += q->rel->row_bits();
     masks += q->rel->sg_masks();
   }
-  L->log_cap = std::min(kBatchLogCap, nv_max + 2);
+  L->log_cap = row_log_len(qs[0]->kind, nv_max, kBatchLogCap);
   const int grid = (int)std::min<uint64_t>(
       grid_of(c, occ_rows(c, L->sg, idb, vwords)),
       (uint64_t)nch * kRowChunk);
@@ -2578,7 +2585,7 @@ static int lane_expand(wg_ctx* c, RowLane* L) {
     q->iterations = capped ? I.max_iters : I.last + 1;
     const unsigned long long* log =
         (const unsigned long long*)L->host(L->o_log) + (size_t)L->slot[i] * L->log_cap;
-    q->log.assign(log, log + std::min(q->iterations + 1, kBatchLogCap));
+    q->log.assign(log, log + std::min(q->iterations + 1, L->log_cap));
     q->error = capped ? WG_E_ITER_CAP : WG_OK;
     q->res_ptr = q->res_own.p;
     I.out = q->res_own.p;
