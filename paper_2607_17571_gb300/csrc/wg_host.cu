@@ -654,6 +654,13 @@ static int tri_count(wg_ctx* c, Relation* R, unsigned long long* count) {
   return rc;
 }
 
+// Per-iteration sizes to keep for a query over nv vertices, at most `cap`: a TC
+// row's levels are distinct vertices, an SG pair's distinct pairs (two cycles of
+// lengths 31 and 32 under one parent: 64 vertices, 992 iterations).
+static uint32_t row_log_len(int kind, uint64_t nv, uint32_t cap) {
+  return (uint32_t)std::min<uint64_t>(cap, (kind == WG_SG ? nv * nv : nv) + 2);
+}
+
 // ------------------------------------------------------------------ engine
 struct KStat {
   const char* name;
@@ -1049,7 +1056,7 @@ struct Engine : EngineBase {
     AllocScope scope(c, st);
     const uint32_t nv = Rl->nv, words = Rl->row_words();
     const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
-    const uint32_t nlog = std::min<uint32_t>(1u << 16, nv + 2);
+    const uint32_t nlog = row_log_len(kind, nv, 1u << 16);
     row_sg = kind == WG_SG;
     const bool small = !row_sg && Rl->small_rows();
     id_bytes = Rl->id_bytes();
@@ -2392,13 +2399,6 @@ static void release_lanes(wg_ctx* c) {
 // most), and instances per launch.
 constexpr size_t kLaneBits = 256u << 20;
 constexpr uint32_t kLaneQueries = 1024;
-
-// Per-iteration sizes to keep for a query over nv vertices, at most `cap`: a TC
-// row's levels are distinct vertices, an SG pair's distinct pairs (two cycles of
-// lengths 31 and 32 under one parent: 64 vertices, 992 iterations).
-static uint32_t row_log_len(int kind, uint64_t nv, uint32_t cap) {
-  return (uint32_t)std::min<uint64_t>(cap, (kind == WG_SG ? nv * nv : nv) + 2);
-}
 
 // Start the queued queries `ids` (one key width) on lane L.
 static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {

@@ -1,7 +1,7 @@
 """Same-generation fixpoints that take more iterations than the relation has
 vertices: two cycles of coprime lengths under one parent meet in lcm(p, q)
 levels.  Every per-iteration size against the oracle's log, for queries
-submitted alone, beside others, and past what a batched query keeps."""
+run singly, submitted alone or beside others, and past what a query keeps."""
 import numpy as np
 import pytest
 
@@ -46,3 +46,18 @@ def test_submitted(lengths):
                 h.free()
             for r in rels:
                 r.free()
+
+
+@pytest.mark.parametrize("p,q", [(2, 3), (3, 4), (20, 21), (31, 32), (40, 41), (256, 257)])
+def test_single(p, q):
+    from paper_2607_17571_gb300 import wg
+    e = _cycles(p, q)
+    want = oracle_sg(*e)  # (256 * 257 = 65,792 iterations: more than a query keeps)
+    with wg.Context(0) as c:
+        for kw in ({}, dict(side_run="never")):
+            rel = c.load(*e)
+            h = c.sg(rel, **kw)
+            h.wait()
+            _same(h, want, 1 << 16)
+            h.free()
+            rel.free()
