@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <set>
 #include <memory>
 #include <string>
 #include <thread>
@@ -101,6 +102,7 @@ struct wg_ctx {
   uint32_t tune_count[2] = {0, 0}, tune_fuse[2] = {0, 0}, tune_emit[2] = {0, 0};
   uint32_t tune_sort[2] = {WG_SORT_SEGMENT16, WG_SORT_SEGMENT16};  // enum wg_sort_mode
   cudaStream_t alloc_stream = nullptr;            // stream of allocations in progress (NULL: stream)
+  bool keep_layouts = false;                      // a row layout is being made (see dev_alloc)
   // scratch of the standalone primitives
   void* s_tmp = nullptr; size_t s_tmp_bytes = 0;
   unsigned long long* s_status = nullptr; size_t s_status_n = 0;
@@ -113,12 +115,15 @@ struct wg_ctx {
 
 static void drop_idle_engines(wg_ctx* c, size_t bytes);
 static void drop_idle_lanes(wg_ctx* c);
+static size_t idle_layouts(wg_ctx* c, bool drop);
 static int dev_alloc(wg_ctx* c, size_t bytes, void** out, cudaStream_t st) {
   *out = nullptr;
   if (bytes == 0) return WG_OK;
   bytes = round_up(bytes);
   if (c->used + bytes > c->budget) drop_idle_engines(c, bytes);  // unused pools go first
   if (c->used + bytes > c->budget) drop_idle_lanes(c);
+  // layouts of other relations last (made again when a query wants one, see row_layout)
+  if (c->used + bytes > c->budget && !c->keep_layouts) idle_layouts(c, true);
   if (c->used + bytes > c->budget)
     return set_err(WG_E_BUDGET, "allocation of " + std::to_string(bytes) +
                                     " bytes exceeds the memory budget");
@@ -502,21 +507,42 @@ static int build_edges(wg_ctx* c, Relation* R, const uint32_t* d_src, const uint
   launch_csr<K>((const K*)ke.p, ne, R->nv, R->w, (uint32_t*)R->off.p, (uint32_t*)R->adj.p,
                 grid_of(c, 4), c->stream);
   CK(cudaGetLastError());
-  if (R->nv <= kRowMaxVertices && ne < (1ull << 31)) {  // (units are counted in 32 bits)
-    R->o_ns = round_up((size_t)R->nv * 16);
-    R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
-    R->o_mp = R->o_units + round_up(row_units(ne, R->nv, R->id_bytes()) * 16);
-    TRY(R->rowv.get(c, R->o_mp + (size_t)R->row_words() * 8));
-    char* v = (char*)R->rowv.p;
-    launch_row_layout<K>((const K*)ke.p, (uint32_t)ne, R->w, (const uint32_t*)R->off.p,
-                         (const uint32_t*)R->adj.p, R->nv, v, (uint32_t*)(v + R->o_ns),
-                         R->row_words(), v + R->o_units, (uint32_t*)(v + R->o_mp), R->id_bytes(),
-                         grid_of(c, 8), c->stream);
-    CK(cudaGetLastError());
-  }
   return WG_OK;
 }
 
+// The layout the row fixpoints read (up to kRowMaxVertices vertices; units are counted
+// in 32 bits).  It is optional: a relation without one runs on the sorted-array
+// pipeline, so where the budget has no room for it the load succeeds without.  A query
+// that wants rows tries again, and may take the room of other relations' layouts
+// (in_load: not).
+static int row_layout(wg_ctx* c, Relation* R, bool in_load) {
+  if (R->rowv.p || R->ne == 0 || R->nv > kRowMaxVertices || R->ne >= (1ull << 31)) return WG_OK;
+  R->o_ns = round_up((size_t)R->nv * 16);
+  R->o_units = R->o_ns + round_up((size_t)R->row_words() * 4);
+  R->o_mp = R->o_units + round_up(row_units(R->ne, R->nv, R->id_bytes()) * 16);
+  AllocScope scope(c, c->stream);
+  c->keep_layouts = in_load;
+  const int rc = R->rowv.get(c, R->o_mp + (size_t)R->row_words() * 8);
+  c->keep_layouts = false;
+  if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
+    cudaGetLastError();
+    return WG_OK;
+  }
+  TRY(rc);
+  char* v = (char*)R->rowv.p;
+  uint32_t *ns = (uint32_t*)(v + R->o_ns), *mp = (uint32_t*)(v + R->o_mp);
+  const uint32_t *off = (const uint32_t*)R->off.p, *adj = (const uint32_t*)R->adj.p;
+  if (R->kb == 4)
+    launch_row_layout<uint32_t>((const uint32_t*)R->keys.p, (uint32_t)R->ne, R->w, off, adj, R->nv, v,
+                                ns, R->row_words(), v + R->o_units, mp, R->id_bytes(),
+                                grid_of(c, 8), c->stream);
+  else
+    launch_row_layout<unsigned long long>((const unsigned long long*)R->keys.p, (uint32_t)R->ne, R->w,
+                                          off, adj, R->nv, v, ns, R->row_words(), v + R->o_units,
+                                          mp, R->id_bytes(), grid_of(c, 8), c->stream);
+  CK(cudaGetLastError());
+  return WG_OK;
+}
 static int load_relation(wg_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, size_t n,
                          Relation* R) {
   if (n >= (1ull << 32)) return set_err(WG_E_INVAL, "at most 2^32 - 1 edges");
@@ -544,8 +570,9 @@ static int load_relation(wg_ctx* c, const uint32_t* d_src, const uint32_t* d_dst
   R->nv = (uint32_t)nv;
   R->w = bits_for(nv);
   R->kb = 2 * R->w <= 32 ? 4 : 8;
-  if (R->kb == 4) return build_edges<uint32_t>(c, R, d_src, d_dst, n);
-  return build_edges<unsigned long long>(c, R, d_src, d_dst, n);
+  if (R->kb == 4) TRY(build_edges<uint32_t>(c, R, d_src, d_dst, n));
+  else TRY(build_edges<unsigned long long>(c, R, d_src, d_dst, n));
+  return row_layout(c, R, true);
 }
 
 // ------------------------------------------------------------------ triangle counting
@@ -1587,6 +1614,21 @@ struct Engine : EngineBase {
   }
 };
 
+// Bytes of the row layouts of relations that no queued or running query uses; freed
+// where asked.
+static size_t idle_layouts(wg_ctx* c, bool drop) {
+  std::set<const Relation*> live;
+  for (auto& kv : c->queries)
+    if (kv.second->state == WG_PENDING || kv.second->state == WG_RUNNING) live.insert(kv.second->rel);
+  size_t b = 0;
+  for (auto& kv : c->rels) {
+    if (live.count(kv.second.get())) continue;
+    b += kv.second->rowv.bytes;
+    if (drop) kv.second->rowv.release(c);
+  }
+  return b;
+}
+
 // Free the pools of idle single-query engines, least recently used first,
 // until `bytes` more fit in the budget (a cached engine only saves the next
 // query of its kind a pool allocation and a graph capture).
@@ -2324,16 +2366,20 @@ static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R) {
 // whose bit sets take at most half of the free budget -- the sorted
 // pipeline needs more than twice the result, so whatever fits there fits here.
 static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
-  const Relation* R = q->rel;
-  if (q->opts.flags || q->opts.reserve_cand || !R->rowv.p) return false;
-  if (q->kind == WG_SG && R->nv > kSgMaxVertices) return false;
+  Relation* R = q->rel;
+  if (q->opts.flags || q->opts.reserve_cand) return false;
+  if (R->ne == 0 || R->nv > (q->kind == WG_SG ? kSgMaxVertices : kRowMaxVertices)) return false;
   size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
   for (auto& e : c->idle) idle += e->held();
   // (small rows apart: their lists, and bit sets for whatever is left)
   const size_t need = q->kind == WG_SG ? 3 * (R->row_bits() + R->sg_masks()) + (size_t)R->nv * 16
                       : R->small_rows() && !batched ? (size_t)R->nv * kSmallRow * 8
                                                     : R->row_bits();
-  return need <= (c->budget - std::min(c->budget, c->used) + idle) / 2;
+  const size_t room = c->budget - std::min(c->budget, c->used) + idle;
+  if (need > room / 2 && need > (room + idle_layouts(c, false)) / 2) return false;
+  if (R->rowv.p) return true;
+  // (made here, it is complete before a lane reads it on its own stream)
+  return row_layout(c, R, false) == WG_OK && R->rowv.p && cudaStreamSynchronize(c->stream) == cudaSuccess;
 }
 static bool row_query(wg_ctx* c, const Query* q) {
   return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->rel->no_rows &&
