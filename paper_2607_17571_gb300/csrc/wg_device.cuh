@@ -310,6 +310,11 @@ struct SgJob {
   SgInst* sg;
   uint32_t* list[2];            // rows with a non-empty delta, by iteration mod 2
 };
+// Whether the barrier's running count of arrivals has reached `target`.  Both wrap
+// after 2^32 (1.8 million iterations of 2,432 CTAs); they are never half of that apart.
+__host__ __device__ inline bool sg_arrived(uint32_t arrived, uint32_t target) {
+  return (int32_t)(arrived - target) >= 0;
+}
 constexpr int kSgThreads = 64;
 constexpr uint32_t kSgList = 1024;            // vertices of 8 pieces
 constexpr uint32_t kSgMaxVertices = 131072;   // 32 mask words

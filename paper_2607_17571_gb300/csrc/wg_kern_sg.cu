@@ -71,7 +71,7 @@ __device__ __forceinline__ bool sg_barrier(SgCtl* c, uint32_t target) {
     __threadfence();
     atomicAdd(&c->arrived, 1u);
     uint32_t spins = 0, ok = 1;
-    while (*(volatile uint32_t*)&c->arrived < target) {
+    while (!sg_arrived(*(volatile uint32_t*)&c->arrived, target)) {
       if (++spins > kSgSpinLimit || *(volatile uint32_t*)&c->error) {
         atomicExch(&c->error, DEV_TIMEOUT);
         ok = 0;

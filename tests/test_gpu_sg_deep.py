@@ -61,3 +61,23 @@ def test_single(p, q):
             _same(h, want, 1 << 16)
             h.free()
             rel.free()
+
+
+def test_iterations_past_2_to_32_arrivals():
+    # every row listed at the start: a full grid of CTAs meets at each of 1,770,230
+    # barriers.  Coprime cycles: each vertex of one with each of the other, two new
+    # tuples an iteration
+    from paper_2607_17571_gb300 import wg
+    p, q = 1330, 1331
+    with wg.Context(0) as c:
+        rel = c.load(*_cycles(p, q))
+        h = c.sg(rel, max_iters=1 << 22)
+        h.wait()
+        st = h.poll()
+        assert (st.n_tuples, st.iterations) == (2 * p * q, p * q)
+        assert h.delta_sizes() == [2] * (1 << 16)
+        a, b = np.arange(p, dtype=np.uint64), np.arange(q, dtype=np.uint64) + np.uint64(10_000)
+        ab = (a[:, None] << np.uint64(32) | b).ravel()
+        ba = (b[:, None] << np.uint64(32) | a).ravel()
+        assert np.array_equal(h.result(), np.concatenate([ab, ba]))
+        h.free()
