@@ -298,9 +298,10 @@ struct SgInst {
   uint32_t* fm;                 // valid pieces of the relation's rows (RowInst::bits)
   uint32_t* dm[2];              // ... and of the delta rows
   uint32_t* act;                // iteration a row was last listed for
+  uint32_t* done;               // slices of a row that have read its delta
   uint32_t mw, pad;
 };
-struct SgCtl {                  // cleared before the launch, with fm, dm and act
+struct SgCtl {                  // cleared before the launch, with fm, dm, act and done
   uint32_t arrived, error;
   uint32_t next[3], count[3];   // items claimed / listed, by iteration mod 3
 };
@@ -308,8 +309,15 @@ struct SgJob {
   RowJob rows;
   SgCtl* ctl;
   SgInst* sg;
-  uint32_t* list[2];            // rows with a non-empty delta, by iteration mod 2
+  uint2* list[2];               // rows with a non-empty delta and their slices, by iteration mod 2
 };
+// Children of one item: a row of more is several items, so that a hub's work is
+// spread over the chip (see k_sg).
+constexpr uint32_t kSgSlice = 256;
+// Items of an iteration at most.
+__host__ __device__ inline unsigned long long sg_items(unsigned long long rows, unsigned long long ne) {
+  return rows + ne / kSgSlice;
+}
 // Whether the barrier's running count of arrivals has reached `target`.  Both wrap
 // after 2^32 (1.8 million iterations of 2,432 CTAs); they are never half of that apart.
 __host__ __device__ inline bool sg_arrived(uint32_t arrived, uint32_t target) {

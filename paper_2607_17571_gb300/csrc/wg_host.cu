@@ -469,7 +469,7 @@ struct Relation {
   bool small_rows() const { return nv > 65536u; }
   bool no_rows = false;           // the rows' bit sets did not fit the budget
   // Same-generation rows (wg_kern_sg.cu): mask words of a row, and bytes beside
-  // the bit sets: two deltas as large, three masks, iteration marks, row lists.
+  // the bit sets: two deltas as large, three masks, marks, row lists.
   uint32_t sg_mask_words() const { return (row_words() / 4 + 31) / 32; }
   size_t sg_masks() const { return (size_t)nv * sg_mask_words() * 4; }
   void row_inst(RowInst* I) const {
@@ -1097,12 +1097,14 @@ struct Engine : EngineBase {
     const size_t o_ctl = at(end, sizeof(RowCtl) + sizeof(SgCtl)), o_sum = at(end, (size_t)nch * 4),
                  o_log = at(end, (size_t)nlog * 8), masks = row_sg ? Rl->sg_masks() : 0,
                  o_fm = at(end, masks), o_dm0 = at(end, masks), o_dm1 = at(end, masks),
-                 o_act = at(end, row_sg ? (size_t)nv * 4 : 0);
+                 o_act = at(end, row_sg ? (size_t)nv * 4 : 0),
+                 o_done = at(end, row_sg ? (size_t)nv * 4 : 0);
     row_clear = end;
     const size_t o_inst = at(end, sizeof(RowInst)), o_sgi = at(end, sizeof(SgInst)),
                  o_base = at(end, (size_t)nch * 8), o_cnt = at(end, (size_t)nv * 4),
-                 o_rows = at(end, small || row_sg ? (size_t)nv * 4 : 0),
-                 o_rows1 = at(end, row_sg ? (size_t)nv * 4 : 0);
+                 items = row_sg ? sg_items(nv, Rl->ne) * sizeof(uint2) : 0,
+                 o_rows = at(end, row_sg ? items : small ? (size_t)nv * 4 : 0),
+                 o_rows1 = at(end, items);
     TRY(row_meta.get(c, end));
     // bit sets of every row, or (small rows apart) of as many as a quarter of
     // the free budget holds: more are made room for when they turn up (settle)
@@ -1139,7 +1141,7 @@ struct Engine : EngineBase {
       sgi.d[1] = (uint4*)((char*)row_bits.p + 2 * Rl->row_bits());
       sgi.fm = (uint32_t*)(m + o_fm);
       sgi.dm[0] = (uint32_t*)(m + o_dm0); sgi.dm[1] = (uint32_t*)(m + o_dm1);
-      sgi.act = (uint32_t*)(m + o_act);
+      sgi.act = (uint32_t*)(m + o_act); sgi.done = (uint32_t*)(m + o_done);
       sgi.mw = Rl->sg_mask_words();
       job.sg = (SgInst*)(m + o_sgi);
       job.sg_ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
@@ -1147,7 +1149,7 @@ struct Engine : EngineBase {
       sg.rows = job;
       sg.ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
       sg.sg = (SgInst*)(m + o_sgi);
-      sg.list[0] = (uint32_t*)(m + o_rows); sg.list[1] = (uint32_t*)(m + o_rows1);
+      sg.list[0] = (uint2*)(m + o_rows); sg.list[1] = (uint2*)(m + o_rows1);
     }
     log_cap = nlog;
     expand_only = false;
@@ -2372,7 +2374,7 @@ static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
   size_t idle = lanes_busy(c) ? 0 : lanes_held(c);
   for (auto& e : c->idle) idle += e->held();
   // (small rows apart: their lists, and bit sets for whatever is left)
-  const size_t need = q->kind == WG_SG ? 3 * (R->row_bits() + R->sg_masks()) + (size_t)R->nv * 16
+  const size_t need = q->kind == WG_SG ? 3 * (R->row_bits() + R->sg_masks()) + sg_items(R->nv, R->ne) * 24
                       : R->small_rows() && !batched ? (size_t)R->nv * kSmallRow * 8
                                                     : R->row_bits();
   const size_t room = c->budget - std::min(c->budget, c->used) + idle;
@@ -2464,8 +2466,9 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   const uint32_t nv_max = qs[by[0]]->rel->nv, vwords = qs[by[0]]->rel->row_words();
   const int idb = qs[0]->rel->id_bytes();
   uint32_t nch = 0;
-  size_t bits = 0, masks = 0;
+  size_t bits = 0, masks = 0, slices = 0;  // (slices: of the rows past their first)
   for (Query* q : qs) {
+    slices += sg_items(0, q->rel->ne);
     nch += (q->rel->nv + kRowChunk - 1) / kRowChunk;
     bits += q->rel->row_bits();
     masks += q->rel->sg_masks();
@@ -2480,6 +2483,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
   if (!L->sg) masks = 0;
   const size_t o_sum = at(end, (size_t)nch * 4), o_fm = at(end, masks), o_dm0 = at(end, masks),
                o_dm1 = at(end, masks), o_act = at(end, L->sg ? rows4 : 0),
+               o_done = at(end, L->sg ? rows4 : 0),
                o_ctl = at(end, sizeof(RowCtl) + sizeof(SgCtl));
   L->o_ctl = o_ctl;
   L->o_log = at(end, (size_t)L->n * L->log_cap * 8);
@@ -2489,7 +2493,8 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
                o_sgi = at(end, L->sg ? (size_t)L->n * sizeof(SgInst) : 0);
   L->up_end = end;
   const size_t o_base = at(end, (size_t)nch * 8), o_cnt = at(end, rows4),
-               o_l0 = at(end, L->sg ? rows4 : 0), o_l1 = at(end, L->sg ? rows4 : 0);
+               items = L->sg ? sg_items(rows4 / 4, 0) * sizeof(uint2) + slices * sizeof(uint2) : 0,
+               o_l0 = at(end, items), o_l1 = at(end, items);
   L->phase = 1;  // (its buffers are not to be dropped while it allocates)
   int rc = L->meta.get(c, end);
   if (rc == WG_OK) rc = L->bits.get(c, L->sg ? 3 * bits : bits);
@@ -2529,7 +2534,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
       g.d[1] = (uint4*)((char*)I.bits + 2 * bits);
       g.fm = (uint32_t*)(m + o_fm + mat);
       g.dm[0] = (uint32_t*)(m + o_dm0 + mat); g.dm[1] = (uint32_t*)(m + o_dm1 + mat);
-      g.act = (uint32_t*)(m + o_act) + I.row0;
+      g.act = (uint32_t*)(m + o_act) + I.row0; g.done = (uint32_t*)(m + o_done) + I.row0;
       g.mw = R->sg_mask_words();
       mat += R->sg_masks();
       hs[k] = g;
@@ -2552,7 +2557,7 @@ static int lane_start(wg_ctx* c, RowLane* L, const std::vector<uint64_t>& ids) {
     S.rows = J;
     S.ctl = (SgCtl*)(m + o_ctl + sizeof(RowCtl));
     S.sg = (SgInst*)(m + o_sgi);
-    S.list[0] = (uint32_t*)(m + o_l0); S.list[1] = (uint32_t*)(m + o_l1);
+    S.list[0] = (uint2*)(m + o_l0); S.list[1] = (uint2*)(m + o_l1);
     CK(launch_sg(S, idb, grid, c->num_sms, L->st));
   } else {
     launch_rows(J, idb, grid, L->st);

@@ -18,6 +18,13 @@
 // atomics.  One cooperative launch runs every iteration of all its instances,
 // a barrier over the grid between two.
 //
+// A row of more than kSgSlice children is several items, each with its own S_a: with
+// one item per row a hub's children (|S_a| / 128 pieces each) were one CTA's work
+// while the grid waited, at the barrier's limit even a timeout.  Stars of 4,000 /
+// 10,000 / 40,000 children, whole call: one item 1.45 / 9.7 / 154 ms (sorted-array
+// pipeline 0.94 / 5.0 / 73), slices of 1,024 0.49 / 1.24 / 5.5, of 512 0.29 / 0.73 / 3.6,
+// of 256 0.20 / 0.47 / 2.6; R-MAT 2^12 / 9,000 0.82, 0.80, 0.80, 0.70.
+//
 // Bound by the latency of an item's steps (delta pieces, records, row pieces) and
 // the barriers between them (ncu: 24% of the issue slots, DRAM 1%), so CTAs are
 // small: 256 / 128 / 64 / 32 threads 1.71 / 1.05 / 0.86 / 0.88 ms on the forest of
@@ -33,11 +40,16 @@ __device__ __forceinline__ uint32_t popc4(const uint4& v) {
   return __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
 }
 __device__ __forceinline__ bool any4(const uint4& v) { return (v.x | v.y | v.z | v.w) != 0; }
+__device__ __forceinline__ uint32_t sg_slices(uint32_t deg) {
+  return (deg + kSgSlice - 1) / kSgSlice;
+}
+constexpr uint32_t kNone = 0xFFFFFFFFu;
 __device__ __forceinline__ bool bit_of(const uint32_t* s, uint32_t i) {
   return s[i >> 5] >> (i & 31) & 1u;
 }
 
-// Clears the rows of vertices with several parents (their pieces are all valid).
+// Clears the rows of vertices with several parents (their pieces are all valid), and
+// lists the slices of every row past its first for iteration 0, which takes all rows.
 __global__ void __launch_bounds__(kThreads) k_sg_init(SgJob J) {
   const uint32_t lane = threadIdx.x & 31;
   for (uint32_t r = (blockIdx.x * kThreads + threadIdx.x) / 32; r < J.rows.nrows;
@@ -45,7 +57,15 @@ __global__ void __launch_bounds__(kThreads) k_sg_init(SgJob J) {
     const uint32_t q = J.rows.chunk_inst ? J.rows.chunk_inst[r / kRowChunk] : 0u;
     const RowInst& I = J.rows.inst[q];
     const uint32_t x = r - I.row0;
-    if (x >= I.nv || !bit_of(I.mp, x)) continue;
+    if (x >= I.nv) continue;
+    const uint32_t more = sg_slices(I.off[x + 1] - I.off[x]) - 1;
+    if (more != 0 && more != kNone) {
+      uint32_t at = 0;
+      if (lane == 0) at = atomicAdd(&J.ctl->count[0], more);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      for (uint32_t i = lane; i < more; i += 32) J.list[0][at + i] = uint2{r, i + 1};
+    }
+    if (!bit_of(I.mp, x)) continue;
     const SgInst& G = J.sg[q];
     const uint32_t quads = I.words / 4;
     const size_t at = (size_t)x * quads;
@@ -86,16 +106,14 @@ __device__ __forceinline__ bool sg_barrier(SgCtl* c, uint32_t target) {
   return s_ok != 0;
 }
 
-constexpr uint32_t kSgKids = 1024;  // children whose listing goes through shared memory
-
 template <typename IdT>
 __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
   constexpr uint32_t kW = kSgThreads / 32;
   extern __shared__ uint4 S4[];
   __shared__ RowInst I;
   __shared__ SgInst G;
-  __shared__ uint32_t s_row[2], s_nq, s_nz, s_kids[kSgKids / 32];  // children with new tuples
-  constexpr uint32_t kNone = 0xFFFFFFFFu;
+  __shared__ uint2 s_item[2];                                // {row, slice of its children}
+  __shared__ uint32_t s_nq, s_nz, s_last, s_kids[kSgSlice / 32];  // children with new tuples
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* S = (uint32_t*)S4;
   uint32_t* strip = S + J.rows.vwords + warp * 32;
@@ -104,7 +122,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
   IdT* list = (IdT*)(vql + J.rows.vwords / 4) + warp * kSgList;
   for (uint32_t i = tid; i < J.rows.vwords / 4; i += kSgThreads) S4[i] = uint4{0, 0, 0, 0};
   if (tid == 0) s_nz = 0;
-  if (tid < kSgKids / 32) s_kids[tid] = 0;
+  if (tid < kSgSlice / 32) s_kids[tid] = 0;
   unsigned long long cand = 0, got = 0;
   uint32_t cur = 0xFFFFFFFFu;
   SgCtl* ctl = J.ctl;
@@ -124,21 +142,22 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
       cand = got = 0;
     };
     const uint32_t in = k & 1, out = in ^ 1u;
-    const uint32_t n = k == 0 ? J.rows.nrows : __ldcg(&ctl->count[k % 3]);
+    const uint32_t first = k == 0 ? J.rows.nrows : 0u;  // (all rows, before what is listed)
+    const uint32_t n = first + __ldcg(&ctl->count[k % 3]);
     uint32_t* const next_n = &ctl->count[(k + 1) % 3];
     if (blockIdx.x == 0 && tid == 0) {  // (the slots no CTA uses in this iteration)
       ctl->count[(k + 2) % 3] = 0;
       ctl->next[(k + 2) % 3] = 0;
     }
-    const uint32_t* const listed = in ? J.list[1] : J.list[0];
-    uint32_t* const to_list = in ? J.list[0] : J.list[1];
-    auto row_of = [&](uint32_t i) {
-      return i >= n ? kNone : k == 0 ? i : __ldcg(listed + i);
+    const uint2* const listed = in ? J.list[1] : J.list[0];
+    uint2* const to_list = in ? J.list[0] : J.list[1];
+    auto item_of = [&](uint32_t i) {
+      return i >= n ? uint2{kNone, 0} : i < first ? uint2{i, 0} : __ldcg(listed + (i - first));
     };
-    if (tid == 0) s_row[0] = row_of(atomicAdd(&ctl->next[k % 3], 1u));
+    if (tid == 0) s_item[0] = item_of(atomicAdd(&ctl->next[k % 3], 1u));
     __syncthreads();
     for (uint32_t p = 0;; p ^= 1) {
-      const uint32_t row = s_row[p];
+      const uint32_t row = s_item[p].x, c0 = s_item[p].y * kSgSlice;
       if (row == kNone) break;
       const uint32_t q = J.rows.chunk_inst ? J.rows.chunk_inst[row / kRowChunk] : 0u;
       if (q != cur) {
@@ -158,22 +177,23 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
         deg = I.off[a + 1] - o;
       }
       if (deg == 0) {
-        if (tid == 0) s_row[p ^ 1] = row_of(next);
+        if (tid == 0) s_item[p ^ 1] = item_of(next);
         __syncthreads();
         continue;
       }
       const uint32_t* adj = I.adj + o;
+      const uint32_t kids = min(deg - c0, kSgSlice), slices = sg_slices(deg);
       if (k == 0) {
         for (uint32_t i = tid; i < deg; i += kSgThreads) {
           const uint32_t z = adj[i];
           atomicOr(S + (z >> 5), 1u << (z & 31));
         }
-        if (tid == 0) cand += (unsigned long long)deg * (deg - 1);
+        if (tid == 0) cand += (unsigned long long)kids * (deg - 1);
       } else {
         if (warp == 0) {  // valid pieces of the delta row (at most 32 mask words)
           uint32_t m = 0;
           uint32_t* dm = G.dm[in] + (size_t)a * G.mw + lane;
-          if (lane < G.mw && (m = __ldcg(dm)) != 0) *dm = 0;
+          if (lane < G.mw && (m = __ldcg(dm)) != 0 && slices == 1) *dm = 0;
           const uint32_t valid = list_pieces(m, vql);
           if (lane == 0) s_nq = valid;
         }
@@ -188,7 +208,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
             w = vql[g + lane];
             uint4* p = G.d[in] + (size_t)a * quads + w;
             v = __ldcg(p);
-            if (many) *p = uint4{0, 0, 0, 0};
+            if (many && slices == 1) *p = uint4{0, 0, 0, 0};
             const uint4 ns = __ldg((const uint4*)I.ns + w);
             v.x &= ns.x; v.y &= ns.y; v.z &= ns.z; v.w &= ns.w;
           }
@@ -203,7 +223,21 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
           dsum += expand_vertices<IdT, true>(I, list, 0, len, 32, S, strip);
           __syncwarp();
         }
-        cand += (unsigned long long)dsum * deg;
+        cand += (unsigned long long)dsum * kids;
+        if (slices > 1) {  // the last of the row's items to have read the delta clears it
+          __syncthreads();
+          if (tid == 0) {
+            __threadfence();
+            s_last = atomicAdd(G.done + a, 1u) == slices - 1;
+            if (s_last) G.done[a] = 0;
+          }
+          __syncthreads();
+          if (s_last) {
+            for (uint32_t i = tid; i < G.mw; i += kSgThreads) G.dm[in][(size_t)a * G.mw + i] = 0;
+            for (uint32_t i = tid; many && i < nq; i += kSgThreads)
+              G.d[in][(size_t)a * quads + vql[i]] = uint4{0, 0, 0, 0};
+          }
+        }
       }
       __syncthreads();
       for (uint32_t w0 = warp * 32; w0 < quads; w0 += kSgThreads) {
@@ -218,9 +252,10 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
       }
       __syncthreads();
       const uint32_t nz = s_nz, more = k < I.max_iters ? 1u : 0u;
-      if (tid == 0) next = row_of(next);
-      for (uint32_t i = tid; i < nz * deg; i += kSgThreads) {
-        const uint32_t c = i / nz, w = nzl[i - c * nz], x = __ldg(adj + c);
+      uint2 item;
+      if (tid == 0) item = item_of(next);
+      for (uint32_t i = tid; i < nz * kids; i += kSgThreads) {
+        const uint32_t c = i / nz, w = nzl[i - c * nz], x = __ldg(adj + c0 + c);
         uint4 s = S4[w];
         if (k == 0 && w == x >> 7) {  // (x, x) is not in the base
           const uint32_t keep = ~(1u << (x & 31)), p = x >> 5 & 3;
@@ -261,24 +296,24 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
         got += popc4(d);
         if (on) {
           atomicOr(G.dm[out] + mat, bit);
-          if (c < kSgKids) atomicOr(s_kids + (c >> 5), 1u << (c & 31));
-          else if (__ldcg(G.act + x) != k + 1 && atomicExch(G.act + x, k + 1) != k + 1)
-            to_list[atomicAdd(next_n, 1u)] = I.row0 + x;
+          atomicOr(s_kids + (c >> 5), 1u << (c & 31));
         }
       }
       __syncthreads();
       // list the children with new tuples: a child of one parent only here, so
       // without asking; one of several once per iteration
-      for (uint32_t c = tid; c < min(deg, kSgKids); c += kSgThreads) {
+      for (uint32_t c = tid; c < kids; c += kSgThreads) {
         if (!(s_kids[c >> 5] >> (c & 31) & 1u)) continue;
-        const uint32_t x = __ldg(adj + c);
-        if (!bit_of(I.mp, x) || atomicExch(G.act + x, k + 1) != k + 1)
-          to_list[atomicAdd(next_n, 1u)] = I.row0 + x;
+        const uint32_t x = __ldg(adj + c0 + c), b = __ldg(I.off + x), e = __ldg(I.off + x + 1);
+        if (bit_of(I.mp, x) && atomicExch(G.act + x, k + 1) == k + 1) continue;
+        const uint32_t s = sg_slices(e - b);
+        uint2* to = to_list + atomicAdd(next_n, s);
+        for (uint32_t i = 0; i < s; ++i) to[i] = uint2{I.row0 + x, i};
       }
       for (uint32_t i = tid; i < nz; i += kSgThreads) S4[nzl[i]] = uint4{0, 0, 0, 0};
-      if (tid == 0) { s_nz = 0; s_row[p ^ 1] = next; }
+      if (tid == 0) { s_nz = 0; s_item[p ^ 1] = item; }
       __syncthreads();  // (every read of s_kids is done)
-      if (tid < kSgKids / 32) s_kids[tid] = 0;
+      if (tid < kSgSlice / 32) s_kids[tid] = 0;
     }
     if (cur != 0xFFFFFFFFu) flush();
     if (!sg_barrier(ctl, (k + 1) * gridDim.x)) return;
