@@ -808,9 +808,10 @@ struct Engine : EngineBase {
   SgJob sg{};
   SgInst sgi{};
   RowReport* report = nullptr;       // page-locked: what a run found, written by k_row_plan
-  size_t row_clear = 0;              // leading bytes of row_meta cleared before a launch
+  size_t row_clear = 0, row_ctl = 0; // leading bytes of row_meta cleared before a run; and a resumed one
   int id_bytes = 2, g_rows = 0;
   bool expand_only = false;          // the rows are done; the result waits for a larger buffer
+  bool resume = false;               // the small rows are done; the long ones waited for bit sets
   bool row_short = false;            // the long rows' bit sets did not fit the budget
   Engine(wg_ctx* ctx, bool single_, uint32_t n, uint32_t bits, uint32_t logcap, bool fuse_,
          bool xseg_, bool copy_back_ = false, bool hash_join_ = false, uint32_t side = 0)
@@ -1100,19 +1101,21 @@ struct Engine : EngineBase {
                  o_act = at(end, row_sg ? (size_t)nv * 4 : 0),
                  o_done = at(end, row_sg ? (size_t)nv * 4 : 0);
     row_clear = end;
+    row_ctl = o_sum;
     const size_t o_inst = at(end, sizeof(RowInst)), o_sgi = at(end, sizeof(SgInst)),
                  o_base = at(end, (size_t)nch * 8), o_cnt = at(end, (size_t)nv * 4),
                  items = row_sg ? sg_items(nv, Rl->ne) * sizeof(uint2) : 0,
                  o_rows = at(end, row_sg ? items : small ? (size_t)nv * 4 : 0),
                  o_rows1 = at(end, items);
     TRY(row_meta.get(c, end));
-    // bit sets of every row, or (small rows apart) of as many as a quarter of
-    // the free budget holds: more are made room for when they turn up (settle)
+    // bit sets of every row, or (small rows apart) what the engine has: once the long
+    // rows are counted, settle makes room for exactly them.  (A sparse relation has
+    // few: ER 400,000 / 360,000 0.5 GB in place of the 14 GB that all rows would take,
+    // for a result of 24 MB.)
     size_t sets = std::max<size_t>(Rl->row_bits(), 16);
     if (small) {
       TRY(row_small.get(c, (size_t)nv * kSmallRow * 4));
-      const size_t room = (c->budget - std::min(c->budget, c->used) + row_bits.bytes) / 4;
-      sets = std::max(std::min(sets, room), (size_t)words * 4);
+      sets = (size_t)words * 4;
     }
     if (row_sg) sets = 3 * std::max<size_t>(Rl->row_bits(), 16);
     TRY(row_bits.get(c, sets));
@@ -1152,13 +1155,13 @@ struct Engine : EngineBase {
       sg.list[0] = (uint2*)(m + o_rows); sg.list[1] = (uint2*)(m + o_rows1);
     }
     log_cap = nlog;
-    expand_only = false;
+    expand_only = resume = row_short = false;
     hi[0] = Inst{};
     hi[0].state = INST_ACTIVE;
     hi[0].log = ri.log;
     return WG_OK;
   }
-  // Room for the bit sets of the long rows the last run found.
+  // Room for the bit sets of the long rows that k_rows_small left.
   int rows_room() {
     AllocScope scope(c, st);
     const size_t set = (size_t)ri.words * 4;
@@ -1168,19 +1171,19 @@ struct Engine : EngineBase {
     row_short = false;
     ri.bits = (uint32_t*)row_bits.p;
     job.slots = (uint32_t)std::min<size_t>(ri.nv, row_bits.bytes / set);
-    ri.n_big = 0; ri.last = 0; ri.cand = 0;
     return WG_OK;
   }
   int rows_launch() {
     ri.out = F[0].p;
     ri.out_cap = capF;
     if (expand_only) ri.fits = 1;
-    launch_row_begin(job, ri, sgi, row_meta.p, expand_only ? 0 : row_clear, c->num_sms, st);
+    launch_row_begin(job, ri, sgi, row_meta.p, expand_only ? 0 : resume ? row_ctl : row_clear,
+                     c->num_sms, st);
     launches_issued += 1;
     if (!expand_only) {
-      if (job.rows) {
+      if (job.rows && !resume) {
         launch_rows_small(job, grid_of(c, 6), st);
-        launches_issued += 2;  // (and k_row_expand_small)
+        launches_issued += 1;
       }
       if (row_sg) {
         CK(launch_sg(sg, id_bytes, g_rows, c->num_sms, st));
@@ -1193,7 +1196,7 @@ struct Engine : EngineBase {
       launches_issued += 1;
     }
     launch_row_expand<K>(job, grid_of(c, 6), st);
-    launches_issued += 1;
+    launches_issued += job.rows ? 2 : 1;
     CK(cudaGetLastError());
     CK(cudaEventRecord(ev_done, st));
     in_flight = true;
@@ -1212,9 +1215,10 @@ struct Engine : EngineBase {
     Inst& I = hi[0];
     I.n_full = ri.n_total;
     I.cand_total = ri.cand;
-    if (job.rows && ri.n_big > job.slots) {  // more long rows than bit sets: start over
+    if (job.rows && ri.n_big > job.slots) {  // more long rows than bit sets: k_rows did nothing
       ++regrows;
       *again = true;
+      resume = true;
       return rows_room();
     }
     if (!ri.fits) {
