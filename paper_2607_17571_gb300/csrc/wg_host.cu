@@ -467,7 +467,6 @@ struct Relation {
   // with 32-bit ranks, where a row's bit set takes 8 KB and more (sparse ER
   // 400,000 / 360,000: 15.5 -> 1.1 ms; dense R-MAT 2^19 / 400k: no change).
   bool small_rows() const { return nv > 65536u; }
-  bool no_rows = false;           // the rows' bit sets did not fit the budget
   // Same-generation rows (wg_kern_sg.cu): mask words of a row, and bytes beside
   // the bit sets: two deltas as large, three masks, marks, row lists.
   uint32_t sg_mask_words() const { return (row_words() / 4 + 31) / 32; }
@@ -743,6 +742,7 @@ struct Query {
   uint32_t slot = 0;
   bool rowb = false;             // batched row by row (see RowLane); bclass is -1
   bool row_alone = false;        // ... once its result did not fit beside others
+  bool no_rows = false;          // its rows' bit sets did not fit the budget
   // served through a single-query engine (a large request, see solo_round)
   bool solo = false;
   bool solo_wait = false;        // paused after a growth over the budget
@@ -1795,7 +1795,7 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->row_short) {
       // the long rows' bit sets do not fit: the sorted-array pipeline takes it
       cudaGetLastError();
-      q->rel->no_rows = true;
+      q->no_rows = true;
       q->own.reset();
       q->eng = nullptr;
       rc = single_begin(c, q);
@@ -2388,7 +2388,7 @@ static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
   return row_layout(c, R, false) == WG_OK && R->rowv.p && cudaStreamSynchronize(c->stream) == cudaSuccess;
 }
 static bool row_query(wg_ctx* c, const Query* q) {
-  return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->rel->no_rows &&
+  return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->no_rows &&
          row_fits(c, q, false);
 }
 // (loop and profile are ignored in batches)

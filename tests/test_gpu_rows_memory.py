@@ -30,3 +30,39 @@ def test_bit_sets_of_the_long_rows_only(nodes, edges):
                     max(4 * edges, 2 * want.keys.shape[0]) * 8 + (8 << 20))
             assert c.mem_used() - before <= most
             q.free()
+
+
+def _long_rows(rows):
+    """`rows` rows of 261 tuples over 400,000 vertices."""
+    i, hubs = np.arange(rows), np.arange(30_000, 30_010)
+    src = np.concatenate([np.arange(0, 400_000, 2), i, np.repeat(hubs, 260)]).astype(np.uint32)
+    dst = np.concatenate([np.arange(1, 400_001, 2), 30_000 + i % 10,
+                          np.tile(np.arange(50_000, 50_260), 10)]).astype(np.uint32)
+    return src, dst
+
+
+def test_a_passing_shortage_marks_no_relation():
+    # 26,000 bit sets take 1.4 GB beside 0.4 GB of lists: too much while another
+    # query's result (0.5 GB) is held, and room enough once it is freed
+    from oracle import oracle_tc_reach
+    from paper_2607_17571_gb300 import wg
+    src, dst = _long_rows(26_000)
+    n, iters, log, dg = oracle_tc_reach(src, dst, n_threads=8)
+    g = I.er_graph(12_000, 36_000, 3)
+    with wg.Context(0, mem_budget=2250 << 20, torch_memory=False) as c:
+        rel, other = c.load(src, dst), c.load(g.src, g.dst)
+
+        def launches():
+            q = c.tc(rel)
+            st = q.wait()
+            assert (st.n_tuples, st.iterations, q.digest()) == (n, iters, dg)
+            k = st.gpu_launches
+            q.free()
+            return k
+
+        held = c.tc(other)
+        held.wait()
+        assert launches() > 20   # the sorted-array pipeline: some ten kernels an iteration
+        held.free()
+        other.free()
+        assert launches() < 20   # rows again
