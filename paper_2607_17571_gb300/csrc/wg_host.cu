@@ -1777,6 +1777,14 @@ static int single_start(wg_ctx* c, Query* q) {
 extern "C" {
 static int single_begin(wg_ctx* c, Query* q);
 }
+// Query q's rows do not fit the memory there is: start it over on the pipeline.
+static int rows_to_pipeline(wg_ctx* c, Query* q) {
+  q->no_rows = true;
+  q->own.reset();
+  q->eng = nullptr;
+  return single_begin(c, q);
+}
+
 template <typename K>
 static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget = false) {
   auto* E = static_cast<Engine<K>*>(q->eng);
@@ -1792,17 +1800,12 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     }
     bool again = false;
     int rc = E->settle(&again);
-    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->row_short) {
-      // the long rows' bit sets do not fit: the sorted-array pipeline takes it
+    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->job.rows) {
+      // the long rows' bit sets, or the result beside them, do not fit: the
+      // sorted-array pipeline, which has no such scratch, takes it
       cudaGetLastError();
-      q->no_rows = true;
-      q->own.reset();
-      q->eng = nullptr;
-      rc = single_begin(c, q);
+      rc = rows_to_pipeline(c, q);
       if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
-      q->state = WG_FAILED;
-      q->error = rc;
-      return rc;
     }
     if (rc != WG_OK && pause_on_budget && (rc == WG_E_BUDGET || rc == WG_E_NOMEM)) {
       cudaGetLastError();  // the pools stay whole at their old capacities

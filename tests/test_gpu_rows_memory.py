@@ -66,3 +66,17 @@ def test_a_passing_shortage_marks_no_relation():
         held.free()
         other.free()
         assert launches() < 20   # rows again
+
+
+@pytest.mark.parametrize("budget_mb", range(1730, 1830, 10))
+def test_result_that_does_not_fit_beside_the_bit_sets(budget_mb):
+    # lists and bit sets take some 1,743 MB, the result 50 MB more
+    from oracle import oracle_tc_reach
+    from paper_2607_17571_gb300 import wg
+    src, dst = _long_rows(26_000)
+    n, iters, log, dg = oracle_tc_reach(src, dst, n_threads=8)
+    with wg.Context(0, mem_budget=budget_mb << 20, torch_memory=False) as c:
+        q = c.tc(c.load(src, dst))
+        st = q.wait()
+        assert (st.n_tuples, st.iterations, q.digest()) == (n, iters, dg)
+        assert q.delta_sizes() == list(log)
