@@ -3166,7 +3166,7 @@ static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
       return WG_OK;  // the request failed; the server carries on
     }
     cudaGetLastError();
-    bool held = false;
+    bool held = lanes_busy(c);
     for (auto& kv : c->batch) held |= kv.second != nullptr;
     if (held && (!x || x == q)) {  // wait for the whole budget
       solo_requeue(c, q);
