@@ -1162,12 +1162,15 @@ struct Engine : EngineBase {
     return WG_OK;
   }
   // Room for the bit sets of the long rows that k_rows_small left.
+  size_t row_sets() const {
+    return std::min((size_t)ri.n_big + ri.n_big / 16 + 64, (size_t)ri.nv) * ri.words * 4;
+  }
   int rows_room() {
     AllocScope scope(c, st);
     const size_t set = (size_t)ri.words * 4;
     row_bits.release(c);
     row_short = true;
-    TRY(row_bits.get(c, std::min((size_t)ri.n_big + ri.n_big / 16 + 64, (size_t)ri.nv) * set));
+    TRY(row_bits.get(c, row_sets()));
     row_short = false;
     ri.bits = (uint32_t*)row_bits.p;
     job.slots = (uint32_t)std::min<size_t>(ri.nv, row_bits.bytes / set);
@@ -1548,7 +1551,7 @@ struct Engine : EngineBase {
   size_t grow_peak() const override {
     unsigned long long wantC, wantF, wantR;
     grow_target(&wantC, &wantF, &wantR);
-    if (rows_ && row_short) return held() + ((size_t)ri.n_big + 64) * ri.words * 4;
+    if (rows_ && row_short) return held() + row_sets();
     if (rows_)
       return held() - F[0].bytes + round_up((h.ctl.need_full + h.ctl.need_full / 16 + 4096) * sizeof(K));
     wantC = std::max<unsigned long long>(wantC, 1ull << 16);
@@ -1800,9 +1803,10 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     }
     bool again = false;
     int rc = E->settle(&again);
-    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->job.rows) {
+    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->job.rows && !pause_on_budget) {
       // the long rows' bit sets, or the result beside them, do not fit: the
-      // sorted-array pipeline, which has no such scratch, takes it
+      // sorted-array pipeline, which has no such scratch, takes it (a served
+      // request waits for memory first, see solo_pipeline)
       cudaGetLastError();
       rc = rows_to_pipeline(c, q);
       if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
@@ -3089,6 +3093,29 @@ static void solo_finish(wg_ctx* c, Query* q, int rc) {
   if (c->solo_run == q->id) c->solo_run = 0;
 }
 
+// Request q on a single-query engine paused for memory that it does not get: it
+// fails, except that one whose wide rows do not fit goes on to the sorted-array
+// pipeline -- queued again, as the exclusive query, while others hold memory the
+// pipeline needs for its start.
+static void solo_give_up(wg_ctx* c, Query* q, int why, bool others) {
+  const bool k4 = q->eng->kb() == 4;
+  if (!q->eng->rows() || !(k4 ? static_cast<Engine<uint32_t>*>(q->eng)->job.rows
+                              : static_cast<Engine<unsigned long long>*>(q->eng)->job.rows)) {
+    solo_finish(c, q, why);
+    return;
+  }
+  q->solo_wait = false;
+  const int rc = rows_to_pipeline(c, q);
+  if (rc == WG_OK) return;  // (running)
+  if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) cudaGetLastError();
+  if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && others) {
+    solo_requeue(c, q);
+    c->excl = q->id;
+  } else {
+    solo_finish(c, q, rc);
+  }
+}
+
 static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
   *busy = false;
   if (c->solo_run && !solo_running(c)) c->solo_run = 0;  // freed while running
@@ -3111,7 +3138,7 @@ static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
         bool held = lanes_busy(c);  // memory that may still come back
         for (auto& kv : c->batch) held |= kv.second != nullptr;
         if (!held) {
-          solo_finish(c, q, WG_E_BUDGET);
+          solo_give_up(c, q, WG_E_BUDGET, false);
           *progressed = true;
         }
         return WG_OK;
@@ -3119,13 +3146,15 @@ static int solo_round(wg_ctx* c, bool* progressed, bool* busy) {
     }
     const int rc = k4 ? single_progress<uint32_t>(c, q, false, true)
                       : single_progress<unsigned long long>(c, q, false, true);
+    Query* x = excl_query(c);
     if (q->solo_wait && !growth_could_fit(c, q->eng)) {  // hopeless: fail now
-      solo_finish(c, q, set_err(WG_E_BUDGET, "the request does not fit the memory budget"));
+      bool others = (!x || x == q) && lanes_busy(c);
+      for (auto& kv : c->batch) others |= (!x || x == q) && kv.second != nullptr;
+      solo_give_up(c, q, set_err(WG_E_BUDGET, "the request does not fit the memory budget"), others);
       *progressed = true;
       return WG_OK;
     }
     if (q->solo_wait) {  // paused: exclusive from now on, unless another query is
-      Query* x = excl_query(c);
       if (x && x != q) solo_requeue(c, q);
       else c->excl = q->id;
       *progressed = true;

@@ -38,3 +38,43 @@ def test_first_buffers_beside_running_lanes():
             h.wait()
             assert np.array_equal(h.result(), _closed(*e))
             h.free()
+
+
+def _long_rows(rows):
+    """`rows` rows of 261 tuples over 400,000 vertices."""
+    i, hubs = np.arange(rows), np.arange(30_000, 30_010)
+    src = np.concatenate([np.arange(0, 400_000, 2), i, np.repeat(hubs, 260)]).astype(np.uint32)
+    dst = np.concatenate([np.arange(1, 400_001, 2), 30_000 + i % 10,
+                          np.tile(np.arange(50_000, 50_260), 10)]).astype(np.uint32)
+    return src, dst
+
+
+@pytest.mark.parametrize("budget_mb,reserve_mb", [
+    (2600, 900),   # rows never fit (1.8 GB beside the reserve); the pipeline's start waits
+    (2600, 300),   # rows fit once the engine of the small request is gone
+    (2600, 20),    # ... with less to reserve
+    (2000, 20)])   # the relation's lists are over half of what is free: the pipeline
+def test_long_rows_beside_a_batch_engine(budget_mb, reserve_mb):
+    # a submitted query that asks for candidate buffers has a batch engine, whose
+    # pools take a third of the budget; bit sets of the large one's rows 1.4 GB
+    from oracle import oracle_tc_reach
+    from paper_2607_17571_gb300 import wg
+    src, dst = _long_rows(26_000)
+    n, iters, log, dg = oracle_tc_reach(src, dst, n_threads=8)
+    small = _pairs(5000)
+    with wg.Context(0, mem_budget=budget_mb * MB, torch_memory=False) as c:
+        a, b = c.load(*small), c.load(src, dst)
+        hs = c.submit([(wg.WG_TC, a, dict(reserve_cand=1)),
+                       (wg.WG_TC, b, dict(reserve_full=reserve_mb * MB // 8))])
+        _drain(c)
+        hs[0].wait()
+        assert np.array_equal(hs[0].result(), _closed(*small))
+        st = hs[1].wait()
+        assert (st.n_tuples, st.iterations, hs[1].digest()) == (n, iters, dg)
+        assert hs[1].delta_sizes() == list(log)
+        for h in hs:
+            h.free()
+        # and the context serves on
+        h, = c.submit([(wg.WG_TC, a)])
+        _drain(c)
+        assert np.array_equal(h.result(), _closed(*small))
