@@ -2268,9 +2268,10 @@ static int batch_round(wg_ctx* c, int cls, uint32_t iters, bool wait_launch, boo
 static int ensure_batch_engine(wg_ctx* c, int cls, Relation* R);
 
 // A dropped engine is built again for the requests of its class still queued
-// (not while another class's exclusive query waits for the memory).  If its
-// first pools do not fit although no other batch engine holds any, those
-// requests fail with the allocation's error.
+// (not while another class's exclusive query waits for the memory).  Engines that
+// hold no work make room for its first pools (left alone, one would keep the memory
+// for good, and a waiting caller would poll forever).  If they do not fit although
+// no other batch engine holds any, those requests fail with the allocation's error.
 static int rebuild_batch(wg_ctx* c, int cls) {
   Query* x = excl_query(c);
   if (x && (x->solo || x->bclass != cls)) return WG_OK;
@@ -2283,11 +2284,15 @@ static int rebuild_batch(wg_ctx* c, int cls) {
     }
   }
   if (!p) return WG_OK;
-  const int rc = ensure_batch_engine(c, cls, p->rel);
+  int rc = ensure_batch_engine(c, cls, p->rel);
+  if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && drop_idle_batch(c, cls)) {
+    cudaGetLastError();
+    rc = ensure_batch_engine(c, cls, p->rel);
+  }
   if (rc != WG_E_BUDGET && rc != WG_E_NOMEM) return rc;
   cudaGetLastError();
   for (auto& kv : c->batch)
-    if (kv.second) return WG_OK;  // memory may come back: retry next round
+    if (kv.second) return WG_OK;  // it holds work, so memory may come back: retry next round
   if (held_elsewhere(c, cls)) return WG_OK;
   std::vector<uint64_t> still;
   for (uint64_t qid : c->pending) {
