@@ -2714,6 +2714,10 @@ static int lane_admit(wg_ctx* c, RowLane* L, bool* progressed) {
   }
   if (ids.empty()) return WG_OK;
   int rc = lane_start(c, L, ids);
+  if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && drop_idle_batch(c, -1)) {
+    cudaGetLastError();  // (engines that hold no work would keep their pools for good)
+    rc = lane_start(c, L, ids);
+  }
   if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) {
     cudaGetLastError();
     if (ids.size() > 1) {  // fewer at once

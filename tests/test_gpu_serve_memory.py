@@ -78,3 +78,19 @@ def test_long_rows_beside_a_batch_engine(budget_mb, reserve_mb):
         h, = c.submit([(wg.WG_TC, a)])
         _drain(c)
         assert np.array_equal(h.result(), _closed(*small))
+
+
+def test_lane_beside_an_idle_engine():
+    # the batch engine of an earlier request holds a third of the budget; a relation
+    # loaded after the submission leaves too little for the lane's 112 MB of bit sets
+    from paper_2607_17571_gb300 import wg
+    first, e, fill = _pairs(5000), _pairs(15_000), _pairs(4_300_000)
+    with wg.Context(0, mem_budget=400 * MB, torch_memory=False) as c:
+        h, = c.submit([(wg.WG_TC, c.load(*first), dict(reserve_cand=1))])
+        h.wait()
+        h.free()
+        h, = c.submit([(wg.WG_TC, c.load(*e))])
+        c.load(*fill)
+        assert c.mem_used() > (400 - 112) * MB
+        h.wait()
+        assert np.array_equal(h.result(), _closed(*e))
