@@ -254,14 +254,17 @@ struct RowInst {
   unsigned long long n_total, cand;
 };
 struct RowCtl {
-  uint32_t next_row, pad;
+  uint32_t next_row, deepest;   // deepest, levels, tuples: of the sampled rows
+  unsigned long long levels, tuples;
 };
 constexpr uint32_t kRowLog = 64;        // levels counted in shared memory
 // What a single query's run found, in page-locked host memory.
 struct RowReport {
   unsigned long long n_total, cand;
   uint32_t last, fits, n_big, error;
+  unsigned long long levels, tuples;  // of the sampled rows
   unsigned long long log[kRowLog];
+  uint32_t deepest, pad;
 };
 // One launch over the rows of one or more instances.
 struct RowJob {
@@ -275,7 +278,8 @@ struct RowJob {
   // has room for `slots`, and kSmallRow ids per row (or NULL, 0, NULL)
   uint32_t* rows;
   uint32_t* small;
-  uint32_t slots, pad;
+  uint32_t slots, few;          // (more long rows than `few`: a sample of them first)
+  uint32_t sample, pad;         // long rows of this launch if it only samples, else 0
   const struct SgInst* sg;      // same-generation: which pieces of the rows are valid (or NULL)
   const struct SgCtl* sg_ctl;   // ... and its control block (or NULL)
   RowReport* report;            // written by k_row_plan (or NULL)

@@ -709,6 +709,7 @@ struct EngineBase {
   virtual uint32_t sort_mode() const = 0;
   virtual uint32_t side_mode() const = 0;
   virtual bool rows() const = 0;
+  virtual bool wide_rows() const = 0;    // ... with the small rows apart
   virtual size_t held() const = 0;       // device bytes of the engine's buffers
   virtual size_t grow_peak() const = 0;  // held() at the peak of the growth the last run asked for
   virtual void release() = 0;
@@ -742,7 +743,9 @@ struct Query {
   uint32_t slot = 0;
   bool rowb = false;             // batched row by row (see RowLane); bclass is -1
   bool row_alone = false;        // ... once its result did not fit beside others
-  bool no_rows = false;          // its rows' bit sets did not fit the budget
+  bool no_rows = false;          // it is not run by rows: their scratch did not fit, or:
+  int deep = 0;                  // 1: its rows are deep (see rows_deep); 2: rows all the same, the
+                                 // pipeline does not fit
   // served through a single-query engine (a large request, see solo_round)
   bool solo = false;
   bool solo_wait = false;        // paused after a growth over the budget
@@ -813,6 +816,8 @@ struct Engine : EngineBase {
   bool expand_only = false;          // the rows are done; the result waits for a larger buffer
   bool resume = false;               // the small rows are done; the long ones waited for bit sets
   bool row_short = false;            // the long rows' bit sets did not fit the budget
+  bool row_deep = false;             // the pipeline is the faster one for this relation
+  unsigned long long small_total = 0;  // tuples of the small rows
   Engine(wg_ctx* ctx, bool single_, uint32_t n, uint32_t bits, uint32_t logcap, bool fuse_,
          bool xseg_, bool copy_back_ = false, bool hash_join_ = false, uint32_t side = 0)
       : c(ctx), single(single_), fuse(fuse_), xseg(xseg_), n_slots(n), bits_(bits),
@@ -838,6 +843,7 @@ struct Engine : EngineBase {
   uint32_t sort_mode() const override { return sort_mode_; }
   uint32_t side_mode() const override { return side_; }
   bool rows() const override { return rows_; }
+  bool wide_rows() const override { return rows_ && job.rows; }
   uint32_t bits() const override { return bits_; }
   uint32_t slots() const override { return n_slots; }
 
@@ -1080,7 +1086,7 @@ struct Engine : EngineBase {
 
   // Row-by-row TC: buffers for relation R and a result of wantF keys.  A
   // result that turns out larger only needs the expansion again (settle).
-  int rows_begin(Relation* Rl, int kind, uint32_t max_iters, unsigned long long wantF) {
+  int rows_begin(Relation* Rl, int kind, uint32_t max_iters, unsigned long long wantF, bool sample) {
     AllocScope scope(c, st);
     const uint32_t nv = Rl->nv, words = Rl->row_words();
     const uint32_t nch = (nv + kRowChunk - 1) / kRowChunk;
@@ -1137,6 +1143,7 @@ struct Engine : EngineBase {
       job.rows = (uint32_t*)(m + o_rows);
       job.small = (uint32_t*)row_small.p;
       job.slots = (uint32_t)std::min<size_t>(nv, row_bits.bytes / ((size_t)words * 4));
+      job.few = sample && Rl->w > kDeepBits ? kDeepRows * (uint32_t)g_rows : 0xFFFFFFFFu;
     }
     if (row_sg) {
       sgi = SgInst{};
@@ -1155,26 +1162,42 @@ struct Engine : EngineBase {
       sg.list[0] = (uint2*)(m + o_rows); sg.list[1] = (uint2*)(m + o_rows1);
     }
     log_cap = nlog;
-    expand_only = resume = row_short = false;
+    expand_only = resume = row_short = row_deep = false;
     hi[0] = Inst{};
     hi[0].state = INST_ACTIVE;
     hi[0].log = ri.log;
     return WG_OK;
   }
-  // Room for the bit sets of the long rows that k_rows_small left.
+  // Room for the bit sets of the long rows that k_rows_small left (or a sample of them).
   size_t row_sets() const {
-    return std::min((size_t)ri.n_big + ri.n_big / 16 + 64, (size_t)ri.nv) * ri.words * 4;
+    const size_t n = job.sample ? job.sample : (size_t)ri.n_big + ri.n_big / 16 + 64;
+    return std::min(n, (size_t)ri.nv) * ri.words * 4;
   }
   int rows_room() {
     AllocScope scope(c, st);
-    const size_t set = (size_t)ri.words * 4;
-    row_bits.release(c);
     row_short = true;
     TRY(row_bits.get(c, row_sets()));
     row_short = false;
     ri.bits = (uint32_t*)row_bits.p;
-    job.slots = (uint32_t)std::min<size_t>(ri.nv, row_bits.bytes / set);
+    job.slots = (uint32_t)std::min<size_t>(ri.nv, row_bits.bytes / ((size_t)ri.words * 4));
     return WG_OK;
+  }
+  // Whether the sampled long rows are so deep that the sorted-array pipeline is the
+  // faster one.  A level of a wide row scans its whole candidate set, so it costs a
+  // CTA kLevelNs however few vertices are new; an iteration of the pipeline costs
+  // kIterNs and, per tuple of the result, kTupleNs and kMergeNs more for each
+  // iteration (Full is merged as it grows).  Whole calls, rows | pipeline, P paths of
+  // n vertices: 300 x 1,000 725 | 547 ms, 786 x 1,000 4,513 | 1,050, 2,600 x 300
+  // 402 | 169; up to 2^18 vertices the pipeline's deep iterations are slower (262 x
+  // 1,000 596 | 3,482) and rows always win, as they do with so few long rows (kDeepRows
+  // a CTA) that even the deepest cost less than the pipeline's iterations.
+  static constexpr uint32_t kDeepBits = 18, kDeepRows = 128;
+  bool rows_deep() const {
+    constexpr double kLevelNs = 1600, kIterNs = 240e3, kTupleNs = 0.2, kMergeNs = 0.0019;
+    const double scale = (double)ri.n_big / std::max<uint32_t>(job.sample, 1);
+    const double d = std::max(report->deepest, ri.last);
+    const double rows_ns = report->levels * scale * kLevelNs / g_rows;
+    return rows_ns > d * kIterNs + (small_total + report->tuples * scale) * (kTupleNs + kMergeNs * d);
   }
   int rows_launch() {
     ri.out = F[0].p;
@@ -1218,7 +1241,22 @@ struct Engine : EngineBase {
     Inst& I = hi[0];
     I.n_full = ri.n_total;
     I.cand_total = ri.cand;
-    if (job.rows && ri.n_big > job.slots) {  // more long rows than bit sets: k_rows did nothing
+    if (job.sample) {
+      if (rows_deep()) {
+        row_deep = true;
+        return WG_OK;
+      }
+      job.sample = 0;
+      job.few = 0xFFFFFFFFu;
+      *again = true;
+      return ri.n_big > job.slots ? rows_room() : WG_OK;
+    }
+    // more long rows than bit sets, or not yet sampled: k_rows did nothing
+    if (job.rows && ri.n_big > std::min(job.slots, job.few)) {
+      if (ri.n_big > job.few) {
+        small_total = ri.n_total;
+        job.sample = 2 * (uint32_t)g_rows;  // two rows a CTA
+      }
       ++regrows;
       *again = true;
       resume = true;
@@ -1683,7 +1721,7 @@ static int single_start(wg_ctx* c, Query* q) {
   const unsigned long long wantF = std::max<unsigned long long>(
       {q->opts.reserve_full, Rl->peak_full, 4ull * Rl->ne, 1ull << 16});
   if (E->rows_) {
-    TRY(E->rows_begin(Rl, q->kind, q->opts.max_iters, wantF));
+    TRY(E->rows_begin(Rl, q->kind, q->opts.max_iters, wantF, q->deep == 0));
     CK(cudaEventRecord(q->ev0, c->stream));
     TRY(E->rows_launch());
     CK(cudaEventRecord(q->ev1, c->stream));
@@ -1780,12 +1818,21 @@ static int single_start(wg_ctx* c, Query* q) {
 extern "C" {
 static int single_begin(wg_ctx* c, Query* q);
 }
-// Query q's rows do not fit the memory there is: start it over on the pipeline.
-static int rows_to_pipeline(wg_ctx* c, Query* q) {
-  q->no_rows = true;
+// Query q, which does not fit the memory there is (or is deep), has another way to
+// run: rows of a wide relation go to the sorted-array pipeline, which has none of
+// their scratch, and a query that is there because its rows are deep back to rows.
+static bool other_way(Query* q) {
+  if (q->eng->wide_rows()) {
+    q->no_rows = true;
+  } else if (!q->eng->rows() && q->deep == 1) {
+    q->deep = 2;
+    q->no_rows = false;
+  } else {
+    return false;
+  }
   q->own.reset();
   q->eng = nullptr;
-  return single_begin(c, q);
+  return true;
 }
 
 template <typename K>
@@ -1803,13 +1850,25 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
     }
     bool again = false;
     int rc = E->settle(&again);
-    if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && E->rows_ && E->job.rows && !pause_on_budget) {
-      // the long rows' bit sets, or the result beside them, do not fit: the
-      // sorted-array pipeline, which has no such scratch, takes it (a served
-      // request waits for memory first, see solo_pipeline)
+    const bool short_of = rc == WG_E_BUDGET || rc == WG_E_NOMEM;
+    const bool deep = rc == WG_OK && E->row_deep;
+    if (deep) q->deep = 1;
+    // (a served request that is short of memory waits for it first, see solo_give_up)
+    if ((deep || (short_of && !pause_on_budget)) && other_way(q)) {
       cudaGetLastError();
-      rc = rows_to_pipeline(c, q);
+      rc = single_begin(c, q);
       if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
+      if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && deep) {  // no room for the pipeline's start
+        cudaGetLastError();
+        q->deep = 2;
+        q->no_rows = false;
+        q->own.reset();
+        rc = single_begin(c, q);
+        if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
+      }
+      q->state = WG_FAILED;
+      q->error = rc;
+      return rc;
     }
     if (rc != WG_OK && pause_on_budget && (rc == WG_E_BUDGET || rc == WG_E_NOMEM)) {
       cudaGetLastError();  // the pools stay whole at their old capacities
@@ -3103,18 +3162,15 @@ static void solo_finish(wg_ctx* c, Query* q, int rc) {
 }
 
 // Request q on a single-query engine paused for memory that it does not get: it
-// fails, except that one whose wide rows do not fit goes on to the sorted-array
-// pipeline -- queued again, as the exclusive query, while others hold memory the
-// pipeline needs for its start.
+// goes on the other way if it has one -- queued again, as the exclusive query, while
+// others hold memory that its start needs -- or fails.
 static void solo_give_up(wg_ctx* c, Query* q, int why, bool others) {
-  const bool k4 = q->eng->kb() == 4;
-  if (!q->eng->rows() || !(k4 ? static_cast<Engine<uint32_t>*>(q->eng)->job.rows
-                              : static_cast<Engine<unsigned long long>*>(q->eng)->job.rows)) {
+  if (!other_way(q)) {
     solo_finish(c, q, why);
     return;
   }
   q->solo_wait = false;
-  const int rc = rows_to_pipeline(c, q);
+  const int rc = single_begin(c, q);
   if (rc == WG_OK) return;  // (running)
   if (rc == WG_E_BUDGET || rc == WG_E_NOMEM) cudaGetLastError();
   if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && others) {

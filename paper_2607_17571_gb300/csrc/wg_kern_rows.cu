@@ -79,6 +79,9 @@ __device__ __forceinline__ void cta_sync() {
 // barriers per iteration; a delta of more than row_list(T) such vertices takes
 // several rounds, the bits not yet listed waiting in the row's place in `bits`.
 //
+// kDry: a sample of the listed rows, of which only levels and tuples are counted
+// (deep rows of wide relations go to the sorted-array pipeline, see rows_deep).
+//
 // Bound by the L1 / shared pipe, issue slots and barriers (ncu on R-MAT 2^15 / 100k,
 // 324 us: pipe 76%, issue 62%, DRAM 0.05%; on ER 16,384 / 34,000 82% and 68%).
 // What it measured on R-MAT 2^17 / 400k, whole call: winners of each
@@ -91,7 +94,7 @@ __device__ __forceinline__ void cta_sync() {
 // shared memory and one global atomic per iteration past its log, 1.02 with 32
 // iterations' counts to an atomic, 0.84 with the list's length and the delta's size
 // in registers, 0.72 without scan and barriers where no lane has two new vertices.
-template <typename IdT, int T, int kMin>
+template <typename IdT, int T, int kMin, bool kDry = false>
 __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   constexpr uint32_t kW = T / 32, kList = row_list(T);
   constexpr bool kOne = kW == 1;  // one warp: counts stay in registers
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
   if (tid == 0) s_row[0] = atomicAdd(&J.ctl->next_row, 1u);
   __syncthreads();
   auto flush = [&]() {  // the counters of the current instance
+    if (kDry) return;
     for (int o = 16; o > 0; o >>= 1) cand += __shfl_xor_sync(0xffffffffu, cand, o);
     if (lane == 0 && cand) atomicAdd(&J.inst[cur].cand, cand);
     cand = 0;
@@ -120,12 +124,16 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
     }
   };
   // listed rows (k_rows_small's leftovers): their bit sets lie in list order
-  const uint32_t nrows = J.rows ? J.inst->n_big : J.nrows;
-  if (J.rows && nrows > J.slots) return;  // no room: the host grows it and starts over
+  const uint32_t n_list = J.rows ? J.inst->n_big : J.nrows;
+  const uint32_t nrows = kDry ? min(J.sample, n_list) : n_list;
+  // no room, or a sample is wanted: the host sees to it and launches again
+  if (J.rows && (nrows > J.slots || nrows > J.few)) return;
   for (uint32_t p = 0;; p ^= 1) {
     const uint32_t at_row = s_row[p];
     if (at_row >= nrows) break;
-    const uint32_t row = J.rows ? J.rows[at_row] : at_row;
+    // (a sample is spread over the list: neighbours are alike)
+    const uint32_t at_list = kDry ? (uint32_t)(at_row * 4294967291ull % n_list) : at_row;
+    const uint32_t row = J.rows ? J.rows[at_list] : at_row;
     const uint32_t q = J.chunk_inst ? J.chunk_inst[row / kRowChunk] : 0u;
     if (q != cur) {
       __syncthreads();
@@ -158,7 +166,7 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
       // iterations past the log in shared memory: warp 0's lanes hold 32 of them
       uint32_t held = 0;
       auto log_held = [&](uint32_t first) {
-        if (held && first + lane < I.log_cap) atomicAdd(I.log + first + lane, (unsigned long long)held);
+        if (held && !kDry && first + lane < I.log_cap) atomicAdd(I.log + first + lane, (unsigned long long)held);
         held = 0;
       };
       uint4* const n4 = (uint4*)N;
@@ -244,7 +252,13 @@ __global__ void __launch_bounds__(T, kMin) k_rows(RowJob J) {
         turn ^= 1;
       }
       if (warp == 0 && lvl > kRowLog) log_held((lvl - 1) & ~31u);
-      if (tid == 0) {  // (the delta of iteration lvl - 1 was the last that is not empty)
+      if (kDry) {
+        if (tid == 0) {
+          atomicMax(&J.ctl->deepest, lvl);
+          atomicAdd(&J.ctl->levels, (unsigned long long)lvl);
+          atomicAdd(&J.ctl->tuples, (unsigned long long)total);
+        }
+      } else if (tid == 0) {  // (the delta of iteration lvl - 1 was the last that is not empty)
         atomicMax(&J.inst[q].last, lvl - 1);
         I.cnt[x] = total;
         atomicAdd(J.csum + row / kRowChunk, total);
@@ -455,7 +469,7 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
   if (threadIdx.x == 0) {
     I->n_total = carry;
     // an output buffer that is too small: the expansion waits for a larger one
-    I->fits = carry <= I->out_cap && !(J.rows && I->n_big > J.slots) ? 1u : 0u;
+    I->fits = carry <= I->out_cap && !(J.rows && (J.sample || I->n_big > min(J.slots, J.few))) ? 1u : 0u;
     if (RowReport* r = J.report) {
       r->n_total = carry;
       r->cand = I->cand;
@@ -463,6 +477,11 @@ __global__ void __launch_bounds__(1024) k_row_plan(RowJob J) {
       r->fits = I->fits;
       r->n_big = I->n_big;
       r->error = J.sg_ctl ? J.sg_ctl->error : 0u;
+      if (J.sample) {
+        r->levels = J.ctl->levels;
+        r->tuples = J.ctl->tuples;
+        r->deepest = J.ctl->deepest;
+      }
     }
   }
   if (J.report && threadIdx.x < kRowLog)
@@ -599,6 +618,12 @@ int occupancy_rows(int id_bytes, uint32_t vwords) {
 void launch_rows(const RowJob& J, int id_bytes, int grid, cudaStream_t s) {
   const int t = row_threads(J.vwords);
   const uint32_t smem = row_smem(J.vwords, id_bytes, t);
+  if (J.sample) {  // (more than 2^18 vertices)
+    auto k = t == 512 ? k_rows<uint32_t, 512, 2, true> : k_rows<uint32_t, 1024, 1, true>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+    k<<<grid, t, smem, s>>>(J);
+    return;
+  }
   rows_kernel(J.vwords, id_bytes, [&](auto k) {
     k<<<grid, t, smem, s>>>(J);
     return 0;
