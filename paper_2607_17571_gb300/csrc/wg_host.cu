@@ -460,6 +460,8 @@ struct Relation {
   DBuf htab;                      // hash-join ablation: E in a linear-probing table (lazy)
   unsigned long long hmask = 0;
   uint64_t peak_cand = 0, peak_full = 0;  // capacities seen by earlier queries
+  bool paths_known = false;       // two-paths from a source: most, and all (see one_heavy_row)
+  unsigned long long paths[2] = {0, 0};
   int id_bytes() const { return nv <= 65536u ? 2 : 4; }  // of a rank in the units
   uint32_t row_words() const { return (nv + 127) / 128 * 4; }  // of a row's bit set
   size_t row_bits() const { return (size_t)nv * row_words() * 4; }  // bytes of all rows' sets
@@ -744,8 +746,8 @@ struct Query {
   bool rowb = false;             // batched row by row (see RowLane); bclass is -1
   bool row_alone = false;        // ... once its result did not fit beside others
   bool no_rows = false;          // it is not run by rows: their scratch did not fit, or:
-  int deep = 0;                  // 1: its rows are deep (see rows_deep); 2: rows all the same, the
-                                 // pipeline does not fit
+  int deep = 0;                  // 1: the pipeline is faster (see rows_deep, one_heavy_row);
+                                 // 2: rows all the same, the pipeline does not fit
   // served through a single-query engine (a large request, see solo_round)
   bool solo = false;
   bool solo_wait = false;        // paused after a growth over the budget
@@ -1858,14 +1860,6 @@ static int single_progress(wg_ctx* c, Query* q, bool block, bool pause_on_budget
       cudaGetLastError();
       rc = single_begin(c, q);
       if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
-      if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && deep) {  // no room for the pipeline's start
-        cudaGetLastError();
-        q->deep = 2;
-        q->no_rows = false;
-        q->own.reset();
-        rc = single_begin(c, q);
-        if (rc == WG_OK) return block ? single_progress<K>(c, q, block, pause_on_budget) : WG_OK;
-      }
       q->state = WG_FAILED;
       q->error = rc;
       return rc;
@@ -2458,6 +2452,36 @@ static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
   // (made here, it is complete before a lane reads it on its own stream)
   return row_layout(c, R, false) == WG_OK && R->rowv.p && cudaStreamSynchronize(c->stream) == cudaSuccess;
 }
+// Whether one source's row would hold up the others: a row is one CTA's work, so a
+// source with many two-paths and little beside it leaves the chip idle.  Shortest
+// times from the edges alone: rows one CTA's candidates (row_candidate_ns), pipeline
+// 0.45 ms and 0.04 ns a candidate.  Hubs of m children with the same n children each,
+// rows | pipeline: 600 x 600 0.46 | 0.99 ms, 1,000 x 1,000 1.13 | 0.55, 2,000 x 2,000
+// 4.3 | 0.76, 500 x 60,000 17.9 | 2.3; 300 x 3,000 among 200,000 vertices 0.39 | 3.2.
+constexpr uint64_t kHeavyEdges = 400'000;  // (fewer two-paths than that cost rows less)
+static bool one_heavy_row(wg_ctx* c, Relation* R) {
+  if (R->ne < kHeavyEdges) return false;
+  if (!R->paths_known) {
+    DBuf b;
+    const size_t head = 256;
+    if (b.get(c, head + (size_t)R->nv * 4) != WG_OK) return false;
+    cudaMemsetAsync(b.p, 0, head + (size_t)R->nv * 4, c->stream);
+    uint32_t* p = (uint32_t*)((char*)b.p + head);
+    const uint32_t *off = (const uint32_t*)R->off.p, *adj = (const uint32_t*)R->adj.p;
+    if (R->kb == 4)
+      launch_row_paths<uint32_t>((const uint32_t*)R->keys.p, (uint32_t)R->ne, R->w, off, adj, p,
+                                 (unsigned long long*)b.p, grid_of(c, 8), c->stream);
+    else
+      launch_row_paths<unsigned long long>((const unsigned long long*)R->keys.p, (uint32_t)R->ne,
+                                           R->w, off, adj, p, (unsigned long long*)b.p,
+                                           grid_of(c, 8), c->stream);
+    R->paths_known = cudaMemcpyAsync(R->paths, b.p, 16, cudaMemcpyDeviceToHost, c->stream) == cudaSuccess &&
+                     cudaStreamSynchronize(c->stream) == cudaSuccess;
+    b.release(c);
+    if (!R->paths_known) return false;
+  }
+  return R->paths[0] * row_candidate_ns(R->row_words()) > 450e3 + 0.04 * (double)(R->paths[1] + R->ne);
+}
 static bool row_query(wg_ctx* c, const Query* q) {
   return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->no_rows &&
          row_fits(c, q, false);
@@ -3025,9 +3049,13 @@ static int make_query(wg_ctx* c, int kind, wg_rel edges, const wg_opts* opts, Qu
 
 // Give query q a single-query engine (an idle one of the same key width, pass
 // plan and stage layout, else a new one) and start its fixpoint.
-static int single_begin(wg_ctx* c, Query* q) {
+static int single_try(wg_ctx* c, Query* q) {
   Relation* R = q->rel;
-  const bool rows = row_query(c, q);
+  bool rows = row_query(c, q);
+  if (rows && q->deep == 0 && q->kind == WG_TC && one_heavy_row(c, R)) {
+    q->deep = 1;
+    rows = false;
+  }
   const int kind = q->kind;
   const bool fuse = !(q->opts.flags & WG_FLAG_SEPARATE_STAGES);
   const bool full_width = (q->opts.flags & WG_FLAG_FULL_WIDTH) != 0;
@@ -3096,6 +3124,18 @@ static int single_begin(wg_ctx* c, Query* q) {
   auto* E = static_cast<Engine<unsigned long long>*>(q->eng);
   E->regrows = 0; E->launches_issued = 0;
   return single_start<unsigned long long>(c, q);
+}
+static int single_begin(wg_ctx* c, Query* q) {
+  int rc = single_try(c, q);
+  if ((rc == WG_E_BUDGET || rc == WG_E_NOMEM) && q->deep == 1) {  // no room for the pipeline's start
+    cudaGetLastError();
+    q->deep = 2;
+    q->no_rows = false;
+    q->own.reset();
+    q->eng = nullptr;
+    rc = single_try(c, q);
+  }
+  return rc;
 }
 
 static int single_query(wg_ctx* c, int kind, wg_rel edges, const wg_opts* opts, wg_query* out) {

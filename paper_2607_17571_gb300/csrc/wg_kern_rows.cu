@@ -60,6 +60,36 @@ __global__ void __launch_bounds__(kThreads) k_row_layout(const K* E, uint32_t ne
   }
 }
 
+// Two-paths from every source (scratch `paths`, nv zeros): out[0] their maximum,
+// out[1] their sum (zero before).  The edges are in source order, so most warps add
+// once.
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_row_paths(const K* E, uint32_t ne, uint32_t w,
+                                                        const uint32_t* off, const uint32_t* adj,
+                                                        uint32_t* paths, unsigned long long* out) {
+  const uint32_t stride = gridDim.x * kThreads, lane = threadIdx.x & 31;
+  unsigned long long sum = 0;
+  uint32_t top = 0;
+  for (uint32_t i0 = (blockIdx.x * kThreads + threadIdx.x) & ~31u; i0 < ne; i0 += stride) {
+    const uint32_t i = min(i0 + lane, ne - 1);
+    const uint32_t x = (uint32_t)(E[i] >> w), z = adj[i];
+    uint32_t d = i0 + lane < ne ? off[z + 1] - off[z] : 0u;
+    sum += d;
+    const bool same = __all_sync(0xffffffffu, x == __shfl_sync(0xffffffffu, x, 0));
+    if (same) {
+      d = __reduce_add_sync(0xffffffffu, d);
+      if (lane) d = 0;
+    }
+    if (d) top = max(top, atomicAdd(paths + x, d) + d);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) {
+    atomicMax(out, (unsigned long long)top);
+    atomicAdd(out + 1, sum);
+  }
+}
+
 template <int T>
 __device__ __forceinline__ void cta_sync() {
   if (T == 32) __syncwarp();
@@ -593,6 +623,13 @@ static int row_threads(uint32_t vwords) {
                            : 1024;
 }
 
+// Time of one candidate in a row that has its CTA to itself and the others idle:
+// one hub of 500 to 5,000 children with the same 1,000 to 60,000 children each.
+double row_candidate_ns(uint32_t vwords) {
+  const int t = row_threads(vwords);
+  return t == 32 ? 1.08 : t == 64 ? 0.68 : t <= 256 ? 0.57 : t == 512 ? 0.27 : 0.17;
+}
+
 template <typename F>
 static auto rows_kernel(uint32_t vwords, int id_bytes, F f) {
   const int t = row_threads(vwords);
@@ -647,6 +684,17 @@ void launch_row_expand(const RowJob& J, int grid, cudaStream_t s) {
   if (J.sg) k_row_expand<K, true><<<grid, kThreads, 0, s>>>(J);
   else k_row_expand<K, false><<<grid, kThreads, 0, s>>>(J);
 }
+template <typename K>
+void launch_row_paths(const K* E, uint32_t ne, uint32_t w, const uint32_t* off, const uint32_t* adj,
+                      uint32_t* paths, unsigned long long* out, int grid, cudaStream_t s) {
+  k_row_paths<K><<<grid, kThreads, 0, s>>>(E, ne, w, off, adj, paths, out);
+}
+template void launch_row_paths<uint32_t>(const uint32_t*, uint32_t, uint32_t, const uint32_t*,
+                                         const uint32_t*, uint32_t*, unsigned long long*, int,
+                                         cudaStream_t);
+template void launch_row_paths<unsigned long long>(const unsigned long long*, uint32_t, uint32_t,
+                                                   const uint32_t*, const uint32_t*, uint32_t*,
+                                                   unsigned long long*, int, cudaStream_t);
 size_t row_units(uint64_t ne, uint32_t nv, int id_bytes) {
   const uint64_t U = 16 / id_bytes;
   return (size_t)((ne + (U - 1) * ((uint64_t)nv + 1)) / U + 1);

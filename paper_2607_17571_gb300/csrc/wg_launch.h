@@ -80,6 +80,11 @@ void launch_row_begin(const RowJob& J, const RowInst& I, const SgInst& G, void* 
 void launch_rows_small(const RowJob& J, int grid, cudaStream_t s);
 void launch_row_plan(const RowJob& J, uint32_t n_inst, cudaStream_t s);
 template <typename K> void launch_row_expand(const RowJob& J, int grid, cudaStream_t s);
+double row_candidate_ns(uint32_t vwords);
+// two-paths from every source: paths (nv zeros before), out: their maximum and sum (zeros)
+template <typename K>
+void launch_row_paths(const K* E, uint32_t ne, uint32_t w, const uint32_t* off, const uint32_t* adj,
+                      uint32_t* paths, unsigned long long* out, int grid, cudaStream_t s);
 // adjacency units of a relation: their number, and the layout of vertex records
 // (16 bytes each), out-edge bit set (words), further units (16 bytes each), bit set
 // of the vertices with several parents (words; followed by as many of scratch)
