@@ -214,15 +214,26 @@ def run_ours(args):
     def run(r, **kw):
         return run0(r, loop=loop, **kw)
     kb = 4 if 2 * info["field_bits"] <= 32 else 8
-    tiles = None if args.no_autotune else autotune_ctx(
-        ctx, [rel], wg.WG_TC if wl["kind"] == "tc" else wg.WG_SG)
+
+    def tune():
+        return None if args.no_autotune else autotune_ctx(
+            ctx, [rel], wg.WG_TC if wl["kind"] == "tc" else wg.WG_SG)
 
     # warm-up: also sizes the pools (a relation remembers the capacities it needed)
-    st = None
-    for _ in range(args.warmup):
-        q = run(rel)
-        st = q.wait()
-        q.free()
+    def warm_up():
+        st = None
+        for _ in range(args.warmup):
+            q = run(rel)
+            st = q.wait()
+            q.free()
+        return st
+    # a query run by rows takes a dozen launches at most, the sorted-array pipeline
+    # more than ten per iteration and two iterations at least; only that has tiles
+    rows = warm_up().gpu_launches <= 16
+    tiles = "none (rows)"
+    if not rows:
+        tiles = tune()
+        warm_up()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=f"cuda:{local}")  # > L2 (129 MB)
 
     if world > 1:
@@ -258,6 +269,8 @@ def run_ours(args):
 
     # the sorted-array pipeline's stages: the same fixpoint once more with CUDA events
     # around every kernel (a profiled query always takes that pipeline)
+    if rows:
+        tune()
     q = run(rel, profile=True)
     q.wait()
     prof = q.profile()
@@ -269,9 +282,6 @@ def run_ours(args):
                               "GBps": round(p["bytes"] / (p["total_ms"] / 1e3) / 1e9, 1),
                               "share": round(p["total_ms"] / sum(x["total_ms"] for x in prof), 4)}
                              for p in sorted(prof, key=lambda p: -p["total_ms"])]}
-    # the timed path: a plain query runs row by row in a handful of launches (the
-    # sorted-array pipeline issues more than ten per iteration)
-    rows = launches <= 8 * args.steps
     traffic = None
     if rows:
         # what the fixpoint cannot do without: the edges and their index read once,
@@ -411,9 +421,6 @@ def run_batch(args):
             torch.cuda.empty_cache()  # the next context's budget sees the memory again
         ctx = wg.Context(0)
         rels = [ctx.load(g.src, g.dst) for g in graphs]
-        if not args.no_autotune:
-            tuned.update(autotune_ctx(ctx, rels))
-    tuned = {}
     # every query is checked against the oracle's closure size, iteration
     # count and digest of the sorted result (tests/golden/batch4096.json,
     # written by tests/golden/make_mix_golden.py, which calls only oracle/);
@@ -422,7 +429,7 @@ def run_batch(args):
 
     failed = []
 
-    def check(i, h, st):
+    def check(i, h, st, digest=True):
         if st.state != wg.WG_DONE:
             failed.append({"query": i, "edges": int(sizes[i][1]), "error": int(st.error)})
             return 1
@@ -430,30 +437,11 @@ def run_batch(args):
         if g is None:
             return 0
         return int(st.n_tuples != g["n_tuples"] or st.iterations != g["iterations"]
-                   or h.digest() != int(g["digest"]))
+                   or (digest and h.digest() != int(g["digest"])))
 
-    def batched():
-        t0 = time.perf_counter()
-        hs = ctx.submit([(wg.WG_TC, r) for r in rels])
-        idx = {h.id: i for i, h in enumerate(hs)}
-        lat, tuples, launches, bad, chk = [0.0] * len(hs), 0, 0, 0, 0.0
-        left = len(hs)
-        while left:
-            ctx.serve_step(args.batch_iters)
-            for qid in ctx.take_completed():
-                i = idx[qid]
-                h = hs[i]
-                st = h.poll()
-                lat[i] = (time.perf_counter() - t0 - chk) * 1e3
-                tuples += st.n_tuples
-                # checked and freed at once (a batched result stays in the
-                # engine's result pool until freed); the check is not timed
-                c0 = time.perf_counter()
-                bad += check(i, h, st)
-                h.free()
-                chk += time.perf_counter() - c0
-                left -= 1
-        return time.perf_counter() - t0 - chk, lat, tuples, bad
+    def batched(digest=False):
+        return batched_pass(ctx, [(wg.WG_TC, r) for r in rels], args.batch_iters,
+                            lambda i, h, st: check(i, h, st, digest))
 
     def plain():
         t0 = time.perf_counter()
@@ -483,8 +471,9 @@ def run_batch(args):
     torch.cuda.synchronize()
     clocks = Clocks(0)
     clocks.start()
-    tb, lb, nb, bad_b = batched()
+    tb, lb, nb, bad_b = batched()  # sizes and iterations checked
     clk_b = clocks.stop()
+    bad_b += batched(digest=True)[3]  # the digests, on the same requests once more
     open_ctx()
     for r in rels[:4]:
         q = ctx.tc(r)
@@ -503,16 +492,16 @@ def run_batch(args):
             "config": {"workload": "batch4096", "queries": n,
                        "desc": "ER TC queries, n log-uniform [64,16384], mean degree U[1.2,3.0], "
                                "seeds 40000+q", "closure_tuples_total": int(nb),
-                       "iterations_per_launch": args.batch_iters,
-                       "tiles": tuned or "compiled defaults"},
+                       "iterations_per_launch": args.batch_iters},
             "batched": {"seconds": round(tb, 3), "queries_per_s": n / tb, "tuples_per_s": nb / tb,
                         "p50_ms": _pct(lb, 50), "p99_ms": _pct(lb, 99), "parity_failures": bad_b,
                         "clocks": clk_b},
             "plain_loop": {"seconds": round(tp, 3), "queries_per_s": n / tp,
                            "tuples_per_s": npl / tp, "p50_ms": _pct(lp, 50), "p99_ms": _pct(lp, 99),
                            "parity_failures": bad_p, "gpu_launches": launches, "clocks": clk_p},
-            "parity_checked": f"{len(want)} of {n} queries: closure size, iterations and "
-                              "result digest against the oracle",
+            "parity_checked": f"{len(want)} of {n} queries against the oracle: closure size and "
+                              "iterations as timed, result digests in one more untimed pass "
+                              "(plain loop: between queries)",
             "same_total": nb == npl, "failed_queries": failed[:20], "clocks": clk_b}
     print(json.dumps(line))
     for r in rels:
@@ -717,6 +706,68 @@ def run_ablations(args):
     return 0
 
 
+def batched_pass(ctx, reqs, iters, check):
+    """All of `reqs` submitted at once and served to the end: seconds, latencies
+    (ms), tuples, failures.  check(i, handle, status) is called on each completed
+    query, which is then freed; its time counts, because the launches of the other
+    queries run on meanwhile (so a timed pass checks nothing that waits)."""
+    t0 = time.perf_counter()
+    hs = ctx.submit(reqs)
+    idx = {h.id: i for i, h in enumerate(hs)}
+    lat, tuples, bad, left = [0.0] * len(hs), 0, 0, len(hs)
+    while left:
+        ctx.serve_step(iters)
+        for qid in ctx.take_completed():
+            i = idx[qid]
+            st = hs[i].poll()
+            lat[i] = (time.perf_counter() - t0) * 1e3
+            tuples += st.n_tuples
+            bad += check(i, hs[i], st)
+            hs[i].free()
+            left -= 1
+    return time.perf_counter() - t0, lat, tuples, bad
+
+
+def served_pass(ctx, reqs, arr, limit, iters, check):
+    """Arrival a asks for reqs[a % len(reqs)] at arr[a] seconds.  As in
+    batched_pass the checks' time counts."""
+    n, npool = len(arr), len(reqs)
+    lat, ok, rej, tuples, bad = [None] * n, 0, 0, 0, 0
+    idx, nxt, done = {}, 0, 0
+    t0 = time.perf_counter()
+    while done < n and time.perf_counter() - t0 < limit:
+        now = time.perf_counter() - t0
+        new = []
+        while nxt < n and arr[nxt] <= now:
+            new.append(nxt)
+            nxt += 1
+        if new:
+            for a, h in zip(new, ctx.submit([reqs[a % npool] for a in new])):
+                idx[h.id] = (a, h)
+        running = ctx.serve_step(iters)
+        t = time.perf_counter() - t0
+        for qid in ctx.take_completed():
+            a, h = idx.pop(qid)
+            st = h.poll()
+            lat[a] = (t - arr[a]) * 1e3
+            if st.error == 0:
+                ok += 1
+                tuples += st.n_tuples
+                bad += check(a % npool, h, st)
+            else:
+                rej += 1
+            h.free()
+            done += 1
+        if running == 0 and nxt < n:
+            time.sleep(max(0.0, min(0.002, arr[nxt] - (time.perf_counter() - t0))))
+    el = time.perf_counter() - t0
+    good = [x for x in lat if x is not None]
+    unfinished = n - done  # closing the context waits only for the launch in flight
+    return dict(seconds=round(el, 3), queries_per_s=ok / el, tuples_per_s=tuples / el,
+                p50_ms=_pct(good, 50), p99_ms=_pct(good, 99), completed=ok, rejected=rej,
+                unfinished_in_time=unfinished, parity_failures=bad)
+
+
 def run_serve(args):
     """Open-loop Poisson arrivals of a mixed TC / SG request stream (see
     inputs.serve_request), served under a fixed device-memory budget: the
@@ -726,7 +777,7 @@ def run_serve(args):
     for request a % pool of a pool of --n-requests distinct seeded requests
     (relations resident); each arm stops after --arm-seconds.  Every completed
     request is checked against the oracle's figures (closure size,
-    iterations, result digest), outside the timed region."""
+    iterations; the result digests on the pool once more, untimed)."""
     import torch
 
     from paper_2607_17571_gb300 import inputs as I
@@ -744,17 +795,12 @@ def run_serve(args):
     npool = len(reqs)
     ctx, rels = None, None
 
-    failed = []
-
-    def check(i, h, st):
-        if st.state != wg.WG_DONE:
-            failed.append({"query": i, "edges": int(sizes[i][1]), "error": int(st.error)})
-            return 1
+    def check(i, h, st, digest=True):
         g = want.get(i)
         if g is None:
             return 0
         return int(st.n_tuples != g["n_tuples"] or st.iterations != g["iterations"]
-                   or h.digest() != int(g["digest"]))
+                   or (digest and h.digest() != int(g["digest"])))
 
     def single(i):
         return (ctx.tc if kinds[i] == wg.WG_TC else ctx.sg)(rels[i])
@@ -782,44 +828,13 @@ def run_serve(args):
                 q.free()
 
     def served(arr):
-        # arrival a asks for pool request a % npool
-        n = len(arr)
-        lat, ok, rej, tuples, bad, chk = [None] * n, 0, 0, 0, 0, 0.0
-        idx, nxt, done = {}, 0, 0
-        t0 = time.perf_counter()
-        while done < n and time.perf_counter() - t0 - chk < args.arm_seconds:
-            now = time.perf_counter() - t0 - chk
-            new = []
-            while nxt < n and arr[nxt] <= now:
-                new.append(nxt)
-                nxt += 1
-            if new:
-                for a, h in zip(new, ctx.submit([(kinds[a % npool], rels[a % npool]) for a in new])):
-                    idx[h.id] = (a, h)
-            running = ctx.serve_step(args.serve_iters)
-            t = time.perf_counter() - t0 - chk
-            for qid in ctx.take_completed():
-                a, h = idx.pop(qid)
-                st = h.poll()
-                lat[a] = (t - arr[a]) * 1e3
-                if st.state == wg.WG_DONE:
-                    ok += 1
-                    tuples += st.n_tuples
-                    c0 = time.perf_counter()  # the check is not part of the served time
-                    bad += check(a % npool, h, st)
-                    chk += time.perf_counter() - c0
-                else:
-                    rej += 1
-                h.free()
-                done += 1
-            if running == 0 and nxt < n:
-                time.sleep(max(0.0, min(0.002, arr[nxt] - (time.perf_counter() - t0 - chk))))
-        el = time.perf_counter() - t0 - chk
-        good = [x for x in lat if x is not None]
-        unfinished = n - done  # closing the context waits only for the launch in flight
-        return dict(seconds=round(el, 3), queries_per_s=ok / el, tuples_per_s=tuples / el,
-                    p50_ms=_pct(good, 50), p99_ms=_pct(good, 99), completed=ok, rejected=rej,
-                    unfinished_in_time=unfinished, parity_failures=bad)
+        # (sizes and iterations checked; the digests in pool_digests, untimed)
+        return served_pass(ctx, [(kinds[i], rels[i]) for i in range(npool)], arr, args.arm_seconds,
+                           args.serve_iters, lambda i, h, st: check(i, h, st, digest=False))
+
+    def pool_digests():
+        return served_pass(ctx, [(kinds[i], rels[i]) for i in range(npool)], [0.0] * npool, 600.0,
+                           args.serve_iters, check)["parity_failures"]
 
     def plain(arr):
         n = len(arr)
@@ -860,6 +875,9 @@ def run_serve(args):
         clocks.start()
         b = served(arr)
         b["clocks"] = clocks.stop()
+        if rate == rates[-1]:  # (every rate serves the same pool)
+            open_ctx(True)
+            b["parity_failures"] += pool_digests()
         open_ctx(False)
         clocks = Clocks(0)
         clocks.start()
@@ -873,9 +891,9 @@ def run_serve(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "u32/u64", "data": "synthetic",
             "config": {"workload": "serve", "arrivals_per_rate": args.n_arrivals,
                        "request_pool": npool, "arm_seconds_cap": args.arm_seconds,
-                       "parity": f"every completed request: closure size, iterations and result "
-                                 f"digest against the oracle ({len(want)} of {npool} pool "
-                                 f"requests have oracle figures)",
+                       "parity": f"every completed request: closure size and iterations, and the "
+                                 f"pool's result digests once more untimed, against the oracle "
+                                 f"({len(want)} of {npool} pool requests have oracle figures)",
                        "mix": "TC 75% (70% ER batch-mix sizes, 30% R-MAT DAG 1e4..1e6 edges), "
                               "SG 25% (forests, batch-mix sizes)",
                        "budget_gb": args.budget_gb, "iterations_per_round": args.serve_iters},
