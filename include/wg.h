@@ -19,7 +19,10 @@
  * set difference and merge are one bit test and set.  A plain SG query over at
  * most 131,072 vertices keeps such rows in device memory and gives all children
  * of a row the same candidate set at once.  The result, iteration count,
- * per-iteration sizes and candidate count are the same.
+ * per-iteration sizes and candidate count are the same.  A TC query runs on the
+ * sorted-array pipeline where that is the faster one (more than 2^18 vertices and a
+ * sample of the long rows is deep; one source's two-paths outweigh all else) or the
+ * rows' scratch does not fit the budget.
  *
  * Conventions for every entry point
  *  - Return value: WG_OK (0) or a negative WG_E_* code.  Nothing aborts, traps

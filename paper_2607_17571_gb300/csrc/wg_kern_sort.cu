@@ -860,9 +860,11 @@ __device__ __forceinline__ unsigned long long merge_path(const K* A, unsigned lo
 // outputs, one merge-path search for their start and then one comparison each,
 // and the tile goes out through shared memory, coalesced.  (A search per output:
 // 0.28 ms for 2.8e7 64-bit keys, now 0.13.)  Tiles are dealt out by CTA and the
-// splits read by every thread, so nothing waits before the loads; at 5 CTAs an SM
-// the registers just fit (whole call, 2^24 + 2^24 64-bit keys: claimed tiles and 4
-// CTAs 229 us, dealt out 223, and 5 CTAs 201; 32-bit keys 140, 136, 134).
+// splits read by every thread, so nothing waits before the loads.  The kernel wants
+// 127 registers with 64-bit keys and 80 with 32-bit ones (two and three CTAs an SM);
+// held to 48 for five CTAs it spills 120 and 24 bytes a thread, and the warps in flight
+// are worth more (whole call, 2^24 + 2^24 64-bit keys: claimed tiles, no bound 229 us,
+// dealt out 223, and 5 CTAs 201; 32-bit keys 140, 136, 134).
 template <typename K>
 __global__ void __launch_bounds__(kThreads, 5) k_merge(Stage* stp) {
   __shared__ K sm[Padded<kTileM>::n];
