@@ -2455,12 +2455,21 @@ static bool row_fits(wg_ctx* c, const Query* q, bool batched) {
 // Whether one source's row would hold up the others: a row is one CTA's work, so a
 // source with many two-paths and little beside it leaves the chip idle.  Shortest
 // times from the edges alone: rows one CTA's candidates (row_candidate_ns), pipeline
-// 0.45 ms and 0.04 ns a candidate.  Hubs of m children with the same n children each,
-// rows | pipeline: 600 x 600 0.46 | 0.99 ms, 1,000 x 1,000 1.13 | 0.55, 2,000 x 2,000
-// 4.3 | 0.76, 500 x 60,000 17.9 | 2.3; 300 x 3,000 among 200,000 vertices 0.39 | 3.2.
-constexpr uint64_t kHeavyEdges = 400'000;  // (fewer two-paths than that cost rows less)
+// 0.45 ms, 13 ns a vertex where it sorts by source (17- and 18-bit ranks), and 0.03 ns
+// a candidate (0.05 with 64-bit keys).  Hubs of m children with the same n children
+// each, rows | pipeline: 600 x 600 0.46 | 0.99 ms, 1,000 x 1,000 1.13 | 0.55, 2,000 x
+// 2,000 4.3 | 0.76, 500 x 60,000 17.9 | 2.3; among 200,000 other vertices 300 x 3,000
+// 0.39 | 3.2, 3,000 x 3,000 2.9 | 3.8, 3,000 x 20,000 17.9 | 8.3.
+// The two-paths are counted where every edge could be on the one source's: from 440,000
+// edges over 4,096 vertices, 900,000 over 65,536, 2.6 million over 409,600.
 static bool one_heavy_row(wg_ctx* c, Relation* R) {
-  if (R->ne < kHeavyEdges) return false;
+  const double row_ns = row_candidate_ns(R->row_words());
+  const double start_ns = 450e3 + (R->w == 17 || R->w == 18 ? 13.0 * R->nv : 0.0);
+  const double cand_ns = R->kb == 4 ? 0.03 : 0.05;
+  auto slower = [&](double most, double all) {
+    return most * row_ns > start_ns + cand_ns * (all + R->ne);
+  };
+  if (!slower(R->ne, R->ne)) return false;
   if (!R->paths_known) {
     DBuf b;
     const size_t head = 256;
@@ -2480,7 +2489,7 @@ static bool one_heavy_row(wg_ctx* c, Relation* R) {
     b.release(c);
     if (!R->paths_known) return false;
   }
-  return R->paths[0] * row_candidate_ns(R->row_words()) > 450e3 + 0.04 * (double)(R->paths[1] + R->ne);
+  return slower(R->paths[0], R->paths[1]);
 }
 static bool row_query(wg_ctx* c, const Query* q) {
   return q->opts.loop == WG_LOOP_DEVICE && !q->opts.profile && !q->no_rows &&

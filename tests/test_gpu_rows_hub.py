@@ -27,8 +27,8 @@ def _run(c, rel, **kw):
 @pytest.mark.parametrize("m,n,pairs,rows", [
     (2000, 2000, 0, False), (500, 15_000, 0, False), (100, 60_000, 0, False),
     (1000, 5000, 40_000, False),   # 32-bit ranks
-    (632, 632, 0, True),           # 399,424 two-paths: not looked at
-    (633, 633, 0, True),           # 400,689 edges beside the hub's own: a light row
+    (650, 650, 0, True), (680, 680, 0, False),  # about 440,000 edges: the line
+    (3000, 3000, 100_000, True),   # 17-bit ranks, where the pipeline starts slowly
     (300, 3000, 100_000, True)])
 def test_routes(m, n, pairs, rows):
     from paper_2607_17571_gb300 import wg
