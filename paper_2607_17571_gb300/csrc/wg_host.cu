@@ -544,6 +544,7 @@ static int row_layout(wg_ctx* c, Relation* R, bool in_load) {
   CK(cudaGetLastError());
   return WG_OK;
 }
+
 static int load_relation(wg_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, size_t n,
                          Relation* R) {
   if (n >= (1ull << 32)) return set_err(WG_E_INVAL, "at most 2^32 - 1 edges");
@@ -764,6 +765,7 @@ struct Query {
   const void* res_ptr = nullptr;
   DBuf res_own;                  // batch results copied out of the retire pool
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  bool begun = false;            // ev0 is recorded: a query that goes another way keeps it
 };
 
 template <typename K>
@@ -1714,6 +1716,12 @@ static int loop_mode(const Query* q) {
   return q->opts.profile && q->opts.loop == WG_LOOP_DEVICE ? (int)WG_LOOP_HOST : (int)q->opts.loop;
 }
 
+static int record_begin(wg_ctx* c, Query* q) {
+  if (!q->begun) CK(cudaEventRecord(q->ev0, c->stream));
+  q->begun = true;
+  return WG_OK;
+}
+
 template <typename K>
 static int single_start(wg_ctx* c, Query* q) {
   auto* E = static_cast<Engine<K>*>(q->eng);
@@ -1724,7 +1732,7 @@ static int single_start(wg_ctx* c, Query* q) {
       {q->opts.reserve_full, Rl->peak_full, 4ull * Rl->ne, 1ull << 16});
   if (E->rows_) {
     TRY(E->rows_begin(Rl, q->kind, q->opts.max_iters, wantF, q->deep == 0));
-    CK(cudaEventRecord(q->ev0, c->stream));
+    TRY(record_begin(c, q));
     TRY(E->rows_launch());
     CK(cudaEventRecord(q->ev1, c->stream));
     q->state = WG_RUNNING;
@@ -1735,7 +1743,7 @@ static int single_start(wg_ctx* c, Query* q) {
   TRY(E->ensure(wantC, wantF, 0, false));
   TRY(E->admit(0, Rl, q->kind, q->opts.max_iters, 0));
   TRY(E->init_deltas(0, 1));
-  CK(cudaEventRecord(q->ev0, c->stream));
+  TRY(record_begin(c, q));
   if (q->opts.profile) {
     // profiled run: host loop with CUDA events around every stage kernel
     for (;;) {
@@ -3192,7 +3200,7 @@ static int solo_resume(wg_ctx* c, Query* q) {
 static void solo_requeue(wg_ctx* c, Query* q) {
   if (q->own) c->idle.push_back(std::move(q->own));  // its pools may be dropped meanwhile
   q->eng = nullptr;
-  q->solo_wait = false;
+  q->solo_wait = q->begun = false;
   q->state = WG_PENDING;
   q->regrows += 1;
   c->pending.insert(c->pending.begin(), q->id);
