@@ -1101,15 +1101,15 @@ struct Engine : EngineBase {
     g_rows = (int)std::min<uint64_t>(
         grid_of(c, occ_rows(c, row_sg, id_bytes, words)),
         std::max<uint32_t>(nv, 1));
-    // control block | chunk sums | log | same-generation: masks, marks (cleared) |
+    // control block | chunk sums | same-generation: masks, marks | log (all cleared) |
     // instance | chunk offsets | row counts | row lists
     auto at = [](size_t& o, size_t b) { const size_t r = o; o += round_up(b); return r; };
     size_t end = 0;
     const size_t o_ctl = at(end, sizeof(RowCtl) + sizeof(SgCtl)), o_sum = at(end, (size_t)nch * 4),
-                 o_log = at(end, (size_t)nlog * 8), masks = row_sg ? Rl->sg_masks() : 0,
+                 masks = row_sg ? Rl->sg_masks() : 0,
                  o_fm = at(end, masks), o_dm0 = at(end, masks), o_dm1 = at(end, masks),
                  o_act = at(end, row_sg ? (size_t)nv * 4 : 0),
-                 o_done = at(end, row_sg ? (size_t)nv * 4 : 0);
+                 o_done = at(end, row_sg ? (size_t)nv * 4 : 0), o_log = at(end, (size_t)nlog * 8);
     row_clear = end;
     row_ctl = o_sum;
     const size_t o_inst = at(end, sizeof(RowInst)), o_sgi = at(end, sizeof(SgInst)),

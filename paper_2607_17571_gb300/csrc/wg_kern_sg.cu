@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
   unsigned long long cand = 0, got = 0;
   uint32_t cur = 0xFFFFFFFFu;
   SgCtl* ctl = J.ctl;
+  bool hubs = false;  // some row has several slices
   for (uint32_t k = 0;; ++k) {
     auto flush = [&]() {  // the counters of the current instance and iteration
       for (int o = 16; o > 0; o >>= 1) {
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
     const uint32_t in = k & 1, out = in ^ 1u;
     const uint32_t first = k == 0 ? J.rows.nrows : 0u;  // (all rows, before what is listed)
     const uint32_t n = first + __ldcg(&ctl->count[k % 3]);
+    if (k == 0) hubs = n > first;
     uint32_t* const next_n = &ctl->count[(k + 1) % 3];
     if (blockIdx.x == 0 && tid == 0) {  // (the slots no CTA uses in this iteration)
       ctl->count[(k + 2) % 3] = 0;
@@ -304,9 +306,14 @@ __global__ void __launch_bounds__(kSgThreads, 16) k_sg(SgJob J) {
       // without asking; one of several once per iteration
       for (uint32_t c = tid; c < kids; c += kSgThreads) {
         if (!(s_kids[c >> 5] >> (c & 31) & 1u)) continue;
-        const uint32_t x = __ldg(adj + c0 + c), b = __ldg(I.off + x), e = __ldg(I.off + x + 1);
+        const uint32_t x = __ldg(adj + c0 + c);
+        uint32_t s = 1;
+        if (hubs) s = sg_slices(__ldg(I.off + x + 1) - __ldg(I.off + x));
         if (bit_of(I.mp, x) && atomicExch(G.act + x, k + 1) == k + 1) continue;
-        const uint32_t s = sg_slices(e - b);
+        if (s == 1) {
+          to_list[atomicAdd(next_n, 1u)] = uint2{I.row0 + x, 0};
+          continue;
+        }
         uint2* to = to_list + atomicAdd(next_n, s);
         for (uint32_t i = 0; i < s; ++i) to[i] = uint2{I.row0 + x, i};
       }
